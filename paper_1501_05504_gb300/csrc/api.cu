@@ -72,6 +72,10 @@ dmrg3s_status upload_plan(Plan&& host, std::unique_ptr<DevicePlan>* out) {
                  bytes_of(h.g12.tc.segs) + bytes_of(h.g12.tc.packA) + bytes_of(h.g12.tc.packB) +
                  bytes_of(h.g1.tc.cta_start) + bytes_of(h.g3s.tc.cta_start) +
                  bytes_of(h.g12.tc.cta_start);
+  for (const SlStage* q : {&h.s12, &h.s3})
+    total += bytes_of(q->segs) + bytes_of(q->units) + bytes_of(q->chunks) + bytes_of(q->words) +
+             bytes_of(q->cta_unit) + bytes_of(q->cta_chunk) + bytes_of(q->gA) + bytes_of(q->gB) + bytes_of(q->mA) + bytes_of(q->mB);
+  total += bytes_of(h.s3r.chunks) + bytes_of(h.s3r.tasks) + bytes_of(h.s3r.terms);
   if (total == 0) total = 256;
   if (cudaMalloc(&dp->mem, total) != cudaSuccess) return DMRG3S_ERR_CUDA;
   std::vector<char> staging(total, 0);
@@ -107,11 +111,91 @@ dmrg3s_status upload_plan(Plan&& host, std::unique_ptr<DevicePlan>* out) {
   dp->c3r_chunks = place(base, &off, h.c3r.chunks, &staging);
   dp->c3r_tasks = place(base, &off, h.c3r.tasks, &staging);
   dp->c3r_terms = place(base, &off, h.c3r.terms, &staging);
+  auto place_sliced = [&](DevicePlan::Sliced* d, const SlStage& q) {
+    d->segs = place(base, &off, q.segs, &staging);
+    d->units = place(base, &off, q.units, &staging);
+    d->chunks = place(base, &off, q.chunks, &staging);
+    d->words = place(base, &off, q.words, &staging);
+    d->cta_unit = place(base, &off, q.cta_unit, &staging);
+    d->cta_chunk = place(base, &off, q.cta_chunk, &staging);
+    d->gA = place(base, &off, q.gA, &staging);
+    d->gB = place(base, &off, q.gB, &staging);
+    d->mA = place(base, &off, q.mA, &staging);
+    d->mB = place(base, &off, q.mB, &staging);
+  };
+  place_sliced(&dp->s12, h.s12);
+  place_sliced(&dp->s3, h.s3);
+  dp->s3r_chunks = place(base, &off, h.s3r.chunks, &staging);
+  dp->s3r_tasks = place(base, &off, h.s3r.tasks, &staging);
+  dp->s3r_terms = place(base, &off, h.s3r.terms, &staging);
   if (cudaMemcpy(dp->mem, staging.data(), total, cudaMemcpyHostToDevice) != cudaSuccess)
     return DMRG3S_ERR_CUDA;
   *out = std::move(dp);
   return DMRG3S_OK;
 }
+
+namespace {
+SlTables tables(const DevicePlan::Sliced& d, const SlStage& s) {
+  return SlTables{d.units,    d.chunks, d.words, d.cta_unit, d.cta_chunk, d.segs,
+                  s.cta_unit.empty() ? 0 : (int)s.cta_unit.size() - 1};
+}
+
+// FP64 by exact FP16 slices (kernels_sliced.cu): slice the operands, stages
+// 1 + 2 in one grouped GEMM, slice T2, stage 3 (split-K: partials and sum).
+dmrg3s_status run_sliced(Context* c, const DevicePlan& p, const double* g1A, const double* g1B,
+                         double* out2, double scale, const double* g3A, const double* g3B,
+                         double* g3C, cudaStream_t st, const SplitHints& hn) {
+  const Plan& h = p.host;
+  Profiler& pr = c->prof;
+  const SlSlots sl = sl_slots(h);
+  double* base = reinterpret_cast<double*>(c->ws);
+  auto pk = [&](int64_t slot) { return reinterpret_cast<uint16_t*>(base + slot); };
+  int32_t* e1A = reinterpret_cast<int32_t*>(base + sl.e);
+  int32_t* e1B = e1A + h.s12.neA;
+  int32_t* e3A = e1B + h.s12.neB;
+  int32_t* e3B = e3A + h.s3.neA;
+  const bool left = h.kind == Kind::Heff || h.kind == Kind::ExpandLR || h.kind == Kind::EnvLR;
+  double* t2 = h.has_g3 ? base + sl.t2 : out2;
+  if (!hn.g1A)
+    launch_slice(p.s12.gA, (int)h.s12.gA.size(), h.s12.ctasA, p.s12.mA, g1A, pk(sl.a1), e1A,
+                 left ? scale : 1.0, st);
+  if (!hn.g1B)
+    launch_slice(p.s12.gB, (int)h.s12.gB.size(), h.s12.ctasB, p.s12.mB, g1B, pk(sl.b1), e1B,
+                 left ? 1.0 : scale, st);
+  if (!h.s12.units.empty()) {
+    const int id = pr.on ? pr.begin(kProfGemm, h.f12.flops, h.f12.bytes, st) : -1;
+    launch_gemm_sliced(tables(p.s12, h.s12), hn.s1A ? hn.s1A : pk(sl.a1), pk(sl.b1),
+                       hn.s1A ? hn.e1A : e1A, e1B, g1A, g1B, h.f12.ta, h.f12.tb, scale, t2,
+                       c->d_err, c->wait_ns, st);
+    if (id >= 0) pr.end(id, st);
+  }
+  if (h.has_g3) {
+    const bool t2_is_a = h.kind == Kind::Heff;
+    const double* a3 = t2_is_a ? t2 : g3A;
+    const double* b3 = t2_is_a ? g3B : t2;
+    if (t2_is_a || !hn.g3A)
+      launch_slice(p.s3.gA, (int)h.s3.gA.size(), h.s3.ctasA, p.s3.mA, a3, pk(sl.a3), e3A, 1.0, st);
+    if (!t2_is_a || !hn.g3B)
+      launch_slice(p.s3.gB, (int)h.s3.gB.size(), h.s3.ctasB, p.s3.mB, b3, pk(sl.b3), e3B, 1.0, st);
+    const bool split = !h.s3r.chunks.empty();
+    double* c3 = split ? base + sl.p3 : g3C;
+    if (!h.s3.units.empty()) {
+      const int id = pr.on ? pr.begin(kProfGemm, h.g3.flops, h.g3.bytes, st) : -1;
+      launch_gemm_sliced(tables(p.s3, h.s3), pk(sl.a3), hn.s3B ? hn.s3B : pk(sl.b3), e3A,
+                         hn.s3B ? hn.e3B : e3B, a3, b3, h.f3.ta, h.f3.tb, 1.0, c3, c->d_err,
+                         c->wait_ns, st);
+      if (id >= 0) pr.end(id, st);
+    }
+    if (split) {
+      const int id = pr.on ? pr.begin(kProfCombine, 0.0, 0.0, st) : -1;
+      launch_combine_f64(p.s3r_chunks, (int)h.s3r.chunks.size(), p.s3r_tasks, p.s3r_terms, c3, g3C,
+                         1.0, st);
+      if (id >= 0) pr.end(id, st);
+    }
+  }
+  return cudaGetLastError() == cudaSuccess ? DMRG3S_OK : DMRG3S_ERR_CUDA;
+}
+}  // namespace
 
 dmrg3s_status run_plan(Context* c, const DevicePlan& p, const double* g1A, const double* g1B,
                        double* ws1, double* c2out, double c2scale, const double* g3A,
@@ -120,7 +204,11 @@ dmrg3s_status run_plan(Context* c, const DevicePlan& p, const double* g1A, const
   const Plan& h = p.host;
   Profiler& pr = c->prof;
   const int passes = prec == DMRG3S_TF32X3 ? 3 : prec == DMRG3S_TF32 ? 1 : 0;
+  const SplitHints none;
+  const SplitHints& hn = hints ? *hints : none;
   if (!passes) {
+    if (hn.f64 == kF64Sliced || (hn.f64 == kF64Auto && sliced_fits(h, c->ws_bytes)))
+      return run_sliced(c, p, g1A, g1B, c2out, c2scale, g3A, g3B, g3C, st, hn);
     if (!h.g1.tiles.empty()) {
       const int id = pr.on ? pr.begin(kProfGemm, h.g1.flops, h.g1.bytes, st) : -1;
       launch_gemm_f64(h.g1.ta, h.g1.tb, p.g1_tiles, (int)h.g1.tiles.size(), p.g1_tasks,
@@ -148,8 +236,6 @@ dmrg3s_status run_plan(Context* c, const DevicePlan& p, const double* g1A, const
   auto lo = [&](int64_t slot, int64_t n) {
     return passes == 3 ? reinterpret_cast<float*>(base + slot) + n : nullptr;
   };
-  const SplitHints none;
-  const SplitHints& hn = hints ? *hints : none;
   // the tensor-core stages write double-float pairs (8 bytes per element, in
   // place of the FP64 intermediates), combined on the FP32 pipe
   float2* t1p = reinterpret_cast<float2*>(ws1);

@@ -49,6 +49,19 @@ struct DevicePlan {
   CombTerm* c3r_terms = nullptr;
   GemmTask* g3_tasks = nullptr;
   GemmSeg* g3_segs = nullptr;
+  // sliced FP64 form: stages 1 + 2, stage 3, the sum of its partials
+  struct Sliced {
+    SlSeg* segs = nullptr;
+    SlUnit* units = nullptr;
+    SlChunk* chunks = nullptr;
+    uint32_t* words = nullptr;
+    int32_t *cta_unit = nullptr, *cta_chunk = nullptr;
+    SlGroup *gA = nullptr, *gB = nullptr;
+    SlMember *mA = nullptr, *mB = nullptr;
+  } s12, s3;
+  CombChunk* s3r_chunks = nullptr;
+  CombTask* s3r_tasks = nullptr;
+  CombTerm* s3r_terms = nullptr;
   ~DevicePlan();
 };
 
@@ -229,7 +242,14 @@ struct SplitHints {
   // H_eff only: packed L (stage-1 A) and R (stage-3 B) held outside the
   // workspace (a prepared operator); when set they replace those slots
   const float *g1A_hi = nullptr, *g1A_lo = nullptr, *g3B_hi = nullptr, *g3B_lo = nullptr;
+  // FP64: which form runs (kF64Auto: sliced when the plan has it and its
+  // intermediates fit the workspace), and, H_eff only, sliced L and R held
+  // outside the workspace with their row scales
+  int f64 = 0;
+  const uint16_t *s1A = nullptr, *s3B = nullptr;
+  const int32_t *e1A = nullptr, *e3B = nullptr;
 };
+constexpr int kF64Auto = 0, kF64Plain = 1, kF64Sliced = 2;
 struct TcSlots {
   int64_t t2p, a1, b1, x3, p3, end;   // offsets in doubles from the workspace start
 };
@@ -247,7 +267,29 @@ inline TcSlots tc_slots(const Plan& p) {
   s.end = s.p3 + slot_round(p.ws3);
   return s;
 }
-// Workspace (in doubles) a plan needs in the given precision.
+// Sliced FP64 mode:
+//   [T2][s12 A][s12 B][s3 A][s3 B][row scales: s12 A, s12 B, s3 A, s3 B][stage-3 partials]
+// (offsets in doubles, 1 KB aligned; without stage 3 the output is not here).
+struct SlSlots {
+  int64_t t2, a1, b1, a3, b3, e, p3, end;
+};
+inline SlSlots sl_slots(const Plan& p) {
+  SlSlots s;
+  s.t2 = 0;
+  s.a1 = slot_round(p.has_g3 ? p.ws2 : 0);
+  s.b1 = s.a1 + slot_round((p.s12.nA + 3) / 4);
+  s.a3 = s.b1 + slot_round((p.s12.nB + 3) / 4);
+  s.b3 = s.a3 + slot_round((p.s3.nA + 3) / 4);
+  s.e = s.b3 + slot_round((p.s3.nB + 3) / 4);
+  s.p3 = s.e + slot_round(((int64_t)p.s12.neA + p.s12.neB + p.s3.neA + p.s3.neB + 1) / 2);
+  s.end = s.p3 + slot_round(p.ws3s);
+  return s;
+}
+inline bool sliced_fits(const Plan& p, size_t ws_bytes) {
+  return p.sliced && (size_t)sl_slots(p).end * sizeof(double) <= ws_bytes;
+}
+// Workspace (in doubles) a plan needs at least in the given precision (FP64:
+// the plain form; the sliced one runs where it fits).
 inline int64_t plan_ws_doubles(const Plan& p, dmrg3s_precision prec) {
   return prec == DMRG3S_FP64 ? p.ws1 + p.ws2 : tc_slots(p).end;
 }

@@ -68,6 +68,20 @@ dmrg3s_status lanczos_batch(Context* c, const DevicePlan& heff, const double* Ld
   // from, several elements per thread
   lz_layout(ranges, plan_ctas(), &hch, &hcn);
   const int nchunks = (int)hch.size();
+  // FP64 products in the sliced form when the Krylov basis fits behind its
+  // intermediates, else in the plain form (the caller's cursor)
+  SplitHints hints;
+  if (prec == DMRG3S_FP64) {
+    const size_t after = (size_t)sl_slots(heff.host).end * sizeof(double);
+    const size_t krylov = sizeof(double) * ((size_t)ldv * (kp + 2) + (size_t)nchunks * kp * 2 +
+                                            (size_t)nchunks * (kLzLag + 1) + (size_t)np * kp * 2 +
+                                            (size_t)np * kp * kp) +
+                          sizeof(TridiagOut) * (size_t)np * kp + sizeof(LzChunk) * (size_t)nchunks +
+                          (sizeof(LzChain) + sizeof(int32_t)) * (size_t)np + 14 * 256;
+    const bool sl = heff.host.sliced && after + krylov <= c->ws_bytes;
+    hints.f64 = sl ? kF64Sliced : kF64Plain;
+    if (sl) cursor = after;
+  }
   void *pV, *pw, *pvc, *ppart, *pnp, *palpha, *pbeta, *py, *pout, *pch, *pcn, *pks, *pk;
   dmrg3s_status s;
   if ((s = carve(c, &cursor, sizeof(double) * ldv * kp, &pV)) ||
@@ -110,7 +124,18 @@ dmrg3s_status lanczos_batch(Context* c, const DevicePlan& heff, const double* Ld
   double* ws1 = reinterpret_cast<double*>(c->ws);
   double* ws2 = ws1 + heff.host.ws1;
   // tensor-core products: pack the environments once for the whole run
-  SplitHints hints;
+  if (hints.f64 == kF64Sliced) {
+    const Plan& hp = heff.host;
+    const SlSlots sl = sl_slots(hp);
+    int32_t* e = reinterpret_cast<int32_t*>(ws1 + sl.e);
+    launch_slice(heff.s12.gA, (int)hp.s12.gA.size(), hp.s12.ctasA, heff.s12.mA, Ldata,
+                 reinterpret_cast<uint16_t*>(ws1 + sl.a1), e, 1.0, st);
+    launch_slice(heff.s3.gB, (int)hp.s3.gB.size(), hp.s3.ctasB, heff.s3.mB, Rdata,
+                 reinterpret_cast<uint16_t*>(ws1 + sl.b3),
+                 e + hp.s12.neA + hp.s12.neB + hp.s3.neA, 1.0, st);
+    hints.g1A = true;
+    hints.g3B = true;
+  }
   if (prec != DMRG3S_FP64) {
     const Plan& hp = heff.host;
     const TcSlots sl = tc_slots(hp);

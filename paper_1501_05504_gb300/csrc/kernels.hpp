@@ -88,6 +88,84 @@ struct PackOut {
   int32_t R8, KC, trans, tile0;
 };
 
+// ---- FP64 products by exact FP16 slices (kernels_sliced.cu) ----
+// A sliced operand block (R rows x K) is stored in tiles of 8 rows x 64 k of
+// FP16 digits, one tile per slice: tile (chunk c, slice i, row group g) at
+// element offset dst + ((c * kSlices + i) * R8 + g) * kSlTile, with R8 the row
+// groups rounded up to an even number (so that a tile column is a multiple of
+// 16 columns of an MMA).  A tile is one 1 KB atom of the K-major 128-byte
+// swizzled layout: row r % 8 is a 128-byte line (64 k), its 16-byte piece j =
+// (k % 64) / 8 at position j ^ (r % 8).
+constexpr int kSlices = 7;
+constexpr int kSlTile = 512;               // FP16 elements of a tile
+constexpr int32_t kSlSpecial = 0x40000000; // row scale of a row with Inf or NaN
+// One block of a scale group: element (r, k) is coef * src[src + r ld + k]
+// (trans = 0) or coef * src[src + k ld + r] (trans = 1).
+struct SlMember {
+  int64_t src, dst;
+  double coef;
+  int32_t ld, K, KC, trans;
+};
+// Blocks with the same rows whose rows share scales: scales[e0 + r]; one CTA
+// of the slicing kernel per row group, from cta0 on.
+// `shift` raises the scales by that power of two: headroom of the integer sums.
+struct SlGroup {
+  int32_t R, R8, m0, nm, e0, cta0, shift;
+};
+// Spans a unit may sum before the headroom has to grow (the levels of a span
+// stay below 2^58.1 in the 64-bit sum).
+constexpr int kSlSpans = 28;
+// One K-segment of a task where its FP64 operands are (read for rows with Inf
+// or NaN only); GemmTask / GemmSeg order.
+struct SlSeg {
+  int64_t offA, offB;
+  double scale;
+  int32_t lda, ldb, K, pad;
+};
+// One output tile of up to 128 rows x tile_n columns (rows and cols: what lies
+// inside the block), written at C + offC with leading dimension ldc; row scales
+// of A from ea, column scales of B from eb; spans accumulation spans.
+// m0, n0: its place in the task (for rows with Inf or NaN).
+struct SlUnit {
+  int64_t offC;
+  int32_t ldc, rows, cols, nw, spans, ea, eb, m0, n0, seg0, nseg, pad;
+};
+// The units' 64-wide k-chunks in the order a CTA runs them.  The copies: slice
+// i of A is `ga` tiles at a + i sa, slice j of B `gb` tiles at b + j sb (FP16
+// elements); `word` is the MMA issuer's view: kSlSteps = its k16 steps (1-4),
+// kSlFirst / kSlLast = first / last chunk of a span (at most 64 k),
+// kSlLongFirst / kSlLongLast = of a long span (four spans, levels 4-6), kSlMove
+// = the accumulators' columns move (another nw than the chunk before), and nw
+// from bit kSlNw on.
+struct SlChunk {
+  int64_t a, b;
+  int32_t sa, sb;
+  int32_t ga, gb;
+};
+constexpr uint32_t kSlSteps = 7, kSlFirst = 8, kSlLast = 16, kSlLongFirst = 32, kSlLongLast = 64,
+                   kSlMove = 128, kSlNw = 8;
+constexpr int kSlLongSpan = 4;
+// Row scales and slices of every block of the groups (`scale` multiplies every
+// coefficient).  nctas: the sum of the groups' R8.
+void launch_slice(const SlGroup* groups, int ngroups, int nctas, const SlMember* members,
+                  const double* src, uint16_t* out, int32_t* scales, double scale, cudaStream_t st);
+// C = sum over the task's segments of op(A) op(B), one rounding to FP64 (see
+// kernels_sliced.cu).  CTA b runs units [cta_unit[b], cta_unit[b + 1]) and
+// chunks [cta_chunk[b], cta_chunk[b + 1]).  A, B, ta, tb, scale, segs: the FP64
+// operands, read for rows with Inf or NaN only.
+struct SlTables {
+  const SlUnit* units;
+  const SlChunk* chunks;
+  const uint32_t* words;
+  const int32_t *cta_unit, *cta_chunk;
+  const SlSeg* segs;
+  int ncta;
+};
+void launch_gemm_sliced(const SlTables& t, const uint16_t* pA, const uint16_t* pB,
+                        const int32_t* eA, const int32_t* eB, const double* A, const double* B,
+                        Trans ta, Trans tb, double scale, double* C, int* err, uint64_t wait_ns,
+                        cudaStream_t st);
+
 // Blockwise inner products: out[task.out] = sum over the task's segments of
 // <A[offA .. offA+len), B[offB .. offB+len)> (FP64, fixed summation order).
 struct DotSeg {

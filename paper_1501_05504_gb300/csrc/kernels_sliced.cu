@@ -1,0 +1,765 @@
+// FP64 block products on the tensor cores: operands cut into exact FP16 slices
+// (the splitting of Ozaki, Ogita, Oishi and Rump, 2012, with the integer slices
+// that Mukunoki, Ozaki, Ogita and Imamura, 2020, run on tensor cores).
+//
+// Every row of a packed operand (an output row of A, an output column of B)
+// carries one power-of-two scale over the whole contracted index; relative to
+// it an element is a 62-bit fixed-point number v (|v| <= 2^62, rounded to
+// nearest), written in seven balanced digits of 9 bits,
+//   v = sum_i q_i 2^(54 - 9 i),   -256 <= q_i <= 256,
+// each exact in FP16.  With both operands sliced,
+//   C = 2^(scales) sum_l 2^(108 - 9 l) S_l,   S_l = sum_{i + j = l} A_i B_j,
+// and the 28 digit products of the levels l = 0 .. 6 are formed (levels >= 7
+// lie below 2^-62 of the row scales).  One S_l collects at most 64 k before
+// it is drained, so |S_l| <= (l + 1) 64 2^16: levels 0-3 are exact integers in
+// the FP32 accumulators (<= 2^24), levels 4-6 carry weights below 2^-36.  The
+// drained levels 0-3 are summed exactly in a 64-bit integer (H; the row scales
+// leave it room for the task's spans); levels 4-6 run on for 256 k, level 4 then
+// joins H and levels 5-6 are summed in FP32 (L: 2^-24 of weights below 2^-45),
+// and the output is H 2^18 + L rounded once to FP64 with integer instructions.
+// Besides that rounding only the slices' own (2^-63 of the row scale) enters an
+// output element, however long its contraction.
+//
+// Why: GB300 multiplies FP64 at 2 multiply-adds per SM and clock (1.1 TFLOP/s
+// measured) and FP16 with FP32 accumulation at ~1700 times that, so 28 exact
+// products cost less than a sixtieth of one FP64 product.
+//
+// Kernel: persistent CTAs (one per SM, 576 threads) over output tiles of
+// 128 x 64.  The seven levels are seven accumulators of nw <= 64 columns side
+// by side in tensor memory, and the B slices lie back to back in shared
+// memory, so digit A_i meets the slices B_0 .. B_(6-i) in MMAs of up to 256
+// columns (one issue serves up to four digit products, and the A digit is read
+// from shared memory once for all of them).  A tile of 128 x 128 would need 896
+// tensor-memory columns of the 512.
+//   warp 0     one lane issues the bulk copies: the seven B slices of a 64-wide
+//              k-chunk in one of two 56 KB buffers, the A slices through a ring
+//              of 16 KB slabs
+//   warp 1     one lane issues tcgen05.mma (kind::f16); level l is committed to
+//              its own barrier right after digit A_l, while the later digits
+//              still run
+//   warps 2-17 drain: 32 rows x 16 columns each, H and L in registers
+// Every wait is bounded as in the other tensor-core kernel.
+#include <atomic>
+#include <cstdint>
+
+#include "kernels.hpp"
+#include "tc_common.cuh"
+
+namespace dmrg3s {
+
+namespace {
+
+constexpr int kFirstDrainWarp = 2, kDrainWarps = 16;
+constexpr int kThreads = 32 * (kFirstDrainWarp + kDrainWarps);
+constexpr int kSlabA = 16384;                          // 128 rows x 64 k of one slice
+constexpr int kSlots = 5;                              // A ring
+constexpr int kBufB = kSlices * 8192;                  // 64 columns x 64 k of all slices
+constexpr int kOffA = 2 * kBufB;
+constexpr int kOffStage = kOffA + kSlots * kSlabA;
+constexpr int kStageRow = 5;                           // doubles per staged row (4 + 1 pad)
+constexpr int kStageWarp = 32 * kStageRow * 8;
+constexpr int kSmemBytes = kOffStage + kDrainWarps * kStageWarp;
+constexpr uint32_t kTmemCols = 512;
+// A drained level is turned into an integer by an FP32 addition (the low bits
+// of x + 1.5 2^23 are x + 2^22; a conversion instruction takes 8 cycles a warp
+// and sub-partition, the addition one).  Two levels of at most 2^21 make one
+// unsigned 32-bit word, (a + 2^21) 512 + b + (the bits of 1.5 2^23), so H grows
+// by kBiasH per span, and by kBiasOne per long span, besides the levels; larger
+// levels (possible, but far outside what rounding digits give) take the
+// conversion.
+constexpr unsigned long long kBiasOne = 0x4B400000ull;
+constexpr unsigned long long kBiasPair = (2097152ull << 9) + kBiasOne;
+constexpr unsigned long long kBiasH = (kBiasPair << 27) + (kBiasPair << 9);
+
+// Instruction descriptor of kind::f16: D = F32, A = B = F16, both K-major.
+__device__ __forceinline__ uint32_t idesc_f16(uint32_t n) {
+  return (1u << 4) | ((n >> 3) << 17) | ((128u >> 4) << 24);
+}
+
+// Lower word of the shared-memory descriptor (smem_desc) of an address; the
+// upper word is the same for all.  A K step of 16 (32 bytes) adds 2.
+__device__ __forceinline__ uint32_t desc_lo(uint32_t addr) { return ((addr >> 4) & 0x3FFF) | (1u << 16); }
+constexpr uint32_t kDescHi = 64u | (1u << 14) | (2u << 29);
+__device__ __forceinline__ uint64_t desc(uint32_t lo) { return ((uint64_t)kDescHi << 32) | lo; }
+
+__device__ __forceinline__ bool elect_one() {
+  uint32_t r;
+  asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n" : "=r"(r));
+  return r != 0;
+}
+
+__device__ __forceinline__ void mma_f16(uint32_t dtmem, uint64_t ad, uint64_t bd, uint32_t idesc,
+                                        uint32_t acc) {
+  asm volatile(
+      "{\n .reg .pred p;\n setp.ne.u32 p, %4, 0;\n"
+      " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(dtmem),
+      "l"(ad), "l"(bd), "r"(idesc), "r"(acc)
+      : "memory");
+}
+
+// ks MMAs of 16 k each from one pair of slabs (acc: whether the first adds).
+__device__ __forceinline__ void mma_steps(uint32_t d, uint32_t a, uint32_t b, uint32_t idesc, int ks,
+                                          uint32_t acc) {
+  if (ks == 4) {
+    mma_f16(d, desc(a), desc(b), idesc, acc);
+    mma_f16(d, desc(a + 2), desc(b + 2), idesc, 1u);
+    mma_f16(d, desc(a + 4), desc(b + 4), idesc, 1u);
+    mma_f16(d, desc(a + 6), desc(b + 6), idesc, 1u);
+  } else {
+    for (int kk = 0; kk < ks; ++kk) mma_f16(d, desc(a + 2 * kk), desc(b + 2 * kk), idesc, kk ? 1u : acc);
+  }
+}
+
+// Loads of 8 columns (32 lanes); several in flight before one wait.
+__device__ __forceinline__ void tmem_ld8_async(uint32_t taddr, uint32_t* v) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+               : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]),
+                 "=r"(v[6]), "=r"(v[7])
+               : "r"(taddr));
+}
+// Waits for the loads; v passes through it, so that no use moves before it.
+__device__ __forceinline__ void tmem_wait_ld(uint32_t (&v)[16]) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;"
+               : "+r"(v[0]), "+r"(v[1]), "+r"(v[2]), "+r"(v[3]), "+r"(v[4]), "+r"(v[5]),
+                 "+r"(v[6]), "+r"(v[7]), "+r"(v[8]), "+r"(v[9]), "+r"(v[10]), "+r"(v[11]),
+                 "+r"(v[12]), "+r"(v[13]), "+r"(v[14]), "+r"(v[15])::"memory");
+}
+
+// (H 2^14 + L) 2^(ex + 4) rounded to the nearest FP64 value: 32-bit integer
+// instructions on the 96-bit sum (an FP64 conversion or addition holds GB300's
+// FP64 unit for 64 cycles a warp), without branches, so that several elements
+// are in flight.  (A negative sum is complemented, one unit below its
+// magnitude: 2^-66 of the scales.)  Sets `out` when the result needs the
+// general form below: exponent outside the normal range, or no bit above the
+// last 32 of the 96.
+__device__ __forceinline__ double fixed_to_f64(long long H, int L, int ex, bool* out) {
+  const uint32_t h0 = (uint32_t)H, h1 = (uint32_t)((unsigned long long)H >> 32);
+  uint32_t x0 = h0 << 14, x1 = __funnelshift_l(h0, h1, 14), x2 = (uint32_t)((int32_t)h1 >> 18);
+  asm("add.cc.u32 %0, %0, %3;\n\taddc.cc.u32 %1, %1, %4;\n\taddc.u32 %2, %2, %4;"
+      : "+r"(x0), "+r"(x1), "+r"(x2)
+      : "r"(L), "r"(L >> 31));
+  const uint32_t s = (uint32_t)((int32_t)x2 >> 31);
+  x0 ^= s;
+  x1 ^= s;
+  x2 ^= s;
+  const bool z = x2 == 0;                           // the leading limb first
+  const uint32_t y2 = z ? x1 : x2, y1 = z ? x0 : x1, y0 = z ? 0u : x0;
+  uint32_t lz;
+  asm("bfind.shiftamt.u32 %0, %1;" : "=r"(lz) : "r"(y2));
+  const uint32_t w1 = __funnelshift_l(y1, y2, lz), w0 = __funnelshift_l(y0, y1, lz);
+  uint32_t r0, r1, c;
+  asm("add.cc.u32 %0, %3, 0x400;\n\taddc.cc.u32 %1, %4, 0;\n\taddc.u32 %2, 0, 0;"
+      : "=r"(r0), "=r"(r1), "=r"(c)
+      : "r"(w0), "r"(w1));
+  // exponent field less one: the leading bit of r1 >> 11 adds it (it is gone
+  // when the rounding carried out)
+  const int f = ex + (4 + 95 + 1022) - (z ? 32 : 0) - (int)lz + 2 * (int)c;
+  const bool zero = (y2 | y1) == 0;
+  *out = *out || (!zero && ((uint32_t)f >= 2045u || y2 == 0));
+  const uint32_t hi = ((r1 >> 11) + ((uint32_t)f << 20)) | (s & 0x80000000u);
+  return __hiloint2double((int)(zero ? 0u : hi), (int)(zero ? 0u : __funnelshift_r(r0, r1, 11)));
+}
+
+// The same sum, (H 2^18 + L) 2^ex, for any range, in FP64 arithmetic.
+__device__ __noinline__ double fixed_to_f64_any(long long H, float L, int ex) {
+  const long long l = __float2ll_rn(L);
+  const long long h = H + (l >> 18);
+  const double top = (double)(h >> 32) * 4294967296.0, low = (double)(h & 0xFFFFFFFFll);
+  return ldexp(fma(top + low, 262144.0, (double)(l & 0x3FFFF)), ex);
+}
+
+// One output element the plain way (rows or columns with Inf or NaN).
+__device__ __noinline__ double element_f64(const SlSeg* __restrict__ segs, int nseg,
+                                           const double* __restrict__ A,
+                                           const double* __restrict__ B, int ta, int tb, int m,
+                                           int n, double scale) {
+  double acc = 0.0;
+  for (int k = 0; k < nseg; ++k) {
+    const SlSeg s = segs[k];
+    double part = 0.0;
+    for (int q = 0; q < s.K; ++q) {
+      const double a = ta ? A[s.offA + (int64_t)q * s.lda + m] : A[s.offA + (int64_t)m * s.lda + q];
+      const double b = tb ? B[s.offB + (int64_t)n * s.ldb + q] : B[s.offB + (int64_t)q * s.ldb + n];
+      part = fma(a, b, part);
+    }
+    acc = fma(s.scale, part, acc);
+  }
+  return scale * acc;
+}
+
+__global__ void __launch_bounds__(kThreads, 1)
+    gemm_sliced_kernel(const SlTables tab, const uint16_t* __restrict__ pA,
+                       const uint16_t* __restrict__ pB, const int32_t* __restrict__ eA,
+                       const int32_t* __restrict__ eB, const double* __restrict__ A,
+                       const double* __restrict__ B, int ta, int tb, double scale,
+                       double* __restrict__ C, int* __restrict__ err, uint64_t wait_ns) {
+  extern __shared__ __align__(1024) unsigned char smem[];
+  __shared__ __align__(8) uint64_t afull[kSlots], aempty[kSlots], bfull[2], bempty[2];
+  __shared__ __align__(8) uint64_t lfull[kSlices], lempty[kSlices], done;
+  __shared__ uint32_t tmem_base;
+  __shared__ volatile int abort_flag;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+
+  if (tid == 0) {
+    for (int s = 0; s < kSlots; ++s) {
+      mbar_init(&afull[s], 1);
+      mbar_init(&aempty[s], 1);
+    }
+    for (int s = 0; s < 2; ++s) {
+      mbar_init(&bfull[s], 1);
+      mbar_init(&bempty[s], 1);
+    }
+    for (int l = 0; l < kSlices; ++l) {
+      mbar_init(&lfull[l], 1);
+      mbar_init(&lempty[l], kDrainWarps);
+    }
+    mbar_init(&done, 1);
+    abort_flag = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                     smem_u32(&tmem_base)),
+                 "r"(kTmemCols)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const uint32_t tmem = tmem_base;
+  const WaitCtl wc{&abort_flag, err, wait_ns};
+
+  if (warp == 0) {
+    // ---------------- bulk-copy producer ----------------
+    if (lane == 0) {
+      const int c_end = tab.cta_chunk[blockIdx.x + 1];
+      int ci = tab.cta_chunk[blockIdx.x];
+      uint32_t qa = 0, bf = 0;               // A slabs and B buffers filled
+      SlChunk next{};
+      if (ci < c_end) next = tab.chunks[ci];
+      for (bool ok = true; ci < c_end && ok; ++ci) {
+        const SlChunk ch = next;
+        if (ci + 1 < c_end) next = tab.chunks[ci + 1];
+        const int bs = (int)(bf & 1);
+        if (bf >= 2 && !mbar_wait(&bempty[bs], ((bf >> 1) - 1) & 1, wc)) break;
+        unsigned char* bb = smem + bs * kBufB;
+        mbar_expect_tx(&bfull[bs], (uint32_t)(kSlices * ch.gb) * 1024u);
+        if (ch.gb * kSlTile == ch.sb) {      // all slices of the chunk are contiguous
+          bulk_g2s(bb, pB + ch.b, (uint32_t)(kSlices * ch.gb) * 1024u, &bfull[bs]);
+        } else {
+          for (int j = 0; j < kSlices; ++j)
+            bulk_g2s(bb + j * ch.gb * 1024, pB + ch.b + (int64_t)j * ch.sb, (uint32_t)ch.gb * 1024u,
+                     &bfull[bs]);
+        }
+        ++bf;
+        for (int i = 0; i < kSlices; ++i, ++qa) {
+          const int st = (int)(qa % kSlots);
+          if (qa >= (uint32_t)kSlots && !mbar_wait(&aempty[st], ((qa / kSlots) - 1) & 1, wc)) {
+            ok = false;
+            break;
+          }
+          mbar_expect_tx(&afull[st], (uint32_t)ch.ga * 1024u);
+          bulk_g2s(smem + kOffA + st * kSlabA, pA + ch.a + (int64_t)i * ch.sa,
+                   (uint32_t)ch.ga * 1024u, &afull[st]);
+        }
+      }
+      // copies still in flight must land before the CTA's memory is released:
+      // the last phase of every slot and buffer that was filled
+      for (uint32_t s = 0; s < (uint32_t)kSlots; ++s) {
+        const uint32_t n = qa > s ? (qa - s + kSlots - 1) / kSlots : 0;
+        if (n) mbar_drain(&afull[s], (n - 1) & 1);
+      }
+      for (uint32_t s = 0; s < 2; ++s) {
+        const uint32_t n = bf > s ? (bf - s + 1) / 2 : 0;
+        if (n) mbar_drain(&bfull[s], (n - 1) & 1);
+      }
+    }
+    __syncwarp();
+  } else if (warp == 1) {
+    // ---------------- MMA issuer ----------------
+    // the whole warp walks the chunks and one elected lane issues: the operands
+    // of tcgen05.mma sit in uniform registers, and inside a branch of a single
+    // known lane moving them there costs ~150 cycles an MMA instead of ~44.  The
+    // next slab's barrier is tested while this one's MMAs are issued, and the
+    // chunk words are read one ahead.
+    const bool one = elect_one();
+    const int c_end = tab.cta_chunk[blockIdx.x + 1];
+    int ci = tab.cta_chunk[blockIdx.x];
+    uint32_t slot = 0, aph = 0, bs = 0, bph = 0;
+    uint32_t ph = 0, pl = 0;             // spans (levels 0-3), long spans (levels 4-6)
+    uint32_t next = ci < c_end ? tab.words[ci] : 0u;
+    const uint32_t s0 = smem_u32(smem);
+    const uint32_t tmem_u = __reduce_or_sync(0xffffffffu, tmem);
+    bool ok = true;
+    bool b_ready = false, a_ready = false;
+    // levels [l0, l1) drained since their last commit
+    auto drained = [&](int l0, int l1, uint32_t n) {
+      bool w = true;
+      for (int l = l0; l < l1 && w; ++l) w = mbar_wait(&lempty[l], (n - 1) & 1, wc);
+      return __all_sync(0xffffffffu, w) != 0;
+    };
+    for (; ci < c_end && ok; ++ci) {
+      const uint32_t w = __reduce_or_sync(0xffffffffu, next);   // in a uniform register
+      if (ci + 1 < c_end) next = tab.words[ci + 1];
+      const uint32_t nw = w >> kSlNw;
+      const int ks = (int)(w & kSlSteps);
+      if (!__all_sync(0xffffffffu, b_ready) &&
+          !__all_sync(0xffffffffu, mbar_wait(&bfull[bs], bph, wc)))
+        break;
+      const uint32_t sb = desc_lo(s0 + bs * kBufB);
+      if ((w & kSlFirst) && ph > 0) {
+        // levels 0-3 (after a change of nw, which moves the levels' columns: all)
+        ok = drained(0, 4, ph) && (!(w & kSlMove) || pl == 0 || drained(4, kSlices, pl));
+        if (!ok) break;
+      }
+#pragma unroll
+      for (int i = 0; i < kSlices; ++i) {
+        if (!__all_sync(0xffffffffu, a_ready) &&
+            !__all_sync(0xffffffffu, mbar_wait(&afull[slot], aph, wc))) {
+          ok = false;
+          break;
+        }
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        const uint32_t sa = desc_lo(s0 + kOffA + slot * kSlabA);
+        const uint32_t cur = slot;
+        if (++slot == kSlots) {
+          slot = 0;
+          aph ^= 1;
+        }
+        a_ready = mbar_test(&afull[slot], aph);
+        // B slices 0 .. 6 - i in one MMA, or in two when they are more than 256
+        // columns (the first digit always: its levels 4-6 are drained later)
+        const uint32_t all = (uint32_t)(7 - i);
+        const uint32_t n1 = i == 0 ? 4u : (i < 3 && all * nw > 256u) ? 3u : all;
+        const bool two = i < 3 && n1 < all;
+        const bool wait2 = i == 0 && (w & kSlLongFirst) && pl > 0;
+        if (wait2) {
+          if (one)
+            mma_steps(tmem_u, sa, sb, idesc_f16(n1 * nw), ks, (w & kSlFirst) ? 0u : 1u);
+          __syncwarp();
+          if (!drained(4, kSlices, pl)) {
+            ok = false;
+            break;
+          }
+          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        }
+        if (one) {
+          if (!wait2)
+            mma_steps(tmem_u + (uint32_t)i * nw, sa, sb, idesc_f16(n1 * nw), ks,
+                      (i == 0 && (w & kSlFirst)) ? 0u : 1u);
+          if (two)
+            mma_steps(tmem_u + ((uint32_t)i + n1) * nw, sa, sb + n1 * nw * 8u,
+                      idesc_f16((all - n1) * nw), ks, (i == 0 && (w & kSlLongFirst)) ? 0u : 1u);
+          mma_commit(&aempty[cur]);
+          if (w & (i < 4 ? kSlLast : kSlLongLast)) mma_commit(&lfull[i]);   // level i is complete
+          if (i == kSlices - 1) mma_commit(&bempty[bs]);
+        }
+        __syncwarp();
+      }
+      if (!ok) break;
+      if (w & kSlLast) ++ph;
+      if (w & kSlLongLast) ++pl;
+      bs ^= 1;
+      if (bs == 0) bph ^= 1;
+      b_ready = ci + 1 < c_end && mbar_test(&bfull[bs], bph);
+    }
+    // every product issued must finish before the tensor memory is freed
+    if (one) {
+      mma_commit(&done);
+      mbar_drain(&done, 0);
+    }
+    __syncwarp();
+  } else {
+    // ---------------- drain and epilogue ----------------
+    // 16 warps (four per scheduler hide the tensor memory's latency), each the
+    // 32 rows of its quarter and 16 columns
+    const int quarter = warp & 3, part = (warp - kFirstDrainWarp) >> 2;
+    const uint32_t tcol = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(part * 16);
+    double* stage =
+        reinterpret_cast<double*>(smem + kOffStage + (warp - kFirstDrainWarp) * kStageWarp);
+    uint32_t ph = 0, pl = 0;
+    bool ok = true;
+    const int u_end = tab.cta_unit[blockIdx.x + 1];
+    for (int u = tab.cta_unit[blockIdx.x]; u < u_end && ok; ++u) {
+      const SlUnit& un = tab.units[u];
+      if (u + 1 < u_end)
+        asm volatile("prefetch.global.L1 [%0];" ::"l"(reinterpret_cast<const char*>(&tab.units[u + 1]) + lane * 2));
+      const uint32_t nw = (uint32_t)un.nw;
+      const int spans = un.spans;
+      // (a warp beyond the tile only arrives)
+      const bool mine = (uint32_t)(part * 16) < nw && quarter * 32 < un.rows;
+      unsigned long long H[16];                          // levels 0-4, biased
+      float L[16];                                       // levels 5-6, FP32
+#pragma unroll
+      for (int j = 0; j < 16; ++j) {
+        H[j] = 0;
+        L[j] = 0.f;
+      }
+      const int row0 = quarter * 32, row = row0 + lane, n0 = part * 16;
+      // (rows and columns of the padding get a scale in the normal range)
+      const int fa = row < un.rows && spans > 0 ? eA[un.ea + row] : 1057;
+      const int fb_lane = lane < 16 && n0 + lane < un.cols && spans > 0 ? eB[un.eb + n0 + lane] : 1057;
+      for (int sp = 0; sp < spans && ok; ++sp, ++ph) {
+        const bool longer = sp % kSlLongSpan == kSlLongSpan - 1 || sp == spans - 1;
+#pragma unroll
+        for (int l = 0; l < 4; l += 2) {                 // levels (0, 1), (2, 3)
+          // one decision per warp: tcgen05.ld is a warp-wide instruction
+          if (!__all_sync(0xffffffffu, mbar_wait(&lfull[l + 1], ph & 1, wc))) {
+            ok = false;
+            break;
+          }
+          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+          if (mine) {
+#pragma unroll
+            for (int h = 0; h < 16; h += 8) {
+              uint32_t v[16];
+              tmem_ld8_async(tcol + (uint32_t)l * nw + h, v);
+              tmem_ld8_async(tcol + (uint32_t)(l + 1) * nw + h, v + 8);
+              tmem_wait_ld(v);
+              float m = 0.f;
+#pragma unroll
+              for (int j = 0; j < 8; ++j)
+                m = fmaxf(m, fmaxf(fabsf(__uint_as_float(v[j])), fabsf(__uint_as_float(v[8 + j]))));
+              if (!__any_sync(0xffffffffu, !(m < 2097152.f))) {
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                  const uint32_t w =
+                      __float_as_uint(__fadd_rn(__uint_as_float(v[j]), 10485760.f)) * 512u +
+                      __float_as_uint(__fadd_rn(__uint_as_float(v[8 + j]), 12582912.f));
+                  H[h + j] += (unsigned long long)w * (l == 0 ? 134217728u : 512u);
+                }
+              } else {
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                  const long long a = (long long)__float2int_rn(__uint_as_float(v[j])) * 512 +
+                                      __float2int_rn(__uint_as_float(v[8 + j]));
+                  H[h + j] += ((unsigned long long)a + kBiasPair) * (l == 0 ? 134217728u : 512u);
+                }
+              }
+            }
+          }
+          asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+          __syncwarp();
+          if (lane == 0) {
+            mbar_arrive(&lempty[l]);
+            mbar_arrive(&lempty[l + 1]);
+          }
+        }
+        if (!ok || !longer) continue;
+#pragma unroll
+        for (int l = 4; l < kSlices; ++l) {
+          if (!__all_sync(0xffffffffu, mbar_wait(&lfull[l], pl & 1, wc))) {
+            ok = false;
+            break;
+          }
+          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+          if (mine) {
+            uint32_t v[16];
+            tmem_ld8_async(tcol + (uint32_t)l * nw, v);
+            tmem_ld8_async(tcol + (uint32_t)l * nw + 8, v + 8);
+            tmem_wait_ld(v);
+            if (l == 4) {
+              float m = 0.f;
+#pragma unroll
+              for (int j = 0; j < 16; ++j) m = fmaxf(m, fabsf(__uint_as_float(v[j])));
+              if (!__any_sync(0xffffffffu, !(m < 4194304.f))) {
+#pragma unroll
+                for (int j = 0; j < 16; ++j)
+                  H[j] += __float_as_uint(__fadd_rn(__uint_as_float(v[j]), 12582912.f));
+              } else {
+#pragma unroll
+                for (int j = 0; j < 16; ++j)
+                  H[j] += (unsigned long long)(long long)__float2int_rn(__uint_as_float(v[j])) + kBiasOne;
+              }
+            } else {
+#pragma unroll
+              for (int j = 0; j < 16; ++j)
+                L[j] = __fmaf_rn(__uint_as_float(v[j]), l == 5 ? 512.f : 1.f, L[j]);
+            }
+          }
+          asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&lempty[l]);
+        }
+        ++pl;
+      }
+      if (!ok) break;
+      if (!mine) continue;
+      // rows of 4 consecutive doubles through the warp's staging rows
+      const unsigned long long bh =
+          (unsigned long long)spans * kBiasH +
+          (unsigned long long)((spans + kSlLongSpan - 1) / kSlLongSpan) * kBiasOne;
+      const int rows = un.rows, cols = un.cols;
+      double* Cu = C + un.offC + n0;
+      const int64_t ldc = un.ldc;
+      // (the vote first: every lane takes part in it)
+      const bool special_col = __any_sync(0xffffffffu, fb_lane == kSlSpecial);
+      const bool special = special_col || fa == kSlSpecial;
+#pragma unroll
+      for (int c4 = 0; c4 < 16; c4 += 4) {
+        if (n0 + c4 >= cols) break;
+        bool out = false;                    // of this lane's elements inside the tile
+        int ex[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const float lf = L[c4 + i];
+          bool o = !(fabsf(lf) < 17179869184.f);           // 2^34: the range of the conversion
+          ex[i] = fa + __shfl_sync(0xffffffffu, fb_lane, c4 + i) - 2114;
+          stage[lane * kStageRow + i] =
+              fixed_to_f64((long long)(H[c4 + i] - bh), __float2int_rn(lf * 0.0625f), ex[i], &o);
+          out = out || (o && row < rows && n0 + c4 + i < cols);
+        }
+        if (out)
+#pragma unroll
+          for (int i = 0; i < 4; ++i)
+            stage[lane * kStageRow + i] =
+                fixed_to_f64_any((long long)(H[c4 + i] - bh), L[c4 + i], ex[i]);
+        __syncwarp();
+#pragma unroll
+        for (int it = 0; it < 4; ++it) {
+          const int r = it * 8 + (lane >> 2), cc = lane & 3;
+          if (row0 + r < rows && n0 + c4 + cc < cols)
+            Cu[(row0 + r) * ldc + c4 + cc] = stage[r * kStageRow + cc];
+        }
+        __syncwarp();
+      }
+      // rows and columns with Inf or NaN (their slices are zero): the FP64 sum
+      if (special && row < rows) {
+        for (int j = 0; j < 16 && n0 + j < cols; ++j)
+          if (fa == kSlSpecial || eB[un.eb + n0 + j] == kSlSpecial)
+            Cu[row * ldc + j] = element_f64(tab.segs + un.seg0, un.nseg, A, B, ta, tb, un.m0 + row,
+                                            un.n0 + n0 + j, scale);
+      }
+      __syncwarp();
+    }
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  if (warp == 1)
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem),
+                 "r"(kTmemCols)
+                 : "memory");
+}
+
+// ---- slicing -----------------------------------------------------------------------
+// One CTA per 8 rows of a scale group (the packed blocks that share row
+// scales): the largest exponent of every row over all blocks of the group,
+// then the slices.  A warp handles 8 rows x 64 k of one block at a time, lane
+// l row l / 4 and the 16-byte pieces l % 4 and l % 4 + 4 (8 k each); the
+// elements of a warp's first tile stay in registers between the two passes,
+// any further tile is read again (from L2).  Integer arithmetic only: the
+// significand is shifted to the row scale and cut into digits.
+
+// Significand and exponent field of coef * x: |coef x| = m 2^(f - 1075)
+// (m < 2^53) when the coefficient is a power of two, else m 2^(f - 1086)
+// with m < 2^64 (the upper 64 bits of the product of the significands).
+struct Coef {
+  unsigned long long m;   // significand << 11
+  int f;                  // exponent field
+  bool pow2, neg, bad;
+};
+__device__ __forceinline__ Coef make_coef(double c) {
+  Coef r;
+  const unsigned long long b = (unsigned long long)__double_as_longlong(c);
+  int f = (int)((b >> 52) & 0x7FF);
+  unsigned long long m = b & 0xFFFFFFFFFFFFFull;
+  r.neg = (b >> 63) != 0;
+  r.bad = f == 0x7FF;
+  if (f) m |= 1ull << 52;
+  else f = 1;
+  r.pow2 = m == (1ull << 52);
+  r.m = m << 11;
+  r.f = f;
+  return r;
+}
+
+// Effective exponent field of coef * x (see slice digits); kMin for a zero.
+constexpr int kMinField = -1000000;
+__device__ __forceinline__ int eff_field(double x, const Coef& c) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+  const int f = (int)((b >> 52) & 0x7FF);
+  if (f == 0x7FF) return kSlSpecial;
+  if ((b << 1) == 0ull) return kMinField;
+  return (f ? f : 1) + c.f - (c.pow2 ? 1023 : 1022);
+}
+
+// The seven digits of coef * x relative to the row field F, biased by 256 each
+// and packed in one 64-bit word (digit i in bits 54 - 9 i ..; digit 0 takes 10).
+__device__ __forceinline__ unsigned long long digits(double x, const Coef& c, int F) {
+  constexpr unsigned long long kBias = (256ull << 54) | (256ull << 45) | (256ull << 36) |
+                                       (256ull << 27) | (256ull << 18) | (256ull << 9) | 256ull;
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+  int f = (int)((b >> 52) & 0x7FF);
+  unsigned long long m = b & 0xFFFFFFFFFFFFFull;
+  if (f) m |= 1ull << 52;
+  else f = 1;
+  unsigned long long t;
+  int s;
+  if (c.pow2) {
+    t = m << 9;
+    s = F - (f + c.f - 1023);
+  } else {
+    t = __umul64hi(m << 11, c.m);
+    s = F - (f + c.f - 1022) + 2;
+  }
+  unsigned long long v = 0;
+  if (s <= 0) v = t;
+  else if (s < 64) v = (t >> s) + ((t >> (s - 1)) & 1ull);   // to nearest, half away from zero
+  const bool neg = ((b >> 63) != 0) != c.neg;
+  return kBias + (neg ? 0ull - v : v);
+}
+
+__global__ void __launch_bounds__(256)
+    slice_kernel(const SlGroup* __restrict__ groups, int ngroups, const SlMember* __restrict__ members,
+                 const double* __restrict__ src, uint16_t* __restrict__ out,
+                 int32_t* __restrict__ scales, double scale) {
+  __shared__ int smax[8];
+  int gi = 0;
+  {
+    int lo = 0, hi = ngroups - 1;
+    const int b = (int)blockIdx.x;
+    while (lo < hi) {
+      const int mid = (lo + hi + 1) >> 1;
+      if (groups[mid].cta0 <= b) lo = mid;
+      else hi = mid - 1;
+    }
+    gi = lo;
+  }
+  const SlGroup gr = groups[gi];
+  const int g = (int)blockIdx.x - gr.cta0;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int rr = lane >> 2, j4 = lane & 3, r = g * 8 + rr;
+  if (threadIdx.x < 8) smax[threadIdx.x] = kMinField;
+  __syncthreads();
+  auto load = [&](const SlMember& mb, int c, double (&x)[16]) {
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        const int k = c * 64 + (j4 + 4 * h) * 8 + q;
+        double v = 0.0;
+        if (r < gr.R && k < mb.K)
+          v = mb.trans ? src[mb.src + (int64_t)k * mb.ld + r] : src[mb.src + (int64_t)r * mb.ld + k];
+        x[h * 8 + q] = v;
+      }
+  };
+  double keep[16];
+  int kept_m = -1, kept_c = -1;
+  int mx = kMinField;
+  {
+    // tiles (member, chunk) of the group, warp-strided
+    int t = warp;
+    for (int m = 0; m < gr.nm; ++m) {
+      const SlMember mb = members[gr.m0 + m];
+      if (t >= mb.KC) {
+        t -= mb.KC;
+        continue;
+      }
+      const Coef cf = make_coef(mb.coef * scale);
+      for (; t < mb.KC; t += 8) {
+        double x[16];
+        load(mb, t, x);
+        if (cf.bad) mx = kSlSpecial;
+#pragma unroll
+        for (int e = 0; e < 16; ++e) mx = max(mx, eff_field(x[e], cf));
+        if (kept_m < 0) {
+          kept_m = m;
+          kept_c = t;
+#pragma unroll
+          for (int e = 0; e < 16; ++e) keep[e] = x[e];
+        }
+      }
+      t -= mb.KC;
+    }
+  }
+  mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
+  mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
+  if (j4 == 0) atomicMax(&smax[rr], mx);
+  __syncthreads();
+  const int F = smax[rr] + gr.shift;
+  if (threadIdx.x < 8 && g * 8 + (int)threadIdx.x < gr.R) {
+    const int v = smax[threadIdx.x];
+    scales[gr.e0 + g * 8 + threadIdx.x] = v == kMinField ? 0 : v == kSlSpecial ? v : v + gr.shift;
+  }
+  const bool zero = smax[rr] == kMinField || smax[rr] == kSlSpecial;
+  int t = warp;
+  for (int m = 0; m < gr.nm; ++m) {
+    const SlMember mb = members[gr.m0 + m];
+    if (t >= mb.KC) {
+      t -= mb.KC;
+      continue;
+    }
+    const Coef cf = make_coef(mb.coef * scale);
+    for (; t < mb.KC; t += 8) {
+      double x[16];
+      if (m == kept_m && t == kept_c) {
+#pragma unroll
+        for (int e = 0; e < 16; ++e) x[e] = keep[e];
+      } else {
+        load(mb, t, x);
+      }
+      uint16_t* base = out + mb.dst + ((int64_t)t * kSlices * gr.R8 + g) * kSlTile + rr * 64;
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        uint32_t w[kSlices][4];
+#pragma unroll
+        for (int q = 0; q < 8; q += 2) {
+          const unsigned long long d0 = digits(zero ? 0.0 : x[h * 8 + q], cf, zero ? 0 : F);
+          const unsigned long long d1 = digits(zero ? 0.0 : x[h * 8 + q + 1], cf, zero ? 0 : F);
+#pragma unroll
+          for (int i = 0; i < kSlices; ++i) {
+            // digit + 256 in 0 .. 512: as FP16, 1024 + (digit + 256) has these
+            // bits exactly; one packed subtraction of 1280 leaves the digits
+            const uint32_t f0 = (uint32_t)(d0 >> (54 - 9 * i)) & (i == 0 ? 0x3FFu : 0x1FFu);
+            const uint32_t f1 = (uint32_t)(d1 >> (54 - 9 * i)) & (i == 0 ? 0x3FFu : 0x1FFu);
+            const uint32_t hw = (f0 | (f1 << 16)) | 0x64006400u;
+            uint32_t res;
+            asm("sub.rn.f16x2 %0, %1, %2;" : "=r"(res) : "r"(hw), "r"(0x65006500u));
+            w[i][q >> 1] = res;
+          }
+        }
+        const int pos = ((j4 + 4 * h) ^ rr) << 3;       // swizzled 16-byte piece
+#pragma unroll
+        for (int i = 0; i < kSlices; ++i)
+          *reinterpret_cast<uint4*>(base + (int64_t)i * gr.R8 * kSlTile + pos) =
+              make_uint4(w[i][0], w[i][1], w[i][2], w[i][3]);
+      }
+    }
+    t -= mb.KC;
+  }
+}
+
+}  // namespace
+
+void launch_slice(const SlGroup* groups, int ngroups, int nctas, const SlMember* members,
+                  const double* src, uint16_t* out, int32_t* scales, double scale, cudaStream_t st) {
+  if (nctas <= 0) return;
+  count_launch();
+  slice_kernel<<<nctas, 256, 0, st>>>(groups, ngroups, members, src, out, scales, scale);
+}
+
+void launch_gemm_sliced(const SlTables& t, const uint16_t* pA, const uint16_t* pB,
+                        const int32_t* eA, const int32_t* eB, const double* A, const double* B,
+                        Trans ta, Trans tb, double scale, double* C, int* err, uint64_t wait_ns,
+                        cudaStream_t st) {
+  if (t.ncta <= 0) return;
+  // the shared-memory limit is a per-device attribute of the kernel
+  static std::atomic<uint64_t> done{0};
+  int dev = 0;
+  cudaGetDevice(&dev);
+  const uint64_t bit = dev >= 0 && dev < 64 ? (1ull << dev) : 0ull;
+  if (!bit || !(done.load() & bit)) {
+    cudaFuncSetAttribute(gemm_sliced_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         kSmemBytes);
+    if (bit) done.fetch_or(bit);
+  }
+  count_launch();
+  gemm_sliced_kernel<<<t.ncta, kThreads, kSmemBytes, st>>>(t, pA, pB, eA, eB, A, B,
+                                                           ta == Trans::T ? 1 : 0,
+                                                           tb == Trans::T ? 1 : 0, scale, C, err,
+                                                           wait_ns);
+}
+
+}  // namespace dmrg3s

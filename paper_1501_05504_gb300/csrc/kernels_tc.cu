@@ -49,6 +49,7 @@
 #include <cstdint>
 
 #include "kernels.hpp"
+#include "tc_common.cuh"
 
 namespace dmrg3s {
 
@@ -64,30 +65,7 @@ constexpr int kStageBytes = 4 * kSlab;              // A hi, A lo, B hi, B lo
 constexpr int kEpiRow = 9;                          // float2 per staged row (8 + 1 pad)
 constexpr int kEpiWarp = 4096;                      // bytes of one drain warp's staging (4 atoms)
 constexpr int kSmemBytes = kStages * kStageBytes + kDrainWarps * kEpiWarp;
-constexpr uint64_t kDrainLimitNs = 1000000000ull;   // waits for work already in flight
 constexpr int kSpanChunks = 4;                      // k-chunks per drain of the main accumulator
-
-__device__ __forceinline__ uint32_t smem_u32(const void* p) {
-  return (uint32_t)__cvta_generic_to_shared(p);
-}
-
-__device__ __forceinline__ uint64_t globaltimer() {
-  uint64_t t;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-  return t;
-}
-
-// Shared-memory matrix descriptor (tcgen05) of a K-major operand in the
-// 128-byte swizzled layout: start address >> 4, leading byte offset 16 (not
-// used by swizzled K-major layouts), stride byte offset 1024 (8-row atoms),
-// descriptor version 1, swizzle mode 2 (128 bytes) in bits 61-63.  The atoms
-// must start on 1 KB boundaries; a K step inside the 128-byte line advances
-// the start address (the hardware applies the swizzle to the full address).
-__device__ __forceinline__ uint64_t smem_desc(uint32_t addr) {
-  const uint64_t lbo = 16, sbo = 1024;
-  return (uint64_t)((addr >> 4) & 0x3FFF) | ((uint64_t)((lbo >> 4) & 0x3FFF) << 16) |
-         ((uint64_t)((sbo >> 4) & 0x3FFF) << 32) | (1ull << 46) | (2ull << 61);
-}
 
 // Instruction descriptor of kind::tf32: D = F32, A = B = TF32, both K-major,
 // N >> 3 at bit 17, M >> 4 at bit 24.
@@ -101,87 +79,6 @@ __device__ __forceinline__ float to_tf32(float x) {
   return __uint_as_float(r);
 }
 
-__device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count));
-}
-
-__device__ __forceinline__ bool mbar_try(uint64_t* bar, uint32_t parity) {
-  uint32_t done;
-  asm volatile(
-      "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
-      " selp.u32 %0, 1, 0, p;\n}\n"
-      : "=r"(done)
-      : "r"(smem_u32(bar)), "r"(parity)
-      : "memory");
-  return done != 0;
-}
-
-// Shared state of one CTA's bounded waits.
-struct WaitCtl {
-  volatile int* abort;
-  int* err;
-  uint64_t limit_ns;
-};
-
-// Waits for the phase of `bar` with the given parity.  Gives up when another
-// thread has aborted, or after limit_ns (then aborts the CTA itself).
-__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, const WaitCtl& w) {
-  if (mbar_try(bar, parity)) return true;
-  const uint64_t t0 = globaltimer();
-  for (;;) {
-    if (mbar_try(bar, parity)) return true;
-    if (*w.abort) return false;
-    if (globaltimer() - t0 > w.limit_ns) {
-      *w.abort = 1;
-      atomicExch(w.err, 1);
-      return false;
-    }
-  }
-}
-
-// Waits for work already in flight (copies, products) before the CTA exits:
-// ignores the abort flag, fixed limit.
-__device__ __forceinline__ bool mbar_drain(uint64_t* bar, uint32_t parity) {
-  const uint64_t t0 = globaltimer();
-  while (!mbar_try(bar, parity))
-    if (globaltimer() - t0 > kDrainLimitNs) return false;
-  return true;
-}
-
-__device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
-}
-
-__device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)),
-               "r"(bytes)
-               : "memory");
-}
-
-// Bulk copy global -> shared, completion counted on `bar` (16-byte aligned
-// addresses, size a multiple of 16).
-__device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
-  asm volatile(
-      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-          smem_u32(dst)),
-      "l"(src), "r"(bytes), "r"(smem_u32(bar))
-      : "memory");
-}
-
-// Bulk copy shared -> global (bulk-group completion), and its waits.
-__device__ __forceinline__ void bulk_s2g(void* dst, const void* src, uint32_t bytes) {
-  asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(dst),
-               "r"(smem_u32(src)), "r"(bytes)
-               : "memory");
-  asm volatile("cp.async.bulk.commit_group;" ::: "memory");
-}
-__device__ __forceinline__ void bulk_wait_read() {
-  asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
-}
-__device__ __forceinline__ void bulk_wait_all() {
-  asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
-}
-
 __device__ __forceinline__ void mma_tf32(uint32_t dtmem, uint64_t ad, uint64_t bd, uint32_t idesc,
                                          uint32_t acc) {
   asm volatile(
@@ -189,24 +86,6 @@ __device__ __forceinline__ void mma_tf32(uint32_t dtmem, uint64_t ad, uint64_t b
       " tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n}\n" ::"r"(dtmem),
       "l"(ad), "l"(bd), "r"(idesc), "r"(acc)
       : "memory");
-}
-
-__device__ __forceinline__ void mma_commit(uint64_t* bar) {
-  asm volatile(
-      "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-          smem_u32(bar))
-      : "memory");
-}
-
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&v)[16]) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,"
-      "%15}, [%16];"
-      : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]),
-        "=r"(v[7]), "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]),
-        "=r"(v[14]), "=r"(v[15])
-      : "r"(taddr));
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
 
 // Knuth's two-sum: (s, e) with s + e = a + b exactly.

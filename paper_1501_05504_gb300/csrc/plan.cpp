@@ -82,19 +82,11 @@ int plan_ctas() { return g_plan_ctas.load(); }
 namespace {
 
 // Static schedule of a stage's units over the persistent CTAs: longest
-// processing time first onto the least loaded CTA.  A unit's cost is its
-// k-chunks, each weighted 0.7 as a fixed share (the A slab's copy and the
-// issue latency, the same for every width) and 0.3 by its MMA width, plus a
-// fixed share for its drain and store.
-void schedule_units(TcStage& tc, const std::vector<GemmTask>& tasks) {
-  const int n = (int)tc.units.size();
+// processing time first onto the least loaded CTA.
+void schedule(std::vector<TcUnit>& units, std::vector<int32_t>& cta_start,
+              const std::vector<double>& cost) {
+  const int n = (int)units.size();
   const int nc = std::max(1, std::min(plan_ctas(), n));
-  std::vector<double> cost(n);
-  for (int i = 0; i < n; ++i) {
-    const TcUnit& u = tc.units[i];
-    const int nrem = std::min(128, tasks[u.task].N - u.tn * 128);
-    cost[i] = u.nchunks * (0.7 + 0.3 * (double)((nrem + 15) / 16 * 16) / 128.0) + 4.0;
-  }
   std::vector<int> order(n);
   for (int i = 0; i < n; ++i) order[i] = i;
   std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return cost[a] > cost[b]; });
@@ -107,13 +99,27 @@ void schedule_units(TcStage& tc, const std::vector<GemmTask>& tasks) {
   }
   std::vector<TcUnit> out;
   out.reserve(n);
-  tc.cta_start.assign(nc + 1, 0);
+  cta_start.assign(nc + 1, 0);
   for (int c = 0; c < nc; ++c) {
-    tc.cta_start[c] = (int32_t)out.size();
-    for (int i : lists[c]) out.push_back(tc.units[i]);
+    cta_start[c] = (int32_t)out.size();
+    for (int i : lists[c]) out.push_back(units[i]);
   }
-  tc.cta_start[nc] = (int32_t)out.size();
-  tc.units.swap(out);
+  cta_start[nc] = (int32_t)out.size();
+  units.swap(out);
+}
+
+// A 128 x 128 unit's cost is its k-chunks, each weighted 0.7 as a fixed share
+// (the A slab's copy and the issue latency, the same for every width) and 0.3
+// by its MMA width, plus a fixed share for its drain and store.
+void schedule_units(TcStage& tc, const std::vector<GemmTask>& tasks) {
+  const int n = (int)tc.units.size();
+  std::vector<double> cost(n);
+  for (int i = 0; i < n; ++i) {
+    const TcUnit& u = tc.units[i];
+    const int nrem = std::min(128, tasks[u.task].N - u.tn * 128);
+    cost[i] = u.nchunks * (0.7 + 0.3 * (double)((nrem + 15) / 16 * 16) / 128.0) + 4.0;
+  }
+  schedule(tc.units, tc.cta_start, cost);
 }
 
 using Key = std::array<int, 4>;
@@ -405,6 +411,277 @@ bool build_fused(Plan* p, const std::map<int64_t, CombPacked>& c2p, std::string*
   return true;
 }
 
+// ---- sliced FP64 form ----
+
+// Blocks of one operand of a stage, grouped by the tasks that use them: blocks
+// that meet in one task share their row scales.
+struct Slicer {
+  struct Blk {
+    SlMember m;
+    int32_t R, spans;      // spans: of the longest task that uses the block
+  };
+  std::vector<Blk> blks;
+  std::vector<int> parent;
+  std::map<std::pair<std::array<int64_t, 5>, double>, int> seen;   // (view, coef) -> block
+  int find(int i) {
+    while (parent[i] != i) i = parent[i] = parent[parent[i]];
+    return i;
+  }
+  int add(int64_t src, int64_t ld, int64_t R, int64_t K, int trans, double coef) {
+    const auto key = std::make_pair(std::array<int64_t, 5>{src, ld, R, K, trans}, coef);
+    auto it = seen.find(key);
+    if (it != seen.end()) return it->second;
+    Blk b{};
+    b.m.src = src;
+    b.m.coef = coef;
+    b.m.ld = (int32_t)ld;
+    b.m.K = (int32_t)K;
+    b.m.KC = (int32_t)((K + 63) / 64);
+    b.m.trans = trans;
+    b.R = (int32_t)R;
+    const int id = (int)blks.size();
+    blks.push_back(b);
+    parent.push_back(id);
+    seen[key] = id;
+    return id;
+  }
+  void join(int a, int b) {
+    a = find(a);
+    b = find(b);
+    if (a != b) parent[std::max(a, b)] = std::min(a, b);
+  }
+  static int32_t groups(int64_t R) { return (int32_t)((R + 15) / 16 * 2); }
+  // Places every block and group; e0[block] = first scale of its group.
+  void layout(bool headroom, std::vector<SlGroup>* g, std::vector<SlMember>* m, int64_t* n, int32_t* ctas,
+              int32_t* ne, std::vector<int32_t>* e0) {
+    std::map<int, std::vector<int>> by;
+    for (int i = 0; i < (int)blks.size(); ++i) by[find(i)].push_back(i);
+    e0->assign(blks.size(), 0);
+    for (const auto& kv : by) {
+      SlGroup gr{};
+      gr.R = blks[kv.first].R;
+      gr.R8 = groups(gr.R);
+      gr.m0 = (int32_t)m->size();
+      gr.nm = (int32_t)kv.second.size();
+      gr.e0 = *ne;
+      gr.cta0 = *ctas;
+      int spans = 0;
+      for (int i : kv.second) spans = std::max(spans, blks[i].spans);
+      while (headroom && spans > kSlSpans << gr.shift) ++gr.shift;
+      for (int i : kv.second) {
+        blks[i].m.dst = *n;
+        *n += (int64_t)gr.R8 * blks[i].m.KC * kSlices * kSlTile;
+        (*e0)[i] = gr.e0;
+        m->push_back(blks[i].m);
+      }
+      *ne += gr.R;
+      *ctas += gr.R8;
+      g->push_back(gr);
+    }
+  }
+};
+
+// Sliced form of a stage: GemmSeg.scale is the coefficient of A (coefA) or B.
+bool build_sliced(const GemmStage& g, bool coefA, SlStage* out, std::string* err) {
+  SlStage& s = *out;
+  s = SlStage();
+  Slicer a, b;
+  std::vector<int> ia(g.segs.size()), ib(g.segs.size());
+  for (const GemmTask& t : g.tasks) {
+    // at most this many spans (a span takes consecutive chunks up to 4 k16 steps)
+    int chunks = 0;
+    for (int k = 0; k < t.nseg; ++k) chunks += (g.segs[t.seg0 + k].K + 63) / 64;
+    for (int k = 0; k < t.nseg; ++k) {
+      const GemmSeg& q = g.segs[t.seg0 + k];
+      // A (rows M): ta = N stores M x K; B (rows N): tb = T stores N x K
+      ia[t.seg0 + k] = a.add(q.offA, q.lda, t.M, q.K, g.ta == Trans::T ? 1 : 0, coefA ? q.scale : 1.0);
+      ib[t.seg0 + k] = b.add(q.offB, q.ldb, t.N, q.K, g.tb == Trans::N ? 1 : 0, coefA ? 1.0 : q.scale);
+      a.blks[ia[t.seg0 + k]].spans = std::max(a.blks[ia[t.seg0 + k]].spans, chunks);
+      if (k) {
+        a.join(ia[t.seg0], ia[t.seg0 + k]);
+        b.join(ib[t.seg0], ib[t.seg0 + k]);
+      }
+    }
+  }
+  for (size_t i = 0; i < a.blks.size(); ++i)
+    if (a.blks[i].R != a.blks[a.find((int)i)].R) {
+      *err = "sliced stage: blocks of unequal rows share scales";
+      return false;
+    }
+  for (size_t i = 0; i < b.blks.size(); ++i)
+    if (b.blks[i].R != b.blks[b.find((int)i)].R) {
+      *err = "sliced stage: blocks of unequal rows share scales";
+      return false;
+    }
+  std::vector<int32_t> ea, eb;
+  a.layout(true, &s.gA, &s.mA, &s.nA, &s.ctasA, &s.neA, &ea);
+  b.layout(false, &s.gB, &s.mB, &s.nB, &s.ctasB, &s.neB, &eb);
+  for (const GemmSeg& q : g.segs) s.segs.push_back(SlSeg{q.offA, q.offB, q.scale, q.lda, q.ldb, q.K, 0});
+  // narrower units when the 64-wide ones leave SMs without work
+  auto count = [&](int tn) {
+    int64_t n = 0;
+    for (const GemmTask& t : g.tasks) n += (int64_t)((t.M + 127) / 128) * ((t.N + tn - 1) / tn);
+    return n;
+  };
+  int tile_n = 64;
+  while (tile_n > 16 && count(tile_n - 16) <= plan_ctas()) tile_n -= 16;
+  std::vector<TcUnit> units;
+  std::vector<double> cost;
+  for (const GemmTask& t : g.tasks) {
+    int steps = 0, chunks = 0;
+    for (int k = 0; k < t.nseg; ++k) {
+      steps += (g.segs[t.seg0 + k].K + 15) / 16;
+      chunks += (g.segs[t.seg0 + k].K + 63) / 64;
+    }
+    const int id = (int)(&t - g.tasks.data());
+    for (int i = 0; i < (t.M + 127) / 128; ++i)
+      for (int j = 0; j < (t.N + tile_n - 1) / tile_n; ++j) {
+        units.push_back(TcUnit{id, i, j, 0});
+        // cycles: 14 per column and k16 step of the 28 digit products, against
+        // the slabs' copies at ~48 B per cycle; then the drains and the store
+        const int nw = std::min(tile_n, (t.N + 15) / 16 * 16 - j * tile_n);
+        const int ga = std::min(16, Slicer::groups(t.M) - i * 16);
+        const double mma = 14.0 * nw * steps, copy = chunks * 7.0 * 1024.0 * (ga + nw / 8) / 48.0;
+        cost.push_back(std::max(std::max(mma, copy), 2200.0 * chunks) + 3000.0);
+      }
+  }
+  std::vector<int32_t> cta;
+  schedule(units, cta, cost);
+  // what each CTA runs: its units, and their chunks one after the other
+  s.cta_unit = cta;
+  s.cta_chunk.assign(cta.size(), 0);
+  for (size_t c = 0; c + 1 < cta.size(); ++c) {
+    s.cta_chunk[c] = (int32_t)s.chunks.size();
+    int prev_nw = 0;
+    for (int32_t ui = cta[c]; ui < cta[c + 1]; ++ui) {
+      const GemmTask& t = g.tasks[units[ui].task];
+      SlUnit un{};
+      un.m0 = units[ui].tm * 128;
+      un.n0 = units[ui].tn * tile_n;
+      un.offC = t.offC + (int64_t)un.m0 * t.ldc + un.n0;
+      un.ldc = t.ldc;
+      un.rows = std::min(128, t.M - un.m0);
+      un.cols = std::min(tile_n, t.N - un.n0);
+      un.nw = (un.cols + 15) / 16 * 16;
+      un.seg0 = t.seg0;
+      un.nseg = t.nseg;
+      if (t.nseg > 0) {
+        un.ea = ea[ia[t.seg0]] + un.m0;
+        un.eb = eb[ib[t.seg0]] + un.n0;
+      }
+      const int ra8 = Slicer::groups(t.M), rb8 = Slicer::groups(t.N);
+      const size_t first = s.words.size();
+      int used = 0;
+      for (int k = 0; k < t.nseg; ++k) {
+        const int k16 = (g.segs[t.seg0 + k].K + 15) / 16;
+        for (int q = 0; 4 * q < k16; ++q) {
+          const int ks = std::min(4, k16 - 4 * q);
+          uint32_t w = (uint32_t)ks | (uint32_t)un.nw << kSlNw;
+          // spans: consecutive chunks while their k16 steps sum to at most 4
+          if (s.words.size() == first || used + ks > 4) {
+            if (s.words.size() > first) s.words.back() |= kSlLast;
+            w |= kSlFirst;
+            if (un.spans % kSlLongSpan == 0) {
+              if (un.spans) s.words.back() |= kSlLongLast;
+              w |= kSlLongFirst;
+            }
+            ++un.spans;
+            used = 0;
+          }
+          if (s.words.size() == first && un.nw != prev_nw) w |= kSlMove;
+          used += ks;
+          s.words.push_back(w);
+          SlChunk ch{};
+          ch.sa = ra8 * kSlTile;
+          ch.sb = rb8 * kSlTile;
+          ch.a = a.blks[ia[t.seg0 + k]].m.dst + (int64_t)q * kSlices * ch.sa + (int64_t)(un.m0 / 8) * kSlTile;
+          ch.b = b.blks[ib[t.seg0 + k]].m.dst + (int64_t)q * kSlices * ch.sb + (int64_t)(un.n0 / 8) * kSlTile;
+          ch.ga = std::min(16, ra8 - un.m0 / 8);
+          ch.gb = un.nw / 8;
+          s.chunks.push_back(ch);
+        }
+      }
+      if (s.words.size() > first) {
+        s.words.back() |= kSlLast | kSlLongLast;
+        prev_nw = un.nw;
+      }
+      s.units.push_back(un);
+    }
+  }
+  if (!cta.empty()) s.cta_chunk.back() = (int32_t)s.chunks.size();
+  return true;
+}
+
+// Stages 1 + 2 as one grouped GEMM in FP64: one task per stage-2 block, one
+// K-segment per MPO term, scaled by its coefficient.
+bool fuse_f64(const Plan& p, GemmStage* out, std::string* err) {
+  std::map<int64_t, int> t1_task;      // T1 element offset -> stage-1 task
+  for (size_t i = 0; i < p.g1.tasks.size(); ++i) t1_task[p.g1.tasks[i].offC] = (int)i;
+  GemmStage& g = *out;
+  g = GemmStage();
+  g.ta = p.g1.ta;
+  g.tb = p.g1.tb;
+  for (const CombTask& ct : p.c2.tasks) {
+    GemmTask t{};
+    t.offC = ct.offOut;
+    t.ldc = ct.ldo;
+    t.M = ct.rows;
+    t.N = ct.cols;
+    t.seg0 = (int32_t)g.segs.size();
+    t.nseg = ct.nt;
+    for (int k = 0; k < ct.nt; ++k) {
+      const CombTerm& tm = p.c2.terms[ct.t0 + k];
+      auto jt = t1_task.find(tm.offIn);
+      if (jt == t1_task.end()) {
+        *err = "fused stage: MPO term without a stage-1 block";
+        return false;
+      }
+      const GemmTask& t1 = p.g1.tasks[jt->second];
+      if (t1.nseg != 1 || t1.M != ct.rows || t1.N != ct.cols) {
+        *err = "fused stage: stage-1 block shape";
+        return false;
+      }
+      GemmSeg q = p.g1.segs[t1.seg0];
+      q.scale = tm.coef;
+      g.segs.push_back(q);
+    }
+    g.tasks.push_back(t);
+  }
+  g.flops = p.g1.flops + p.c2.flops;   // algorithmic: the stages it replaces
+  g.bytes = p.g1.bytes + p.c2.bytes;
+  return true;
+}
+
+// Stage 3 in `groups` consecutive groups of K-segments per output block, each
+// into its own partial block (offsets from 0), and the sum of the partials.
+void split_k(const GemmStage& g3, int groups, GemmStage* parts, CombStage* sum, int64_t* n) {
+  parts->ta = g3.ta;
+  parts->tb = g3.tb;
+  int64_t poff = 0;
+  for (const GemmTask& t : g3.tasks) {
+    std::vector<CombTerm> terms;
+    const int ng = std::min<int>(groups, std::max(1, (int)t.nseg));
+    for (int gi = 0; gi < ng; ++gi) {
+      const int k0 = (int)((int64_t)t.nseg * gi / ng), k1 = (int)((int64_t)t.nseg * (gi + 1) / ng);
+      std::vector<GemmSeg> sg(g3.segs.begin() + t.seg0 + k0, g3.segs.begin() + t.seg0 + k1);
+      if (sg.empty() && t.nseg > 0) continue;
+      parts->add(poff, t.N, t.M, t.N, sg);
+      CombTerm tm{};
+      tm.offIn = poff;
+      tm.ldi = t.N;
+      tm.coef = 1.0;
+      terms.push_back(tm);
+      poff += (int64_t)t.M * t.N;
+    }
+    sum->add(t.offC, t.ldc, t.M, t.N, terms);
+  }
+  *n = poff;
+  parts->flops = g3.flops;        // same algorithmic work as stage 3
+  parts->bytes = g3.bytes;
+  sum->flops = 0.0;               // the partial sums are bookkeeping, not algorithm
+  sum->bytes = 0.0;
+}
+
 // Smaller combination chunks when a stage would have fewer than `target`
 // of them (small blocks: more CTAs, each with fewer rows).
 void rechunk(CombStage& c, int target) {
@@ -422,6 +699,53 @@ void rechunk(CombStage& c, int target) {
     for (int r = 0; r < rows; r += rpc)
       c.chunks.push_back(CombChunk{(int32_t)id, r, rows - r < rpc ? rows - r : rpc, 0});
   }
+}
+
+// Least algorithmic work of a contraction that takes the sliced form.
+constexpr double kSlicedMinFlops = 2e6;
+// Largest ratio of the fused stage's work to stage 1's: the sliced products
+// run ~15 times as fast as the plain ones; a model MPO has a ratio near 1.2.
+constexpr double kSlicedMaxTerms = 6.0;
+
+// The sliced FP64 form, where there is enough work for it.
+dmrg3s_status finish_sliced(Plan* p, int64_t nA1, int64_t nB1, int64_t nOut2, int64_t nA3,
+                            int64_t nB3, int64_t nC3, std::string* err) {
+  p->sliced = false;
+  if (p->flops() < kSlicedMinFlops) return DMRG3S_OK;
+  // a dense MPO tensor: too many terms per stage-1 block to form each anew
+  double terms = 0.0, blocks = 0.0;
+  for (const CombTask& t : p->c2.tasks) terms += (double)t.nt * t.rows * t.cols;
+  for (const GemmTask& t : p->g1.tasks) blocks += (double)t.M * t.N;
+  if (terms > kSlicedMaxTerms * blocks) return DMRG3S_OK;
+  const bool left = p->kind == Kind::Heff || p->kind == Kind::ExpandLR || p->kind == Kind::EnvLR;
+  bool ok = fuse_f64(*p, &p->f12, err) && build_sliced(p->f12, left, &p->s12, err) &&
+            sliced_ok(p->f12, p->s12, nA1, nB1, nOut2, err);
+  if (ok && p->has_g3) {
+    int64_t units1 = 0;
+    int maxseg = 1;
+    for (const GemmTask& t : p->g3.tasks) {
+      units1 += (int64_t)((t.M + 127) / 128) * ((t.N + 63) / 64);
+      maxseg = std::max(maxseg, (int)t.nseg);
+    }
+    int G = units1 > 0 ? (int)((kTargetUnits + units1 - 1) / units1) : 1;
+    G = std::max(1, std::min(G, maxseg));
+    if (G > 1) {
+      split_k(p->g3, G, &p->f3, &p->s3r, &p->ws3s);
+      rechunk(p->s3r, 2 * plan_ctas());
+      ok = comb_ok(p->s3r.tasks, p->s3r.terms, std::max<int64_t>(p->ws3s, 1), nC3, err);
+    } else {
+      p->f3 = p->g3;
+      p->f3.tiles.clear();
+    }
+    ok = ok && build_sliced(p->f3, true, &p->s3, err) &&
+         sliced_ok(p->f3, p->s3, nA3, nB3, G > 1 ? std::max<int64_t>(p->ws3s, 1) : nC3, err);
+  }
+  if (!ok) {
+    *err = "internal planning error: " + *err;
+    return DMRG3S_ERR_SHAPE;
+  }
+  p->sliced = true;
+  return DMRG3S_OK;
 }
 
 // Bounds of every table against the buffers the stages address.
@@ -445,32 +769,8 @@ dmrg3s_status finish(Plan* p, int64_t nA1, int64_t nB1, int64_t nOut2, int64_t n
     }
     int G = units1 > 0 ? (int)((kTargetUnits + units1 - 1) / units1) : 1;
     G = std::max(1, std::min(G, maxseg));
-    p->g3s.ta = p->g3.ta;
-    p->g3s.tb = p->g3.tb;
-    int64_t poff = 0;
-    for (const GemmTask& t : p->g3.tasks) {
-      std::vector<CombTerm> terms;
-      const int ng = std::min<int>(G, std::max(1, (int)t.nseg));
-      for (int gi = 0; gi < ng; ++gi) {
-        const int k0 = (int)((int64_t)t.nseg * gi / ng), k1 = (int)((int64_t)t.nseg * (gi + 1) / ng);
-        std::vector<GemmSeg> sg(p->g3.segs.begin() + t.seg0 + k0, p->g3.segs.begin() + t.seg0 + k1);
-        if (sg.empty() && t.nseg > 0) continue;
-        p->g3s.add(poff, t.N, t.M, t.N, sg);
-        CombTerm tm{};
-        tm.offIn = poff;
-        tm.ldi = t.N;
-        tm.coef = 1.0;
-        terms.push_back(tm);
-        poff += (int64_t)t.M * t.N;
-      }
-      p->c3r.add(t.offC, t.ldc, t.M, t.N, terms);
-    }
-    p->ws3 = poff;
-    p->g3s.flops = p->g3.flops;        // same algorithmic work as stage 3
-    p->g3s.bytes = p->g3.bytes;
-    p->c3r.flops = 0.0;                // the partial sums are bookkeeping, not algorithm
-    p->c3r.bytes = 0.0;
-    const int64_t w3 = poff > 0 ? poff : 1;
+    split_k(p->g3, G, &p->g3s, &p->c3r, &p->ws3);
+    const int64_t w3 = p->ws3 > 0 ? p->ws3 : 1;
     if (!gemm_ok(p->g3s.ta, p->g3s.tb, p->g3s.tasks, p->g3s.segs, nA3, nB3, w3, err) ||
         !comb_ok(p->c3r.tasks, p->c3r.terms, w3, nC3, err)) {
       *err = "internal planning error: " + *err;
@@ -514,7 +814,7 @@ dmrg3s_status finish(Plan* p, int64_t nA1, int64_t nB1, int64_t nOut2, int64_t n
   }
   rechunk(p->c2, 2 * plan_ctas());
   rechunk(p->c3r, 2 * plan_ctas());
-  return DMRG3S_OK;
+  return finish_sliced(p, nA1, nB1, nOut2, nA3, nB3, nC3, err);
 }
 
 }  // namespace

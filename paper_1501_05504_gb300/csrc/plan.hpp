@@ -41,6 +41,22 @@ struct TcStage {
   int32_t tilesA = 0, tilesB = 0;
 };
 
+// Sliced FP64 form of a grouped GEMM stage (kernels_sliced.cu): every packed
+// block belongs to a scale group (the blocks that meet in one task share the
+// scales of their rows), units are 128 x tile_n tiles.
+struct SlStage {
+  std::vector<SlSeg> segs;              // parallel to GemmStage::segs
+  std::vector<SlUnit> units;            // grouped by CTA
+  std::vector<SlChunk> chunks;          // grouped by CTA, in the order of its units
+  std::vector<uint32_t> words;          // one per chunk
+  std::vector<int32_t> cta_unit, cta_chunk;
+  std::vector<SlGroup> gA, gB;
+  std::vector<SlMember> mA, mB;
+  int64_t nA = 0, nB = 0;               // FP16 elements of each packed operand
+  int32_t ctasA = 0, ctasB = 0;         // CTAs of the slicing launches
+  int32_t neA = 0, neB = 0;             // row scales of each operand
+};
+
 struct GemmStage {
   Trans ta = Trans::N, tb = Trans::N;
   std::vector<GemmTask> tasks;
@@ -96,6 +112,16 @@ struct Plan {
   // never formed.  g12's A operand is the coefficient-scaled L blocks.
   GemmStage g12;
   bool fused = false;
+  // FP64 mode, sliced form (kernels_sliced.cu): stages 1 and 2 as one grouped
+  // GEMM over the MPO terms (f12: one task per stage-2 block, one K-segment per
+  // term, scaled by its coefficient; the output is the stage-2 output in FP64),
+  // stage 3 split-K into FP64 partial blocks and a sum (no split: written to
+  // the output directly).  sliced = false: too little work (plan.cpp).
+  GemmStage f12, f3;
+  SlStage s12, s3;
+  CombStage s3r;                // sum of the partials (empty: no split)
+  int64_t ws3s = 0;             // doubles of the partial blocks
+  bool sliced = false;
   double flops() const { return g1.flops + c2.flops + (has_g3 ? g3.flops : 0.0); }
 };
 

@@ -127,6 +127,101 @@ inline bool tc_ok(const std::vector<GemmTask>& tasks, const TcStage& tc, int64_t
   return true;
 }
 
+// Sliced FP64 tables: every source view, packed block, row scale, bulk copy and
+// output inside its array.
+inline bool slices_ok(const std::vector<SlGroup>& g, const std::vector<SlMember>& m, int64_t nSrc,
+                      int64_t nPacked, int32_t ctas, int32_t ne, std::string* err) {
+  int32_t at = 0;
+  for (const SlGroup& q : g) {
+    bool ok = q.R > 0 && q.R8 * 8 >= q.R && q.R8 % 2 == 0 && q.m0 >= 0 && q.nm > 0 &&
+              (size_t)q.m0 + q.nm <= m.size() && q.e0 >= 0 && q.e0 + q.R <= ne && q.cta0 == at &&
+              q.shift >= 0 && q.shift < 16;
+    at += q.R8;
+    for (int k = 0; ok && k < q.nm; ++k) {
+      const SlMember& b = m[q.m0 + k];
+      const int64_t last = b.trans ? (int64_t)(b.K - 1) * b.ld + q.R - 1
+                                   : (int64_t)(q.R - 1) * b.ld + b.K - 1;
+      ok = b.K > 0 && span_ok(b.src, last, nSrc) && b.ld >= (b.trans ? q.R : b.K) &&
+           (int64_t)b.KC * 64 >= b.K && b.dst >= 0 && b.dst % kSlTile == 0 &&
+           b.dst + (int64_t)q.R8 * b.KC * kSlices * kSlTile <= nPacked;
+    }
+    if (!ok) {
+      *err = "sliced operand out of bounds";
+      return false;
+    }
+  }
+  if (at != ctas) {
+    *err = "sliced operand launch";
+    return false;
+  }
+  return true;
+}
+
+inline bool sliced_ok(const GemmStage& g, const SlStage& s, int64_t nA, int64_t nB, int64_t nC,
+                      std::string* err) {
+  if (!gemm_ok(g.ta, g.tb, g.tasks, g.segs, nA, nB, nC, err) ||
+      !slices_ok(s.gA, s.mA, nA, s.nA, s.ctasA, s.neA, err) ||
+      !slices_ok(s.gB, s.mB, nB, s.nB, s.ctasB, s.neB, err))
+    return false;
+  bool ok = s.segs.size() == g.segs.size() && s.words.size() == s.chunks.size() &&
+            s.cta_unit.size() == s.cta_chunk.size() &&
+            (s.units.empty() ||
+             (s.cta_unit.size() >= 2 && s.cta_unit.front() == 0 && s.cta_chunk.front() == 0 &&
+              s.cta_unit.back() == (int32_t)s.units.size() &&
+              s.cta_chunk.back() == (int32_t)s.chunks.size()));
+  for (const SlChunk& c : s.chunks) {
+    ok = ok && c.ga >= 1 && c.ga <= 16 && c.gb >= 2 && c.gb <= 8 && c.gb % 2 == 0 && c.a >= 0 &&
+         c.b >= 0 && c.sa >= c.ga * kSlTile && c.sb >= c.gb * kSlTile && c.a % kSlTile == 0 &&
+         c.b % kSlTile == 0 && c.sa % kSlTile == 0 && c.sb % kSlTile == 0 &&
+         c.a + (int64_t)(kSlices - 1) * c.sa + c.ga * kSlTile <= s.nA &&
+         c.b + (int64_t)(kSlices - 1) * c.sb + c.gb * kSlTile <= s.nB;
+  }
+  // every CTA: its units' spans are what its chunk words describe
+  for (size_t b = 0; ok && b + 1 < s.cta_unit.size(); ++b) {
+    int32_t w = s.cta_chunk[b];
+    ok = s.cta_unit[b] <= s.cta_unit[b + 1] && w <= s.cta_chunk[b + 1];
+    uint32_t nw = 0;
+    for (int32_t u = s.cta_unit[b]; ok && u < s.cta_unit[b + 1]; ++u) {
+      const SlUnit& x = s.units[u];
+      ok = x.rows >= 1 && x.rows <= 128 && x.cols >= 1 && x.cols <= x.nw && x.nw <= 64 &&
+           x.nw % 16 == 0 && x.ldc >= x.cols && x.spans >= 0 && x.seg0 >= 0 &&
+           (size_t)x.seg0 + x.nseg <= s.segs.size() && x.m0 >= 0 && x.n0 >= 0 &&
+           span_ok(x.offC, (int64_t)(x.rows - 1) * x.ldc + x.cols - 1, nC);
+      if (ok && x.spans > 0)
+        ok = x.ea >= 0 && x.ea + x.rows <= s.neA && x.eb >= 0 && x.eb + x.cols <= s.neB;
+      for (int sp = 0; ok && sp < x.spans; ++sp) {
+        int steps = 0;
+        for (bool first = true;; first = false, ++w) {
+          if (w >= s.cta_chunk[b + 1]) {
+            ok = false;
+            break;
+          }
+          const uint32_t q = s.words[w];
+          const bool last = (q & kSlLast) != 0;
+          const bool long_first = first && sp % kSlLongSpan == 0;
+          const bool long_last =
+              last && (sp % kSlLongSpan == kSlLongSpan - 1 || sp == x.spans - 1);
+          ok = ok && (q & kSlSteps) >= 1 && (q & kSlSteps) <= 4 && (q >> kSlNw) == (uint32_t)x.nw &&
+               ((q & kSlFirst) != 0) == first && ((q & kSlLongFirst) != 0) == long_first &&
+               ((q & kSlLongLast) != 0) == long_last &&
+               ((q & kSlMove) != 0) == (first && sp == 0 && (uint32_t)x.nw != nw) &&
+               s.chunks[w].gb * 8 == x.nw;
+          steps += (int)(q & kSlSteps);
+          if (!ok || last) {
+            ++w;
+            break;
+          }
+        }
+        ok = ok && steps <= 4;
+        nw = (uint32_t)x.nw;
+      }
+    }
+    ok = ok && w == s.cta_chunk[b + 1];
+  }
+  if (!ok) *err = "sliced stage tables";
+  return ok;
+}
+
 // Tasks whose output is a packed operand (offC = float offset, ldc = R8).
 inline bool packed_tasks_ok(const std::vector<GemmTask>& tasks, int64_t nPacked, std::string* err) {
   for (const GemmTask& t : tasks) {
