@@ -41,6 +41,14 @@ void Hasher::mpo(const MpoLayout& w) {
 DevicePlan::~DevicePlan() {
   if (mem) cudaFree(mem);
 }
+DeviceGradPlan::~DeviceGradPlan() {
+  if (mem) cudaFree(mem);
+}
+
+SlTables sliced_tables(const DeviceSliced& d, const SlStage& s) {
+  return SlTables{d.units,    d.chunks, d.words, d.cta_unit, d.cta_chunk, d.segs,
+                  s.cta_unit.empty() ? 0 : (int)s.cta_unit.size() - 1};
+}
 
 namespace {
 template <class T>
@@ -53,6 +61,18 @@ T* place(char* base, size_t* off, const std::vector<T>& v, std::vector<char>* st
   if (!v.empty()) std::memcpy(staging->data() + *off, v.data(), v.size() * sizeof(T));
   *off += bytes_of(v);
   return v.empty() ? nullptr : p;
+}
+size_t bytes_of(const SlStage& q) {
+  return bytes_of(q.segs) + bytes_of(q.units) + bytes_of(q.chunks) + bytes_of(q.words) +
+         bytes_of(q.cta_unit) + bytes_of(q.cta_chunk);
+}
+void place_sliced(char* base, size_t* off, DeviceSliced* d, const SlStage& q, std::vector<char>* staging) {
+  d->segs = place(base, off, q.segs, staging);
+  d->units = place(base, off, q.units, staging);
+  d->chunks = place(base, off, q.chunks, staging);
+  d->words = place(base, off, q.words, staging);
+  d->cta_unit = place(base, off, q.cta_unit, staging);
+  d->cta_chunk = place(base, off, q.cta_chunk, staging);
 }
 }  // namespace
 
@@ -72,9 +92,9 @@ dmrg3s_status upload_plan(Plan&& host, std::unique_ptr<DevicePlan>* out) {
                  bytes_of(h.g12.tc.segs) + bytes_of(h.g12.tc.packA) + bytes_of(h.g12.tc.packB) +
                  bytes_of(h.g1.tc.cta_start) + bytes_of(h.g3s.tc.cta_start) +
                  bytes_of(h.g12.tc.cta_start);
-  for (const SlStage* q : {&h.s12, &h.s3})
-    total += bytes_of(q->segs) + bytes_of(q->units) + bytes_of(q->chunks) + bytes_of(q->words) +
-             bytes_of(q->cta_unit) + bytes_of(q->cta_chunk) + bytes_of(q->gA) + bytes_of(q->gB) + bytes_of(q->mA) + bytes_of(q->mB);
+  total += bytes_of(h.s12) + bytes_of(h.s3);
+  total += bytes_of(h.slices.groups) + bytes_of(h.slices.members) +
+           bytes_of(h.slices.cta_group) + bytes_of(h.t2) + bytes_of(h.t2_first);
   total += bytes_of(h.s3r.chunks) + bytes_of(h.s3r.tasks) + bytes_of(h.s3r.terms);
   if (total == 0) total = 256;
   if (cudaMalloc(&dp->mem, total) != cudaSuccess) return DMRG3S_ERR_CUDA;
@@ -111,20 +131,13 @@ dmrg3s_status upload_plan(Plan&& host, std::unique_ptr<DevicePlan>* out) {
   dp->c3r_chunks = place(base, &off, h.c3r.chunks, &staging);
   dp->c3r_tasks = place(base, &off, h.c3r.tasks, &staging);
   dp->c3r_terms = place(base, &off, h.c3r.terms, &staging);
-  auto place_sliced = [&](DevicePlan::Sliced* d, const SlStage& q) {
-    d->segs = place(base, &off, q.segs, &staging);
-    d->units = place(base, &off, q.units, &staging);
-    d->chunks = place(base, &off, q.chunks, &staging);
-    d->words = place(base, &off, q.words, &staging);
-    d->cta_unit = place(base, &off, q.cta_unit, &staging);
-    d->cta_chunk = place(base, &off, q.cta_chunk, &staging);
-    d->gA = place(base, &off, q.gA, &staging);
-    d->gB = place(base, &off, q.gB, &staging);
-    d->mA = place(base, &off, q.mA, &staging);
-    d->mB = place(base, &off, q.mB, &staging);
-  };
-  place_sliced(&dp->s12, h.s12);
-  place_sliced(&dp->s3, h.s3);
+  place_sliced(base, &off, &dp->s12, h.s12, &staging);
+  place_sliced(base, &off, &dp->s3, h.s3, &staging);
+  dp->sl_groups = place(base, &off, h.slices.groups, &staging);
+  dp->sl_members = place(base, &off, h.slices.members, &staging);
+  dp->sl_cta_group = place(base, &off, h.slices.cta_group, &staging);
+  dp->t2 = place(base, &off, h.t2, &staging);
+  dp->t2_first = place(base, &off, h.t2_first, &staging);
   dp->s3r_chunks = place(base, &off, h.s3r.chunks, &staging);
   dp->s3r_tasks = place(base, &off, h.s3r.tasks, &staging);
   dp->s3r_terms = place(base, &off, h.s3r.terms, &staging);
@@ -135,9 +148,8 @@ dmrg3s_status upload_plan(Plan&& host, std::unique_ptr<DevicePlan>* out) {
 }
 
 namespace {
-SlTables tables(const DevicePlan::Sliced& d, const SlStage& s) {
-  return SlTables{d.units,    d.chunks, d.words, d.cta_unit, d.cta_chunk, d.segs,
-                  s.cta_unit.empty() ? 0 : (int)s.cta_unit.size() - 1};
+SlSource source(const GemmStage& g, const double* A, const double* B, double scale) {
+  return SlSource{A, B, A, B, g.ta == Trans::T ? 1 : 0, g.tb == Trans::T ? 1 : 0, scale};
 }
 
 // FP64 by exact FP16 slices (kernels_sliced.cu): slice the operands, stages
@@ -156,34 +168,37 @@ dmrg3s_status run_sliced(Context* c, const DevicePlan& p, const double* g1A, con
   int32_t* e3B = e3A + h.s3.neA;
   const bool left = h.kind == Kind::Heff || h.kind == Kind::ExpandLR || h.kind == Kind::EnvLR;
   double* t2 = h.has_g3 ? base + sl.t2 : out2;
-  if (!hn.g1A)
-    launch_slice(p.s12.gA, (int)h.s12.gA.size(), h.s12.ctasA, p.s12.mA, g1A, pk(sl.a1), e1A,
-                 left ? scale : 1.0, st);
-  if (!hn.g1B)
-    launch_slice(p.s12.gB, (int)h.s12.gB.size(), h.s12.ctasB, p.s12.mB, g1B, pk(sl.b1), e1B,
-                 left ? 1.0 : scale, st);
+  const bool t2_is_a = h.kind == Kind::Heff;
+  SlOperands ops{};
+  ops.op[0] = left ? SlOperand{g1A, pk(sl.a1), e1A, scale} : SlOperand{g1B, pk(sl.b1), e1B, scale};
+  ops.op[1] = t2_is_a ? SlOperand{g3B, pk(sl.b3), e3B, 1.0} : SlOperand{g3A, pk(sl.a3), e3A, 1.0};
+  ops.op[2] = left ? SlOperand{g1B, pk(sl.b1), e1B, 1.0} : SlOperand{g1A, pk(sl.a1), e1A, 1.0};
+  int32_t* et2 = t2_is_a ? e3A : e3B;        // row scales of T2, collected by stage 2
+  if (h.has_g3) {
+    ops.clear = et2;
+    ops.nclear = t2_is_a ? h.s3.neA : h.s3.neB;
+  }
+  // (a caller that has sliced the environments does so for both)
+  slice_operands(p, hn.sliced_env ? 2 : 0, 2, ops, st);
   if (!h.s12.units.empty()) {
     const int id = pr.on ? pr.begin(kProfGemm, h.f12.flops, h.f12.bytes, st) : -1;
-    launch_gemm_sliced(tables(p.s12, h.s12), hn.s1A ? hn.s1A : pk(sl.a1), pk(sl.b1),
-                       hn.s1A ? hn.e1A : e1A, e1B, g1A, g1B, h.f12.ta, h.f12.tb, scale, t2,
-                       c->d_err, c->wait_ns, st);
+    launch_gemm_sliced(sliced_tables(p.s12, h.s12), hn.s1A ? hn.s1A : pk(sl.a1), pk(sl.b1),
+                       hn.s1A ? hn.e1A : e1A, e1B, source(h.f12, g1A, g1B, scale), t2, et2,
+                       h.kind == Kind::EnvLR, c->d_err, c->wait_ns, st);
     if (id >= 0) pr.end(id, st);
   }
   if (h.has_g3) {
-    const bool t2_is_a = h.kind == Kind::Heff;
     const double* a3 = t2_is_a ? t2 : g3A;
     const double* b3 = t2_is_a ? g3B : t2;
-    if (t2_is_a || !hn.g3A)
-      launch_slice(p.s3.gA, (int)h.s3.gA.size(), h.s3.ctasA, p.s3.mA, a3, pk(sl.a3), e3A, 1.0, st);
-    if (!t2_is_a || !hn.g3B)
-      launch_slice(p.s3.gB, (int)h.s3.gB.size(), h.s3.ctasB, p.s3.mB, b3, pk(sl.b3), e3B, 1.0, st);
+    launch_slice_known(p.t2, (int)h.t2.size(), p.t2_first, h.t2_tiles, t2, pk(t2_is_a ? sl.a3 : sl.b3),
+                       et2, st);
     const bool split = !h.s3r.chunks.empty();
     double* c3 = split ? base + sl.p3 : g3C;
     if (!h.s3.units.empty()) {
       const int id = pr.on ? pr.begin(kProfGemm, h.g3.flops, h.g3.bytes, st) : -1;
-      launch_gemm_sliced(tables(p.s3, h.s3), pk(sl.a3), hn.s3B ? hn.s3B : pk(sl.b3), e3A,
-                         hn.s3B ? hn.e3B : e3B, a3, b3, h.f3.ta, h.f3.tb, 1.0, c3, c->d_err,
-                         c->wait_ns, st);
+      launch_gemm_sliced(sliced_tables(p.s3, h.s3), pk(sl.a3), hn.s3B ? hn.s3B : pk(sl.b3), e3A,
+                         hn.s3B ? hn.e3B : e3B, source(h.f3, a3, b3, 1.0), c3, nullptr, false,
+                         c->d_err, c->wait_ns, st);
       if (id >= 0) pr.end(id, st);
     }
     if (split) {
@@ -325,6 +340,72 @@ dmrg3s_status run_plan(Context* c, const DevicePlan& p, const double* g1A, const
     if (id >= 0) pr.end(id, st);
   }
   return cudaGetLastError() == cudaSuccess ? DMRG3S_OK : DMRG3S_ERR_CUDA;
+}
+
+}  // namespace dmrg3s
+
+namespace dmrg3s {
+
+dmrg3s_status upload_grad_plan(GradPlan&& host, std::unique_ptr<DeviceGradPlan>* out) {
+  std::unique_ptr<DeviceGradPlan> dp(new (std::nothrow) DeviceGradPlan());
+  if (!dp) return DMRG3S_ERR_OOM;
+  dp->host = std::move(host);
+  const GradPlan& h = dp->host;
+  size_t total = bytes_of(h.tasks) + bytes_of(h.segs) + bytes_of(h.s) + bytes_of(h.slices.groups) +
+                 bytes_of(h.slices.members) + bytes_of(h.slices.cta_group) + 256;
+  for (const GemmStage* g : {&h.g1, &h.gy})
+    total += bytes_of(g->tiles) + bytes_of(g->tasks) + bytes_of(g->segs);
+  if (cudaMalloc(&dp->mem, total) != cudaSuccess) return DMRG3S_ERR_CUDA;
+  std::vector<char> staging(total, 0);
+  char* base = static_cast<char*>(dp->mem);
+  size_t off = 0;
+  DeviceGradPlan::Gemm* dg[2] = {&dp->g1, &dp->gy};
+  const GemmStage* hg[2] = {&h.g1, &h.gy};
+  for (int i = 0; i < 2; ++i) {
+    dg[i]->tiles = place(base, &off, hg[i]->tiles, &staging);
+    dg[i]->tasks = place(base, &off, hg[i]->tasks, &staging);
+    dg[i]->segs = place(base, &off, hg[i]->segs, &staging);
+  }
+  dp->tasks = place(base, &off, h.tasks, &staging);
+  dp->segs = place(base, &off, h.segs, &staging);
+  place_sliced(base, &off, &dp->s, h.s, &staging);
+  dp->sl_groups = place(base, &off, h.slices.groups, &staging);
+  dp->sl_members = place(base, &off, h.slices.members, &staging);
+  dp->sl_cta_group = place(base, &off, h.slices.cta_group, &staging);
+  if (cudaMemcpy(dp->mem, staging.data(), total, cudaMemcpyHostToDevice) != cudaSuccess)
+    return DMRG3S_ERR_CUDA;
+  *out = std::move(dp);
+  return DMRG3S_OK;
+}
+
+// The gradient uses W's structure only, so its values are not in the key.
+dmrg3s_status grad_plan(Context* c, const EnvLayout& le, const MpoLayout& w, const EnvLayout& re,
+                        const SiteLayout& a, const DeviceGradPlan** out) {
+  Hasher h;
+  h.pod(100);
+  h.env(le);
+  h.pod(w.d);
+  h.pod(w.wl);
+  h.pod(w.wr);
+  h.env(re);
+  h.site(a);
+  auto it = c->grad_plans.find(h.h);
+  if (it != c->grad_plans.end()) {
+    *out = it->second.get();
+    return DMRG3S_OK;
+  }
+  GradPlan p;
+  std::string err;
+  dmrg3s_status st = plan_mpo_grad(le, w, re, a, &p, &err);
+  if (st != DMRG3S_OK) return fail(c, st, err);
+  std::unique_ptr<DeviceGradPlan> dp;
+  if ((st = upload_grad_plan(std::move(p), &dp)))
+    return fail(c, st, "uploading a gradient plan failed");
+  // a bounded cache: freeing the tables waits for the device
+  if (c->grad_plans.size() >= kMaxGradPlans) c->grad_plans.clear();
+  *out = dp.get();
+  c->grad_plans[h.h] = std::move(dp);
+  return DMRG3S_OK;
 }
 
 }  // namespace dmrg3s
@@ -477,6 +558,7 @@ dmrg3s_status dmrg3s_destroy(dmrg3s_ctx ctx) {
   use_device(c);
   cudaDeviceSynchronize();
   c->plans.clear();
+  c->grad_plans.clear();
   if (c->ws) cudaFree(c->ws);
   if (c->pinned) cudaFreeHost(c->pinned);
   if (c->d_err) cudaFree(c->d_err);

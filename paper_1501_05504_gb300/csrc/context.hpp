@@ -13,6 +13,35 @@
 
 namespace dmrg3s {
 
+// Tables of a sliced FP64 stage (SlStage).
+struct DeviceSliced {
+  SlSeg* segs = nullptr;
+  SlUnit* units = nullptr;
+  SlChunk* chunks = nullptr;
+  uint32_t* words = nullptr;
+  int32_t *cta_unit = nullptr, *cta_chunk = nullptr;
+};
+SlTables sliced_tables(const DeviceSliced& d, const SlStage& s);
+
+// Device copy of the MPO-entry gradient's tables.
+struct DeviceGradPlan {
+  GradPlan host;
+  void* mem = nullptr;
+  struct Gemm {
+    GemmTile* tiles = nullptr;
+    GemmTask* tasks = nullptr;
+    GemmSeg* segs = nullptr;
+  } g1, gy;
+  DotTask* tasks = nullptr;
+  DotSeg* segs = nullptr;
+  DeviceSliced s;
+  SlGroup* sl_groups = nullptr;
+  SlMember* sl_members = nullptr;
+  int32_t* sl_cta_group = nullptr;
+  ~DeviceGradPlan();
+};
+constexpr size_t kMaxGradPlans = 256;     // cached per context
+
 // Device copy of a plan's task tables.
 struct DevicePlan {
   Plan host;
@@ -50,15 +79,12 @@ struct DevicePlan {
   GemmTask* g3_tasks = nullptr;
   GemmSeg* g3_segs = nullptr;
   // sliced FP64 form: stages 1 + 2, stage 3, the sum of its partials
-  struct Sliced {
-    SlSeg* segs = nullptr;
-    SlUnit* units = nullptr;
-    SlChunk* chunks = nullptr;
-    uint32_t* words = nullptr;
-    int32_t *cta_unit = nullptr, *cta_chunk = nullptr;
-    SlGroup *gA = nullptr, *gB = nullptr;
-    SlMember *mA = nullptr, *mB = nullptr;
-  } s12, s3;
+  DeviceSliced s12, s3;
+  SlGroup* sl_groups = nullptr;
+  SlMember* sl_members = nullptr;
+  int32_t* sl_cta_group = nullptr;
+  SlPiece* t2 = nullptr;
+  int32_t* t2_first = nullptr;
   CombChunk* s3r_chunks = nullptr;
   CombTask* s3r_tasks = nullptr;
   CombTerm* s3r_terms = nullptr;
@@ -136,6 +162,7 @@ struct Context {
   double* pinned_big = nullptr;   // pinned read-back area of the batched Lanczos (grown on demand)
   size_t pinned_big_n = 0;        // its size in doubles
   std::unordered_map<uint64_t, std::unique_ptr<DevicePlan>> plans;
+  std::unordered_map<uint64_t, std::unique_ptr<DeviceGradPlan>> grad_plans;
   std::string last_error;
 };
 
@@ -246,6 +273,7 @@ struct SplitHints {
   // intermediates fit the workspace), and, H_eff only, sliced L and R held
   // outside the workspace with their row scales
   int f64 = 0;
+  bool sliced_env = false;   // L and R are sliced already (in the workspace slots or below)
   const uint16_t *s1A = nullptr, *s3B = nullptr;
   const int32_t *e1A = nullptr, *e3B = nullptr;
 };
@@ -285,6 +313,14 @@ inline SlSlots sl_slots(const Plan& p) {
   s.end = s.p3 + slot_round(p.ws3s);
   return s;
 }
+// Slices operands [first, last] of a plan (Plan::slices); ops[i] describes
+// operand i.
+inline void slice_operands(const DevicePlan& p, int first, int last, const SlOperands& ops,
+                           cudaStream_t st) {
+  const SliceTable& t = p.host.slices;
+  launch_slice(p.sl_groups, p.sl_cta_group, t.cta[first], t.cta[last + 1] - t.cta[first],
+               p.sl_members, ops, st);
+}
 inline bool sliced_fits(const Plan& p, size_t ws_bytes) {
   return p.sliced && (size_t)sl_slots(p).end * sizeof(double) <= ws_bytes;
 }
@@ -303,7 +339,9 @@ dmrg3s_status run_plan(Context* c, const DevicePlan& p, const double* g1A, const
 
 // MPO-entry gradient G (d*d*wl*wr doubles, device, layout of W) of
 // <M|H_eff|M> for the given environments; intermediates in the workspace.
-dmrg3s_status run_mpo_grad(Context* c, const GradPlan& p, const double* L, const double* M,
+dmrg3s_status grad_plan(Context* c, const EnvLayout& le, const MpoLayout& w, const EnvLayout& re,
+                        const SiteLayout& a, const DeviceGradPlan** out);
+dmrg3s_status run_mpo_grad(Context* c, const DeviceGradPlan& p, const double* L, const double* M,
                            const double* R, double* G, cudaStream_t st);
 
 }  // namespace dmrg3s

@@ -128,13 +128,12 @@ dmrg3s_status lanczos_batch(Context* c, const DevicePlan& heff, const double* Ld
     const Plan& hp = heff.host;
     const SlSlots sl = sl_slots(hp);
     int32_t* e = reinterpret_cast<int32_t*>(ws1 + sl.e);
-    launch_slice(heff.s12.gA, (int)hp.s12.gA.size(), hp.s12.ctasA, heff.s12.mA, Ldata,
-                 reinterpret_cast<uint16_t*>(ws1 + sl.a1), e, 1.0, st);
-    launch_slice(heff.s3.gB, (int)hp.s3.gB.size(), hp.s3.ctasB, heff.s3.mB, Rdata,
-                 reinterpret_cast<uint16_t*>(ws1 + sl.b3),
-                 e + hp.s12.neA + hp.s12.neB + hp.s3.neA, 1.0, st);
-    hints.g1A = true;
-    hints.g3B = true;
+    SlOperands ops{};
+    ops.op[0] = SlOperand{Ldata, reinterpret_cast<uint16_t*>(ws1 + sl.a1), e, 1.0};
+    ops.op[1] = SlOperand{Rdata, reinterpret_cast<uint16_t*>(ws1 + sl.b3),
+                          e + hp.s12.neA + hp.s12.neB + hp.s3.neA, 1.0};
+    slice_operands(heff, 0, 1, ops, st);
+    hints.sliced_env = true;
   }
   if (prec != DMRG3S_FP64) {
     const Plan& hp = heff.host;

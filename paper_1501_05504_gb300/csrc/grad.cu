@@ -18,55 +18,51 @@
 
 namespace dmrg3s {
 
-namespace {
-
-template <class T>
-dmrg3s_status put(Context* c, const std::vector<T>& v, T** dev, cudaStream_t st) {
-  *dev = nullptr;
-  if (v.empty()) return DMRG3S_OK;
-  cudaError_t e = cudaMallocAsync((void**)dev, v.size() * sizeof(T), st);
-  if (e == cudaSuccess)
-    e = cudaMemcpyAsync(*dev, v.data(), v.size() * sizeof(T), cudaMemcpyHostToDevice, st);
-  if (e != cudaSuccess) return fail(c, DMRG3S_ERR_CUDA, "gradient table upload");
-  return DMRG3S_OK;
-}
-
-dmrg3s_status gemm_stage(Context* c, const GemmStage& g, const double* A, const double* B,
-                         double* C, cudaStream_t st) {
-  if (g.tiles.empty()) return DMRG3S_OK;
-  GemmTile* dt;
-  GemmTask* dk;
-  GemmSeg* ds;
-  dmrg3s_status s;
-  if ((s = put(c, g.tiles, &dt, st)) || (s = put(c, g.tasks, &dk, st)) ||
-      (s = put(c, g.segs, &ds, st)))
-    return s;
-  const int id = c->prof.on ? c->prof.begin(kProfAuxGemm, g.flops, g.bytes, st) : -1;
-  launch_gemm_f64(g.ta, g.tb, dt, (int)g.tiles.size(), dk, ds, A, B, C, st);
-  if (id >= 0) c->prof.end(id, st);
-  cudaFreeAsync(dt, st);
-  cudaFreeAsync(dk, st);
-  if (ds) cudaFreeAsync(ds, st);
-  return DMRG3S_OK;
-}
-
-}  // namespace
-
-dmrg3s_status run_mpo_grad(Context* c, const GradPlan& p, const double* L, const double* M,
+// Sliced form (kernels_sliced.cu): L and R and both views of M sliced by one
+// launch, T1 and Y by one grouped GEMM, then the inner products.  It runs
+// where its intermediates fit the workspace, else the plain form.
+dmrg3s_status run_mpo_grad(Context* c, const DeviceGradPlan& dp, const double* L, const double* M,
                            const double* R, double* G, cudaStream_t st) {
+  const GradPlan& p = dp.host;
   if ((size_t)(p.ws1 + p.wsy) * sizeof(double) > c->ws_bytes)
     return fail(c, DMRG3S_ERR_OOM, "context workspace too small for the gradient intermediates");
   double* ws1 = reinterpret_cast<double*>(c->ws);
-  double* wsy = ws1 + p.ws1;
-  dmrg3s_status s;
-  if ((s = gemm_stage(c, p.g1, L, M, ws1, st)) || (s = gemm_stage(c, p.gy, M, R, wsy, st)))
-    return s;
-  DotTask* dt;
-  DotSeg* ds;
-  if ((s = put(c, p.tasks, &dt, st)) || (s = put(c, p.segs, &ds, st))) return s;
-  launch_dots(dt, (int)p.tasks.size(), ds, ws1, wsy, G, st);
-  cudaFreeAsync(dt, st);
-  if (ds) cudaFreeAsync(ds, st);
+  const int64_t w1 = p.ws1 > 0 ? p.ws1 : 1, wy = p.wsy > 0 ? p.wsy : 1;
+  double* wsy = ws1 + (p.sliced ? w1 : p.ws1);
+  Profiler& pr = c->prof;
+  const int64_t a = slot_round(w1 + wy), b = a + slot_round((p.s.nA + 3) / 4),
+                e = b + slot_round((p.s.nB + 3) / 4),
+                end = e + slot_round(((int64_t)p.s.neA + p.s.neB + 1) / 2);
+  if (p.sliced && (size_t)end * sizeof(double) <= c->ws_bytes) {
+    uint16_t* pA = reinterpret_cast<uint16_t*>(ws1 + a);
+    uint16_t* pB = reinterpret_cast<uint16_t*>(ws1 + b);
+    int32_t* eA = reinterpret_cast<int32_t*>(ws1 + e);
+    int32_t* eB = eA + p.s.neA;
+    SlOperands ops{};
+    ops.op[0] = SlOperand{L, pA, eA, 1.0};
+    ops.op[1] = SlOperand{M, pA, eA, 1.0};
+    ops.op[2] = SlOperand{M, pB, eB, 1.0};
+    ops.op[3] = SlOperand{R, pB, eB, 1.0};
+    launch_slice(dp.sl_groups, dp.sl_cta_group, 0, p.slices.cta.back(), dp.sl_members, ops, st);
+    const int id = pr.on ? pr.begin(kProfAuxGemm, p.g1.flops + p.gy.flops, p.g1.bytes + p.gy.bytes, st) : -1;
+    launch_gemm_sliced(sliced_tables(dp.s, p.s), pA, pB, eA, eB, SlSource{L, M, M, R, 0, 0, 1.0}, ws1,
+                       nullptr, false, c->d_err, c->wait_ns, st);
+    if (id >= 0) pr.end(id, st);
+  } else {
+    wsy = ws1 + p.ws1;
+    const DeviceGradPlan::Gemm* d[2] = {&dp.g1, &dp.gy};
+    const GemmStage* g[2] = {&p.g1, &p.gy};
+    const double *A[2] = {L, M}, *B[2] = {M, R};
+    double* C[2] = {ws1, wsy};
+    for (int i = 0; i < 2; ++i) {
+      if (g[i]->tiles.empty()) continue;
+      const int id = pr.on ? pr.begin(kProfAuxGemm, g[i]->flops, g[i]->bytes, st) : -1;
+      launch_gemm_f64(g[i]->ta, g[i]->tb, d[i]->tiles, (int)g[i]->tiles.size(), d[i]->tasks, d[i]->segs,
+                      A[i], B[i], C[i], st);
+      if (id >= 0) pr.end(id, st);
+    }
+  }
+  launch_dots(dp.tasks, (int)p.tasks.size(), dp.segs, ws1, wsy, G, st);
   if (cudaGetLastError() != cudaSuccess) return fail(c, DMRG3S_ERR_CUDA, "gradient launch");
   return DMRG3S_OK;
 }
@@ -94,8 +90,8 @@ extern "C" dmrg3s_status dmrg3s_mpo_grad_site(dmrg3s_ctx ctx, const dmrg3s_env* 
       (st = check_env(re, m.right, w.wr, w.tr, "R", &err)))
     return fail(c, st, err);
   if (!L->data || !R->data || !M->data) return fail(c, DMRG3S_ERR_ARG, "NULL device data pointer");
-  GradPlan p;
-  if ((st = plan_mpo_grad(le, w, re, m, &p, &err))) return fail(c, st, err);
   if ((st = use_device(c))) return st;
-  return run_mpo_grad(c, p, L->data, M->data, R->data, G, reinterpret_cast<cudaStream_t>(stream));
+  const DeviceGradPlan* p = nullptr;
+  if ((st = grad_plan(c, le, w, re, m, &p))) return st;
+  return run_mpo_grad(c, *p, L->data, M->data, R->data, G, reinterpret_cast<cudaStream_t>(stream));
 }

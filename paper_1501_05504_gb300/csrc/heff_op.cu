@@ -100,10 +100,10 @@ dmrg3s_status dmrg3s_heff_create(dmrg3s_ctx ctx, const dmrg3s_env* L, const dmrg
     const SlStage& s3 = p->host.s3;
     if (cudaMalloc(&h->sliceL, sliced_bytes(s1.nA, s1.neA)) == cudaSuccess &&
         cudaMalloc(&h->sliceR, sliced_bytes(s3.nB, s3.neB)) == cudaSuccess) {
-      launch_slice(p->s12.gA, (int)s1.gA.size(), s1.ctasA, p->s12.mA, L->data, h->sliceL,
-                   row_scales(h->sliceL, s1.nA), 1.0, s);
-      launch_slice(p->s3.gB, (int)s3.gB.size(), s3.ctasB, p->s3.mB, R->data, h->sliceR,
-                   row_scales(h->sliceR, s3.nB), 1.0, s);
+      SlOperands ops{};
+      ops.op[0] = SlOperand{L->data, h->sliceL, row_scales(h->sliceL, s1.nA), 1.0};
+      ops.op[1] = SlOperand{R->data, h->sliceR, row_scales(h->sliceR, s3.nB), 1.0};
+      slice_operands(*p, 0, 1, ops, s);
       if (cudaGetLastError() != cudaSuccess) {
         cudaFree(h->sliceL);
         cudaFree(h->sliceR);
@@ -147,7 +147,7 @@ dmrg3s_status dmrg3s_heff_apply(dmrg3s_heff op, const double* A, double* HA,
     const Plan& pl = h->plan->host;
     hints.f64 = h->sliceL ? kF64Sliced : kF64Plain;
     if (h->sliceL) {
-      hints.g1A = hints.g3B = true;
+      hints.sliced_env = true;
       hints.s1A = h->sliceL;
       hints.e1A = row_scales(h->sliceL, pl.s12.nA);
       hints.s3B = h->sliceR;

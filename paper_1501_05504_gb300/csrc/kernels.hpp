@@ -101,16 +101,17 @@ constexpr int kSlTile = 512;               // FP16 elements of a tile
 constexpr int32_t kSlSpecial = 0x40000000; // row scale of a row with Inf or NaN
 // One block of a scale group: element (r, k) is coef * src[src + r ld + k]
 // (trans = 0) or coef * src[src + k ld + r] (trans = 1).
+// t0: its first 64-wide chunk among the chunks of its group.
 struct SlMember {
   int64_t src, dst;
   double coef;
-  int32_t ld, K, KC, trans;
+  int32_t ld, K, KC, trans, t0, pad;
 };
 // Blocks with the same rows whose rows share scales: scales[e0 + r]; one CTA
 // of the slicing kernel per row group, from cta0 on.
 // `shift` raises the scales by that power of two: headroom of the integer sums.
 struct SlGroup {
-  int32_t R, R8, m0, nm, e0, cta0, shift;
+  int32_t R, R8, m0, nm, nt, e0, cta0, shift, which, pad;   // nt: chunks; which: its operand
 };
 // Spans a unit may sum before the headroom has to grow (the levels of a span
 // stay below 2^58.1 in the 64-bit sum).
@@ -125,10 +126,14 @@ struct SlSeg {
 // One output tile of up to 128 rows x tile_n columns (rows and cols: what lies
 // inside the block), written at C + offC with leading dimension ldc; row scales
 // of A from ea, column scales of B from eb; spans accumulation spans.
-// m0, n0: its place in the task (for rows with Inf or NaN).
+// m0, n0: its place in the task (for rows with Inf or NaN).  The largest
+// exponent of every output row (column) is collected in the scales from em on.
 struct SlUnit {
   int64_t offC;
-  int32_t ldc, rows, cols, nw, spans, ea, eb, m0, n0, seg0, nseg, pad;
+  int32_t ldc, rows, cols, nw, spans, ea, eb, m0, n0, seg0, nseg;
+  int32_t shift;    // of A's row scales (SlGroup.shift)
+  int32_t em;       // first row scale of the output as a later operand, or -1
+  int32_t sel;      // which pair of FP64 operands (SlSource) its segments read
 };
 // The units' 64-wide k-chunks in the order a CTA runs them.  The copies: slice
 // i of A is `ga` tiles at a + i sa, slice j of B `gb` tiles at b + j sb (FP16
@@ -145,14 +150,41 @@ struct SlChunk {
 constexpr uint32_t kSlSteps = 7, kSlFirst = 8, kSlLast = 16, kSlLongFirst = 32, kSlLongLast = 64,
                    kSlMove = 128, kSlNw = 8;
 constexpr int kSlLongSpan = 4;
-// Row scales and slices of every block of the groups (`scale` multiplies every
-// coefficient).  nctas: the sum of the groups' R8.
-void launch_slice(const SlGroup* groups, int ngroups, int nctas, const SlMember* members,
-                  const double* src, uint16_t* out, int32_t* scales, double scale, cudaStream_t st);
+// An operand: its FP64 array, its packed array, its row scales; `scale`
+// multiplies every coefficient.
+struct SlOperand {
+  const double* src;
+  uint16_t* out;
+  int32_t* scales;
+  double scale;
+};
+// The launch also clears `nclear` scales (which a later launch collects).
+struct SlOperands {
+  SlOperand op[4];
+  int32_t* clear;
+  int32_t nclear;
+};
+// A block of an operand whose row scales are known (collected by the launch
+// that wrote it): tiles [tile0, tile0 + R8 KC), tile t = (chunk, row group) with
+// t = chunk R8 + group.
+struct SlPiece {
+  int64_t src, dst;
+  int32_t ld, K, KC, trans, R, R8, e0, shift, tile0, pad;
+};
+// Row scales and slices of every block of the groups whose CTAs are
+// [cta0, cta0 + nctas) (a group has R8 CTAs from its cta0 on; cta_group[c] = the
+// group of CTA c).
+void launch_slice(const SlGroup* groups, const int32_t* cta_group, int cta0, int nctas,
+                  const SlMember* members, const SlOperands& ops, cudaStream_t st);
+// Slices of the pieces, a warp per tile; first[c] = the piece of tile 8 c.
+void launch_slice_known(const SlPiece* pieces, int npieces, const int32_t* first, int ntiles,
+                        const double* src, uint16_t* out, const int32_t* scales, cudaStream_t st);
+
 // C = sum over the task's segments of op(A) op(B), one rounding to FP64 (see
 // kernels_sliced.cu).  CTA b runs units [cta_unit[b], cta_unit[b + 1]) and
-// chunks [cta_chunk[b], cta_chunk[b + 1]).  A, B, ta, tb, scale, segs: the FP64
-// operands, read for rows with Inf or NaN only.
+// chunks [cta_chunk[b], cta_chunk[b + 1]).  src, segs: the FP64
+// operands, read for rows with Inf or NaN only.  collect: the row scales of the
+// output as an operand (of its rows, or of its columns), cleared before.
 struct SlTables {
   const SlUnit* units;
   const SlChunk* chunks;
@@ -161,9 +193,14 @@ struct SlTables {
   const SlSeg* segs;
   int ncta;
 };
+struct SlSource {
+  const double *A, *B, *A1, *B1;     // A1, B1: of the units with sel = 1
+  int32_t ta, tb;                    // stored transposed (as in launch_gemm_f64)
+  double scale;
+};
 void launch_gemm_sliced(const SlTables& t, const uint16_t* pA, const uint16_t* pB,
-                        const int32_t* eA, const int32_t* eB, const double* A, const double* B,
-                        Trans ta, Trans tb, double scale, double* C, int* err, uint64_t wait_ns,
+                        const int32_t* eA, const int32_t* eB, const SlSource& src, double* C,
+                        int32_t* collect, bool collect_cols, int* err, uint64_t wait_ns,
                         cudaStream_t st);
 
 // Blockwise inner products: out[task.out] = sum over the task's segments of

@@ -171,18 +171,39 @@ __global__ void __launch_bounds__(256) combine_pairs_f64_kernel(
 
 std::atomic<int64_t> g_launches{0};
 
+// One CTA per entry.  Each segment is cut into pieces of 1024 elements, dealt to
+// the CTA's warps in turn: the blocks of a charge-conserving tensor are often
+// only a few hundred elements, which a CTA-wide loop per segment visits one
+// memory latency after the other.
+constexpr int kDotPiece = 1024;
 __global__ void __launch_bounds__(256) dots_kernel(const DotTask* __restrict__ tasks,
                                                    const DotSeg* __restrict__ segs,
                                                    const double* __restrict__ A,
                                                    const double* __restrict__ B,
                                                    double* __restrict__ out) {
   const DotTask t = tasks[blockIdx.x];
-  double acc = 0.0;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  double acc0 = 0.0, acc1 = 0.0, acc2 = 0.0, acc3 = 0.0;
+  int turn = 0;                       // pieces dealt so far, modulo the warps
   for (int k = 0; k < t.nseg; ++k) {
     const DotSeg g = segs[t.seg0 + k];
-    for (int64_t e = threadIdx.x; e < g.len; e += blockDim.x)
-      acc = fma(A[g.offA + e], B[g.offB + e], acc);
+    const int64_t np = (g.len + kDotPiece - 1) / kDotPiece;
+    for (int64_t q = (warp - turn) & 7; q < np; q += 8) {
+      const int64_t e1 = min(g.len, (q + 1) * kDotPiece);
+      int64_t e = q * kDotPiece + lane;
+      const double* a = A + g.offA;
+      const double* b = B + g.offB;
+      for (; e + 96 < e1; e += 128) {
+        acc0 = fma(a[e], b[e], acc0);
+        acc1 = fma(a[e + 32], b[e + 32], acc1);
+        acc2 = fma(a[e + 64], b[e + 64], acc2);
+        acc3 = fma(a[e + 96], b[e + 96], acc3);
+      }
+      for (; e < e1; e += 32) acc0 = fma(a[e], b[e], acc0);
+    }
+    turn = (int)((turn + np) & 7);
   }
+  double acc = (acc0 + acc1) + (acc2 + acc3);
   __shared__ double red[8];
   for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;

@@ -190,9 +190,9 @@ __device__ __noinline__ double element_f64(const SlSeg* __restrict__ segs, int n
 __global__ void __launch_bounds__(kThreads, 1)
     gemm_sliced_kernel(const SlTables tab, const uint16_t* __restrict__ pA,
                        const uint16_t* __restrict__ pB, const int32_t* __restrict__ eA,
-                       const int32_t* __restrict__ eB, const double* __restrict__ A,
-                       const double* __restrict__ B, int ta, int tb, double scale,
-                       double* __restrict__ C, int* __restrict__ err, uint64_t wait_ns) {
+                       const int32_t* __restrict__ eB, const __grid_constant__ SlSource src,
+                       double* __restrict__ C, int32_t* __restrict__ collect, int collect_cols,
+                       int* __restrict__ err, uint64_t wait_ns) {
   extern __shared__ __align__(1024) unsigned char smem[];
   __shared__ __align__(8) uint64_t afull[kSlots], aempty[kSlots], bfull[2], bempty[2];
   __shared__ __align__(8) uint64_t lfull[kSlices], lempty[kSlices], done;
@@ -493,6 +493,8 @@ __global__ void __launch_bounds__(kThreads, 1)
       const int rows = un.rows, cols = un.cols;
       double* Cu = C + un.offC + n0;
       const int64_t ldc = un.ldc;
+      const int em = un.em, shift = un.shift;
+      uint32_t hmax = 0;                       // largest |high word| of the row (column `lane`)
       // (the vote first: every lane takes part in it)
       const bool special_col = __any_sync(0xffffffffu, fb_lane == kSlSpecial);
       const bool special = special_col || fa == kSlSpecial;
@@ -501,20 +503,36 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (n0 + c4 >= cols) break;
         bool out = false;                    // of this lane's elements inside the tile
         int ex[4];
+        double val[4];
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
           const float lf = L[c4 + i];
           bool o = !(fabsf(lf) < 17179869184.f);           // 2^34: the range of the conversion
-          ex[i] = fa + __shfl_sync(0xffffffffu, fb_lane, c4 + i) - 2114;
-          stage[lane * kStageRow + i] =
-              fixed_to_f64((long long)(H[c4 + i] - bh), __float2int_rn(lf * 0.0625f), ex[i], &o);
+          ex[i] = fa + shift + __shfl_sync(0xffffffffu, fb_lane, c4 + i) - 2114;
+          val[i] = fixed_to_f64((long long)(H[c4 + i] - bh), __float2int_rn(lf * 0.0625f), ex[i], &o);
           out = out || (o && row < rows && n0 + c4 + i < cols);
         }
         if (out)
 #pragma unroll
           for (int i = 0; i < 4; ++i)
-            stage[lane * kStageRow + i] =
-                fixed_to_f64_any((long long)(H[c4 + i] - bh), L[c4 + i], ex[i]);
+            val[i] = fixed_to_f64_any((long long)(H[c4 + i] - bh), L[c4 + i], ex[i]);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) stage[lane * kStageRow + i] = val[i];
+        if (em >= 0) {
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            // (a nonzero low word alone still counts as a smallest exponent)
+            uint32_t hw = (uint32_t)__double2hiint(val[i]) & 0x7FFFFFFFu;
+            hw |= __double2loint(val[i]) != 0 ? 1u : 0u;
+            if (row >= rows || n0 + c4 + i >= cols) hw = 0;
+            if (collect_cols) {
+              hw = __reduce_max_sync(0xffffffffu, hw);
+              hmax = lane == c4 + i ? hw : hmax;
+            } else {
+              hmax = max(hmax, hw);
+            }
+          }
+        }
         __syncwarp();
 #pragma unroll
         for (int it = 0; it < 4; ++it) {
@@ -524,12 +542,22 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
         __syncwarp();
       }
+      if (em >= 0) {
+        // exponent field of the largest element (0: all zero); rows (columns)
+        // that meet Inf or NaN have no scale
+        const bool inside = collect_cols ? lane < 16 && n0 + lane < cols : row < rows;
+        int f = hmax == 0 ? 0 : max((int)(hmax >> 20), 1);
+        const bool any = __any_sync(0xffffffffu, special && row < rows);
+        if (f >= 0x7FF || (collect_cols ? any : special)) f = kSlSpecial;
+        if (inside && f) atomicMax(collect + em + (collect_cols ? n0 + lane : row), f);
+      }
       // rows and columns with Inf or NaN (their slices are zero): the FP64 sum
       if (special && row < rows) {
         for (int j = 0; j < 16 && n0 + j < cols; ++j)
           if (fa == kSlSpecial || eB[un.eb + n0 + j] == kSlSpecial)
-            Cu[row * ldc + j] = element_f64(tab.segs + un.seg0, un.nseg, A, B, ta, tb, un.m0 + row,
-                                            un.n0 + n0 + j, scale);
+            Cu[row * ldc + j] =
+                element_f64(tab.segs + un.seg0, un.nseg, un.sel ? src.A1 : src.A,
+                            un.sel ? src.B1 : src.B, src.ta, src.tb, un.m0 + row, un.n0 + n0 + j, src.scale);
       }
       __syncwarp();
     }
@@ -546,11 +574,13 @@ __global__ void __launch_bounds__(kThreads, 1)
 // ---- slicing -----------------------------------------------------------------------
 // One CTA per 8 rows of a scale group (the packed blocks that share row
 // scales): the largest exponent of every row over all blocks of the group,
-// then the slices.  A warp handles 8 rows x 64 k of one block at a time, lane
-// l row l / 4 and the 16-byte pieces l % 4 and l % 4 + 4 (8 k each); the
-// elements of a warp's first tile stay in registers between the two passes,
-// any further tile is read again (from L2).  Integer arithmetic only: the
-// significand is shifted to the row scale and cut into digits.
+// then the slices.  A warp handles 8 rows x 64 k of one block at a time, lane l
+// k = 2 l and 2 l + 1 of every row, so that the reads of a row and the writes
+// of a slice's row are whole 128-byte lines; blocks stored with k as the slow
+// index go through shared memory.  The elements of a warp's first tile stay in
+// registers between the two passes, any further tile is read again (from L2).  Integer arithmetic only: the significand is shifted to the row
+// scale and cut into digits.  All operands of a stage that are at hand are
+// sliced by one launch.
 
 // Significand and exponent field of coef * x: |coef x| = m 2^(f - 1075)
 // (m < 2^53) when the coefficient is a power of two, else m 2^(f - 1086)
@@ -611,138 +641,181 @@ __device__ __forceinline__ unsigned long long digits(double x, const Coef& c, in
   return kBias + (neg ? 0ull - v : v);
 }
 
-__global__ void __launch_bounds__(256)
-    slice_kernel(const SlGroup* __restrict__ groups, int ngroups, const SlMember* __restrict__ members,
-                 const double* __restrict__ src, uint16_t* __restrict__ out,
-                 int32_t* __restrict__ scales, double scale) {
-  __shared__ int smax[8];
-  int gi = 0;
-  {
-    int lo = 0, hi = ngroups - 1;
-    const int b = (int)blockIdx.x;
-    while (lo < hi) {
-      const int mid = (lo + hi + 1) >> 1;
-      if (groups[mid].cta0 <= b) lo = mid;
-      else hi = mid - 1;
+constexpr int kTRow = 66;      // doubles per row of a transposed tile (64 + 2 pad)
+
+// x[2 r + h] = element (r0 + r, 64 c + 2 lane + h) of a block (0 outside its nr
+// rows and K columns); tile: the warp's shared memory.
+__device__ __forceinline__ void load_tile(const double* __restrict__ src, int64_t ld, int K, int trans,
+                                          int nr, int c, int lane, double* tile, double (&x)[16]) {
+  const int k = c * 64 + 2 * lane;
+  if (!trans) {
+    const double* p = src + k;
+#pragma unroll
+    for (int r = 0; r < 8; ++r) {
+      x[2 * r] = r < nr && k < K ? p[r * ld] : 0.0;
+      x[2 * r + 1] = r < nr && k + 1 < K ? p[r * ld + 1] : 0.0;
     }
-    gi = lo;
+  } else {
+    const double* p = src + (lane & 7);
+    double v[16];
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+      const int kk = c * 64 + 4 * i + (lane >> 3);
+      v[i] = (lane & 7) < nr && kk < K ? p[kk * ld] : 0.0;
+    }
+    __syncwarp();
+#pragma unroll
+    for (int i = 0; i < 16; ++i) tile[(lane & 7) * kTRow + 4 * i + (lane >> 3)] = v[i];
+    __syncwarp();
+#pragma unroll
+    for (int r = 0; r < 8; ++r) {
+      x[2 * r] = tile[r * kTRow + 2 * lane];
+      x[2 * r + 1] = tile[r * kTRow + 2 * lane + 1];
+    }
   }
-  const SlGroup gr = groups[gi];
-  const int g = (int)blockIdx.x - gr.cta0;
+}
+
+// The digits of row r of a tile (its scale f; zero: no digits): this lane's
+// pair of k, 4 bytes of the swizzled 16-byte piece lane / 4 of every slice.
+__device__ __forceinline__ void store_row(uint16_t* base, int64_t slice, int r, double x0, double x1,
+                                          const Coef& cf, bool zero, int f, int lane) {
+  const unsigned long long d0 = digits(zero ? 0.0 : x0, cf, zero ? 0 : f);
+  const unsigned long long d1 = digits(zero ? 0.0 : x1, cf, zero ? 0 : f);
+  uint16_t* row = base + r * 64 + (((lane >> 2) ^ r) << 3) + 2 * (lane & 3);
+#pragma unroll
+  for (int i = 0; i < kSlices; ++i) {
+    // digit + 256 in 0 .. 512: as FP16, 1024 + (digit + 256) has these bits
+    // exactly; one packed subtraction of 1280 leaves the digits
+    const uint32_t f0 = (uint32_t)(d0 >> (54 - 9 * i)) & (i == 0 ? 0x3FFu : 0x1FFu);
+    const uint32_t f1 = (uint32_t)(d1 >> (54 - 9 * i)) & (i == 0 ? 0x3FFu : 0x1FFu);
+    const uint32_t hw = (f0 | (f1 << 16)) | 0x64006400u;
+    uint32_t res;
+    asm("sub.rn.f16x2 %0, %1, %2;" : "=r"(res) : "r"(hw), "r"(0x65006500u));
+    *reinterpret_cast<uint32_t*>(row + i * slice) = res;
+  }
+}
+
+// The member of a group that holds its chunk t: lanes compare 32 members at a time
+// (a walk would wait for one table entry after the other).
+__device__ __forceinline__ int member_of(const SlMember* __restrict__ m, int nm, int t, int lane) {
+  int n = 0;
+  for (int b = 0; b < nm; b += 32) {
+    const bool le = b + lane < nm && m[b + lane].t0 <= t;
+    const int c = __popc(__ballot_sync(0xffffffffu, le));
+    n += c;
+    if (c < 32) break;
+  }
+  return n - 1;
+}
+
+__global__ void __launch_bounds__(256, 3)
+    slice_kernel(const SlGroup* __restrict__ groups, const int32_t* __restrict__ cta_group,
+                 const SlMember* __restrict__ members, int cta0,
+                 const __grid_constant__ SlOperands ops) {
+  __shared__ int smax[8];
+  __shared__ double tr[8][8 * kTRow];
+  const int cta = cta0 + (int)blockIdx.x;
+  const SlGroup gr = groups[cta_group[cta]];
+  const SlOperand op = ops.op[gr.which];
+  const SlMember* __restrict__ mem = members + gr.m0;
+  const int r0 = (cta - gr.cta0) * 8, nr = min(8, gr.R - r0);      // rows of this CTA (<= 0: padding)
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int rr = lane >> 2, j4 = lane & 3, r = g * 8 + rr;
+  for (int i = (int)(blockIdx.x * blockDim.x + threadIdx.x); i < ops.nclear; i += (int)(gridDim.x * blockDim.x))
+    ops.clear[i] = 0;
   if (threadIdx.x < 8) smax[threadIdx.x] = kMinField;
   __syncthreads();
-  auto load = [&](const SlMember& mb, int c, double (&x)[16]) {
-#pragma unroll
-    for (int h = 0; h < 2; ++h)
-#pragma unroll
-      for (int q = 0; q < 8; ++q) {
-        const int k = c * 64 + (j4 + 4 * h) * 8 + q;
-        double v = 0.0;
-        if (r < gr.R && k < mb.K)
-          v = mb.trans ? src[mb.src + (int64_t)k * mb.ld + r] : src[mb.src + (int64_t)r * mb.ld + k];
-        x[h * 8 + q] = v;
-      }
+  auto load = [&](const SlMember& mb, int t, double (&x)[16]) {
+    load_tile(op.src + mb.src + (mb.trans ? (int64_t)r0 : (int64_t)r0 * mb.ld), mb.ld, mb.K, mb.trans, nr,
+              t - mb.t0, lane, tr[warp], x);
   };
-  double keep[16];
-  int kept_m = -1, kept_c = -1;
-  int mx = kMinField;
-  {
-    // tiles (member, chunk) of the group, warp-strided
-    int t = warp;
-    for (int m = 0; m < gr.nm; ++m) {
-      const SlMember mb = members[gr.m0 + m];
-      if (t >= mb.KC) {
-        t -= mb.KC;
-        continue;
-      }
-      const Coef cf = make_coef(mb.coef * scale);
-      for (; t < mb.KC; t += 8) {
-        double x[16];
-        load(mb, t, x);
-        if (cf.bad) mx = kSlSpecial;
+  double x[16];
+  if (nr > 0) {
+    int mx[8];
 #pragma unroll
-        for (int e = 0; e < 16; ++e) mx = max(mx, eff_field(x[e], cf));
-        if (kept_m < 0) {
-          kept_m = m;
-          kept_c = t;
+    for (int r = 0; r < 8; ++r) mx[r] = kMinField;
+    // the warp's chunks, the last one first: the first stays in registers
+    const int last = gr.nt > warp ? warp + (gr.nt - 1 - warp) / 8 * 8 : -1;
+    for (int t = last; t >= 0; t -= 8) {
+      const SlMember mb = mem[member_of(mem, gr.nm, t, lane)];
+      const Coef cf = make_coef(mb.coef * op.scale);
+      load(mb, t, x);
 #pragma unroll
-          for (int e = 0; e < 16; ++e) keep[e] = x[e];
-        }
-      }
-      t -= mb.KC;
+      for (int e = 0; e < 16; ++e)
+        mx[e >> 1] = max(mx[e >> 1], cf.bad ? kSlSpecial : eff_field(x[e], cf));
+    }
+#pragma unroll
+    for (int r = 0; r < 8; ++r) {
+      const int w = __reduce_max_sync(0xffffffffu, mx[r]);
+      if (lane == r && w != kMinField) atomicMax(&smax[r], w);
     }
   }
-  mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
-  mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
-  if (j4 == 0) atomicMax(&smax[rr], mx);
   __syncthreads();
-  const int F = smax[rr] + gr.shift;
-  if (threadIdx.x < 8 && g * 8 + (int)threadIdx.x < gr.R) {
+  if ((int)threadIdx.x < nr) {
     const int v = smax[threadIdx.x];
-    scales[gr.e0 + g * 8 + threadIdx.x] = v == kMinField ? 0 : v == kSlSpecial ? v : v + gr.shift;
+    op.scales[gr.e0 + r0 + threadIdx.x] = v == kMinField ? 0 : v;
   }
-  const bool zero = smax[rr] == kMinField || smax[rr] == kSlSpecial;
-  int t = warp;
-  for (int m = 0; m < gr.nm; ++m) {
-    const SlMember mb = members[gr.m0 + m];
-    if (t >= mb.KC) {
-      t -= mb.KC;
-      continue;
+  for (int t = warp; t < gr.nt; t += 8) {
+    const SlMember mb = mem[member_of(mem, gr.nm, t, lane)];
+    const Coef cf = make_coef(mb.coef * op.scale);
+    if (t != warp || nr <= 0) load(mb, t, x);
+    uint16_t* base = op.out + mb.dst + ((int64_t)(t - mb.t0) * kSlices * gr.R8 + (r0 >> 3)) * kSlTile;
+#pragma unroll
+    for (int r = 0; r < 8; ++r) {
+      const int f = smax[r];             // zero rows and rows with Inf or NaN have no digits
+      store_row(base, (int64_t)gr.R8 * kSlTile, r, x[2 * r], x[2 * r + 1], cf,
+                f == kMinField || f == kSlSpecial, f + gr.shift, lane);
     }
-    const Coef cf = make_coef(mb.coef * scale);
-    for (; t < mb.KC; t += 8) {
-      double x[16];
-      if (m == kept_m && t == kept_c) {
+  }
+}
+
+// Known row scales (the products that wrote the blocks collected them): one
+// pass, a warp per tile.
+__global__ void __launch_bounds__(256)
+    slice_known_kernel(const SlPiece* __restrict__ pieces, int npieces,
+                       const int32_t* __restrict__ first, int ntiles, const double* __restrict__ src,
+                       uint16_t* __restrict__ out, const int32_t* __restrict__ scales) {
+  __shared__ double tr[8][8 * kTRow];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int t = (int)blockIdx.x * 8 + warp;
+  if (t >= ntiles) return;
+  int pi = first[blockIdx.x];
+  while (pi + 1 < npieces && pieces[pi + 1].tile0 <= t) ++pi;
+  const SlPiece p = pieces[pi];
+  const int local = t - p.tile0, c = local / p.R8, g = local - c * p.R8;
+  const int r0 = g * 8, nr = min(8, p.R - r0);
+  const int fl = lane < nr ? scales[p.e0 + r0 + lane] : 0;
+  double x[16];
+  load_tile(src + p.src + (p.trans ? (int64_t)r0 : (int64_t)r0 * p.ld), p.ld, p.K, p.trans, nr, c, lane,
+            tr[warp], x);
+  const Coef cf{1ull << 63, 1023, true, false, false};     // no coefficient
+  uint16_t* base = out + p.dst + ((int64_t)c * kSlices * p.R8 + g) * kSlTile;
 #pragma unroll
-        for (int e = 0; e < 16; ++e) x[e] = keep[e];
-      } else {
-        load(mb, t, x);
-      }
-      uint16_t* base = out + mb.dst + ((int64_t)t * kSlices * gr.R8 + g) * kSlTile + rr * 64;
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        uint32_t w[kSlices][4];
-#pragma unroll
-        for (int q = 0; q < 8; q += 2) {
-          const unsigned long long d0 = digits(zero ? 0.0 : x[h * 8 + q], cf, zero ? 0 : F);
-          const unsigned long long d1 = digits(zero ? 0.0 : x[h * 8 + q + 1], cf, zero ? 0 : F);
-#pragma unroll
-          for (int i = 0; i < kSlices; ++i) {
-            // digit + 256 in 0 .. 512: as FP16, 1024 + (digit + 256) has these
-            // bits exactly; one packed subtraction of 1280 leaves the digits
-            const uint32_t f0 = (uint32_t)(d0 >> (54 - 9 * i)) & (i == 0 ? 0x3FFu : 0x1FFu);
-            const uint32_t f1 = (uint32_t)(d1 >> (54 - 9 * i)) & (i == 0 ? 0x3FFu : 0x1FFu);
-            const uint32_t hw = (f0 | (f1 << 16)) | 0x64006400u;
-            uint32_t res;
-            asm("sub.rn.f16x2 %0, %1, %2;" : "=r"(res) : "r"(hw), "r"(0x65006500u));
-            w[i][q >> 1] = res;
-          }
-        }
-        const int pos = ((j4 + 4 * h) ^ rr) << 3;       // swizzled 16-byte piece
-#pragma unroll
-        for (int i = 0; i < kSlices; ++i)
-          *reinterpret_cast<uint4*>(base + (int64_t)i * gr.R8 * kSlTile + pos) =
-              make_uint4(w[i][0], w[i][1], w[i][2], w[i][3]);
-      }
-    }
-    t -= mb.KC;
+  for (int r = 0; r < 8; ++r) {
+    const int f = __shfl_sync(0xffffffffu, fl, r);
+    store_row(base, (int64_t)p.R8 * kSlTile, r, x[2 * r], x[2 * r + 1], cf, f == 0 || f == kSlSpecial,
+              f + p.shift, lane);
   }
 }
 
 }  // namespace
 
-void launch_slice(const SlGroup* groups, int ngroups, int nctas, const SlMember* members,
-                  const double* src, uint16_t* out, int32_t* scales, double scale, cudaStream_t st) {
+void launch_slice(const SlGroup* groups, const int32_t* cta_group, int cta0, int nctas,
+                  const SlMember* members, const SlOperands& ops, cudaStream_t st) {
   if (nctas <= 0) return;
   count_launch();
-  slice_kernel<<<nctas, 256, 0, st>>>(groups, ngroups, members, src, out, scales, scale);
+  slice_kernel<<<nctas, 256, 0, st>>>(groups, cta_group, members, cta0, ops);
+}
+
+void launch_slice_known(const SlPiece* pieces, int npieces, const int32_t* first, int ntiles,
+                        const double* src, uint16_t* out, const int32_t* scales, cudaStream_t st) {
+  if (ntiles <= 0) return;
+  count_launch();
+  slice_known_kernel<<<(ntiles + 7) / 8, 256, 0, st>>>(pieces, npieces, first, ntiles, src, out, scales);
 }
 
 void launch_gemm_sliced(const SlTables& t, const uint16_t* pA, const uint16_t* pB,
-                        const int32_t* eA, const int32_t* eB, const double* A, const double* B,
-                        Trans ta, Trans tb, double scale, double* C, int* err, uint64_t wait_ns,
+                        const int32_t* eA, const int32_t* eB, const SlSource& src, double* C,
+                        int32_t* collect, bool collect_cols, int* err, uint64_t wait_ns,
                         cudaStream_t st) {
   if (t.ncta <= 0) return;
   // the shared-memory limit is a per-device attribute of the kernel
@@ -756,10 +829,8 @@ void launch_gemm_sliced(const SlTables& t, const uint16_t* pA, const uint16_t* p
     if (bit) done.fetch_or(bit);
   }
   count_launch();
-  gemm_sliced_kernel<<<t.ncta, kThreads, kSmemBytes, st>>>(t, pA, pB, eA, eB, A, B,
-                                                           ta == Trans::T ? 1 : 0,
-                                                           tb == Trans::T ? 1 : 0, scale, C, err,
-                                                           wait_ns);
+  gemm_sliced_kernel<<<t.ncta, kThreads, kSmemBytes, st>>>(t, pA, pB, eA, eB, src, C, collect,
+                                                           collect_cols ? 1 : 0, err, wait_ns);
 }
 
 }  // namespace dmrg3s

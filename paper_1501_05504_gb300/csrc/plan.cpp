@@ -48,6 +48,21 @@ void GemmStage::finalize_bytes(Trans, Trans) {
   bytes = 8.0 * elems;
 }
 
+void SliceTable::add(const std::vector<SlGroup>& g, const std::vector<SlMember>& m) {
+  const int32_t which = (int32_t)cta.size() - 1, m0 = (int32_t)members.size();
+  int32_t at = cta.back();
+  for (SlGroup q : g) {
+    q.which = which;
+    q.m0 += m0;
+    q.cta0 = at;
+    at += q.R8;
+    cta_group.insert(cta_group.end(), q.R8, (int32_t)groups.size());
+    groups.push_back(q);
+  }
+  members.insert(members.end(), m.begin(), m.end());
+  cta.push_back(at);
+}
+
 void CombStage::add(int64_t offOut, int ldo, int rows, int cols, const std::vector<CombTerm>& t) {
   if (rows <= 0 || cols <= 0) return;
   CombTask task{};
@@ -419,6 +434,7 @@ struct Slicer {
   struct Blk {
     SlMember m;
     int32_t R, spans;      // spans: of the longest task that uses the block
+    int32_t shift;         // of its group (at the group's first block)
   };
   std::vector<Blk> blks;
   std::vector<int> parent;
@@ -452,7 +468,7 @@ struct Slicer {
   }
   static int32_t groups(int64_t R) { return (int32_t)((R + 15) / 16 * 2); }
   // Places every block and group; e0[block] = first scale of its group.
-  void layout(bool headroom, std::vector<SlGroup>* g, std::vector<SlMember>* m, int64_t* n, int32_t* ctas,
+  void layout(bool headroom, std::vector<SlGroup>* g, std::vector<SlMember>* m, int64_t* n,
               int32_t* ne, std::vector<int32_t>* e0) {
     std::map<int, std::vector<int>> by;
     for (int i = 0; i < (int)blks.size(); ++i) by[find(i)].push_back(i);
@@ -464,18 +480,19 @@ struct Slicer {
       gr.m0 = (int32_t)m->size();
       gr.nm = (int32_t)kv.second.size();
       gr.e0 = *ne;
-      gr.cta0 = *ctas;
       int spans = 0;
       for (int i : kv.second) spans = std::max(spans, blks[i].spans);
       while (headroom && spans > kSlSpans << gr.shift) ++gr.shift;
+      blks[kv.first].shift = gr.shift;
       for (int i : kv.second) {
+        blks[i].m.t0 = gr.nt;
+        gr.nt += blks[i].m.KC;
         blks[i].m.dst = *n;
         *n += (int64_t)gr.R8 * blks[i].m.KC * kSlices * kSlTile;
         (*e0)[i] = gr.e0;
         m->push_back(blks[i].m);
       }
       *ne += gr.R;
-      *ctas += gr.R8;
       g->push_back(gr);
     }
   }
@@ -514,8 +531,8 @@ bool build_sliced(const GemmStage& g, bool coefA, SlStage* out, std::string* err
       return false;
     }
   std::vector<int32_t> ea, eb;
-  a.layout(true, &s.gA, &s.mA, &s.nA, &s.ctasA, &s.neA, &ea);
-  b.layout(false, &s.gB, &s.mB, &s.nB, &s.ctasB, &s.neB, &eb);
+  a.layout(true, &s.gA, &s.mA, &s.nA, &s.neA, &ea);
+  b.layout(false, &s.gB, &s.mB, &s.nB, &s.neB, &eb);
   for (const GemmSeg& q : g.segs) s.segs.push_back(SlSeg{q.offA, q.offB, q.scale, q.lda, q.ldb, q.K, 0});
   // narrower units when the 64-wide ones leave SMs without work
   auto count = [&](int tn) {
@@ -556,6 +573,7 @@ bool build_sliced(const GemmStage& g, bool coefA, SlStage* out, std::string* err
     for (int32_t ui = cta[c]; ui < cta[c + 1]; ++ui) {
       const GemmTask& t = g.tasks[units[ui].task];
       SlUnit un{};
+      un.em = -1;
       un.m0 = units[ui].tm * 128;
       un.n0 = units[ui].tn * tile_n;
       un.offC = t.offC + (int64_t)un.m0 * t.ldc + un.n0;
@@ -568,6 +586,7 @@ bool build_sliced(const GemmStage& g, bool coefA, SlStage* out, std::string* err
       if (t.nseg > 0) {
         un.ea = ea[ia[t.seg0]] + un.m0;
         un.eb = eb[ib[t.seg0]] + un.n0;
+        un.shift = a.blks[a.find(ia[t.seg0])].shift;
       }
       const int ra8 = Slicer::groups(t.M), rb8 = Slicer::groups(t.N);
       const size_t first = s.words.size();
@@ -701,6 +720,52 @@ void rechunk(CombStage& c, int target) {
   }
 }
 
+// The stage-2 output as stage 3's operand: its blocks as pieces, and where
+// every unit of stage 2 collects its row scales (EnvLR: its columns' scales).
+bool plan_t2(Plan* p, const std::vector<SlGroup>& groups, const std::vector<SlMember>& members,
+             std::string* err) {
+  std::map<int64_t, int32_t> e0;       // block offset -> its first row scale
+  for (const SlGroup& g : groups)
+    for (int k = 0; k < g.nm; ++k) {
+      const SlMember& m = members[g.m0 + k];
+      SlPiece q{};
+      q.src = m.src;
+      q.dst = m.dst;
+      q.ld = m.ld;
+      q.K = m.K;
+      q.KC = m.KC;
+      q.trans = m.trans;
+      q.R = g.R;
+      q.R8 = g.R8;
+      q.e0 = g.e0;
+      q.shift = g.shift;
+      q.tile0 = p->t2_tiles;
+      p->t2_tiles += g.R8 * m.KC;
+      p->t2.push_back(q);
+      if (!e0.emplace(m.src, g.e0).second) {
+        *err = "sliced stage: a stage-2 block with two sets of scales";
+        return false;
+      }
+    }
+  int32_t at = 0;
+  for (int32_t t = 0; t < p->t2_tiles; t += 8) {
+    while (at + 1 < (int32_t)p->t2.size() && p->t2[at + 1].tile0 <= t) ++at;
+    p->t2_first.push_back(at);
+  }
+  const bool cols = p->kind == Kind::EnvLR;
+  for (SlUnit& u : p->s12.units) {
+    // the unit's block: its offset less the unit's place in it
+    const auto it = e0.find(u.offC - (int64_t)u.m0 * u.ldc - u.n0);
+    u.em = it == e0.end() ? -1 : it->second + (cols ? u.n0 : u.m0);
+    const int32_t ne = p->kind == Kind::Heff ? p->s3.neA : p->s3.neB;
+    if (u.em >= 0 && u.em + (cols ? u.cols : u.rows) > ne) {
+      *err = "sliced stage: collected scales out of bounds";
+      return false;
+    }
+  }
+  return true;
+}
+
 // Least algorithmic work of a contraction that takes the sliced form.
 constexpr double kSlicedMinFlops = 2e6;
 // Largest ratio of the fused stage's work to stage 1's: the sliced products
@@ -739,6 +804,14 @@ dmrg3s_status finish_sliced(Plan* p, int64_t nA1, int64_t nB1, int64_t nOut2, in
     }
     ok = ok && build_sliced(p->f3, true, &p->s3, err) &&
          sliced_ok(p->f3, p->s3, nA3, nB3, G > 1 ? std::max<int64_t>(p->ws3s, 1) : nC3, err);
+  }
+  if (ok) {
+    const bool t2_is_a = p->kind == Kind::Heff;
+    p->slices.add(left ? p->s12.gA : p->s12.gB, left ? p->s12.mA : p->s12.mB);
+    p->slices.add(t2_is_a ? p->s3.gB : p->s3.gA, t2_is_a ? p->s3.mB : p->s3.mA);
+    p->slices.add(left ? p->s12.gB : p->s12.gA, left ? p->s12.mB : p->s12.mA);
+    ok = slice_table_ok(p->slices, err);
+    if (ok && p->has_g3) ok = plan_t2(p, t2_is_a ? p->s3.gA : p->s3.gB, t2_is_a ? p->s3.mA : p->s3.mB, err);
   }
   if (!ok) {
     *err = "internal planning error: " + *err;
@@ -1141,6 +1214,47 @@ dmrg3s_status plan_mpo_grad(const EnvLayout& le, const MpoLayout& W, const EnvLa
       !gemm_ok(p->gy.ta, p->gy.tb, p->gy.tasks, p->gy.segs, M.size, re.size, wy, err)) {
     *err = "internal planning error: " + *err;
     return DMRG3S_ERR_SHAPE;
+  }
+  // sliced form over the virtual operand arrays A = [L | M], B = [M | R] and
+  // the output [T1 | Y]; then each operand's blocks back to its own array
+  p->sliced = false;
+  if (p->flops() >= kSlicedMinFlops) {
+    const int64_t nL = le.size, nM = M.size, nR = re.size;
+    GemmStage g;
+    g.ta = p->g1.ta;
+    g.tb = p->g1.tb;
+    append_gemm(g, p->g1, 0, 0, 0);
+    append_gemm(g, p->gy, nL, nM, w1);
+    bool ok = p->g1.ta == p->gy.ta && p->g1.tb == p->gy.tb && build_sliced(g, true, &p->s, err) &&
+              sliced_ok(g, p->s, nL + nM, nM + nR, w1 + wy, err);
+    auto split = [&](std::vector<SlGroup>& gs, std::vector<SlMember>& ms, int64_t n0) {
+      std::vector<SlGroup> ga, gb;
+      for (SlGroup q : gs) {
+        const bool second = ms[q.m0].src >= n0;
+        for (int k = 0; k < q.nm; ++k) {
+          ok = ok && (ms[q.m0 + k].src >= n0) == second;
+          if (second) ms[q.m0 + k].src -= n0;
+        }
+        (second ? gb : ga).push_back(q);
+      }
+      p->slices.add(ga, ms);
+      p->slices.add(gb, ms);
+    };
+    if (ok) {
+      split(p->s.gA, p->s.mA, nL);
+      split(p->s.gB, p->s.mB, nM);
+      for (size_t k = p->g1.segs.size(); k < p->s.segs.size(); ++k) {
+        p->s.segs[k].offA -= nL;
+        p->s.segs[k].offB -= nM;
+      }
+      for (SlUnit& u : p->s.units) u.sel = u.seg0 >= (int32_t)p->g1.segs.size() ? 1 : 0;
+      ok = slice_table_ok(p->slices, err);
+    }
+    if (!ok) {
+      *err = "internal planning error: " + *err;
+      return DMRG3S_ERR_SHAPE;
+    }
+    p->sliced = true;
   }
   for (const DotSeg& g : p->segs)
     if (g.offA < 0 || g.offB < 0 || g.len < 0 || g.offA + g.len > p->ws1 ||

@@ -50,11 +50,20 @@ struct SlStage {
   std::vector<SlChunk> chunks;          // grouped by CTA, in the order of its units
   std::vector<uint32_t> words;          // one per chunk
   std::vector<int32_t> cta_unit, cta_chunk;
-  std::vector<SlGroup> gA, gB;
+  std::vector<SlGroup> gA, gB;          // (moved into a SliceTable)
   std::vector<SlMember> mA, mB;
   int64_t nA = 0, nB = 0;               // FP16 elements of each packed operand
-  int32_t ctasA = 0, ctasB = 0;         // CTAs of the slicing launches
   int32_t neA = 0, neB = 0;             // row scales of each operand
+};
+
+// The slicing of several operands: operand i (SlGroup.which) has the CTAs
+// [cta[i], cta[i + 1]), so that a launch over a range slices some or all.
+struct SliceTable {
+  std::vector<SlGroup> groups;
+  std::vector<SlMember> members;
+  std::vector<int32_t> cta_group;       // group of every CTA
+  std::vector<int32_t> cta{0};
+  void add(const std::vector<SlGroup>& g, const std::vector<SlMember>& m);
 };
 
 struct GemmStage {
@@ -117,8 +126,15 @@ struct Plan {
   // term, scaled by its coefficient; the output is the stage-2 output in FP64),
   // stage 3 split-K into FP64 partial blocks and a sum (no split: written to
   // the output directly).  sliced = false: too little work (plan.cpp).
+  // slices: operand 0 = stage 1's environment (L, R), 1 = stage 3's operand that
+  // is at hand (R, M), 2 = stage 1's site tensor.  The stage-2 output is sliced
+  // piece by piece (t2), its row scales collected by stage 2.
   GemmStage f12, f3;
   SlStage s12, s3;
+  SliceTable slices;
+  std::vector<SlPiece> t2;
+  std::vector<int32_t> t2_first;   // piece of every eighth tile
+  int32_t t2_tiles = 0;
   CombStage s3r;                // sum of the partials (empty: no split)
   int64_t ws3s = 0;             // doubles of the partial blocks
   bool sliced = false;
@@ -178,6 +194,11 @@ struct GradPlan {
   std::vector<DotTask> tasks;     // one per entry of G, row-major [s'][s][bl][br]
   std::vector<DotSeg> segs;       // A = ws1, B = wsy
   int64_t ws1 = 0, wsy = 0, nG = 0;
+  // sliced form: g1 and gy as one grouped GEMM (A = L or M, B = M or R; the
+  // outputs T1 and Y back to back); slices: L, M (A), M (B), R
+  SlStage s;
+  SliceTable slices;
+  bool sliced = false;
   double dot_flops = 0.0;
   double flops() const { return g1.flops + gy.flops + dot_flops; }
 };

@@ -1688,11 +1688,10 @@ dmrg3s_status grad_all(State* S, cudaStream_t st, std::vector<double>* hGout,
   // environment of the current tensors on the far side of the centre
   auto grad_at = [&](int i, const EnvLayout& ll, const double* L, const EnvLayout& rl,
                      const double* R) -> dmrg3s_status {
-    GradPlan p;
-    std::string err;
-    dmrg3s_status r = plan_mpo_grad(ll, S->W[i], rl, S->M[i].lay, &p, &err);
-    if (r) return fail(c, r, "site " + std::to_string(i) + ": " + err);
-    return run_mpo_grad(c, p, L, S->M[i].data, R, dG + goff[i], st);
+    const DeviceGradPlan* p = nullptr;
+    dmrg3s_status r = grad_plan(c, ll, S->W[i], rl, S->M[i].lay, &p);
+    if (r) return fail(c, r, "site " + std::to_string(i) + ": " + c->last_error);
+    return run_mpo_grad(c, *p, L, S->M[i].data, R, dG + goff[i], st);
   };
   s = grad_at(cen, S->Lenv[cen].lay, S->Lenv[cen].data, S->Renv[cen].lay, S->Renv[cen].data);
   for (int dir = -1; dir <= 1 && !s; dir += 2) {

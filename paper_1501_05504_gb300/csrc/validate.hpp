@@ -130,28 +130,44 @@ inline bool tc_ok(const std::vector<GemmTask>& tasks, const TcStage& tc, int64_t
 // Sliced FP64 tables: every source view, packed block, row scale, bulk copy and
 // output inside its array.
 inline bool slices_ok(const std::vector<SlGroup>& g, const std::vector<SlMember>& m, int64_t nSrc,
-                      int64_t nPacked, int32_t ctas, int32_t ne, std::string* err) {
-  int32_t at = 0;
+                      int64_t nPacked, int32_t ne, std::string* err) {
   for (const SlGroup& q : g) {
     bool ok = q.R > 0 && q.R8 * 8 >= q.R && q.R8 % 2 == 0 && q.m0 >= 0 && q.nm > 0 &&
-              (size_t)q.m0 + q.nm <= m.size() && q.e0 >= 0 && q.e0 + q.R <= ne && q.cta0 == at &&
-              q.shift >= 0 && q.shift < 16;
-    at += q.R8;
+              (size_t)q.m0 + q.nm <= m.size() && q.e0 >= 0 && q.e0 + q.R <= ne && q.shift >= 0 &&
+              q.shift < 16;
+    int32_t t = 0;
     for (int k = 0; ok && k < q.nm; ++k) {
       const SlMember& b = m[q.m0 + k];
       const int64_t last = b.trans ? (int64_t)(b.K - 1) * b.ld + q.R - 1
                                    : (int64_t)(q.R - 1) * b.ld + b.K - 1;
       ok = b.K > 0 && span_ok(b.src, last, nSrc) && b.ld >= (b.trans ? q.R : b.K) &&
            (int64_t)b.KC * 64 >= b.K && b.dst >= 0 && b.dst % kSlTile == 0 &&
-           b.dst + (int64_t)q.R8 * b.KC * kSlices * kSlTile <= nPacked;
+           b.dst + (int64_t)q.R8 * b.KC * kSlices * kSlTile <= nPacked && b.t0 == t;
+      t += b.KC;
     }
+    ok = ok && t == q.nt;
     if (!ok) {
       *err = "sliced operand out of bounds";
       return false;
     }
   }
-  if (at != ctas) {
-    *err = "sliced operand launch";
+  return true;
+}
+
+inline bool slice_table_ok(const SliceTable& t, std::string* err) {
+  int32_t at = 0;
+  bool ok = t.cta.size() >= 2 && t.cta.size() <= 5 && t.cta.front() == 0 &&
+            (int32_t)t.cta_group.size() == t.cta.back();
+  for (const SlGroup& q : t.groups) {
+    ok = ok && q.cta0 == at && q.which >= 0 && (size_t)q.which + 1 < t.cta.size() &&
+         q.cta0 >= t.cta[q.which] && q.cta0 + q.R8 <= t.cta[q.which + 1] && q.m0 >= 0 &&
+         (size_t)q.m0 + q.nm <= t.members.size();
+    for (int32_t c = at; ok && c < at + q.R8; ++c)
+      ok = t.cta_group[c] == (int32_t)(&q - t.groups.data());
+    at += q.R8;
+  }
+  if (!ok || at != t.cta.back()) {
+    *err = "slicing table";
     return false;
   }
   return true;
@@ -160,8 +176,8 @@ inline bool slices_ok(const std::vector<SlGroup>& g, const std::vector<SlMember>
 inline bool sliced_ok(const GemmStage& g, const SlStage& s, int64_t nA, int64_t nB, int64_t nC,
                       std::string* err) {
   if (!gemm_ok(g.ta, g.tb, g.tasks, g.segs, nA, nB, nC, err) ||
-      !slices_ok(s.gA, s.mA, nA, s.nA, s.ctasA, s.neA, err) ||
-      !slices_ok(s.gB, s.mB, nB, s.nB, s.ctasB, s.neB, err))
+      !slices_ok(s.gA, s.mA, nA, s.nA, s.neA, err) ||
+      !slices_ok(s.gB, s.mB, nB, s.nB, s.neB, err))
     return false;
   bool ok = s.segs.size() == g.segs.size() && s.words.size() == s.chunks.size() &&
             s.cta_unit.size() == s.cta_chunk.size() &&
