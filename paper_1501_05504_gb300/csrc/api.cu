@@ -3,6 +3,7 @@
 #include <new>
 
 #include "context.hpp"
+#include "launch.hpp"
 #include "dmrg3s.h"
 
 using namespace dmrg3s;
@@ -47,7 +48,8 @@ DeviceGradPlan::~DeviceGradPlan() {
 
 SlTables sliced_tables(const DeviceSliced& d, const SlStage& s) {
   return SlTables{d.units,    d.chunks, d.words, d.cta_unit, d.cta_chunk, d.segs,
-                  s.cta_unit.empty() ? 0 : (int)s.cta_unit.size() - 1};
+                  s.cta_unit.empty() ? 0 : (int)s.cta_unit.size() - 1,
+                  s.chunks.size() <= (size_t)kChainChunks * s.cta_unit.size()};
 }
 
 namespace {
@@ -268,7 +270,7 @@ dmrg3s_status run_plan(Context* c, const DevicePlan& p, const double* g1A, const
       const int id = pr.on ? pr.begin(kProfGemm, h.g12.flops, h.g12.bytes, st) : -1;
       launch_gemm_tc(passes, true, p.g12_units, p.g12_cta, (int)t12.cta_start.size() - 1,
                      p.g12_tasks, p.g12_tsegs, aH, aL, hi(sl.b1), lo(sl.b1, t12.nB), hi(sl.t2p),
-                     lo(sl.t2p, h.nT2p), c->d_err, c->wait_ns, st);
+                     lo(sl.t2p, h.nT2p), c->d_err, c->wait_ns, t12.chain, st);
       if (id >= 0) pr.end(id, st);
     }
   } else {
@@ -282,7 +284,7 @@ dmrg3s_status run_plan(Context* c, const DevicePlan& p, const double* g1A, const
       launch_gemm_tc(passes, false, p.g1_units, p.g1_cta, (int)t1.cta_start.size() - 1,
                      p.g1_tasks, p.g1_tsegs,
                      hi(sl.a1), lo(sl.a1, t1.nA), hi(sl.b1), lo(sl.b1, t1.nB),
-                     reinterpret_cast<float*>(t1p), nullptr, c->d_err, c->wait_ns, st);
+                     reinterpret_cast<float*>(t1p), nullptr, c->d_err, c->wait_ns, t1.chain, st);
       if (id >= 0) pr.end(id, st);
     }
   }
@@ -330,7 +332,7 @@ dmrg3s_status run_plan(Context* c, const DevicePlan& p, const double* g1A, const
     launch_gemm_tc(passes, false, p.g3s_units, p.g3s_cta, (int)t3.cta_start.size() - 1,
                    p.g3s_tasks, p.g3s_tsegs,
                    a3h, a3l, b3h, b3l, reinterpret_cast<float*>(part), nullptr, c->d_err,
-                   c->wait_ns, st);
+                   c->wait_ns, t3.chain, st);
     if (id >= 0) pr.end(id, st);
   }
   if (!h.c3r.chunks.empty()) {

@@ -14,6 +14,7 @@
 #include "context.hpp"
 #include "dmrg3s.h"
 #include "kernels.hpp"
+#include "launch.hpp"
 #include "vecops.hpp"
 
 namespace dmrg3s {
@@ -202,6 +203,7 @@ dmrg3s_status lanczos_batch(Context* c, const DevicePlan& heff, const double* Ld
   // the launches are issued directly so that each product is recorded.
   cudaGraphExec_t gexec = nullptr;
   if (!c->prof.on && c->cap) {
+    const PlainLaunches plain;
     cudaGraph_t graph = nullptr;
     bool ok = cudaStreamBeginCapture(c->cap, cudaStreamCaptureModeThreadLocal) == cudaSuccess;
     if (ok) {

@@ -192,6 +192,7 @@ struct SlTables {
   const int32_t *cta_unit, *cta_chunk;
   const SlSeg* segs;
   int ncta;
+  bool chain;       // short enough for a chained launch (launch.hpp)
 };
 struct SlSource {
   const double *A, *B, *A1, *B1;     // A1, B1: of the units with sel = 1
@@ -240,7 +241,7 @@ void launch_gemm_f64(Trans ta, Trans tb, const GemmTile* tiles, int ntiles, cons
 void launch_gemm_tc(int passes, bool packed, const TcUnit* units, const int32_t* cta_start,
                     int ncta, const GemmTask* tasks, const TcSeg* segs, const float* Ahi,
                     const float* Alo, const float* Bhi, const float* Blo, float* Chi, float* Clo,
-                    int* err, uint64_t wait_ns, cudaStream_t st);
+                    int* err, uint64_t wait_ns, bool chain, cudaStream_t st);
 
 // Packs FP64 blocks into tensor-core operands: hi = tf32(x), lo = tf32(x - hi)
 // (lo may be null), in the tile layout above.

@@ -8,6 +8,7 @@
 #include <atomic>
 
 #include "kernels.hpp"
+#include "launch.hpp"
 
 namespace dmrg3s {
 
@@ -19,9 +20,11 @@ template <Trans TA, Trans TB>
 __global__ void __launch_bounds__(NT) gemm_f64_kernel(const GemmTile* __restrict__ tiles,
                                                       const GemmTask* __restrict__ tasks,
                                                       const GemmSeg* __restrict__ segs,
-                                                      const double* __restrict__ A,
-                                                      const double* __restrict__ B,
-                                                      double* __restrict__ C) {
+                                                      const double* A,
+                                                      const double* B,
+                                                      double* C) {
+  grid_next();
+  grid_wait();
   __shared__ double As[BK][BM + 1];
   __shared__ double Bs[BK][BN + 1];
   const GemmTile tile = tiles[blockIdx.x];
@@ -103,9 +106,11 @@ __global__ void __launch_bounds__(NT) gemm_f64_kernel(const GemmTile* __restrict
 __global__ void __launch_bounds__(256) combine_f64_kernel(const CombChunk* __restrict__ chunks,
                                                          const CombTask* __restrict__ tasks,
                                                          const CombTerm* __restrict__ terms,
-                                                         const double* __restrict__ in,
-                                                         double* __restrict__ out,
+                                                         const double* in,
+                                                         double* out,
                                                          double scale) {
+  grid_next();
+  grid_wait();
   const CombChunk ch = chunks[blockIdx.x];
   const CombTask t = tasks[ch.task];
   const int n = ch.nrows * t.cols;
@@ -138,7 +143,7 @@ __device__ __forceinline__ void df_acc(float ch, float cl, float2 x, float& ah, 
 
 // sum_k coef_k in_k for output element (r, c) of a chunk's task, as a pair
 __device__ __forceinline__ void df_combine(const CombTask& t, const CombTerm* __restrict__ terms,
-                                           const float2* __restrict__ in, int r, int c, float sh,
+                                           const float2* in, int r, int c, float sh,
                                            float sl, float& ah, float& al) {
   ah = 0.f;
   al = 0.f;
@@ -156,8 +161,10 @@ __device__ __forceinline__ void df_combine(const CombTask& t, const CombTerm* __
 
 __global__ void __launch_bounds__(256) combine_pairs_f64_kernel(
     const CombChunk* __restrict__ chunks, const CombTask* __restrict__ tasks,
-    const CombTerm* __restrict__ terms, const float2* __restrict__ in, double* __restrict__ out,
+    const CombTerm* __restrict__ terms, const float2* in, double* out,
     float sh, float sl) {
+  grid_next();
+  grid_wait();
   const CombChunk ch = chunks[blockIdx.x];
   const CombTask t = tasks[ch.task];
   const int n = ch.nrows * t.cols;
@@ -178,9 +185,11 @@ std::atomic<int64_t> g_launches{0};
 constexpr int kDotPiece = 1024;
 __global__ void __launch_bounds__(256) dots_kernel(const DotTask* __restrict__ tasks,
                                                    const DotSeg* __restrict__ segs,
-                                                   const double* __restrict__ A,
-                                                   const double* __restrict__ B,
-                                                   double* __restrict__ out) {
+                                                   const double* A,
+                                                   const double* B,
+                                                   double* out) {
+  grid_next();
+  grid_wait();
   const DotTask t = tasks[blockIdx.x];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   double acc0 = 0.0, acc1 = 0.0, acc2 = 0.0, acc3 = 0.0;
@@ -227,13 +236,13 @@ void launch_gemm_f64(Trans ta, Trans tb, const GemmTile* tiles, int ntiles, cons
   count_launch();
   dim3 grid(ntiles), block(NT);
   if (ta == Trans::N && tb == Trans::N)
-    gemm_f64_kernel<Trans::N, Trans::N><<<grid, block, 0, st>>>(tiles, tasks, segs, A, B, C);
+    launch_chain(gemm_f64_kernel<Trans::N, Trans::N>, grid, block, 0, st, tiles, tasks, segs, A, B, C);
   else if (ta == Trans::N && tb == Trans::T)
-    gemm_f64_kernel<Trans::N, Trans::T><<<grid, block, 0, st>>>(tiles, tasks, segs, A, B, C);
+    launch_chain(gemm_f64_kernel<Trans::N, Trans::T>, grid, block, 0, st, tiles, tasks, segs, A, B, C);
   else if (ta == Trans::T && tb == Trans::N)
-    gemm_f64_kernel<Trans::T, Trans::N><<<grid, block, 0, st>>>(tiles, tasks, segs, A, B, C);
+    launch_chain(gemm_f64_kernel<Trans::T, Trans::N>, grid, block, 0, st, tiles, tasks, segs, A, B, C);
   else
-    gemm_f64_kernel<Trans::T, Trans::T><<<grid, block, 0, st>>>(tiles, tasks, segs, A, B, C);
+    launch_chain(gemm_f64_kernel<Trans::T, Trans::T>, grid, block, 0, st, tiles, tasks, segs, A, B, C);
 }
 
 void launch_combine_pairs_f64(const CombChunk* chunks, int nchunks, const CombTask* tasks,
@@ -242,7 +251,7 @@ void launch_combine_pairs_f64(const CombChunk* chunks, int nchunks, const CombTa
   if (nchunks <= 0) return;
   count_launch();
   const float sh = (float)scale, sl = (float)(scale - (double)sh);
-  combine_pairs_f64_kernel<<<nchunks, 256, 0, st>>>(chunks, tasks, terms, in, out, sh, sl);
+  launch_chain(combine_pairs_f64_kernel, nchunks, 256, 0, st, chunks, tasks, terms, in, out, sh, sl);
 }
 
 void launch_combine_f64(const CombChunk* chunks, int nchunks, const CombTask* tasks,
@@ -250,14 +259,14 @@ void launch_combine_f64(const CombChunk* chunks, int nchunks, const CombTask* ta
                         cudaStream_t st) {
   if (nchunks <= 0) return;
   count_launch();
-  combine_f64_kernel<<<nchunks, 256, 0, st>>>(chunks, tasks, terms, in, out, scale);
+  launch_chain(combine_f64_kernel, nchunks, 256, 0, st, chunks, tasks, terms, in, out, scale);
 }
 
 void launch_dots(const DotTask* tasks, int ntasks, const DotSeg* segs, const double* A,
                  const double* B, double* out, cudaStream_t st) {
   if (ntasks <= 0) return;
   count_launch();
-  dots_kernel<<<ntasks, 256, 0, st>>>(tasks, segs, A, B, out);
+  launch_chain(dots_kernel, ntasks, 256, 0, st, tasks, segs, A, B, out);
 }
 
 }  // namespace dmrg3s

@@ -43,6 +43,7 @@
 #include <cstdint>
 
 #include "kernels.hpp"
+#include "launch.hpp"
 #include "tc_common.cuh"
 
 namespace dmrg3s {
@@ -170,8 +171,8 @@ __device__ __noinline__ double fixed_to_f64_any(long long H, float L, int ex) {
 
 // One output element the plain way (rows or columns with Inf or NaN).
 __device__ __noinline__ double element_f64(const SlSeg* __restrict__ segs, int nseg,
-                                           const double* __restrict__ A,
-                                           const double* __restrict__ B, int ta, int tb, int m,
+                                           const double* A,
+                                           const double* B, int ta, int tb, int m,
                                            int n, double scale) {
   double acc = 0.0;
   for (int k = 0; k < nseg; ++k) {
@@ -188,11 +189,11 @@ __device__ __noinline__ double element_f64(const SlSeg* __restrict__ segs, int n
 }
 
 __global__ void __launch_bounds__(kThreads, 1)
-    gemm_sliced_kernel(const SlTables tab, const uint16_t* __restrict__ pA,
-                       const uint16_t* __restrict__ pB, const int32_t* __restrict__ eA,
-                       const int32_t* __restrict__ eB, const __grid_constant__ SlSource src,
-                       double* __restrict__ C, int32_t* __restrict__ collect, int collect_cols,
-                       int* __restrict__ err, uint64_t wait_ns) {
+    gemm_sliced_kernel(const SlTables tab, const uint16_t* pA,
+                       const uint16_t* pB, const int32_t* eA,
+                       const int32_t* eB, const __grid_constant__ SlSource src,
+                       double* C, int32_t* collect, int collect_cols,
+                       int* err, uint64_t wait_ns) {
   extern __shared__ __align__(1024) unsigned char smem[];
   __shared__ __align__(8) uint64_t afull[kSlots], aempty[kSlots], bfull[2], bempty[2];
   __shared__ __align__(8) uint64_t lfull[kSlices], lempty[kSlices], done;
@@ -229,6 +230,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = tmem_base;
   const WaitCtl wc{&abort_flag, err, wait_ns};
+  grid_wait();
 
   if (warp == 0) {
     // ---------------- bulk-copy producer ----------------
@@ -562,6 +564,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       __syncwarp();
     }
   }
+  grid_next();
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -645,7 +648,7 @@ constexpr int kTRow = 66;      // doubles per row of a transposed tile (64 + 2 p
 
 // x[2 r + h] = element (r0 + r, 64 c + 2 lane + h) of a block (0 outside its nr
 // rows and K columns); tile: the warp's shared memory.
-__device__ __forceinline__ void load_tile(const double* __restrict__ src, int64_t ld, int K, int trans,
+__device__ __forceinline__ void load_tile(const double* src, int64_t ld, int K, int trans,
                                           int nr, int c, int lane, double* tile, double (&x)[16]) {
   const int k = c * 64 + 2 * lane;
   if (!trans) {
@@ -712,12 +715,14 @@ __global__ void __launch_bounds__(256, 3)
     slice_kernel(const SlGroup* __restrict__ groups, const int32_t* __restrict__ cta_group,
                  const SlMember* __restrict__ members, int cta0,
                  const __grid_constant__ SlOperands ops) {
+  grid_next();
+  grid_wait();
   __shared__ int smax[8];
   __shared__ double tr[8][8 * kTRow];
   const int cta = cta0 + (int)blockIdx.x;
   const SlGroup gr = groups[cta_group[cta]];
   const SlOperand op = ops.op[gr.which];
-  const SlMember* __restrict__ mem = members + gr.m0;
+  const SlMember* mem = members + gr.m0;
   const int r0 = (cta - gr.cta0) * 8, nr = min(8, gr.R - r0);      // rows of this CTA (<= 0: padding)
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   for (int i = (int)(blockIdx.x * blockDim.x + threadIdx.x); i < ops.nclear; i += (int)(gridDim.x * blockDim.x))
@@ -772,8 +777,10 @@ __global__ void __launch_bounds__(256, 3)
 // pass, a warp per tile.
 __global__ void __launch_bounds__(256)
     slice_known_kernel(const SlPiece* __restrict__ pieces, int npieces,
-                       const int32_t* __restrict__ first, int ntiles, const double* __restrict__ src,
-                       uint16_t* __restrict__ out, const int32_t* __restrict__ scales) {
+                       const int32_t* __restrict__ first, int ntiles, const double* src,
+                       uint16_t* out, const int32_t* scales) {
+  grid_next();
+  grid_wait();
   __shared__ double tr[8][8 * kTRow];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int t = (int)blockIdx.x * 8 + warp;
@@ -803,14 +810,14 @@ void launch_slice(const SlGroup* groups, const int32_t* cta_group, int cta0, int
                   const SlMember* members, const SlOperands& ops, cudaStream_t st) {
   if (nctas <= 0) return;
   count_launch();
-  slice_kernel<<<nctas, 256, 0, st>>>(groups, cta_group, members, cta0, ops);
+  launch_chain(slice_kernel, nctas, 256, 0, st, groups, cta_group, members, cta0, ops);
 }
 
 void launch_slice_known(const SlPiece* pieces, int npieces, const int32_t* first, int ntiles,
                         const double* src, uint16_t* out, const int32_t* scales, cudaStream_t st) {
   if (ntiles <= 0) return;
   count_launch();
-  slice_known_kernel<<<(ntiles + 7) / 8, 256, 0, st>>>(pieces, npieces, first, ntiles, src, out, scales);
+  launch_chain(slice_known_kernel, (ntiles + 7) / 8, 256, 0, st, pieces, npieces, first, ntiles, src, out, scales);
 }
 
 void launch_gemm_sliced(const SlTables& t, const uint16_t* pA, const uint16_t* pB,
@@ -829,8 +836,8 @@ void launch_gemm_sliced(const SlTables& t, const uint16_t* pA, const uint16_t* p
     if (bit) done.fetch_or(bit);
   }
   count_launch();
-  gemm_sliced_kernel<<<t.ncta, kThreads, kSmemBytes, st>>>(t, pA, pB, eA, eB, src, C, collect,
-                                                           collect_cols ? 1 : 0, err, wait_ns);
+  const PlainLaunches plain(!t.chain);
+  launch_chain(gemm_sliced_kernel, t.ncta, kThreads, kSmemBytes, st, t, pA, pB, eA, eB, src, C, collect, collect_cols ? 1 : 0, err, wait_ns);
 }
 
 }  // namespace dmrg3s

@@ -49,6 +49,7 @@
 #include <cstdint>
 
 #include "kernels.hpp"
+#include "launch.hpp"
 #include "tc_common.cuh"
 
 namespace dmrg3s {
@@ -99,10 +100,10 @@ template <int kPasses, int kSpan, bool kPackedOut>
 __global__ void __launch_bounds__(kThreads, 1)
     gemm_tc_kernel(const TcUnit* __restrict__ units, const int32_t* __restrict__ cta_start,
                    const GemmTask* __restrict__ tasks,
-                   const TcSeg* __restrict__ segs, const float* __restrict__ Ahi,
-                   const float* __restrict__ Alo, const float* __restrict__ Bhi,
-                   const float* __restrict__ Blo, float* __restrict__ Chi,
-                   float* __restrict__ Clo, int* __restrict__ err, uint64_t wait_ns) {
+                   const TcSeg* __restrict__ segs, const float* Ahi,
+                   const float* Alo, const float* Bhi,
+                   const float* Blo, float* Chi,
+                   float* Clo, int* err, uint64_t wait_ns) {
   extern __shared__ __align__(1024) unsigned char smem[];
   constexpr bool kLo = kPasses == 3;
   constexpr uint32_t kTmemCols = 512;
@@ -143,6 +144,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = tmem_base;
   const WaitCtl wc{&abort_flag, err, wait_ns};
+  grid_wait();
   const int u_begin = cta_start[blockIdx.x], u_end = cta_start[blockIdx.x + 1];
   if (warp < kFirstDrainWarp) asm volatile("setmaxnreg.dec.sync.aligned.u32 56;" ::: "memory");
 
@@ -389,6 +391,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     if (kPackedOut && lane == 0) bulk_wait_all();   // the tile stores are complete
     __syncwarp();
   }
+  grid_next();
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -429,7 +432,7 @@ __device__ __forceinline__ bool split_bits(double x, float& hi, float& lo) {
 
 // Binary search: the block of tile `tile` (blocks in increasing tile0 order).
 template <class T>
-__device__ __forceinline__ int block_of_tile(const T* __restrict__ b, int n, int tile) {
+__device__ __forceinline__ int block_of_tile(const T* b, int n, int tile) {
   int lo = 0, hi = n - 1;
   while (lo < hi) {
     const int mid = (lo + hi + 1) >> 1;
@@ -443,7 +446,9 @@ __device__ __forceinline__ int block_of_tile(const T* __restrict__ b, int n, int
 // 16-byte chunk j (j = 0..7), stored at its swizzled position.
 __global__ void __launch_bounds__(256)
     pack_kernel(const PackBlock* __restrict__ blocks, int nblocks, int ntiles,
-                const double* __restrict__ src, float* __restrict__ hi, float* __restrict__ lo) {
+                const double* src, float* hi, float* lo) {
+  grid_next();
+  grid_wait();
   const int tile = blockIdx.x * 8 + (threadIdx.x >> 5);
   if (tile >= ntiles) return;
   const int lane = threadIdx.x & 31;
@@ -456,22 +461,25 @@ __global__ void __launch_bounds__(256)
   // applied in FP64 before the split
   const bool f64scale = b.scale != 1.0 && b.pow2 == 0.f;
   const float fs = b.pow2 != 0.f ? b.pow2 : 1.f;
+  double v[8];                   // every load before the first store
 #pragma unroll
   for (int j = 0; j < 8; ++j) {
     const int k = c * 32 + j * 4 + (lane & 3);
-    float h = 0.f, l = 0.f;
-    if (r < b.R && k < b.K) {
-      double x = b.trans ? src[b.src + (int64_t)k * b.ld + r] : src[b.src + (int64_t)r * b.ld + k];
-      if (f64scale) x *= b.scale;
-      if (!split_bits(x, h, l)) {
-        h = to_tf32((float)x);
-        l = to_tf32((float)(x - (double)h));
-      }
-      h *= fs;
-      l *= fs;
+    v[j] = 0.0;
+    if (r < b.R && k < b.K)
+      v[j] = b.trans ? src[b.src + (int64_t)k * b.ld + r] : src[b.src + (int64_t)r * b.ld + k];
+  }
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    double x = v[j];
+    float h, l;
+    if (f64scale) x *= b.scale;
+    if (!split_bits(x, h, l)) {
+      h = to_tf32((float)x);
+      l = to_tf32((float)(x - (double)h));
     }
-    hi[out + ((j ^ rr) << 2)] = h;
-    if (lo) lo[out + ((j ^ rr) << 2)] = l;
+    hi[out + ((j ^ rr) << 2)] = h * fs;
+    if (lo) lo[out + ((j ^ rr) << 2)] = l * fs;
   }
 }
 
@@ -494,8 +502,10 @@ __device__ __forceinline__ void df_acc(float ch, float cl, float2 x, float& ah, 
 __global__ void __launch_bounds__(256)
     combine_pairs_pack_kernel(const PackOut* __restrict__ outs, int ntasks, int ntiles,
                               const CombTask* __restrict__ tasks, const CombTerm* __restrict__ terms,
-                              const float2* __restrict__ in, float* __restrict__ out_hi,
-                              float* __restrict__ out_lo, float sh, float sl) {
+                              const float2* in, float* out_hi,
+                              float* out_lo, float sh, float sl) {
+  grid_next();
+  grid_wait();
   const int tile = blockIdx.x * 8 + (threadIdx.x >> 5);
   if (tile >= ntiles) return;
   const int lane = threadIdx.x & 31;
@@ -549,8 +559,7 @@ void launch_one(const TcUnit* units, const int32_t* cta_start, int ncta, const G
                          cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
     if (bit) done.fetch_or(bit);
   }
-  gemm_tc_kernel<P, kSpanChunks, kPacked><<<ncta, kThreads, kSmemBytes, st>>>(
-      units, cta_start, tasks, segs, Ah, Al, Bh, Bl, Chi, Clo, err, wait_ns);
+  launch_chain(gemm_tc_kernel<P, kSpanChunks, kPacked>, ncta, kThreads, kSmemBytes, st, units, cta_start, tasks, segs, Ah, Al, Bh, Bl, Chi, Clo, err, wait_ns);
 }
 
 }  // namespace
@@ -559,7 +568,7 @@ void launch_pack(const PackBlock* blocks, int nblocks, int ntiles, const double*
                  float* lo, cudaStream_t st) {
   if (ntiles <= 0 || nblocks <= 0) return;
   count_launch();
-  pack_kernel<<<(ntiles + 7) / 8, 256, 0, st>>>(blocks, nblocks, ntiles, src, hi, lo);
+  launch_chain(pack_kernel, (ntiles + 7) / 8, 256, 0, st, blocks, nblocks, ntiles, src, hi, lo);
 }
 
 void launch_combine_pairs_pack(const PackOut* outs, int ntasks, int ntiles, const CombTask* tasks,
@@ -568,15 +577,15 @@ void launch_combine_pairs_pack(const PackOut* outs, int ntasks, int ntiles, cons
   if (ntiles <= 0 || ntasks <= 0) return;
   count_launch();
   const float sh = (float)scale, sl = (float)(scale - (double)sh);
-  combine_pairs_pack_kernel<<<(ntiles + 7) / 8, 256, 0, st>>>(outs, ntasks, ntiles, tasks, terms,
-                                                              in, out_hi, out_lo, sh, sl);
+  launch_chain(combine_pairs_pack_kernel, (ntiles + 7) / 8, 256, 0, st, outs, ntasks, ntiles, tasks, terms, in, out_hi, out_lo, sh, sl);
 }
 
 void launch_gemm_tc(int passes, bool packed, const TcUnit* units, const int32_t* cta_start,
                     int ncta, const GemmTask* tasks, const TcSeg* segs, const float* Ahi,
                     const float* Alo, const float* Bhi, const float* Blo, float* Chi, float* Clo,
-                    int* err, uint64_t wait_ns, cudaStream_t st) {
+                    int* err, uint64_t wait_ns, bool chain, cudaStream_t st) {
   if (ncta <= 0) return;
+  const PlainLaunches plain(!chain);
   count_launch();
   if (passes == 3) {
     if (packed)

@@ -1,6 +1,7 @@
 // Host-side planning of the block-sparse contractions.  See plan.hpp.
 #include "plan.hpp"
 
+#include "launch.hpp"
 #include "validate.hpp"
 
 #include <algorithm>
@@ -135,6 +136,9 @@ void schedule_units(TcStage& tc, const std::vector<GemmTask>& tasks) {
     cost[i] = u.nchunks * (0.7 + 0.3 * (double)((nrem + 15) / 16 * 16) / 128.0) + 4.0;
   }
   schedule(tc.units, tc.cta_start, cost);
+  int64_t chunks = 0;
+  for (const TcUnit& u : tc.units) chunks += u.nchunks;
+  tc.chain = chunks <= (int64_t)kChainChunks * ((int64_t)tc.cta_start.size() - 1);
 }
 
 using Key = std::array<int, 4>;

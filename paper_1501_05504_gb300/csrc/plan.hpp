@@ -37,6 +37,7 @@ struct TcStage {
   std::vector<TcUnit> units;            // grouped by CTA: CTA b runs units [cta_start[b], cta_start[b+1])
   std::vector<int32_t> cta_start;       // one entry per CTA of the persistent launch, plus one
   std::vector<PackBlock> packA, packB;  // empty for an operand packed by stage 2
+  bool chain = false;                   // short enough for a chained launch (launch.hpp)
   int64_t nA = 0, nB = 0;               // floats of one part (hi or lo) of each packed operand
   int32_t tilesA = 0, tilesB = 0;
 };

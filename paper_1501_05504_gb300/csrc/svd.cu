@@ -38,6 +38,7 @@
 #include <thread>
 
 #include "kernels.hpp"
+#include "launch.hpp"
 #include "svd.hpp"
 
 namespace dmrg3s {
@@ -70,7 +71,9 @@ __device__ __forceinline__ T cta_sum(T v, T* red) {
 // j <= i); V1 = I where the left vectors are wanted.  One CTA per column j.
 __global__ void __launch_bounds__(kJacThreads)
 jac_init_kernel(const JacJob* __restrict__ jobs, const int* __restrict__ col_job,
-                const double* __restrict__ A, double* __restrict__ Y, double* __restrict__ V) {
+                const double* A, double* Y, double* V) {
+  grid_next();
+  grid_wait();
   const JacJob J = jobs[col_job[blockIdx.x]];
   const int j = blockIdx.x - J.col0;
   double* y = Y + J.offY + (int64_t)j * J.n;
@@ -85,7 +88,9 @@ jac_init_kernel(const JacJob* __restrict__ jobs, const int* __restrict__ col_job
 // Squared norm of every column of every A (m rows, ld m).  One CTA per column.
 __global__ void __launch_bounds__(kJacThreads)
 jac_anorm_kernel(const JacJob* __restrict__ jobs, const int* __restrict__ col_job,
-                 const double* __restrict__ A, double* __restrict__ nrm) {
+                 const double* A, double* nrm) {
+  grid_next();
+  grid_wait();
   __shared__ double red[kJacThreads / 32];
   const JacJob J = jobs[col_job[blockIdx.x]];
   const int j = blockIdx.x - J.col0;
@@ -99,8 +104,10 @@ jac_anorm_kernel(const JacJob* __restrict__ jobs, const int* __restrict__ col_jo
 // T = A P: column j of T is column perm[j] of A.  One CTA per column.
 __global__ void __launch_bounds__(kJacThreads)
 jac_permute_kernel(const JacJob* __restrict__ jobs, const int* __restrict__ col_job,
-                   const int* __restrict__ perm, const double* __restrict__ A,
-                   double* __restrict__ T) {
+                   const int* perm, const double* A,
+                   double* T) {
+  grid_next();
+  grid_wait();
   const JacJob J = jobs[col_job[blockIdx.x]];
   const int j = blockIdx.x - J.col0;
   const double* x = A + J.offA + (int64_t)perm[blockIdx.x] * J.m;
@@ -152,7 +159,9 @@ __device__ __forceinline__ void jacobi_rotation(double saa, double sbb, double s
 }
 
 // Advances the sweep counter read by the round kernels (first node of a sweep).
-__global__ void jac_next_sweep_kernel(int* sweep) { *sweep += 1; }
+__global__ void jac_next_sweep_kernel(int* sweep) {
+  grid_next();
+  grid_wait(); *sweep += 1; }
 
 // Sums of three per-lane values over the warp, returned to every lane with
 // the same bits in every lane.  The first two levels exchange halves of the
@@ -187,8 +196,10 @@ constexpr int kJacPairsPerCta = 4;
 constexpr int kJacCache = 8;
 __global__ void __launch_bounds__(32 * kJacPairsPerCta)
 jac_round_kernel(const JacJob* __restrict__ jobs, const int* __restrict__ pair_job, int npairs,
-                 int njobs, int r, const int* __restrict__ sweep, int* __restrict__ rot,
-                 double* __restrict__ Y, double* __restrict__ V) {
+                 int njobs, int r, const int* sweep, int* rot,
+                 double* Y, double* V) {
+  grid_next();
+  grid_wait();
   const int p = blockIdx.x * kJacPairsPerCta + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (p >= npairs) return;
@@ -251,7 +262,21 @@ jac_round_kernel(const JacJob* __restrict__ jobs, const int* __restrict__ pair_j
   if (J.offV >= 0) {
     double* va = V + J.offV + (int64_t)a * n;
     double* vb = V + J.offV + (int64_t)b * n;
-    for (int i = lane; i < n; i += 32) {
+#pragma unroll
+    for (int e = 0; e < kJacCache; ++e) {      // every load before the first store
+      const int i = lane + e * 32;
+      ua[e] = i < n ? va[i] : 0.0;
+      ub[e] = i < n ? vb[i] : 0.0;
+    }
+#pragma unroll
+    for (int e = 0; e < kJacCache; ++e) {
+      const int i = lane + e * 32;
+      if (i < n) {
+        va[i] = cs * ua[e] - sn * ub[e];
+        vb[i] = sn * ua[e] + cs * ub[e];
+      }
+    }
+    for (int i = lane + kJacCache * 32; i < n; i += 32) {
       const double u = va[i], v = vb[i];
       va[i] = cs * u - sn * v;
       vb[i] = sn * u + cs * v;
@@ -261,7 +286,9 @@ jac_round_kernel(const JacJob* __restrict__ jobs, const int* __restrict__ pair_j
 
 __global__ void __launch_bounds__(kJacThreads)
 jac_norm_kernel(const JacJob* __restrict__ jobs, const int* __restrict__ col_job,
-                const double* __restrict__ Y, double* __restrict__ sig) {
+                const double* Y, double* sig) {
+  grid_next();
+  grid_wait();
   __shared__ double red[kJacThreads / 32];
   const JacJob J = jobs[col_job[blockIdx.x]];
   const int j = blockIdx.x - J.col0;
@@ -281,9 +308,11 @@ __device__ __forceinline__ double sig_key(double x) { return x != x ? INFINITY :
 // which Q then multiplies.  One CTA per column.
 __global__ void __launch_bounds__(kJacThreads)
 jac_scatter_kernel(const JacJob* __restrict__ jobs, const int* __restrict__ col_job,
-                   const int* __restrict__ perm, const double* __restrict__ Y,
-                   const double* __restrict__ V, const double* __restrict__ sig,
-                   double* __restrict__ S, double* __restrict__ VT, double* __restrict__ U) {
+                   const int* perm, const double* Y,
+                   const double* V, const double* sig,
+                   double* S, double* VT, double* U) {
+  grid_next();
+  grid_wait();
   __shared__ int red[kJacThreads / 32];
   const JacJob J = jobs[col_job[blockIdx.x]];
   const int j = blockIdx.x - J.col0;
@@ -423,7 +452,7 @@ dmrg3s_status svd_jacobi(Context* c, std::vector<SvdLane>& lanes, int nlanes,
   std::vector<int> perm(ncol);
   if (!s) {
     std::vector<double> hn(ncol);
-    jac_anorm_kernel<<<ncol, kJacThreads, 0, st>>>(dt, d_col, A, anrm);
+    launch_chain(jac_anorm_kernel, ncol, kJacThreads, 0, st, dt, d_col, A, anrm);
     count_launch();
     if (!(s = cuda_ok(c, cudaMemcpyAsync(hn.data(), anrm, ncol * sizeof(double),
                                          cudaMemcpyDeviceToHost, st), "column norms")) &&
@@ -435,7 +464,7 @@ dmrg3s_status svd_jacobi(Context* c, std::vector<SvdLane>& lanes, int nlanes,
         std::stable_sort(pj, pj + t.n, [&](int x, int y) { return nj_[x] > nj_[y]; });
       }
       cudaMemcpyAsync(d_perm, perm.data(), ncol * sizeof(int), cudaMemcpyHostToDevice, st);
-      jac_permute_kernel<<<ncol, kJacThreads, 0, st>>>(dt, d_col, d_perm, A, T);
+      launch_chain(jac_permute_kernel, ncol, kJacThreads, 0, st, dt, d_col, d_perm, A, T);
       count_launch();
       s = cuda_ok(c, cudaGetLastError(), "column order");
     }
@@ -529,20 +558,20 @@ dmrg3s_status svd_jacobi(Context* c, std::vector<SvdLane>& lanes, int nlanes,
   if (!s && !qr_ok) s = fail(c, DMRG3S_ERR_CUDA, "QR factorisation");
   // ---- 2. Y = R^T, V1 = I
   if (!s) {
-    jac_init_kernel<<<ncol, kJacThreads, 0, st>>>(dt, d_col, T, Y, V1);
+    launch_chain(jac_init_kernel, ncol, kJacThreads, 0, st, dt, d_col, T, Y, V1);
     count_launch();
     s = cuda_ok(c, cudaGetLastError(), "Jacobi set-up");
   }
   // ---- 3. sweeps: one CUDA graph of (sweep counter, rounds 0 .. maxr-1)
+  const PlainLaunches plain;
   cudaStream_t cap = nullptr;
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t gexec = nullptr;
   if (!s && cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking) == cudaSuccess &&
       cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal) == cudaSuccess) {
-    jac_next_sweep_kernel<<<1, 1, 0, cap>>>(d_sweep);
+    launch_chain(jac_next_sweep_kernel, 1, 1, 0, cap, d_sweep);
     for (int r = 0; r < maxr; ++r)
-      jac_round_kernel<<<ncta, 32 * kJacPairsPerCta, 0, cap>>>(dt, d_pair, npair, nj, r, d_sweep,
-                                                              rot, Y, V1);
+      launch_chain(jac_round_kernel, ncta, 32 * kJacPairsPerCta, 0, cap, dt, d_pair, npair, nj, r, d_sweep, rot, Y, V1);
     if (cudaStreamEndCapture(cap, &graph) != cudaSuccess ||
         cudaGraphInstantiate(&gexec, graph, 0) != cudaSuccess)
       gexec = nullptr;
@@ -559,10 +588,9 @@ dmrg3s_status svd_jacobi(Context* c, std::vector<SvdLane>& lanes, int nlanes,
     if (gexec) {
       s = cuda_ok(c, cudaGraphLaunch(gexec, st), "Jacobi sweep");
     } else {
-      jac_next_sweep_kernel<<<1, 1, 0, st>>>(d_sweep);
+      launch_chain(jac_next_sweep_kernel, 1, 1, 0, st, d_sweep);
       for (int r = 0; r < maxr; ++r)
-        jac_round_kernel<<<ncta, 32 * kJacPairsPerCta, 0, st>>>(dt, d_pair, npair, nj, r, d_sweep,
-                                                              rot, Y, V1);
+        launch_chain(jac_round_kernel, ncta, 32 * kJacPairsPerCta, 0, st, dt, d_pair, npair, nj, r, d_sweep, rot, Y, V1);
       s = cuda_ok(c, cudaGetLastError(), "Jacobi sweep");
     }
     count_launch(maxr + 1);
@@ -602,8 +630,8 @@ dmrg3s_status svd_jacobi(Context* c, std::vector<SvdLane>& lanes, int nlanes,
   if (cap) cudaStreamDestroy(cap);
   // ---- 4. singular values in descending order, VT, (V1; 0) for the left vectors
   if (!s) {
-    jac_norm_kernel<<<ncol, kJacThreads, 0, st>>>(dt, d_col, Y, sig);
-    jac_scatter_kernel<<<ncol, kJacThreads, 0, st>>>(dt, d_col, d_perm, Y, V1, sig, S, VT, U);
+    launch_chain(jac_norm_kernel, ncol, kJacThreads, 0, st, dt, d_col, Y, sig);
+    launch_chain(jac_scatter_kernel, ncol, kJacThreads, 0, st, dt, d_col, d_perm, Y, V1, sig, S, VT, U);
     count_launch(2);
     s = cuda_ok(c, cudaGetLastError(), "singular vectors");
   }

@@ -6,6 +6,7 @@
 #include <cmath>
 
 #include "kernels.hpp"
+#include "launch.hpp"
 #include "vecops.hpp"
 
 namespace dmrg3s {
@@ -37,10 +38,12 @@ __device__ double block_sum(double v, double* sh) {
 // h[j] = <V_j, w> for j < k: block (c, j) sums chunk c of vector j (one block
 // reduction per block); multidot_final adds the chunk partials of vector j
 // in chunk order, so the result is deterministic.
-__global__ void __launch_bounds__(kThreads) multidot_partial(const double* __restrict__ V,
-                                                             int64_t ldv, const double* __restrict__ w,
+__global__ void __launch_bounds__(kThreads) multidot_partial(const double* V,
+                                                             int64_t ldv, const double* w,
                                                              int64_t n, int64_t chunk,
-                                                             double* __restrict__ partial) {
+                                                             double* partial) {
+  grid_next();
+  grid_wait();
   __shared__ double sh[32];
   const int j = blockIdx.y;
   const double* v = V + (int64_t)j * ldv;
@@ -52,8 +55,10 @@ __global__ void __launch_bounds__(kThreads) multidot_partial(const double* __res
   if (threadIdx.x == 0) partial[(int64_t)j * gridDim.x + blockIdx.x] = s;
 }
 
-__global__ void multidot_final(const double* __restrict__ partial, int nchunk, int k,
-                               double* __restrict__ h, double* __restrict__ copy_last) {
+__global__ void multidot_final(const double* partial, int nchunk, int k,
+                               double* h, double* copy_last) {
+  grid_next();
+  grid_wait();
   __shared__ double sh[32];
   const int j = blockIdx.x;
   double acc = 0.0;
@@ -126,8 +131,8 @@ __device__ void tridiag_vector(const double* alpha, const double* beta, int k, d
 // returns the Rayleigh quotient of the vector, which is accurate to FP64
 // rounding whatever the width of the bracket was.
 // bl = the norm of the new residual vector (stored as beta[k - 1]).
-__device__ void tridiag_block(const double* __restrict__ alpha, double* __restrict__ beta, int k,
-                              double bl, double* __restrict__ y, TridiagOut* __restrict__ out) {
+__device__ void tridiag_block(const double* alpha, double* beta, int k,
+                              double bl, double* y, TridiagOut* out) {
   __shared__ double sh_lo, sh_hi, sh_span, sh_c;
   __shared__ int sh_bad, sh_first;
   __shared__ DF sa[128], sbb[128];
@@ -297,8 +302,10 @@ __device__ void tridiag_vector(const double* alpha, const double* beta, int k, d
 }
 
 __global__ void copy_blocks_kernel(const CopyTask* __restrict__ tasks,
-                                   const double* __restrict__ src, double* __restrict__ dst,
-                                   const double* __restrict__ scale) {
+                                   const double* src, double* dst,
+                                   const double* scale) {
+  grid_next();
+  grid_wait();
   const CopyTask t = tasks[blockIdx.x];
   const int n = t.rows * t.cols;
   for (int idx = threadIdx.x; idx < n; idx += blockDim.x) {
@@ -323,7 +330,7 @@ constexpr int kLzWarps = kLzThreads / 32;
 
 // Sum of partial[b * kp + j] over the chunks b of [c0, c0 + nc) in a fixed
 // order (lane-strided sums, then the xor tree); every lane returns the sum.
-__device__ __forceinline__ double chain_sum(const double* __restrict__ partial, int kp, int c0,
+__device__ __forceinline__ double chain_sum(const double* partial, int kp, int c0,
                                             int nc, int j, int lane) {
   double a0 = 0.0, a1 = 0.0;
   int b = lane;
@@ -339,7 +346,7 @@ __device__ __forceinline__ double chain_sum(const double* __restrict__ partial, 
 
 // <v, x> over len elements by one warp (lane-strided), four loads in flight
 // per lane; the lanes' partial sums in a fixed order, then the xor tree.
-__device__ __forceinline__ double warp_dot(const double* __restrict__ v, const double* x, int len,
+__device__ __forceinline__ double warp_dot(const double* v, const double* x, int len,
                                            int lane) {
   double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
   int i = lane;
@@ -356,7 +363,7 @@ __device__ __forceinline__ double warp_dot(const double* __restrict__ v, const d
 
 // x - sum_{j < k1} h[j] V_j[e], the loads of four basis vectors in flight at a
 // time (the basis is L2-resident; the loop is latency-bound otherwise).
-__device__ __forceinline__ double lz_project(const double* __restrict__ V, int64_t ldv, int k1,
+__device__ __forceinline__ double lz_project(const double* V, int64_t ldv, int k1,
                                              const double* h, int64_t e, double x) {
   int j = 0;
   for (; j + 4 <= k1; j += 4) {
@@ -373,12 +380,14 @@ __device__ __forceinline__ double lz_project(const double* __restrict__ V, int64
 
 // The chunk of w is staged in shared memory once; warp q then forms the dot
 // products with V_j for j = q, q + 8, ...
-__global__ void __launch_bounds__(kLzThreads) lz_dots_kernel(const double* __restrict__ V,
+__global__ void __launch_bounds__(kLzThreads) lz_dots_kernel(const double* V,
                                                              int64_t ldv, int k1,
-                                                             const int* __restrict__ kdev,
-                                                             const double* __restrict__ w,
+                                                             const int* kdev,
+                                                             const double* w,
                                                              const LzChunk* __restrict__ chunks,
-                                                             double* __restrict__ partial, int kp) {
+                                                             double* partial, int kp) {
+  grid_next();
+  grid_wait();
   extern __shared__ double wsh[];
   if (kdev) k1 = *kdev + 1;
   const LzChunk ch = chunks[blockIdx.x];
@@ -393,10 +402,12 @@ __global__ void __launch_bounds__(kLzThreads) lz_dots_kernel(const double* __res
 }
 
 __global__ void __launch_bounds__(kLzThreads) lz_update_kernel(
-    const double* __restrict__ V, int64_t ldv, int k1, const int* __restrict__ kdev,
-    double* __restrict__ w, const LzChunk* __restrict__ chunks, const LzChain* __restrict__ chains,
-    const double* __restrict__ partial, int kp, double* __restrict__ alpha,
-    double* __restrict__ nrm_partial, int64_t nrm_stride) {
+    const double* V, int64_t ldv, int k1, const int* kdev,
+    double* w, const LzChunk* __restrict__ chunks, const LzChain* __restrict__ chains,
+    const double* partial, int kp, double* alpha,
+    double* nrm_partial, int64_t nrm_stride) {
+  grid_next();
+  grid_wait();
   __shared__ double h[kLzMaxK];
   __shared__ double red[32];
   if (kdev) {
@@ -429,10 +440,12 @@ __global__ void __launch_bounds__(kLzThreads) lz_update_kernel(
 // The first Gram-Schmidt pass's update fused with the second pass's dots:
 // the updated chunk of w stays in shared memory for the dots against V_j.
 __global__ void __launch_bounds__(kLzThreads) lz_update_dots_kernel(
-    const double* __restrict__ V, int64_t ldv, int k1, double* __restrict__ w,
+    const double* V, int64_t ldv, int k1, double* w,
     const LzChunk* __restrict__ chunks, const LzChain* __restrict__ chains,
-    const double* __restrict__ partial, int kp, double* __restrict__ alpha,
-    double* __restrict__ partial2, const int* __restrict__ kdev) {
+    const double* partial, int kp, double* alpha,
+    double* partial2, const int* kdev) {
+  grid_next();
+  grid_wait();
   extern __shared__ double wsh[];
   __shared__ double h[kLzMaxK];
   if (kdev) k1 = *kdev + 1;
@@ -462,8 +475,10 @@ __global__ void __launch_bounds__(kLzThreads) lz_update_dots_kernel(
 }
 
 __global__ void __launch_bounds__(kLzThreads) lz_normalise_kernel(
-    const double* __restrict__ x, double* __restrict__ y, const LzChunk* __restrict__ chunks,
-    const LzChain* __restrict__ chains, const double* __restrict__ nrm_partial) {
+    const double* x, double* y, const LzChunk* __restrict__ chunks,
+    const LzChain* __restrict__ chains, const double* nrm_partial) {
+  grid_next();
+  grid_wait();
   __shared__ double scale;
   const LzChunk ch = chunks[blockIdx.x];
   if (threadIdx.x < 32) {
@@ -479,10 +494,12 @@ __global__ void __launch_bounds__(kLzThreads) lz_normalise_kernel(
 // v_{k+1} = w / |w| (norm partials of iteration k, k from the device
 // counter), written into the basis and into the fixed product input vcur.
 __global__ void __launch_bounds__(kLzThreads) lz_next_kernel(
-    const double* __restrict__ w, double* __restrict__ V, int64_t ldv, const int* __restrict__ kdev,
-    double* __restrict__ vcur, const LzChunk* __restrict__ chunks,
-    const LzChain* __restrict__ chains, const double* __restrict__ nrm_partial,
+    const double* w, double* V, int64_t ldv, const int* kdev,
+    double* vcur, const LzChunk* __restrict__ chunks,
+    const LzChain* __restrict__ chains, const double* nrm_partial,
     int64_t nrm_stride) {
+  grid_next();
+  grid_wait();
   __shared__ double scale;
   const int k = *kdev;
   const LzChunk ch = chunks[blockIdx.x];
@@ -502,12 +519,16 @@ __global__ void __launch_bounds__(kLzThreads) lz_next_kernel(
   }
 }
 
-__global__ void lz_advance_kernel(int* kdev) { *kdev += 1; }
+__global__ void lz_advance_kernel(int* kdev) {
+  grid_next();
+  grid_wait(); *kdev += 1; }
 
-__global__ void lz_tridiag_kernel(const LzChain* __restrict__ chains, const double* __restrict__ alpha,
-                                  double* __restrict__ beta, int kp, int k,
-                                  const double* __restrict__ nrm_partial, double* __restrict__ y,
-                                  TridiagOut* __restrict__ out) {
+__global__ void lz_tridiag_kernel(const LzChain* __restrict__ chains, const double* alpha,
+                                  double* beta, int kp, int k,
+                                  const double* nrm_partial, double* y,
+                                  TridiagOut* out) {
+  grid_next();
+  grid_wait();
   __shared__ double bl;
   const int c = blockIdx.x;
   const LzChain cn = chains[c];
@@ -521,9 +542,11 @@ __global__ void lz_tridiag_kernel(const LzChain* __restrict__ chains, const doub
 }
 
 __global__ void __launch_bounds__(kLzThreads) lz_ritz_kernel(
-    const double* __restrict__ V, int64_t ldv, const LzChunk* __restrict__ chunks,
-    const LzChain* __restrict__ chains, const int32_t* __restrict__ kstop,
-    const double* __restrict__ y, int kp, double* __restrict__ x, double* __restrict__ nrm_partial) {
+    const double* V, int64_t ldv, const LzChunk* __restrict__ chunks,
+    const LzChain* __restrict__ chains, const int32_t* kstop,
+    const double* y, int kp, double* x, double* nrm_partial) {
+  grid_next();
+  grid_wait();
   __shared__ double red[32];
   const LzChunk ch = chunks[blockIdx.x];
   const int ks = kstop[ch.chain];
@@ -550,16 +573,15 @@ void launch_multidot(const double* V, int64_t ldv, int k, const double* w, int64
   chunk = (chunk + kThreads - 1) / kThreads * kThreads;
   int nchunk = (int)((n + chunk - 1) / chunk);
   if (nchunk < 1) nchunk = 1;
-  multidot_partial<<<dim3(nchunk, k), kThreads, 0, st>>>(V, ldv, w, n, chunk, partial);
-  multidot_final<<<k, 128, 0, st>>>(partial, nchunk, k, h, copy_last);
+  launch_chain(multidot_partial, dim3(nchunk, k), kThreads, 0, st, V, ldv, w, n, chunk, partial);
+  launch_chain(multidot_final, k, 128, 0, st, partial, nchunk, k, h, copy_last);
 }
 
 void launch_lz_dots(const double* V, int64_t ldv, int k1, const double* w, const LzChunk* chunks,
                     int nchunks, double* partial, int kp, cudaStream_t st, const int* kdev) {
   if ((!kdev && k1 <= 0) || nchunks <= 0) return;
   count_launch();
-  lz_dots_kernel<<<nchunks, kLzThreads, kLzChunkMax * sizeof(double), st>>>(V, ldv, k1, kdev, w,
-                                                                             chunks, partial, kp);
+  launch_chain(lz_dots_kernel, nchunks, kLzThreads, kLzChunkMax * sizeof(double), st, V, ldv, k1, kdev, w, chunks, partial, kp);
 }
 
 void launch_lz_update(const double* V, int64_t ldv, int k1, double* w, const LzChunk* chunks,
@@ -568,8 +590,7 @@ void launch_lz_update(const double* V, int64_t ldv, int k1, double* w, const LzC
                       int64_t nrm_stride) {
   if (nchunks <= 0) return;
   count_launch();
-  lz_update_kernel<<<nchunks, kLzThreads, 0, st>>>(V, ldv, k1, kdev, w, chunks, chains, partial,
-                                                   kp, alpha, nrm_partial, nrm_stride);
+  launch_chain(lz_update_kernel, nchunks, kLzThreads, 0, st, V, ldv, k1, kdev, w, chunks, chains, partial, kp, alpha, nrm_partial, nrm_stride);
 }
 
 void launch_lz_next(const double* w, double* V, int64_t ldv, const int* kdev, double* vcur,
@@ -577,13 +598,12 @@ void launch_lz_next(const double* w, double* V, int64_t ldv, const int* kdev, do
                     const double* nrm_partial, int64_t nrm_stride, cudaStream_t st) {
   if (nchunks <= 0) return;
   count_launch();
-  lz_next_kernel<<<nchunks, kLzThreads, 0, st>>>(w, V, ldv, kdev, vcur, chunks, chains,
-                                                 nrm_partial, nrm_stride);
+  launch_chain(lz_next_kernel, nchunks, kLzThreads, 0, st, w, V, ldv, kdev, vcur, chunks, chains, nrm_partial, nrm_stride);
 }
 
 void launch_lz_advance(int* kdev, cudaStream_t st) {
   count_launch();
-  lz_advance_kernel<<<1, 1, 0, st>>>(kdev);
+  launch_chain(lz_advance_kernel, 1, 1, 0, st, kdev);
 }
 
 void launch_lz_update_dots(const double* V, int64_t ldv, int k1, double* w, const LzChunk* chunks,
@@ -591,15 +611,14 @@ void launch_lz_update_dots(const double* V, int64_t ldv, int k1, double* w, cons
                            double* alpha, double* partial2, cudaStream_t st, const int* kdev) {
   if (nchunks <= 0 || (!kdev && k1 <= 0)) return;
   count_launch();
-  lz_update_dots_kernel<<<nchunks, kLzThreads, kLzChunkMax * sizeof(double), st>>>(
-      V, ldv, k1, w, chunks, chains, partial, kp, alpha, partial2, kdev);
+  launch_chain(lz_update_dots_kernel, nchunks, kLzThreads, kLzChunkMax * sizeof(double), st,  V, ldv, k1, w, chunks, chains, partial, kp, alpha, partial2, kdev);
 }
 
 void launch_lz_normalise(const double* x, double* y, const LzChunk* chunks, int nchunks,
                          const LzChain* chains, const double* nrm_partial, cudaStream_t st) {
   if (nchunks <= 0) return;
   count_launch();
-  lz_normalise_kernel<<<nchunks, kLzThreads, 0, st>>>(x, y, chunks, chains, nrm_partial);
+  launch_chain(lz_normalise_kernel, nchunks, kLzThreads, 0, st, x, y, chunks, chains, nrm_partial);
 }
 
 void launch_lz_tridiag(const LzChain* chains, int nchains, const double* alpha, double* beta,
@@ -607,7 +626,7 @@ void launch_lz_tridiag(const LzChain* chains, int nchains, const double* alpha, 
                        cudaStream_t st) {
   if (nchains <= 0) return;
   count_launch();
-  lz_tridiag_kernel<<<nchains, 256, 0, st>>>(chains, alpha, beta, kp, k, nrm_partial, y, out);
+  launch_chain(lz_tridiag_kernel, nchains, 256, 0, st, chains, alpha, beta, kp, k, nrm_partial, y, out);
 }
 
 void launch_lz_ritz(const double* V, int64_t ldv, const LzChunk* chunks, int nchunks,
@@ -615,15 +634,14 @@ void launch_lz_ritz(const double* V, int64_t ldv, const LzChunk* chunks, int nch
                     double* x, double* nrm_partial, cudaStream_t st) {
   if (nchunks <= 0) return;
   count_launch();
-  lz_ritz_kernel<<<nchunks, kLzThreads, 0, st>>>(V, ldv, chunks, chains, kstop, y, kp, x,
-                                                 nrm_partial);
+  launch_chain(lz_ritz_kernel, nchunks, kLzThreads, 0, st, V, ldv, chunks, chains, kstop, y, kp, x, nrm_partial);
 }
 
 void launch_copy_blocks(const CopyTask* tasks, int ntasks, const double* src, double* dst,
                         const double* scale, cudaStream_t st) {
   if (ntasks <= 0) return;
   count_launch();
-  copy_blocks_kernel<<<ntasks, 256, 0, st>>>(tasks, src, dst, scale);
+  launch_chain(copy_blocks_kernel, ntasks, 256, 0, st, tasks, src, dst, scale);
 }
 
 }  // namespace dmrg3s
