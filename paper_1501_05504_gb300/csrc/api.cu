@@ -404,7 +404,10 @@ dmrg3s_status grad_plan(Context* c, const EnvLayout& le, const MpoLayout& w, con
   if ((st = upload_grad_plan(std::move(p), &dp)))
     return fail(c, st, "uploading a gradient plan failed");
   // a bounded cache: freeing the tables waits for the device
-  if (c->grad_plans.size() >= kMaxGradPlans) c->grad_plans.clear();
+  if (c->grad_plans.size() >= kMaxGradPlans) {
+    c->grad_by_args.clear();
+    c->grad_plans.clear();
+  }
   *out = dp.get();
   c->grad_plans[h.h] = std::move(dp);
   return DMRG3S_OK;
@@ -490,6 +493,15 @@ dmrg3s_status check_ws(Context* c, const Plan& p, dmrg3s_precision prec) {
     return fail(c, DMRG3S_ERR_OOM,
                 "context workspace too small: need " + std::to_string(need) + " bytes");
   return DMRG3S_OK;
+}
+
+const DevicePlan* known_plan(Context* c, const RawKey& key) {
+  if (!key.ok) return nullptr;
+  auto it = c->by_args.find(key);
+  return it == c->by_args.end() ? nullptr : it->second;
+}
+void remember_plan(Context* c, const RawKey& key, const DevicePlan* p) {
+  if (key.ok) c->by_args[key] = p;
 }
 
 dmrg3s_status prec_ok(Context* c, dmrg3s_precision prec) {
@@ -765,26 +777,38 @@ dmrg3s_status dmrg3s_apply_heff(dmrg3s_ctx ctx, const dmrg3s_env* L, const dmrg3
   if (!c || !L || !W || !R || !A || !HA) return fail(c, DMRG3S_ERR_ARG, "NULL argument");
   dmrg3s_status st = prec_ok(c, prec);
   if (st != DMRG3S_OK) return st;
-  std::string err;
-  EnvLayout le, re;
-  MpoLayout w;
-  SiteLayout a, ha;
-  if ((st = make_env(L, &le, &err)) || (st = make_env(R, &re, &err)) ||
-      (st = make_mpo(W, &w, &err)) || (st = make_site(A, &a, &err)) ||
-      (st = make_site(HA, &ha, &err)))
-    return fail(c, st, err);
-  if ((st = check_site_mpo(a, w, &err)) ||
-      (st = check_env(le, a.left, w.wl, w.tl, "L", &err)) ||
-      (st = check_env(re, a.right, w.wr, w.tr, "R", &err)))
-    return fail(c, st, err);
-  if (!same_bond(a.left, ha.left) || !same_bond(a.right, ha.right) || a.d != ha.d ||
-      !same_charges(a.qp, ha.qp))
-    return fail(c, DMRG3S_ERR_SHAPE, "HA must have the structure of A");
+  RawKey key;
+  key.word((uint64_t)Kind::Heff);
+  key.env(*L);
+  key.mpo(*W, true);
+  key.env(*R);
+  key.site(*A);
+  key.site(*HA);
+  const DevicePlan* p = known_plan(c, key);
+  if (!p) {
+    std::string err;
+    EnvLayout le, re;
+    MpoLayout w;
+    SiteLayout a, ha;
+    if ((st = make_env(L, &le, &err)) || (st = make_env(R, &re, &err)) ||
+        (st = make_mpo(W, &w, &err)) || (st = make_site(A, &a, &err)) ||
+        (st = make_site(HA, &ha, &err)))
+      return fail(c, st, err);
+    if ((st = check_site_mpo(a, w, &err)) ||
+        (st = check_env(le, a.left, w.wl, w.tl, "L", &err)) ||
+        (st = check_env(re, a.right, w.wr, w.tr, "R", &err)))
+      return fail(c, st, err);
+    if (!same_bond(a.left, ha.left) || !same_bond(a.right, ha.right) || a.d != ha.d ||
+        !same_charges(a.qp, ha.qp))
+      return fail(c, DMRG3S_ERR_SHAPE, "HA must have the structure of A");
+    if (!L->data || !R->data || !A->data || !HA->data)
+      return fail(c, DMRG3S_ERR_ARG, "NULL device data pointer");
+    st = heff_plan(c, le, w, re, a, &p);
+    if (st != DMRG3S_OK) return st;
+    remember_plan(c, key, p);
+  }
   if (!L->data || !R->data || !A->data || !HA->data)
     return fail(c, DMRG3S_ERR_ARG, "NULL device data pointer");
-  const DevicePlan* p = nullptr;
-  st = heff_plan(c, le, w, re, a, &p);
-  if (st != DMRG3S_OK) return st;
   if ((st = check_ws(c, p->host, prec)) || (st = use_device(c))) return st;
   double* ws1 = reinterpret_cast<double*>(c->ws);
   double* ws2 = ws1 + p->host.ws1;
@@ -801,32 +825,42 @@ dmrg3s_status dmrg3s_expand(dmrg3s_ctx ctx, int32_t dir, const dmrg3s_env* env,
   if (dir != 1 && dir != -1) return fail(c, DMRG3S_ERR_ARG, "dir must be +1 or -1");
   dmrg3s_status st = prec_ok(c, prec);
   if (st != DMRG3S_OK) return st;
-  std::string err;
-  EnvLayout e;
-  MpoLayout w;
-  SiteLayout m, pl;
-  if ((st = make_env(env, &e, &err)) || (st = make_mpo(W, &w, &err)) ||
-      (st = make_site(M, &m, &err)) || (st = make_site(P, &pl, &err)))
-    return fail(c, st, err);
-  if ((st = check_site_mpo(m, w, &err))) return fail(c, st, err);
-  if (dir == 1) {
-    if ((st = check_env(e, m.left, w.wl, w.tl, "env (L)", &err))) return fail(c, st, err);
-  } else {
-    if ((st = check_env(e, m.right, w.wr, w.tr, "env (R)", &err))) return fail(c, st, err);
+  RawKey key;
+  key.word((uint64_t)(dir == 1 ? Kind::ExpandLR : Kind::ExpandRL));
+  key.env(*env);
+  key.mpo(*W, true);
+  key.site(*M);
+  key.site(*P);
+  const DevicePlan* p = known_plan(c, key);
+  if (!p) {
+    std::string err;
+    EnvLayout e;
+    MpoLayout w;
+    SiteLayout m, pl;
+    if ((st = make_env(env, &e, &err)) || (st = make_mpo(W, &w, &err)) ||
+        (st = make_site(M, &m, &err)) || (st = make_site(P, &pl, &err)))
+      return fail(c, st, err);
+    if ((st = check_site_mpo(m, w, &err))) return fail(c, st, err);
+    if (dir == 1) {
+      if ((st = check_env(e, m.left, w.wl, w.tl, "env (L)", &err))) return fail(c, st, err);
+    } else {
+      if ((st = check_env(e, m.right, w.wr, w.tr, "env (R)", &err))) return fail(c, st, err);
+    }
+    FusedBond f;
+    fuse_bond(dir == 1 ? m.right : m.left, dir == 1 ? w.wr : w.wl, dir == 1 ? w.tr : w.tl, false,
+              &f);
+    const Bond& keep = dir == 1 ? m.left : m.right;
+    const Bond& pkeep = dir == 1 ? pl.left : pl.right;
+    const Bond& pfused = dir == 1 ? pl.right : pl.left;
+    if (!same_bond(keep, pkeep) || !same_bond(f.bond, pfused) || pl.d != m.d ||
+        !same_charges(pl.qp, m.qp))
+      return fail(c, DMRG3S_ERR_SHAPE, "P does not have the expanded structure of M");
+    if (!env->data || !M->data || !P->data) return fail(c, DMRG3S_ERR_ARG, "NULL device data");
+    st = expand_plan(c, dir, e, w, m, pl, f, &p);
+    if (st != DMRG3S_OK) return st;
+    remember_plan(c, key, p);
   }
-  FusedBond f;
-  fuse_bond(dir == 1 ? m.right : m.left, dir == 1 ? w.wr : w.wl, dir == 1 ? w.tr : w.tl, false,
-            &f);
-  const Bond& keep = dir == 1 ? m.left : m.right;
-  const Bond& pkeep = dir == 1 ? pl.left : pl.right;
-  const Bond& pfused = dir == 1 ? pl.right : pl.left;
-  if (!same_bond(keep, pkeep) || !same_bond(f.bond, pfused) || pl.d != m.d ||
-      !same_charges(pl.qp, m.qp))
-    return fail(c, DMRG3S_ERR_SHAPE, "P does not have the expanded structure of M");
   if (!env->data || !M->data || !P->data) return fail(c, DMRG3S_ERR_ARG, "NULL device data");
-  const DevicePlan* p = nullptr;
-  st = expand_plan(c, dir, e, w, m, pl, f, &p);
-  if (st != DMRG3S_OK) return st;
   if ((st = check_ws(c, p->host, prec)) || (st = use_device(c))) return st;
   double* ws1 = reinterpret_cast<double*>(c->ws);
   const double* g1A = dir == 1 ? env->data : M->data;
@@ -844,27 +878,37 @@ dmrg3s_status dmrg3s_update_env(dmrg3s_ctx ctx, int32_t dir, const dmrg3s_env* e
   if (dir != 1 && dir != -1) return fail(c, DMRG3S_ERR_ARG, "dir must be +1 or -1");
   dmrg3s_status st = prec_ok(c, prec);
   if (st != DMRG3S_OK) return st;
-  std::string err;
-  EnvLayout e, o;
-  MpoLayout w;
-  SiteLayout a;
-  if ((st = make_env(env, &e, &err)) || (st = make_env(out, &o, &err)) ||
-      (st = make_mpo(W, &w, &err)) || (st = make_site(A, &a, &err)))
-    return fail(c, st, err);
-  if ((st = check_site_mpo(a, w, &err))) return fail(c, st, err);
-  if (dir == 1) {
-    if ((st = check_env(e, a.left, w.wl, w.tl, "env (L_{i-1})", &err)) ||
-        (st = check_env(o, a.right, w.wr, w.tr, "out (L_i)", &err)))
+  RawKey key;
+  key.word((uint64_t)(dir == 1 ? Kind::EnvLR : Kind::EnvRL));
+  key.env(*env);
+  key.mpo(*W, true);
+  key.site(*A);
+  key.env(*out);
+  const DevicePlan* p = known_plan(c, key);
+  if (!p) {
+    std::string err;
+    EnvLayout e, o;
+    MpoLayout w;
+    SiteLayout a;
+    if ((st = make_env(env, &e, &err)) || (st = make_env(out, &o, &err)) ||
+        (st = make_mpo(W, &w, &err)) || (st = make_site(A, &a, &err)))
       return fail(c, st, err);
-  } else {
-    if ((st = check_env(e, a.right, w.wr, w.tr, "env (R_{i+1})", &err)) ||
-        (st = check_env(o, a.left, w.wl, w.tl, "out (R_i)", &err)))
-      return fail(c, st, err);
+    if ((st = check_site_mpo(a, w, &err))) return fail(c, st, err);
+    if (dir == 1) {
+      if ((st = check_env(e, a.left, w.wl, w.tl, "env (L_{i-1})", &err)) ||
+          (st = check_env(o, a.right, w.wr, w.tr, "out (L_i)", &err)))
+        return fail(c, st, err);
+    } else {
+      if ((st = check_env(e, a.right, w.wr, w.tr, "env (R_{i+1})", &err)) ||
+          (st = check_env(o, a.left, w.wl, w.tl, "out (R_i)", &err)))
+        return fail(c, st, err);
+    }
+    if (!env->data || !A->data || !out->data) return fail(c, DMRG3S_ERR_ARG, "NULL device data");
+    st = env_plan(c, dir, e, w, a, o, &p);
+    if (st != DMRG3S_OK) return st;
+    remember_plan(c, key, p);
   }
   if (!env->data || !A->data || !out->data) return fail(c, DMRG3S_ERR_ARG, "NULL device data");
-  const DevicePlan* p = nullptr;
-  st = env_plan(c, dir, e, w, a, o, &p);
-  if (st != DMRG3S_OK) return st;
   if ((st = check_ws(c, p->host, prec)) || (st = use_device(c))) return st;
   double* ws1 = reinterpret_cast<double*>(c->ws);
   double* ws2 = ws1 + p->host.ws1;

@@ -4,11 +4,13 @@
 #include <cuda_runtime.h>
 
 #include <cstdint>
+#include <cstring>
 #include <memory>
 #include <string>
 #include <unordered_map>
 #include <vector>
 
+#include "dmrg3s.h"
 #include "plan.hpp"
 
 namespace dmrg3s {
@@ -147,25 +149,6 @@ struct Profiler {
   }
 };
 
-struct Context {
-  Profiler prof;
-  int device = 0;
-  char* ws = nullptr;           // workspace arena
-  size_t ws_bytes = 0;
-  double* pinned = nullptr;     // small pinned host buffer for scalar read-backs (64 doubles)
-  int* d_err = nullptr;         // device error word latched by bounded waits (tensor-core kernel)
-  uint64_t wait_ns = 1000000000ull;   // limit of every bounded device wait (dmrg3s_set_wait_limit)
-  cudaStream_t aux = nullptr;   // side stream: the Lanczos tridiagonal solve beside the next product
-  cudaEvent_t ev_ready = nullptr, ev_done = nullptr;
-  cudaEvent_t ev_lz[3] = {nullptr, nullptr, nullptr};   // Lanczos results of iterations k mod 3
-  cudaStream_t cap = nullptr;   // private stream for capturing the Lanczos iteration graph
-  double* pinned_big = nullptr;   // pinned read-back area of the batched Lanczos (grown on demand)
-  size_t pinned_big_n = 0;        // its size in doubles
-  std::unordered_map<uint64_t, std::unique_ptr<DevicePlan>> plans;
-  std::unordered_map<uint64_t, std::unique_ptr<DeviceGradPlan>> grad_plans;
-  std::string last_error;
-};
-
 // FNV-1a fingerprint builder used as the plan-cache key.
 struct Hasher {
   uint64_t h = 1469598103934665603ull;
@@ -187,6 +170,105 @@ struct Hasher {
   void site(const SiteLayout& s);
   void env(const EnvLayout& e);
   void mpo(const MpoLayout& w);
+};
+
+// 128-bit fingerprint of a call's raw arguments (charges, dimensions, channel
+// charges, MPO entries; not the data pointers).  A call whose arguments have
+// been checked and planned before finds its plan by it, without building the
+// layouts again: two multiplicative hashes over 8-byte words, ~1 us for the 7 KB
+// of a Hubbard site, where layouts, checks and the plan key take ~30 us.
+struct RawKey {
+  uint64_t a = 0x243F6A8885A308D3ull, b = 0x13198A2E03707344ull;
+  bool ok = true;          // false: malformed arguments (the checked path reports them)
+  void word(uint64_t x) {
+    a = (a ^ x) * 0x9E3779B97F4A7C15ull;
+    a ^= a >> 32;
+    b = (b + x) * 0xC2B2AE3D27D4EB4Full;
+    b ^= b >> 29;
+  }
+  void bytes(const void* p, size_t n) {
+    if (n && !p) {
+      ok = false;
+      return;
+    }
+    word(n);
+    const char* c = static_cast<const char*>(p);
+    for (; n >= 8; n -= 8, c += 8) {
+      uint64_t x;
+      std::memcpy(&x, c, 8);
+      word(x);
+    }
+    if (n) {
+      uint64_t x = 0;
+      std::memcpy(&x, c, n);
+      word(x);
+    }
+  }
+  bool range(int64_t v, int64_t lo, int64_t hi) {
+    ok = ok && v >= lo && v <= hi;
+    return ok;
+  }
+  void bond(int nsym, const dmrg3s_bond& q) {
+    if (!range(nsym, 0, DMRG3S_MAX_NSYM) || !range(q.nsec, 1, 1 << 20)) return;
+    word((uint64_t)nsym << 32 | (uint32_t)q.nsec);
+    if (nsym) bytes(q.q, sizeof(int32_t) * (size_t)nsym * q.nsec);
+    bytes(q.dim, sizeof(int64_t) * (size_t)q.nsec);
+  }
+  void site(const dmrg3s_site& s) {
+    if (!range(s.nsym, 0, DMRG3S_MAX_NSYM) || !range(s.d, 1, 1 << 12)) return;
+    word((uint64_t)s.d);
+    if (s.nsym) bytes(s.qp, sizeof(int32_t) * (size_t)s.nsym * s.d);
+    bond(s.nsym, s.left);
+    if (ok) bond(s.nsym, s.right);
+  }
+  void env(const dmrg3s_env& e) {
+    if (!range(e.nsym, 0, DMRG3S_MAX_NSYM) || !range(e.w, 1, 1 << 16)) return;
+    word((uint64_t)e.w);
+    if (e.nsym) bytes(e.t, sizeof(int32_t) * (size_t)e.nsym * e.w);
+    bond(e.nsym, e.bond);
+  }
+  void mpo(const dmrg3s_mpo_site& m, bool values) {
+    if (!range(m.nsym, 0, DMRG3S_MAX_NSYM) || !range(m.d, 1, 1 << 12) || !range(m.wl, 1, 1 << 16) ||
+        !range(m.wr, 1, 1 << 16))
+      return;
+    word((uint64_t)m.d << 32 | (uint32_t)m.nsym);
+    word((uint64_t)m.wl << 32 | (uint32_t)m.wr);
+    if (m.nsym) {
+      bytes(m.qp, sizeof(int32_t) * (size_t)m.nsym * m.d);
+      bytes(m.tl, sizeof(int32_t) * (size_t)m.nsym * m.wl);
+      bytes(m.tr, sizeof(int32_t) * (size_t)m.nsym * m.wr);
+    }
+    const size_t n = (size_t)m.d * m.d * m.wl * m.wr;
+    if (!m.W) ok = false;
+    if (ok && values) bytes(m.W, sizeof(double) * n);
+  }
+  bool operator==(const RawKey& o) const { return a == o.a && b == o.b; }
+};
+struct RawKeyHash {
+  size_t operator()(const RawKey& k) const { return (size_t)(k.a ^ (k.b << 1)); }
+};
+
+struct Context {
+  Profiler prof;
+  int device = 0;
+  char* ws = nullptr;           // workspace arena
+  size_t ws_bytes = 0;
+  double* pinned = nullptr;     // small pinned host buffer for scalar read-backs (64 doubles)
+  int* d_err = nullptr;         // device error word latched by bounded waits (tensor-core kernel)
+  uint64_t wait_ns = 1000000000ull;   // limit of every bounded device wait (dmrg3s_set_wait_limit)
+  cudaStream_t aux = nullptr;   // side stream: the Lanczos tridiagonal solve beside the next product
+  cudaEvent_t ev_ready = nullptr, ev_done = nullptr;
+  cudaEvent_t ev_lz[3] = {nullptr, nullptr, nullptr};   // Lanczos results of iterations k mod 3
+  cudaStream_t cap = nullptr;   // private stream for capturing the Lanczos iteration graph
+  double* pinned_big = nullptr;   // pinned read-back area of the batched Lanczos (grown on demand)
+  size_t pinned_big_n = 0;        // its size in doubles
+  std::unordered_map<uint64_t, std::unique_ptr<DevicePlan>> plans;
+  std::unordered_map<uint64_t, std::unique_ptr<DeviceGradPlan>> grad_plans;
+  // plans by the raw arguments of the calls that use them (entries of `plans`,
+  // which live as long as the context; of `grad_plans`, dropped with them)
+  std::unordered_map<RawKey, const DevicePlan*, RawKeyHash> by_args;
+  std::unordered_map<RawKey, const DeviceGradPlan*, RawKeyHash> grad_by_args;
+  std::string last_error;
 };
 
 inline dmrg3s_status fail(Context* c, dmrg3s_status st, const std::string& msg) {

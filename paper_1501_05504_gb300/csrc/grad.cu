@@ -77,21 +77,35 @@ extern "C" dmrg3s_status dmrg3s_mpo_grad_site(dmrg3s_ctx ctx, const dmrg3s_env* 
                                               dmrg3s_stream stream) {
   Context* c = reinterpret_cast<Context*>(ctx);
   if (!c || !L || !W || !R || !M || !G) return fail(c, DMRG3S_ERR_ARG, "NULL argument");
-  std::string err;
-  EnvLayout le, re;
-  MpoLayout w;
-  SiteLayout m;
   dmrg3s_status st;
-  if ((st = make_env(L, &le, &err)) || (st = make_env(R, &re, &err)) ||
-      (st = make_mpo(W, &w, &err)) || (st = make_site(M, &m, &err)))
-    return fail(c, st, err);
-  if ((st = check_site_mpo(m, w, &err)) ||
-      (st = check_env(le, m.left, w.wl, w.tl, "L", &err)) ||
-      (st = check_env(re, m.right, w.wr, w.tr, "R", &err)))
-    return fail(c, st, err);
+  RawKey key;
+  key.env(*L);
+  key.mpo(*W, true);       // (its values are checked against the charges)
+  key.env(*R);
+  key.site(*M);
+  const DeviceGradPlan* p = nullptr;
+  if (key.ok) {
+    auto it = c->grad_by_args.find(key);
+    if (it != c->grad_by_args.end()) p = it->second;
+  }
+  if (!p) {
+    std::string err;
+    EnvLayout le, re;
+    MpoLayout w;
+    SiteLayout m;
+    if ((st = make_env(L, &le, &err)) || (st = make_env(R, &re, &err)) ||
+        (st = make_mpo(W, &w, &err)) || (st = make_site(M, &m, &err)))
+      return fail(c, st, err);
+    if ((st = check_site_mpo(m, w, &err)) ||
+        (st = check_env(le, m.left, w.wl, w.tl, "L", &err)) ||
+        (st = check_env(re, m.right, w.wr, w.tr, "R", &err)))
+      return fail(c, st, err);
+    if (!L->data || !R->data || !M->data) return fail(c, DMRG3S_ERR_ARG, "NULL device data pointer");
+    if ((st = use_device(c))) return st;
+    if ((st = grad_plan(c, le, w, re, m, &p))) return st;
+    if (key.ok) c->grad_by_args[key] = p;
+  }
   if (!L->data || !R->data || !M->data) return fail(c, DMRG3S_ERR_ARG, "NULL device data pointer");
   if ((st = use_device(c))) return st;
-  const DeviceGradPlan* p = nullptr;
-  if ((st = grad_plan(c, le, w, re, m, &p))) return st;
   return run_mpo_grad(c, *p, L->data, M->data, R->data, G, reinterpret_cast<cudaStream_t>(stream));
 }
