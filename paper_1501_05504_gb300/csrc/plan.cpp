@@ -705,9 +705,19 @@ void split_k(const GemmStage& g3, int groups, GemmStage* parts, CombStage* sum, 
   sum->bytes = 0.0;
 }
 
-// Smaller combination chunks when a stage would have fewer than `target`
-// of them (small blocks: more CTAs, each with fewer rows).
-void rechunk(CombStage& c, int target) {
+// Smaller combination chunks when a stage would have too few of them: up to
+// kCombCtas CTAs per SM (all the threads an SM holds) while each still has
+// kCombElems elements, two per thread; two CTAs per SM when there are fewer
+// elements.  The sum of the cylinder's 0.9 M stage-3 partials, with two CTAs an
+// SM bound by the loads in flight, took 23 us of a 215 us 3xTF32 operator; the
+// operator takes 202 us (with the packing's tile search in one step).
+constexpr int kCombCtas = 8;
+constexpr int kCombElems = 512;
+void rechunk(CombStage& c) {
+  int64_t elems = 0;
+  for (const CombTask& t : c.tasks) elems += (int64_t)t.rows * t.cols;
+  const int64_t target = std::max<int64_t>(
+      2 * plan_ctas(), std::min<int64_t>(elems / kCombElems, kCombCtas * plan_ctas()));
   int rpc = kCombRows;
   auto count = [&](int r) {
     int64_t n = 0;
@@ -800,7 +810,7 @@ dmrg3s_status finish_sliced(Plan* p, int64_t nA1, int64_t nB1, int64_t nOut2, in
     G = std::max(1, std::min(G, maxseg));
     if (G > 1) {
       split_k(p->g3, G, &p->f3, &p->s3r, &p->ws3s);
-      rechunk(p->s3r, 2 * plan_ctas());
+      rechunk(p->s3r);
       ok = comb_ok(p->s3r.tasks, p->s3r.terms, std::max<int64_t>(p->ws3s, 1), nC3, err);
     } else {
       p->f3 = p->g3;
@@ -889,8 +899,8 @@ dmrg3s_status finish(Plan* p, int64_t nA1, int64_t nB1, int64_t nOut2, int64_t n
     *err = "internal planning error: " + *err;
     return DMRG3S_ERR_SHAPE;
   }
-  rechunk(p->c2, 2 * plan_ctas());
-  rechunk(p->c3r, 2 * plan_ctas());
+  rechunk(p->c2);
+  rechunk(p->c3r);
   return finish_sliced(p, nA1, nB1, nOut2, nA3, nB3, nC3, err);
 }
 
