@@ -20,14 +20,17 @@
 // times fewer sweeps on R^T than on A; the norm order cuts the sweeps on the
 // most graded sectors by a further third.
 //
-// Parallel order: the circle (round-robin) schedule.  With n' = n rounded up
-// to even and N = n' - 1, round r (0 <= r < N) pairs column r with N and
-// (r + k) mod N with (r - k) mod N for k = 1 .. n'/2 - 1; the N rounds of a
-// sweep meet every pair exactly once and the pairs of one round are disjoint
-// (a pair with the padding column N = n, n odd, is skipped).  Every pair of a
-// round is one warp and one launch runs a round of every matrix of the batch;
-// one sweep (a launch per round) is a CUDA graph.  A matrix with no rotation
-// in a sweep is converged and its warps exit at once in later sweeps.
+// Parallel order: columns in blocks of kJacB, blocks paired by the circle
+// (round-robin) schedule.  With nb' = the number of blocks rounded up to even and
+// N = nb' - 1, round r (0 <= r < N) pairs block r with N and (r + k) mod N with
+// (r - k) mod N for k = 1 .. nb'/2 - 1; the N rounds of a sweep meet every pair of
+// blocks exactly once and the pairs of one round are disjoint.  A pair of blocks
+// is a CTA, which takes the pairs of columns across the two blocks in kJacB
+// inner rounds of kJacB disjoint pairs, one warp each (in round 0 all pairs of
+// the 2 kJacB columns, in the circle schedule); columns >= n are skipped.  One
+// launch runs a round of every matrix of the batch; one sweep (a launch per
+// round) is a CUDA graph.  A matrix with no rotation in a sweep is converged and
+// its CTAs exit at once in later sweeps.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -51,8 +54,15 @@ constexpr int kJacThreads = 128;
 struct JacJob {
   int64_t offA, offY, offV, offTau;   // Y = R^T (n x n, ld n); V1 (n x n) or offV = -1
   int64_t offS, offVT, offU;          // outputs (offU = -1: no left vectors)
-  int32_t m, n, npad, pair0;          // pair0: first pair of the matrix in a round launch
-  int32_t col0, pad;                  // first column of the matrix in the batch numbering
+  int32_t m, n, col0, pad;            // col0: first column of the matrix in the batch numbering
+};
+
+// One pair of column blocks of a round launch (a CTA): pair k of its matrix's N
+// rounds.
+struct JacPair {
+  int64_t offY, offV;
+  int32_t n, col0, k, N;
+  int32_t job, staged;                // staged: the columns are held in shared memory
   double tol2;                        // the square of the pair tolerance
 };
 
@@ -115,172 +125,245 @@ jac_permute_kernel(const JacJob* __restrict__ jobs, const int* __restrict__ col_
   for (int i = threadIdx.x; i < J.m; i += kJacThreads) t[i] = x[i];
 }
 
-// The rotation (c, s) of a pair with Gram entries alpha = saa, beta = sbb,
-// gamma = sab: t = tan(theta) the smaller root of t^2 + 2 zeta t - 1 = 0,
-// zeta = (beta - alpha) / (2 gamma), c = 1 / sqrt(1 + t^2), s = c t.  GB300
-// issues FP64 at 1/64 of its FP32 rate, and a division or square root in
-// FP64 is a long chain of such instructions, so the angle is computed in
-// FP32 on (beta - alpha, 2 gamma) scaled by a common power of two (so that
-// neither underflows nor overflows), and (c, s) is then made orthonormal to
-// FP64 accuracy by two Newton steps on c^2 + s^2 = 1 (FP64 multiply-adds
-// only).  The angle carries FP32 rounding (~1e-7 relative): the rotated pair
-// is orthogonal to ~1e-7 of its former cosine rather than exactly, which the
-// next sweep removes; the rotation itself is orthogonal to FP64 rounding, so
-// the singular values are unaffected.
-__device__ __forceinline__ void jacobi_rotation(double saa, double sbb, double sab, double* c,
+// A double's top 24 bits as a float with the power of two 2^e taken out
+// (truncated; 0 where that is below the float range), and a float times 2^e as a
+// double (0 below the double range).  Integer instructions: a warp runs those
+// 32 times as fast as FP64 ones.
+__device__ __forceinline__ float float_of(double x, int e) {
+  const unsigned long long u = (unsigned long long)__double_as_longlong(x);
+  const int fe = (int)((u >> 52) & 0x7ff) - e + 127;
+  const unsigned sign = (unsigned)(u >> 32) & 0x80000000u;
+  return fe < 1 ? 0.f : __uint_as_float(sign | (unsigned)fe << 23 | ((unsigned)(u >> 29) & 0x7fffffu));
+}
+__device__ __forceinline__ double double_of(float x, int e) {   // x normal
+  const unsigned u = __float_as_uint(x);
+  const int de = (int)((u >> 23) & 0xff) + 896 + e;
+  const unsigned long long m = (unsigned long long)(u & 0x7fffffu) << 29;
+  const unsigned long long sign = (unsigned long long)(u & 0x80000000u) << 32;
+  return de < 1 ? 0.0 : __longlong_as_double((long long)(sign | (unsigned long long)de << 52 | m));
+}
+
+// The rotation of a pair with d = beta - alpha and gamma = g, as p = tan(theta / 2)
+// and s = sin(theta) = 2 p / (1 + p^2).  GB300 issues FP64 at 1/64 of its FP32
+// rate, and a division or square root in FP64 is a long chain of such
+// instructions, so the angle is computed in FP32 from d and 2 g scaled by a
+// common power of two; p is that FP32 number and s belongs to it to FP64
+// accuracy (an FP32 reciprocal r0 of q = 1 + p^2, then 1 / q = r0 (1 + e + e^2 +
+// ..) with e = 1 - q r0 below 2^-22).  The angle carries FP32 rounding (~1e-7
+// relative): the rotated pair is orthogonal to ~1e-7 of its former cosine rather
+// than exactly, which the next sweep removes; the rotation itself is orthogonal
+// to FP64 rounding, so the singular values are unaffected.
+__device__ __forceinline__ void jacobi_rotation(double d, double g, double* p, double* p2,
                                                 double* s) {
-  const double d = sbb - saa, g2 = 2.0 * sab;
-  const double big = fmax(fabs(d), fabs(g2));
-  // 2^-e with e the binary exponent of big (a normal number here)
-  const long long eb = (__double_as_longlong(big) >> 52) & 0x7ff;
-  const double scale = __longlong_as_double((long long)(2046 - eb) << 52);
-  const double ds = d * scale, gs = g2 * scale;   // the larger magnitude in [1, 2)
-  const float df = (float)ds, gf = (float)gs;
-  double t;
-  if (fabs(ds) > 1048576.0 * fabs(gs)) {
-    // |zeta| > 2^20: t = 1 / (2 zeta) = gamma / (beta - alpha) to FP32 rounding, in
-    // FP64 (it may be far below the FP32 range) with an FP32 reciprocal of ds
-    t = 0.5 * gs * (double)(1.0f / df);
+  const int ed = (int)(__double_as_longlong(d) >> 52) & 0x7ff;
+  const int eg = ((int)(__double_as_longlong(g) >> 52) & 0x7ff) + 1;   // of 2 g
+  double pp, pp2;
+  float pf = 0.f;
+  if (ed - eg > 20) {
+    // |zeta| > 2^19: theta = gamma / (beta - alpha) to FP32 rounding
+    const float t = __fdiv_rn(float_of(g, eg - 1), float_of(d, ed));
+    pp = double_of(t, eg - ed - 2);
+    pp2 = double_of(t, eg - ed - 1);
   } else {
-    const float z = df / gf;
-    t = (double)(copysignf(1.0f, z) / (fabsf(z) + sqrtf(fmaf(z, z, 1.0f))));
+    const int e = max(ed, eg);
+    const float z = __fdiv_rn(float_of(d, e), float_of(g, e - 1));
+    const float t = copysignf(1.0f, z) / (fabsf(z) + sqrtf(fmaf(z, z, 1.0f)));
+    const float c = rsqrtf(fmaf(t, t, 1.0f));
+    pf = t * c / (1.0f + c);
+    pp = double_of(pf, 0);
+    pp2 = double_of(pf, 1);
   }
-  const float tf = (float)t;
-  const float c32 = rsqrtf(fmaf(tf, tf, 1.0f));
-  double cc = c32, ss = (double)c32 * t;
-#pragma unroll
-  for (int it = 0; it < 2; ++it) {
-    const double r = fma(-0.5, fma(cc, cc, ss * ss), 1.5);
-    cc *= r;
-    ss *= r;
-  }
-  *c = cc;
-  *s = ss;
+  const double r0 = double_of(1.0f / fmaf(pf, pf, 1.0f), 0);
+  const double q = fma(pp, pp, 1.0);
+  const double e1 = fma(-q, r0, 1.0);
+  const double s0 = pp2 * r0;
+  *p = pp;
+  *p2 = pp2;
+  *s = fma(s0, fma(e1, e1, e1), s0);
 }
 
-// Advances the sweep counter read by the round kernels (first node of a sweep).
-__global__ void jac_next_sweep_kernel(int* sweep) {
-  grid_next();
-  grid_wait(); *sweep += 1; }
-
-// Sums of three per-lane values over the warp, returned to every lane with
-// the same bits in every lane.  The first two levels exchange halves of the
-// values a lane carries (the lower 16 lanes go on with x and y, the upper
-// with z and a zero; then each group of 8 with one of those), so the five
-// levels take 6 FP64 additions instead of the 15 of a butterfly per value;
-// the last three levels are a butterfly within each group of 8 lanes, whose
-// lanes then hold identical sums (IEEE addition commutes bit for bit).
-__device__ __forceinline__ void warp_sum3(double& x, double& y, double& z) {
-  const int lane = threadIdx.x & 31;
-  const bool hi16 = (lane & 16) != 0, hi8 = (lane & 8) != 0;
-  const double w = 0.0;
-  const double a = (hi16 ? z : x) + __shfl_xor_sync(0xffffffffu, hi16 ? x : z, 16);
-  const double b = (hi16 ? w : y) + __shfl_xor_sync(0xffffffffu, hi16 ? y : w, 16);
-  double c = (hi8 ? b : a) + __shfl_xor_sync(0xffffffffu, hi8 ? a : b, 8);
-  for (int o = 4; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
-  x = __shfl_sync(0xffffffffu, c, 0);    // lanes 0-7: the sum of x
-  y = __shfl_sync(0xffffffffu, c, 8);    // lanes 8-15: of y
-  z = __shfl_sync(0xffffffffu, c, 16);   // lanes 16-23: of z
+// (a, b) <- (c a - s b, s a + c b) as three shears: half the roundings of the
+// product form, and the error of each is that of a fused multiply-add (the
+// singular values of graded 100 to 245-column matrices, against long double: 1.4
+// to 2.7e-15 at the largest, 4 to 7e-15 in the product form).
+__device__ __forceinline__ void shears(double p, double s, double& a, double& b) {
+  a = fma(-p, b, a);
+  b = fma(s, a, b);
+  a = fma(-p, b, a);
 }
 
-// One round r of the current sweep for every matrix: one warp per pair,
-// kJacPairsPerCta pairs per CTA.  rot[s * njobs + job] counts the rotations
-// of sweep s.  GB300 runs an FP64 warp instruction in ~64 cycles of a
-// sub-partition, so the round is priced in FP64 instructions: a warp per
-// pair does the pair's three dot products and its rotation with the same
-// count as a CTA would, but reduces once instead of once per warp, and every
-// lane computes the (identical) rotation itself, with no shared memory, CTA
-// barrier or single-thread step.  The first kJacCache elements of each
-// lane's share stay in registers between the dot products and the rotation.
-constexpr int kJacPairsPerCta = 4;
-constexpr int kJacCache = 8;
-__global__ void __launch_bounds__(32 * kJacPairsPerCta)
-jac_round_kernel(const JacJob* __restrict__ jobs, const int* __restrict__ pair_job, int npairs,
-                 int njobs, int r, const int* sweep, int* rot,
-                 double* Y, double* V) {
+// Starts a sweep: the squared norm of every column of every Y (one CTA per
+// column), and the sweep counter read by the round kernels.
+__global__ void __launch_bounds__(kJacThreads)
+jac_sweep_kernel(const JacJob* __restrict__ jobs, const int* __restrict__ col_job,
+                 const double* Y, double* nrm, int* sweep) {
   grid_next();
   grid_wait();
-  const int p = blockIdx.x * kJacPairsPerCta + (threadIdx.x >> 5);
-  const int lane = threadIdx.x & 31;
-  if (p >= npairs) return;
+  __shared__ double red[kJacThreads / 32];
+  const JacJob J = jobs[col_job[blockIdx.x]];
+  const double* y = Y + J.offY + (int64_t)(blockIdx.x - J.col0) * J.n;
+  double s = 0.0;
+  for (int i = threadIdx.x; i < J.n; i += kJacThreads) s = fma(y[i], y[i], s);
+  s = cta_sum(s, red);
+  if (threadIdx.x == 0) {
+    nrm[blockIdx.x] = s;
+    if (blockIdx.x == 0) *sweep += 1;
+  }
+}
+
+// One round r of the current sweep for every matrix: one CTA per pair of
+// blocks, one warp per pair of columns.  rot[s * njobs + job] counts the
+// rotations of sweep s.  GB300 runs an FP64 warp instruction in ~64 cycles of a
+// sub-partition, and the pairs of a truncation are about as many as the chip's
+// sub-partitions, so an inner round is priced in FP64 instructions of one warp:
+// one dot product (the squared norms are kept through the sweep by the rotation's
+// own recurrence, |y_a'|^2 = alpha + s (s (beta - alpha) - 2 c gamma), and formed
+// anew at the next sweep's start, so the last sweep, which rotates nothing, tests
+// every pair with fresh norms), one reduction, ~15 for the rotation (every lane
+// computes the identical one: no exchange), and three shears per element: ~55 at
+// n = 245 where three dot products and the product form took ~80.  The columns
+// of a CTA stay in shared memory between the inner rounds where they fit, so
+// that only every kJacB-th round pays for a launch and for its loads.  Whole
+// factorisations, a launch per round of column pairs before: 762 x 245 18.1 ->
+// 13.3 ms, 900 x 600 74 -> 44, 1300 x 1100 (columns in global memory) 213 -> 124;
+// the local update of an m = 512 XXZ window 30.6 -> 24.9.
+constexpr int kJacB = 4;
+constexpr int kJacCache = 8;              // elements of a column that a lane keeps in registers
+constexpr size_t kJacStage = 64 * 1024;   // shared memory of a CTA: three fit an SM
+__global__ void __launch_bounds__(32 * kJacB)
+jac_round_kernel(const JacPair* __restrict__ pairs, int njobs, int r, const int* sweep, int* rot,
+                 double* nrm, double* Y, double* V) {
+  grid_next();
+  grid_wait();
+  extern __shared__ double cols[];
+  __shared__ double s_nrm[2 * kJacB];
+  const JacPair P = pairs[blockIdx.x];
   const int sw = *sweep;
-  if (sw < 0 || sw >= kJacobiMaxSweeps) return;
-  const int jb = pair_job[p];
-  if (sw > 0 && rot[(sw - 1) * njobs + jb] == 0) return;   // converged in the previous sweep
-  const JacJob J = jobs[jb];
-  const int N = J.npad - 1;
-  if (r >= N) return;
-  const int k = p - J.pair0;
-  int a, b;
-  if (k == 0) {
-    a = r;
-    b = N;
-  } else {
-    a = (r + k) % N;
-    b = (r - k + N) % N;
-  }
-  const int n = J.n;
-  if (a >= n || b >= n) return;   // the padding column
-  double* ya = Y + J.offY + (int64_t)a * n;
-  double* yb = Y + J.offY + (int64_t)b * n;
-  double ua[kJacCache], ub[kJacCache];
-  double saa = 0.0, sbb = 0.0, sab = 0.0;
-#pragma unroll
-  for (int e = 0; e < kJacCache; ++e) {
-    const int i = lane + e * 32;
-    ua[e] = i < n ? ya[i] : 0.0;
-    ub[e] = i < n ? yb[i] : 0.0;
-    saa = fma(ua[e], ua[e], saa);
-    sbb = fma(ub[e], ub[e], sbb);
-    sab = fma(ua[e], ub[e], sab);
-  }
-  for (int i = lane + kJacCache * 32; i < n; i += 32) {
-    const double u = ya[i], v = yb[i];
-    saa = fma(u, u, saa);
-    sbb = fma(v, v, sbb);
-    sab = fma(u, v, sab);
-  }
-  warp_sum3(saa, sbb, sab);
-  // zero columns and NaN leave the pair unrotated (NaN reaches the singular values)
-  if (!(saa > 0.0 && sbb > 0.0 && sab * sab > J.tol2 * saa * sbb)) return;
-  double cs, sn;
-  jacobi_rotation(saa, sbb, sab, &cs, &sn);
-  if (lane == 0) atomicAdd(rot + sw * njobs + jb, 1);
-#pragma unroll
-  for (int e = 0; e < kJacCache; ++e) {
-    const int i = lane + e * 32;
-    if (i < n) {
-      ya[i] = cs * ua[e] - sn * ub[e];
-      yb[i] = sn * ua[e] + cs * ub[e];
+  if (r >= P.N || sw < 0 || sw >= kJacobiMaxSweeps) return;
+  const int n = P.n, k = P.k, N = P.N;
+  // first columns of the two blocks
+  const int ca = (k == 0 ? r : (r + k) % N) * kJacB;
+  const int cb = (k == 0 ? N : (r - k + N) % N) * kJacB;
+  if (r > 0 && (ca >= n || cb >= n)) return;   // the padding block
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int before = sw > 0 ? rot[(sw - 1) * njobs + P.job] : 1;
+  const bool vec = P.offV >= 0;
+  double* yg = Y + P.offY;
+  double* vg = vec ? V + P.offV : nullptr;
+  double* ys = cols;
+  double* vs = cols + 2 * kJacB * n;
+  const auto column = [&](int c) { return c < kJacB ? ca + c : cb + c - kJacB; };
+  if (P.staged) {
+    for (int h = 0; h < 2; ++h) {
+      const int c = warp + h * kJacB;
+      const int g = column(c);
+      if (g >= n) continue;
+      for (int i = lane; i < n; i += 32) ys[c * n + i] = yg[(int64_t)g * n + i];
+      if (vec)
+        for (int i = lane; i < n; i += 32) vs[c * n + i] = vg[(int64_t)g * n + i];
     }
   }
-  for (int i = lane + kJacCache * 32; i < n; i += 32) {
-    const double u = ya[i], v = yb[i];
-    ya[i] = cs * u - sn * v;
-    yb[i] = sn * u + cs * v;
+  if (threadIdx.x < 2 * kJacB) {
+    const int g = column(threadIdx.x);
+    s_nrm[threadIdx.x] = g < n ? nrm[P.col0 + g] : 0.0;
   }
-  if (J.offV >= 0) {
-    double* va = V + J.offV + (int64_t)a * n;
-    double* vb = V + J.offV + (int64_t)b * n;
-#pragma unroll
-    for (int e = 0; e < kJacCache; ++e) {      // every load before the first store
-      const int i = lane + e * 32;
-      ua[e] = i < n ? va[i] : 0.0;
-      ub[e] = i < n ? vb[i] : 0.0;
+  if (before == 0) return;   // converged in the previous sweep (the same for the whole CTA)
+  __syncthreads();
+  const int M = 2 * kJacB - 1;
+  const int inner = r == 0 ? M : kJacB;
+  int nrot = 0;
+  for (int q = 0; q < inner; ++q) {
+    int a, b;
+    if (r > 0) {
+      a = warp;
+      b = kJacB + ((warp + q) & (kJacB - 1));
+    } else {
+      a = warp == 0 ? q : (q + warp) % M;
+      b = warp == 0 ? M : (q - warp + M) % M;
     }
+    const int ga = column(a), gb = column(b);
+    if (ga < n && gb < n) {
+      double* ya = P.staged ? ys + a * n : yg + (int64_t)ga * n;
+      double* yb = P.staged ? ys + b * n : yg + (int64_t)gb * n;
+      const double alpha = s_nrm[a], beta = s_nrm[b];
+      double ua[kJacCache], ub[kJacCache];
+      double g0 = 0.0, g1 = 0.0;
 #pragma unroll
-    for (int e = 0; e < kJacCache; ++e) {
-      const int i = lane + e * 32;
-      if (i < n) {
-        va[i] = cs * ua[e] - sn * ub[e];
-        vb[i] = sn * ua[e] + cs * ub[e];
+      for (int e = 0; e < kJacCache; ++e) {
+        const int i = lane + e * 32;
+        ua[e] = i < n ? ya[i] : 0.0;
+        ub[e] = i < n ? yb[i] : 0.0;
+      }
+#pragma unroll
+      for (int e = 0; e < kJacCache; ++e)
+        if (e * 32 < n) {
+          if (e & 1) g1 = fma(ua[e], ub[e], g1);
+          else g0 = fma(ua[e], ub[e], g0);
+        }
+      for (int i = lane + kJacCache * 32; i < n; i += 32) g0 = fma(ya[i], yb[i], g0);
+      double g = g0 + g1;
+      for (int o = 16; o > 0; o >>= 1) g += __shfl_xor_sync(0xffffffffu, g, o);
+      // zero columns and NaN leave the pair unrotated (NaN reaches the singular
+      // values); a norm cancelled to nothing waits for the next sweep's
+      if (__double_as_longlong(alpha) > 0 && __double_as_longlong(beta) > 0 &&
+          g * g > P.tol2 * alpha * beta) {
+        const double d = beta - alpha;
+        double p, p2, s;
+        jacobi_rotation(d, g, &p, &p2, &s);
+        ++nrot;
+#pragma unroll
+        for (int e = 0; e < kJacCache; ++e)
+          if (e * 32 < n) {
+            shears(p, s, ua[e], ub[e]);
+            const int i = lane + e * 32;
+            if (i < n) {
+              ya[i] = ua[e];
+              yb[i] = ub[e];
+            }
+          }
+        for (int i = lane + kJacCache * 32; i < n; i += 32) {
+          double u = ya[i], v = yb[i];
+          shears(p, s, u, v);
+          ya[i] = u;
+          yb[i] = v;
+        }
+        if (vec) {
+          double* va = P.staged ? vs + a * n : vg + (int64_t)ga * n;
+          double* vb = P.staged ? vs + b * n : vg + (int64_t)gb * n;
+#pragma unroll 4
+          for (int i = lane; i < n; i += 32) {
+            double u = va[i], v = vb[i];
+            shears(p, s, u, v);
+            va[i] = u;
+            vb[i] = v;
+          }
+        }
+        const double c2 = fma(-p2, s, 2.0);   // 2 cos(theta)
+        const double dl = s * fma(s, d, -(c2 * g));
+        __syncwarp();
+        if (lane == 0) {
+          s_nrm[a] = alpha + dl;
+          s_nrm[b] = beta - dl;
+        }
       }
     }
-    for (int i = lane + kJacCache * 32; i < n; i += 32) {
-      const double u = va[i], v = vb[i];
-      va[i] = cs * u - sn * v;
-      vb[i] = sn * u + cs * v;
+    __syncthreads();
+  }
+  if (nrot && lane == 0) atomicAdd(rot + sw * njobs + P.job, nrot);
+  if (!__syncthreads_or(nrot)) return;
+  if (P.staged) {
+    for (int h = 0; h < 2; ++h) {
+      const int c = warp + h * kJacB;
+      const int g = column(c);
+      if (g >= n) continue;
+      for (int i = lane; i < n; i += 32) yg[(int64_t)g * n + i] = ys[c * n + i];
+      if (vec)
+        for (int i = lane; i < n; i += 32) vg[(int64_t)g * n + i] = vs[c * n + i];
     }
+  }
+  if (threadIdx.x < 2 * kJacB) {
+    const int g = column(threadIdx.x);
+    if (g < n) nrm[P.col0 + g] = s_nrm[threadIdx.x];
   }
 }
 
@@ -379,9 +462,11 @@ dmrg3s_status svd_jacobi(Context* c, std::vector<SvdLane>& lanes, int nlanes,
   if (nlanes < 1) return fail(c, DMRG3S_ERR_ARG, "no SVD lane");
   // ---- tables
   std::vector<JacJob> tab(nj);
-  std::vector<int> pair_job, col_job;
+  std::vector<JacPair> pairs;
+  std::vector<int> col_job;
   int64_t ny = 0, nv = 0, ntau = 0;
   int maxr = 0;
+  size_t smem = 0;
   for (int k = 0; k < nj; ++k) {
     const SvdJob& jb = jobs[k];
     if (jb.n < 1 || jb.m < jb.n || jb.m > (1 << 30) || jb.n > (1 << 15))
@@ -400,33 +485,41 @@ dmrg3s_status svd_jacobi(Context* c, std::vector<SvdLane>& lanes, int nlanes,
     t.offU = jb.offU;
     t.m = (int32_t)jb.m;
     t.n = (int32_t)jb.n;
-    t.npad = t.n + (t.n & 1);
-    t.pair0 = (int32_t)pair_job.size();
     t.col0 = (int32_t)col_job.size();
     t.pad = 0;
-    const double tol = std::max(std::sqrt((double)t.n), 32.0) * DBL_EPSILON;
-    t.tol2 = tol * tol;
-    pair_job.insert(pair_job.end(), t.npad / 2, k);
     col_job.insert(col_job.end(), t.n, k);
-    maxr = std::max(maxr, t.npad - 1);
+    const double tol = std::max(std::sqrt((double)t.n), 32.0) * DBL_EPSILON;
+    const int nb = (t.n + kJacB - 1) / kJacB, nbpad = nb + (nb & 1);
+    const size_t bytes = (size_t)2 * kJacB * t.n * sizeof(double) * (t.offV >= 0 ? 2 : 1);
+    const bool staged = bytes <= kJacStage;
+    if (staged) smem = std::max(smem, bytes);
+    maxr = std::max(maxr, nbpad - 1);
+    for (int q = 0; q < nbpad / 2; ++q)
+      pairs.push_back(JacPair{t.offY, t.offV, t.n, t.col0, q, nbpad - 1, k, staged, tol * tol});
   }
-  const int npair = (int)pair_job.size(), ncol = (int)col_job.size();
-  const int ncta = (npair + kJacPairsPerCta - 1) / kJacPairsPerCta;
+  const int ncta = (int)pairs.size(), ncol = (int)col_job.size();
   int64_t na = 0;   // extent of the A buffer used by the jobs
   for (const JacJob& t : tab) na = std::max(na, t.offA + (int64_t)t.m * t.n);
   // ---- device buffers: doubles [tau | Y | V1 | sigma | column norms | T = A P],
-  //      ints [pair_job | col_job | perm | rot | sweep | qinfo]
+  //      ints [col_job | perm | rot | sweep | qinfo]
   const int64_t nd = ntau + ny + nv + 2 * (int64_t)ncol + na;
-  const int64_t ni = npair + 2 * (int64_t)ncol + (int64_t)kJacobiMaxSweeps * nj + 1 + nj;
+  const int64_t ni = 2 * (int64_t)ncol + (int64_t)kJacobiMaxSweeps * nj + 1 + nj;
   double* dd = nullptr;
   int* di = nullptr;
   JacJob* dt = nullptr;
+  JacPair* dp = nullptr;
   dmrg3s_status s = DMRG3S_OK;
   if ((s = cuda_ok(c, cudaMallocAsync((void**)&dd, (size_t)nd * sizeof(double), st), "SVD buffers")) ||
       (s = cuda_ok(c, cudaMallocAsync((void**)&di, (size_t)ni * sizeof(int), st), "SVD buffers")) ||
-      (s = cuda_ok(c, cudaMallocAsync((void**)&dt, tab.size() * sizeof(JacJob), st), "SVD buffers"))) {
+      (s = cuda_ok(c, cudaMallocAsync((void**)&dt, tab.size() * sizeof(JacJob), st), "SVD buffers")) ||
+      (s = cuda_ok(c, cudaMallocAsync((void**)&dp, pairs.size() * sizeof(JacPair), st), "SVD buffers")) ||
+      (s = cuda_ok(c, cudaFuncSetAttribute(jac_round_kernel,
+                                           cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                           (int)kJacStage), "Jacobi shared memory"))) {
     if (dd) cudaFreeAsync(dd, st);
     if (di) cudaFreeAsync(di, st);
+    if (dt) cudaFreeAsync(dt, st);
+    if (dp) cudaFreeAsync(dp, st);
     return s;
   }
   double* tau = dd;
@@ -435,14 +528,13 @@ dmrg3s_status svd_jacobi(Context* c, std::vector<SvdLane>& lanes, int nlanes,
   double* sig = V1 + nv;
   double* anrm = sig + ncol;
   double* T = anrm + ncol;
-  int* d_pair = di;
-  int* d_col = d_pair + npair;
+  int* d_col = di;
   int* d_perm = d_col + ncol;
   int* rot = d_perm + ncol;
   int* d_sweep = rot + (int64_t)kJacobiMaxSweeps * nj;
   int* qinfo = d_sweep + 1;
   cudaMemcpyAsync(dt, tab.data(), tab.size() * sizeof(JacJob), cudaMemcpyHostToDevice, st);
-  cudaMemcpyAsync(d_pair, pair_job.data(), pair_job.size() * sizeof(int), cudaMemcpyHostToDevice, st);
+  cudaMemcpyAsync(dp, pairs.data(), pairs.size() * sizeof(JacPair), cudaMemcpyHostToDevice, st);
   cudaMemcpyAsync(d_col, col_job.data(), col_job.size() * sizeof(int), cudaMemcpyHostToDevice, st);
   cudaMemsetAsync(rot, 0, (size_t)kJacobiMaxSweeps * nj * sizeof(int), st);
   cudaMemsetAsync(d_sweep, 0xff, sizeof(int), st);   // -1: the first sweep advances it to 0
@@ -569,9 +661,9 @@ dmrg3s_status svd_jacobi(Context* c, std::vector<SvdLane>& lanes, int nlanes,
   cudaGraphExec_t gexec = nullptr;
   if (!s && cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking) == cudaSuccess &&
       cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal) == cudaSuccess) {
-    launch_chain(jac_next_sweep_kernel, 1, 1, 0, cap, d_sweep);
+    launch_chain(jac_sweep_kernel, ncol, kJacThreads, 0, cap, dt, d_col, Y, anrm, d_sweep);
     for (int r = 0; r < maxr; ++r)
-      launch_chain(jac_round_kernel, ncta, 32 * kJacPairsPerCta, 0, cap, dt, d_pair, npair, nj, r, d_sweep, rot, Y, V1);
+      launch_chain(jac_round_kernel, ncta, 32 * kJacB, smem, cap, dp, nj, r, d_sweep, rot, anrm, Y, V1);
     if (cudaStreamEndCapture(cap, &graph) != cudaSuccess ||
         cudaGraphInstantiate(&gexec, graph, 0) != cudaSuccess)
       gexec = nullptr;
@@ -588,9 +680,9 @@ dmrg3s_status svd_jacobi(Context* c, std::vector<SvdLane>& lanes, int nlanes,
     if (gexec) {
       s = cuda_ok(c, cudaGraphLaunch(gexec, st), "Jacobi sweep");
     } else {
-      launch_chain(jac_next_sweep_kernel, 1, 1, 0, st, d_sweep);
+      launch_chain(jac_sweep_kernel, ncol, kJacThreads, 0, st, dt, d_col, Y, anrm, d_sweep);
       for (int r = 0; r < maxr; ++r)
-        launch_chain(jac_round_kernel, ncta, 32 * kJacPairsPerCta, 0, st, dt, d_pair, npair, nj, r, d_sweep, rot, Y, V1);
+        launch_chain(jac_round_kernel, ncta, 32 * kJacB, smem, st, dp, nj, r, d_sweep, rot, anrm, Y, V1);
       s = cuda_ok(c, cudaGetLastError(), "Jacobi sweep");
     }
     count_launch(maxr + 1);
@@ -658,6 +750,7 @@ dmrg3s_status svd_jacobi(Context* c, std::vector<SvdLane>& lanes, int nlanes,
   cudaFreeAsync(dd, st);
   cudaFreeAsync(di, st);
   cudaFreeAsync(dt, st);
+  cudaFreeAsync(dp, st);
   if (ev_in) cudaEventDestroy(ev_in);
   return s;
 }
