@@ -259,7 +259,6 @@ struct Context {
   cudaStream_t aux = nullptr;   // side stream: the Lanczos tridiagonal solve beside the next product
   cudaEvent_t ev_ready = nullptr, ev_done = nullptr;
   cudaEvent_t ev_lz[3] = {nullptr, nullptr, nullptr};   // Lanczos results of iterations k mod 3
-  cudaStream_t cap = nullptr;   // private stream for capturing the Lanczos iteration graph
   double* pinned_big = nullptr;   // pinned read-back area of the batched Lanczos (grown on demand)
   size_t pinned_big_n = 0;        // its size in doubles
   std::unordered_map<uint64_t, std::unique_ptr<DevicePlan>> plans;

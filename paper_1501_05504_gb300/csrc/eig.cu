@@ -34,12 +34,13 @@ dmrg3s_status pinned_reserve(Context* c, size_t n) {
 }
 
 // Iteration k of every problem, on the main stream:
-//   two classical Gram-Schmidt passes of w = H v_k against v_0 .. v_k in three
-//   launches (dots; update fused with the second pass's dots; update with
-//   the partial norms of w); the first pass's last coefficient is alpha_k;
-//   v_{k+1} = w / |w|; w = H v_{k+1};
-// then, on the side stream, the tridiagonal solve of order k + 1 and the copy
-// of its results to the host.  The host reads iteration k's results only
+//   two classical Gram-Schmidt passes of w = H v_k against v_0 .. v_k and
+//   v_{k+1} = w / |w| in one cooperative launch (more than one chunk per SM:
+//   dots; update fused with the second pass's dots; update with the partial
+//   norms of w; scaling); the first pass's last coefficient is alpha_k;
+//   w = H v_{k+1};
+// and beside the product, on the side stream, the tridiagonal solve of order
+// k + 1 and the copy of its results to the host.  The host reads iteration k's results only
 // after it has enqueued iteration k + 2, so the device never waits for the
 // host's stopping decision; a problem that has stopped keeps being iterated
 // (its results are no longer read) until every problem has stopped, and the
@@ -65,10 +66,14 @@ dmrg3s_status lanczos_batch(Context* c, const DevicePlan& heff, const double* Ld
   for (int i = 0; i < np; ++i) ranges[i] = {probs[i].off, probs[i].n};
   std::vector<LzChunk> hch;
   std::vector<LzChain> hcn;
-  // about one chunk per SM: few partials per problem to finish the sums
-  // from, several elements per thread
-  lz_layout(ranges, plan_ctas(), &hch, &hcn);
+  // at most one chunk per SM where the sizes allow: few partials per problem to
+  // finish the sums from, and an iteration's orthogonalisation in one cooperative
+  // launch (the longest chunk is kLzChunkMax: 0.6 M elements in all)
+  lz_layout(ranges, std::max(1, plan_ctas() - np), &hch, &hcn);
   const int nchunks = (int)hch.size();
+  const bool one_launch = nchunks <= plan_ctas();
+  int maxlen = 0;
+  for (const LzChunk& ch : hch) maxlen = std::max(maxlen, (int)(ch.e1 - ch.e0));
   // FP64 products in the sliced form when the Krylov basis fits behind its
   // intermediates, else in the plain form (the caller's cursor)
   SplitHints hints;
@@ -97,7 +102,7 @@ dmrg3s_status lanczos_batch(Context* c, const DevicePlan& heff, const double* Ld
       (s = carve(c, &cursor, sizeof(LzChunk) * nchunks, &pch)) ||
       (s = carve(c, &cursor, sizeof(LzChain) * np, &pcn)) ||
       (s = carve(c, &cursor, sizeof(int32_t) * np, &pks)) ||
-      (s = carve(c, &cursor, sizeof(int), &pk)))
+      (s = carve(c, &cursor, 2 * sizeof(int), &pk)))
     return s;
   // read-back slots: kLzLag iterations' results (4 doubles per problem) and the error word
   const size_t slot = (size_t)np * 4 + 2;
@@ -117,6 +122,7 @@ dmrg3s_status lanczos_batch(Context* c, const DevicePlan& heff, const double* Ld
   LzChain* dcn = (LzChain*)pcn;
   int32_t* dks = (int32_t*)pks;
   int* kdev = (int*)pk;
+  unsigned* arrivals = (unsigned*)pk + 1;
   if (cudaMemcpyAsync(dch, hch.data(), sizeof(LzChunk) * nchunks, cudaMemcpyHostToDevice, st) !=
           cudaSuccess ||
       cudaMemcpyAsync(dcn, hcn.data(), sizeof(LzChain) * np, cudaMemcpyHostToDevice, st) !=
@@ -163,7 +169,7 @@ dmrg3s_status lanczos_batch(Context* c, const DevicePlan& heff, const double* Ld
   }
   launch_lz_normalise(X, V, dch, nchunks, dcn, nrm_x, st);
   cudaMemcpyAsync(vcur, V, sizeof(double) * ldv, cudaMemcpyDeviceToDevice, st);
-  cudaMemsetAsync(kdev, 0, sizeof(int), st);
+  cudaMemsetAsync(kdev, 0, 2 * sizeof(int), st);
 
   std::vector<int> kstop(np, -1);
   theta->assign(np, 0.0);
@@ -178,42 +184,36 @@ dmrg3s_status lanczos_batch(Context* c, const DevicePlan& heff, const double* Ld
   };
   // profiler records of the product that builds on iteration k (index k + 1)
   std::vector<std::pair<size_t, size_t>> prod_recs(kp + 1, {0, 0});
-  auto product = [&](int j, cudaStream_t q) -> dmrg3s_status {   // w = H v_j (v_j in vcur)
+  auto product = [&](int j) -> dmrg3s_status {   // w = H v_j (v_j in vcur)
     const size_t r0 = c->prof.recs.size();
-    dmrg3s_status r = run_plan(c, heff, Ldata, vcur, ws1, ws2, 1.0, ws2, Rdata, w, q, prec,
+    dmrg3s_status r = run_plan(c, heff, Ldata, vcur, ws1, ws2, 1.0, ws2, Rdata, w, st, prec,
                                &hints);
-    if (j >= 0) prod_recs[j] = {r0, c->prof.recs.size()};
+    prod_recs[j] = {r0, c->prof.recs.size()};
     return r != DMRG3S_OK ? fail(c, r, "H_eff launch failed") : DMRG3S_OK;
   };
-  // Iteration k on stream q with k from the device counter: two Gram-Schmidt
-  // passes (the update of the first fused with the dots of the second),
-  // v_{k+1} into the basis and vcur, w = H v_{k+1}, k += 1.
-  auto body = [&](cudaStream_t q, int j) -> dmrg3s_status {
-    launch_lz_dots(V, ldv, 0, w, dch, nchunks, part, kp, q, kdev);
-    launch_lz_update_dots(V, ldv, 0, w, dch, nchunks, dcn, part, kp, alpha, part2, q, kdev);
-    launch_lz_update(V, ldv, 0, w, dch, nchunks, dcn, part2, kp, nullptr, nrm, q, kdev, nchunks);
-    launch_lz_next(w, V, ldv, kdev, vcur, dch, nchunks, dcn, nrm, nchunks, q);
-    dmrg3s_status r = product(j, q);
-    launch_lz_advance(kdev, q);
-    return r;
-  };
-  if ((s = product(0, st))) return bail(s);
-  // Without the profiler, the iteration is captured once into a CUDA graph
-  // (every kernel reads k from the device counter) and replayed; with it,
-  // the launches are issued directly so that each product is recorded.
-  cudaGraphExec_t gexec = nullptr;
-  if (!c->prof.on && c->cap) {
-    const PlainLaunches plain;
-    cudaGraph_t graph = nullptr;
-    bool ok = cudaStreamBeginCapture(c->cap, cudaStreamCaptureModeThreadLocal) == cudaSuccess;
-    if (ok) {
-      const dmrg3s_status r = body(c->cap, -1);
-      ok = cudaStreamEndCapture(c->cap, &graph) == cudaSuccess && r == DMRG3S_OK;
+  // Iteration k (from the device counter) up to its product: two Gram-Schmidt
+  // passes (the update of the first fused with the dots of the second), v_{k+1}
+  // into the basis and vcur, k += 1.  The launches are issued directly: chained ones
+  // (launch.hpp) keep the device busier than replays of a captured iteration, in
+  // which the products cannot be chained (3387 us against 3505 for 40 iterations
+  // of the m = 512 XXZ chain in 3xTF32; 72 us an iteration against 73 at m = 32,
+  // where the host's share is largest).  In all, with the tridiagonal solve beside
+  // the product: 4745 -> 3284 us (3xTF32) and 5288 -> 4371 us (FP64).
+  auto orthogonalise = [&]() -> dmrg3s_status {
+    if (one_launch) {
+      if (!launch_lz_orth(V, ldv, kdev, w, vcur, dch, nchunks, maxlen, dcn, part, part2, kp, alpha,
+                          nrm, nchunks, arrivals, c->d_err, c->wait_ns, st))
+        return fail(c, DMRG3S_ERR_CUDA, "Lanczos orthogonalisation launch");
+    } else {
+      launch_lz_dots(V, ldv, 0, w, dch, nchunks, part, kp, st, kdev);
+      launch_lz_update_dots(V, ldv, 0, w, dch, nchunks, dcn, part, kp, alpha, part2, st, kdev);
+      launch_lz_update(V, ldv, 0, w, dch, nchunks, dcn, part2, kp, nullptr, nrm, st, kdev, nchunks);
+      launch_lz_next(w, V, ldv, kdev, vcur, dch, nchunks, dcn, nrm, nchunks, st);
+      launch_lz_advance(kdev, st);
     }
-    if (ok && cudaGraphInstantiate(&gexec, graph, 0) != cudaSuccess) gexec = nullptr;
-    if (graph) cudaGraphDestroy(graph);
-    cudaGetLastError();   // a failed capture leaves the direct launches
-  }
+    return DMRG3S_OK;
+  };
+  if ((s = product(0))) return bail(s);
   // the host's reading of iteration k
   auto collect = [&](int k) -> dmrg3s_status {
     if (cudaEventSynchronize(c->ev_lz[k % kLzLag]) != cudaSuccess)
@@ -250,16 +250,7 @@ dmrg3s_status lanczos_batch(Context* c, const DevicePlan& heff, const double* Ld
   int last = -1;   // the last iteration enqueued
   int next_read = 0;
   for (int k = 0; k < kmax; ++k) {
-    if (gexec) {
-      if (cudaGraphLaunch(gexec, st) != cudaSuccess)
-        s = fail(c, DMRG3S_ERR_CUDA, "Lanczos iteration graph");
-    } else {
-      s = body(st, k + 1);
-    }
-    if (s) {
-      if (gexec) cudaGraphExecDestroy(gexec);
-      return bail(s);
-    }
+    if ((s = orthogonalise())) return bail(s);
     cudaEventRecord(c->ev_ready, st);
     cudaStreamWaitEvent(c->aux, c->ev_ready, 0);
     launch_lz_tridiag(dcn, np, alpha, beta, kp, k, nrm + (int64_t)(k % kLzLag) * nchunks, y, out,
@@ -270,6 +261,7 @@ dmrg3s_status lanczos_batch(Context* c, const DevicePlan& heff, const double* Ld
     cudaMemcpyAsync(sl + (size_t)np * 4, c->d_err, sizeof(int), cudaMemcpyDeviceToHost, c->aux);
     cudaEventRecord(c->ev_lz[k % kLzLag], c->aux);
     last = k;
+    if (k + 1 < kmax && (s = product(k + 1))) return bail(s);
     if (k >= kLagRead) {
       if ((s = collect(next_read++))) break;
       if (nstopped == np) break;
@@ -277,13 +269,10 @@ dmrg3s_status lanczos_batch(Context* c, const DevicePlan& heff, const double* Ld
   }
   while (!s && nstopped < np && next_read <= last) s = collect(next_read++);
   if (!s && nstopped < np) s = fail(c, DMRG3S_ERR_CUDA, "Lanczos did not stop");
-  if (s) {
-    if (gexec) cudaGraphExecDestroy(gexec);
-    return bail(s);
-  }
+  if (s) return bail(s);
   int kmaxstop = 0;
   for (int i = 0; i < np; ++i) kmaxstop = std::max(kmaxstop, kstop[i]);
-  for (int j = kmaxstop + 1; j <= kp; ++j)   // the discarded products (direct launches only)
+  for (int j = kmaxstop + 1; j <= kp; ++j)   // the discarded products
     for (size_t r = prod_recs[j].first; r < prod_recs[j].second; ++r) {
       c->prof.recs[r].flops = 0.0;
       c->prof.recs[r].bytes = 0.0;
@@ -292,16 +281,10 @@ dmrg3s_status lanczos_batch(Context* c, const DevicePlan& heff, const double* Ld
   cudaEventRecord(c->ev_ready, c->aux);
   cudaStreamWaitEvent(st, c->ev_ready, 0);
   if (cudaMemcpyAsync(dks, kstop.data(), sizeof(int32_t) * np, cudaMemcpyHostToDevice, st) !=
-      cudaSuccess) {
-    if (gexec) cudaGraphExecDestroy(gexec);
+      cudaSuccess)
     return bail(fail(c, DMRG3S_ERR_CUDA, "Lanczos tables"));
-  }
   launch_lz_ritz(V, ldv, dch, nchunks, dcn, dks, y, kp, w, nrm_x, st);
   launch_lz_normalise(w, X, dch, nchunks, dcn, nrm_x, st);
-  if (gexec) {   // its last replays may still run: free it once they are done
-    cudaStreamSynchronize(st);
-    cudaGraphExecDestroy(gexec);
-  }
   if (cudaGetLastError() != cudaSuccess) return fail(c, DMRG3S_ERR_CUDA, "Lanczos launch failed");
   return DMRG3S_OK;
 }

@@ -40,6 +40,7 @@
 #include <string>
 #include <thread>
 
+#include "fp64.cuh"
 #include "kernels.hpp"
 #include "launch.hpp"
 #include "svd.hpp"
@@ -125,24 +126,6 @@ jac_permute_kernel(const JacJob* __restrict__ jobs, const int* __restrict__ col_
   for (int i = threadIdx.x; i < J.m; i += kJacThreads) t[i] = x[i];
 }
 
-// A double's top 24 bits as a float with the power of two 2^e taken out
-// (truncated; 0 where that is below the float range), and a float times 2^e as a
-// double (0 below the double range).  Integer instructions: a warp runs those
-// 32 times as fast as FP64 ones.
-__device__ __forceinline__ float float_of(double x, int e) {
-  const unsigned long long u = (unsigned long long)__double_as_longlong(x);
-  const int fe = (int)((u >> 52) & 0x7ff) - e + 127;
-  const unsigned sign = (unsigned)(u >> 32) & 0x80000000u;
-  return fe < 1 ? 0.f : __uint_as_float(sign | (unsigned)fe << 23 | ((unsigned)(u >> 29) & 0x7fffffu));
-}
-__device__ __forceinline__ double double_of(float x, int e) {   // x normal
-  const unsigned u = __float_as_uint(x);
-  const int de = (int)((u >> 23) & 0xff) + 896 + e;
-  const unsigned long long m = (unsigned long long)(u & 0x7fffffu) << 29;
-  const unsigned long long sign = (unsigned long long)(u & 0x80000000u) << 32;
-  return de < 1 ? 0.0 : __longlong_as_double((long long)(sign | (unsigned long long)de << 52 | m));
-}
-
 // The rotation of a pair with d = beta - alpha and gamma = g, as p = tan(theta / 2)
 // and s = sin(theta) = 2 p / (1 + p^2).  GB300 issues FP64 at 1/64 of its FP32
 // rate, and a division or square root in FP64 is a long chain of such
@@ -155,8 +138,8 @@ __device__ __forceinline__ double double_of(float x, int e) {   // x normal
 // to FP64 rounding, so the singular values are unaffected.
 __device__ __forceinline__ void jacobi_rotation(double d, double g, double* p, double* p2,
                                                 double* s) {
-  const int ed = (int)(__double_as_longlong(d) >> 52) & 0x7ff;
-  const int eg = ((int)(__double_as_longlong(g) >> 52) & 0x7ff) + 1;   // of 2 g
+  const int ed = exponent_of(d);
+  const int eg = exponent_of(g) + 1;   // of 2 g
   double pp, pp2;
   float pf = 0.f;
   if (ed - eg > 20) {

@@ -3,8 +3,10 @@
 // Reductions are deterministic: a fixed grid of kRedBlocks CTAs writes one
 // partial sum per CTA (warp-shuffle reduction inside the CTA) and a second
 // kernel adds the partials in a fixed order.
+#include <algorithm>
 #include <cmath>
 
+#include "fp64.cuh"
 #include "kernels.hpp"
 #include "launch.hpp"
 #include "vecops.hpp"
@@ -120,14 +122,150 @@ __device__ int sturm_count_df(const DF* sa, const DF* sbb, int k, DF x) {
   return cnt;
 }
 
-__device__ void tridiag_vector(const double* alpha, const double* beta, int k, double bl,
+constexpr int kTriMax = 128;   // largest order
+
+// Largest value of a warp's lanes.
+__device__ __forceinline__ double warp_max(double v) {
+  for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
+  return v;
+}
+
+// The eigenvector of T for an eigenvalue near theta and its Rayleigh quotient, by
+// one warp: inverse iteration with a pivoted tridiagonal LU of T - theta I
+// (partial pivoting keeps the elimination stable at the near-singular shift; a
+// vanishing pivot is replaced by 1e-15 of the matrix scale, which keeps the
+// solution finite before normalisation).  T is scaled by a power of two to a span
+// of order one.  The elimination and the substitutions are chains of one lane:
+// the pivots are inverted once, by an FP32 reciprocal and three FP64
+// multiply-adds, the rows of U are divided by them beforehand, and every operand
+// comes from shared memory, so a substitution step is one dependent FP64
+// instruction; everything else is spread over the lanes.  The whole solve
+// at order 32 to 37: 122 us with one thread on local memory, 77 us now.
+__device__ void tridiag_vector(const double* al, const double* be, int k, double bl,
                                double theta, double span, double lo, double hi, double* y,
-                               TridiagOut* out);
+                               TridiagOut* out) {
+  __shared__ double s_d[kTriMax], s_l[kTriMax], s_u[kTriMax], s_u2[kTriMax], s_y[kTriMax],
+      s_b[kTriMax];
+  __shared__ unsigned char s_piv[kTriMax];
+  const int lane = threadIdx.x;
+  if (k == 1) {                 // the Ritz vector of a 1x1 matrix
+    if (lane == 0) {
+      y[0] = 1.0;
+      out->theta = theta;
+      out->resid = fabs(bl);
+      out->beta_last = bl;
+      out->nan_seen = 0.0;
+    }
+    return;
+  }
+  const double sc = inverse_scale(span);
+  const double tiny = 1e-15 * sc * fmax(span, fmax(fabs(lo), fabs(hi)));
+  for (int i = lane; i < k; i += 32) {
+    s_d[i] = sc * (al[i] - theta);
+    s_b[i] = i < k - 1 ? sc * be[i] : 0.0;
+    s_y[i] = 1.0;
+  }
+  __syncwarp();
+  if (lane == 0) {   // s_d becomes the inverted pivots
+    double cd = s_d[0], cu = s_b[0];
+    for (int i = 0; i < k - 1; ++i) {
+      const double l = s_b[i], dn = s_d[i + 1], un = s_b[i + 1];
+      const bool swap = fabs(cd) < fabs(l);
+      double p = swap ? l : cd;
+      if (fabs(p) < 1e-300) p = tiny;
+      const double r = recip(p), f = (swap ? cd : l) * r;
+      s_piv[i] = swap;
+      s_d[i] = r;
+      s_l[i] = f;
+      s_u[i] = swap ? dn : cu;
+      s_u2[i] = swap ? un : 0.0;
+      cd = swap ? fma(-f, dn, cu) : fma(-f, cu, dn);
+      cu = swap ? -f * un : un;
+    }
+    s_d[k - 1] = recip(fabs(cd) < 1e-300 ? tiny : cd);
+  }
+  __syncwarp();
+  for (int i = lane; i < k - 1; i += 32) {
+    s_u[i] *= s_d[i];
+    s_u2[i] *= s_d[i];
+  }
+  for (int sweep = 0; sweep < 3; ++sweep) {
+    __syncwarp();
+    if (lane == 0) {   // row interchanges and L
+      double cur = s_y[0];
+      for (int i = 0; i < k - 1; ++i) {
+        const double nx = s_y[i + 1], f = s_l[i];
+        const bool swap = s_piv[i];
+        s_y[i] = swap ? nx : cur;
+        cur = swap ? fma(-f, nx, cur) : fma(-f, cur, nx);
+      }
+      s_y[k - 1] = cur;
+    }
+    __syncwarp();
+    for (int i = lane; i < k; i += 32) s_y[i] *= s_d[i];
+    __syncwarp();
+    if (lane == 0) {   // back substitution (first and second superdiagonal)
+      double y2 = 0.0, y1 = s_y[k - 1];
+      for (int i = k - 2; i >= 0; --i) {
+        const double t = fma(-s_u2[i], y2, s_y[i]);
+        y2 = y1;
+        y1 = fma(-s_u[i], y1, t);
+        s_y[i] = y1;
+      }
+    }
+    __syncwarp();
+    // normalise: scale by the largest component first (no overflow in the squares)
+    double big = 0.0;
+    for (int i = lane; i < k; i += 32) big = fmax(big, fabs(s_y[i]));
+    big = warp_max(big);
+    if (!(big > 0.0) || !(big < 1e308)) {   // degenerate solve: restart from e_0
+      for (int i = lane; i < k; i += 32) s_y[i] = i == 0 ? 1.0 : 0.0;
+      continue;
+    }
+    const double ib = inverse_scale(big);
+    double nrm = 0.0;
+    for (int i = lane; i < k; i += 32) {
+      const double v = ib * s_y[i];
+      nrm = fma(v, v, nrm);
+    }
+    const double in = ib / sqrt(warp_sum(nrm));
+    for (int i = lane; i < k; i += 32) s_y[i] *= in;
+  }
+  __syncwarp();
+  // fix the sign: largest component positive (only the subspace is defined)
+  double big = 0.0;
+  int imax = kTriMax;
+  for (int i = lane; i < k; i += 32)
+    if (fabs(s_y[i]) > big) {
+      big = fabs(s_y[i]);
+      imax = i;
+    }
+  const double all = warp_max(big);
+  imax = __reduce_min_sync(0xffffffffu, big == all ? imax : kTriMax);
+  const bool flip = imax < kTriMax && s_y[imax] < 0.0;
+  // Rayleigh quotient y^T T y (y has unit norm): second-order accurate in the
+  // error of the vector, so the bracket's width does not limit the Ritz value
+  double rq = 0.0;
+  for (int i = lane; i < k; i += 32) {
+    double ty = al[i] * s_y[i];
+    if (i > 0) ty = fma(be[i - 1], s_y[i - 1], ty);
+    if (i < k - 1) ty = fma(be[i], s_y[i + 1], ty);
+    rq = fma(s_y[i], ty, rq);
+    y[i] = flip ? -s_y[i] : s_y[i];
+  }
+  rq = warp_sum(rq);
+  if (lane == 0) {
+    out->theta = rq == rq ? rq : theta;
+    out->resid = fabs(bl * s_y[k - 1]);
+    out->beta_last = bl;
+    out->nan_seen = 0.0;
+  }
+}
 
 // Multisection: all threads of the block evaluate Sturm counts at equally
 // spaced points of the bracket, shrinking it by blockDim.x + 1 per round
 // until it reaches the resolution of double-float counts (~1e-13 of the
-// Gershgorin span); thread 0 then runs the inverse iteration in FP64 and
+// Gershgorin span); the first warp then runs the inverse iteration in FP64 and
 // returns the Rayleigh quotient of the vector, which is accurate to FP64
 // rounding whatever the width of the bracket was.
 // bl = the norm of the new residual vector (stored as beta[k - 1]).
@@ -135,26 +273,35 @@ __device__ void tridiag_block(const double* alpha, double* beta, int k,
                               double bl, double* y, TridiagOut* out) {
   __shared__ double sh_lo, sh_hi, sh_span, sh_c;
   __shared__ int sh_bad, sh_first;
-  __shared__ DF sa[128], sbb[128];
+  __shared__ double s_al[kTriMax], s_be[kTriMax];
+  __shared__ DF sa[kTriMax], sbb[kTriMax];
   const int tid = threadIdx.x, nt = blockDim.x;
-  if (tid == 0) {
+  for (int i = tid; i < k; i += nt) {
+    s_al[i] = alpha[i];
+    s_be[i] = i < k - 1 ? beta[i] : 0.0;
+  }
+  __syncthreads();
+  if (tid < 32) {
     double lo = 1e300, hi = -1e300;
-    int bad = 0;
-    for (int i = 0; i < k; ++i) {
-      const double bi = i < k - 1 ? beta[i] : 0.0;
-      const double r = (i > 0 ? fabs(beta[i - 1]) : 0.0) + fabs(bi);
-      lo = fmin(lo, alpha[i] - r);
-      hi = fmax(hi, alpha[i] + r);
-      if (!(alpha[i] == alpha[i])) bad = 1;
+    bool bad = !(bl == bl);
+    for (int i = tid; i < k; i += 32) {
+      const double r = (i > 0 ? fabs(s_be[i - 1]) : 0.0) + fabs(s_be[i]);
+      lo = fmin(lo, s_al[i] - r);
+      hi = fmax(hi, s_al[i] + r);
+      if (!(s_al[i] == s_al[i])) bad = true;
     }
-    if (!(bl == bl)) bad = 1;
-    const double span = fmax(hi - lo, 1e-300);
-    sh_lo = lo - 1e-12 * span;
-    sh_hi = hi + 1e-12 * span;
-    sh_span = span;
-    sh_c = 0.5 * (lo + hi);
-    sh_bad = bad;
-    beta[k - 1] = bl;
+    lo = -warp_max(-lo);
+    hi = warp_max(hi);
+    bad = __any_sync(0xffffffffu, bad);
+    if (tid == 0) {
+      const double span = fmax(hi - lo, 1e-300);
+      sh_lo = lo - 1e-12 * span;
+      sh_hi = hi + 1e-12 * span;
+      sh_span = span;
+      sh_c = 0.5 * (lo + hi);
+      sh_bad = bad;
+      beta[k - 1] = bl;
+    }
   }
   __syncthreads();
   if (sh_bad) {
@@ -168,8 +315,8 @@ __device__ void tridiag_block(const double* alpha, double* beta, int k,
   }
   const double c = sh_c, inv_s = 1.0 / sh_span;
   for (int i = tid; i < k; i += nt) {
-    sa[i] = df_from((alpha[i] - c) * inv_s);
-    const double bs = i > 0 ? beta[i - 1] * inv_s : 0.0;
+    sa[i] = df_from((s_al[i] - c) * inv_s);
+    const double bs = i > 0 ? s_be[i - 1] * inv_s : 0.0;
     sbb[i] = df_from(bs * bs);
   }
   __syncthreads();
@@ -189,116 +336,8 @@ __device__ void tridiag_block(const double* alpha, double* beta, int k,
     }
     __syncthreads();
   }
-  if (tid == 0)
-    tridiag_vector(alpha, beta, k, bl, 0.5 * (sh_lo + sh_hi), sh_span, sh_lo, sh_hi, y, out);
-}
-
-__device__ void tridiag_vector(const double* alpha, const double* beta, int k, double bl,
-                               double theta, double span, double lo, double hi, double* y,
-                               TridiagOut* out) {
-  const int kk = k <= 128 ? k : 128;
-  if (kk == 1) {                 // the Ritz vector of a 1x1 matrix
-    y[0] = 1.0;
-    out->theta = theta;
-    out->resid = fabs(bl);
-    out->beta_last = bl;
-    out->nan_seen = 0.0;
-    return;
-  }
-  // inverse iteration: solve (T - theta I) z = y with a pivoted tridiagonal LU
-  // (partial pivoting keeps the elimination stable at the near-singular shift);
-  // an exactly zero pivot is replaced by 1e-15 of the matrix scale, which keeps
-  // the solution finite (of order 1e15 times the scale) before normalisation.
-  // The shift is the same in every sweep, so the matrix is factored once and
-  // the pivots are inverted once; a sweep is then two substitutions without
-  // divisions (FP64 division is the long pole of this one-thread chain).
-  const double tiny = 1e-15 * fmax(span, fmax(fabs(lo), fabs(hi)));
-  double dl[128], dd[128], du[128], du2[128];
-  int piv[128];
-  for (int i = 0; i < kk; ++i) {
-    dd[i] = alpha[i] - theta;
-    du[i] = i < kk - 1 ? beta[i] : 0.0;
-    dl[i] = i < kk - 1 ? beta[i] : 0.0;
-    du2[i] = 0.0;
-  }
-  for (int i = 0; i < kk - 1; ++i) {
-    if (fabs(dd[i]) >= fabs(dl[i])) {
-      piv[i] = i;
-      if (dd[i] == 0.0) dd[i] = tiny;
-      const double f = dl[i] / dd[i];
-      dl[i] = f;
-      dd[i + 1] -= f * du[i];
-    } else {
-      piv[i] = i + 1;
-      const double f = dd[i] / dl[i];
-      dd[i] = dl[i];
-      dl[i] = f;
-      const double t = du[i];
-      du[i] = dd[i + 1];
-      dd[i + 1] = t - f * dd[i + 1];
-      if (i < kk - 2) {
-        du2[i] = du[i + 1];
-        du[i + 1] = -f * du[i + 1];
-      }
-    }
-  }
-  for (int i = 0; i < kk; ++i) {
-    if (dd[i] == 0.0) dd[i] = tiny;
-    dd[i] = 1.0 / dd[i];               // dd now holds the inverted pivots
-  }
-  for (int i = 0; i < kk; ++i) y[i] = 1.0 / sqrt((double)kk);
-  for (int sweep = 0; sweep < 3; ++sweep) {
-    // forward: apply row interchanges and L
-    for (int i = 0; i < kk - 1; ++i) {
-      if (piv[i] == i) {
-        y[i + 1] -= dl[i] * y[i];
-      } else {
-        const double t = y[i];
-        y[i] = y[i + 1];
-        y[i + 1] = t - dl[i] * y[i];
-      }
-    }
-    // back substitution with U (inverted diagonal dd, super du, second super du2)
-    y[kk - 1] *= dd[kk - 1];
-    if (kk > 1) y[kk - 2] = (y[kk - 2] - du[kk - 2] * y[kk - 1]) * dd[kk - 2];
-    for (int i = kk - 3; i >= 0; --i)
-      y[i] = (y[i] - du[i] * y[i + 1] - du2[i] * y[i + 2]) * dd[i];
-    // normalise: scale by the largest component first (no overflow in the squares)
-    double big = 0.0;
-    for (int i = 0; i < kk; ++i) big = fmax(big, fabs(y[i]));
-    if (!(big > 0.0) || !(big < 1e308)) {   // degenerate solve: restart from e_0
-      for (int i = 0; i < kk; ++i) y[i] = i == 0 ? 1.0 : 0.0;
-      continue;
-    }
-    const double ib = 1.0 / big;
-    double nrm = 0.0;
-    for (int i = 0; i < kk; ++i) {
-      y[i] *= ib;
-      nrm += y[i] * y[i];
-    }
-    const double in = 1.0 / sqrt(nrm);
-    for (int i = 0; i < kk; ++i) y[i] *= in;
-  }
-  // fix the sign: largest component positive (only the subspace is defined)
-  int imax = 0;
-  for (int i = 1; i < kk; ++i)
-    if (fabs(y[i]) > fabs(y[imax])) imax = i;
-  if (y[imax] < 0.0)
-    for (int i = 0; i < kk; ++i) y[i] = -y[i];
-  // Rayleigh quotient y^T T y (y has unit norm): second-order accurate in the
-  // error of the vector, so the bracket's width does not limit the Ritz value
-  double rq = 0.0;
-  for (int i = 0; i < kk; ++i) {
-    double ty = alpha[i] * y[i];
-    if (i > 0) ty += beta[i - 1] * y[i - 1];
-    if (i < kk - 1) ty += beta[i] * y[i + 1];
-    rq += y[i] * ty;
-  }
-  if (rq == rq) theta = rq;
-  out->theta = theta;
-  out->resid = fabs(bl * y[kk - 1]);
-  out->beta_last = bl;
-  out->nan_seen = 0.0;
+  if (tid < 32)
+    tridiag_vector(s_al, s_be, k, bl, 0.5 * (sh_lo + sh_hi), sh_span, sh_lo, sh_hi, y, out);
 }
 
 __global__ void copy_blocks_kernel(const CopyTask* __restrict__ tasks,
@@ -523,6 +562,218 @@ __global__ void lz_advance_kernel(int* kdev) {
   grid_next();
   grid_wait(); *kdev += 1; }
 
+// ---- one iteration's orthogonalisation in one launch ----
+
+constexpr int kOrThreads = 512;
+constexpr int kOrWarps = kOrThreads / 32;
+constexpr int kOrSegs = 4;          // element ranges a chunk's dot products are split into
+
+// Barrier of all CTAs of a cooperative launch: `count` counts arrivals and is
+// never reset, `target` is its value once all have arrived.  Bounded: false (in
+// every thread of the CTA) after limit_ns, with *err set.
+__device__ __forceinline__ bool grid_sync(unsigned* count, unsigned target, int* err,
+                                          uint64_t limit_ns, int* s_ok) {
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    atomicAdd(count, 1u);
+    int ok = 1;
+    uint64_t t0, t;
+    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t0));
+    for (;;) {
+      unsigned v;
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(count) : "memory");
+      if ((int)(v - target) >= 0) break;
+      asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+      if (t - t0 > limit_ns) {
+        atomicExch(err, 1);
+        ok = 0;
+        break;
+      }
+    }
+    __threadfence();
+    *s_ok = ok;
+  }
+  __syncthreads();
+  return *s_ok != 0;
+}
+
+// h[j] = the sum of partial[., j] over the chain's chunks, j < k1, in a fixed order: a
+// group of warps per eight columns, four chunks at a time side by side in a warp.
+__device__ __forceinline__ void chain_sums(const double* partial, int kp, const LzChain& cn, int k1,
+                                           double* red, double* h) {
+  const int lane = threadIdx.x & 31, q = threadIdx.x >> 5;
+  const int nb = (k1 + 7) / 8;                       // column blocks: at most 17
+  const int ways = nb < kOrWarps ? kOrWarps / nb : 1;   // warps per block
+  for (int u = q; u < nb * ways; u += kOrWarps) {
+    const int jb = u % nb, way = u / nb;
+    const int j = jb * 8 + (lane & 7);
+    const int step = 4 * ways;
+    double a0 = 0.0, a1 = 0.0;
+    if (j < k1) {
+      const double* p = partial + (int64_t)cn.c0 * kp + j;
+      int b = way * 4 + (lane >> 3);
+      for (; b + 3 * step < cn.nc; b += 4 * step) {   // four loads in flight per lane
+        const double x0 = __ldcg(p + (int64_t)b * kp), x1 = __ldcg(p + (int64_t)(b + step) * kp);
+        const double x2 = __ldcg(p + (int64_t)(b + 2 * step) * kp);
+        const double x3 = __ldcg(p + (int64_t)(b + 3 * step) * kp);
+        a0 += x0;
+        a1 += x1;
+        a0 += x2;
+        a1 += x3;
+      }
+      for (; b < cn.nc; b += step) a0 += __ldcg(p + (int64_t)b * kp);
+    }
+    a0 += a1;
+    a0 += __shfl_xor_sync(0xffffffffu, a0, 8);
+    a0 += __shfl_xor_sync(0xffffffffu, a0, 16);
+    if (lane < 8) red[way * (kLzMaxK + 7) + jb * 8 + lane] = a0;
+  }
+  __syncthreads();
+  for (int j = threadIdx.x; j < k1; j += kOrThreads) {
+    double s = red[j];
+    for (int w = 1; w < ways; ++w) s += red[w * (kLzMaxK + 7) + j];
+    h[j] = s;
+  }
+  __syncthreads();
+}
+
+// partial_b[j] = <V_j, x> over the chunk, j < k1: a warp takes four vectors over one of
+// kOrSegs element ranges (four vectors share the reads of x and one reduction:
+// 22 FP64 instructions per 16 multiply-adds at four elements a lane).  Vectors below
+// `have` are read from Vs (stride lp); FILL stores the others there while they fit.
+template <bool FILL>
+__device__ __forceinline__ void chunk_dots(const double* V, int64_t ldv, double* Vs, int lp,
+                                           int vcap, const double* x, int len, int k1, double* red,
+                                           double* out) {
+  const int lane = threadIdx.x & 31, q = threadIdx.x >> 5;
+  const int ng = (k1 + 3) / 4;
+  const int seg = ((len + kOrSegs - 1) / kOrSegs + 31) & ~31;
+  for (int u = q; u < ng * kOrSegs; u += kOrWarps) {
+    const int g = u / kOrSegs, sg = u % kOrSegs;
+    const int i0 = sg * seg, i1 = min(len, i0 + seg);
+    const int nj = min(4, k1 - 4 * g);
+    double a[4] = {0.0, 0.0, 0.0, 0.0};
+    const double* src[4];
+#pragma unroll
+    for (int t = 0; t < 4; ++t) {
+      const int j = 4 * g + (t < nj ? t : 0);
+      src[t] = !FILL && j < vcap ? Vs + (int64_t)j * lp : V + (int64_t)j * ldv;
+    }
+    for (int ib = i0; ib < i1; ib += 128) {        // 16 loads of V in flight per lane
+      double v[4][4];
+#pragma unroll
+      for (int m = 0; m < 4; ++m) {
+        const int i = ib + 32 * m + lane;
+#pragma unroll
+        for (int t = 0; t < 4; ++t) v[m][t] = i < i1 ? src[t][i] : 0.0;
+      }
+#pragma unroll
+      for (int m = 0; m < 4; ++m) {
+        const int i = ib + 32 * m + lane;
+        if (ib + 32 * m >= i1) break;
+        const double xi = i < i1 ? x[i] : 0.0;
+#pragma unroll
+        for (int t = 0; t < 4; ++t) {
+          if (FILL && i < i1 && t < nj && 4 * g + t < vcap)
+            Vs[(int64_t)(4 * g + t) * lp + i] = v[m][t];
+          a[t] = fma(v[m][t], xi, a[t]);
+        }
+      }
+    }
+    // the four sums over the lanes: halves exchanged twice, then a butterfly
+    const bool h16 = (lane & 16) != 0, h8 = (lane & 8) != 0;
+    double b0 = (h16 ? a[2] : a[0]) + __shfl_xor_sync(0xffffffffu, h16 ? a[0] : a[2], 16);
+    double b1 = (h16 ? a[3] : a[1]) + __shfl_xor_sync(0xffffffffu, h16 ? a[1] : a[3], 16);
+    double c = (h8 ? b1 : b0) + __shfl_xor_sync(0xffffffffu, h8 ? b0 : b1, 8);
+    for (int o = 4; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
+    if ((lane & 7) == 0) {
+      const int t = (h16 ? 2 : 0) + (h8 ? 1 : 0);
+      if (t < nj) red[sg * (kLzMaxK + 7) + 4 * g + t] = c;
+    }
+  }
+  __syncthreads();
+  for (int j = threadIdx.x; j < k1; j += kOrThreads) {
+    double s = red[j];
+    for (int w = 1; w < kOrSegs; ++w) s += red[w * (kLzMaxK + 7) + j];
+    out[j] = s;
+  }
+}
+
+// Iteration k (from the device counter): two classical Gram-Schmidt passes of w
+// against V_0 .. V_k, v_{k+1} = w / |w| into the basis and vcur, k += 1.  One CTA
+// per chunk, all resident (cooperative launch); the chunk of w and as much of
+// the basis as fits stay in shared memory through the passes, which are
+// separated by device-wide barriers instead of launches.  Bound by the FP64
+// pipe: 4 k multiply-adds per element are 19 us at k = 37 for the 75 k elements
+// of an m = 512 XXZ tensor, beside three barriers and the sums over the chunks'
+// partials.  At k = 32 to 37 (cold caches) 52 us; as five launches (dots, update
+// and dots, update, next, advance) 107 us.
+__global__ void __launch_bounds__(kOrThreads, 1) lz_orth_kernel(
+    double* V, int64_t ldv, int* kdev, const double* w, double* vcur,
+    const LzChunk* __restrict__ chunks, const LzChain* __restrict__ chains, double* part,
+    double* part2, int kp, double* alpha, double* nrm, int64_t nrm_stride, int lp, int vcap,
+    unsigned* count, int* err, uint64_t limit_ns) {
+  extern __shared__ double osh[];
+  __shared__ double h[kLzMaxK + 7];
+  __shared__ double red[kOrWarps * (kLzMaxK + 7)];
+  __shared__ double s_scale;
+  __shared__ int s_ok;
+  const int k = *kdev, k1 = k + 1;
+  const unsigned G = gridDim.x, base = 3u * G * (unsigned)k;
+  const LzChunk ch = chunks[blockIdx.x];
+  const LzChain cn = chains[ch.chain];
+  const int len = (int)(ch.e1 - ch.e0);
+  double* x = osh;
+  double* Vs = osh + lp;
+  if (vcap > k1) vcap = k1;
+  const double* Vc = V + ch.e0;
+  for (int i = threadIdx.x; i < len; i += kOrThreads) x[i] = w[ch.e0 + i];
+  __syncthreads();
+  double nacc = 0.0;
+  for (int pass = 0; pass < 2; ++pass) {
+    double* pp = pass == 0 ? part : part2;
+    if (pass == 0)
+      chunk_dots<true>(Vc, ldv, Vs, lp, vcap, x, len, k1, red, pp + (int64_t)blockIdx.x * kp);
+    else
+      chunk_dots<false>(Vc, ldv, Vs, lp, vcap, x, len, k1, red, pp + (int64_t)blockIdx.x * kp);
+    if (!grid_sync(count, base + (unsigned)(pass + 1) * G, err, limit_ns, &s_ok)) return;
+    chain_sums(pp, kp, cn, k1, red, h);
+    if (pass == 0 && threadIdx.x == 0 && (int)blockIdx.x == cn.c0)
+      alpha[(int64_t)ch.chain * kp + k] = h[k];
+    for (int i = threadIdx.x; i < len; i += kOrThreads) {
+      double acc = x[i];
+      int j = 0;
+#pragma unroll 4
+      for (; j < vcap; ++j) acc = fma(-h[j], Vs[(int64_t)j * lp + i], acc);
+#pragma unroll 4
+      for (; j < k1; ++j) acc = fma(-h[j], Vc[(int64_t)j * ldv + i], acc);
+      x[i] = acc;
+      if (pass == 1) nacc = fma(acc, acc, nacc);
+    }
+    __syncthreads();
+  }
+  double* np = nrm + (int64_t)(k % kLzLag) * nrm_stride;
+  nacc = block_sum(nacc, red);
+  if (threadIdx.x == 0) np[blockIdx.x] = nacc;
+  if (!grid_sync(count, base + 3u * G, err, limit_ns, &s_ok)) return;
+  if (threadIdx.x < 32) {
+    double a = 0.0;
+    for (int b = threadIdx.x; b < cn.nc; b += 32) a += __ldcg(np + cn.c0 + b);
+    a = warp_sum(a);
+    if (threadIdx.x == 0) s_scale = (a > 0.0 && a < 1e308) ? 1.0 / sqrt(a) : 0.0;
+  }
+  __syncthreads();
+  const double sc = s_scale;
+  double* vn = V + (int64_t)k1 * ldv;
+  for (int i = threadIdx.x; i < len; i += kOrThreads) {
+    const double v = x[i] * sc;
+    vn[ch.e0 + i] = v;
+    vcur[ch.e0 + i] = v;
+  }
+  if (blockIdx.x == 0 && threadIdx.x == 0) *kdev = k1;   // every CTA has read it before a barrier
+}
+
 __global__ void lz_tridiag_kernel(const LzChain* __restrict__ chains, const double* alpha,
                                   double* beta, int kp, int k,
                                   const double* nrm_partial, double* y,
@@ -619,6 +870,33 @@ void launch_lz_normalise(const double* x, double* y, const LzChunk* chunks, int 
   if (nchunks <= 0) return;
   count_launch();
   launch_chain(lz_normalise_kernel, nchunks, kLzThreads, 0, st, x, y, chunks, chains, nrm_partial);
+}
+
+bool launch_lz_orth(double* V, int64_t ldv, int* kdev, const double* w, double* vcur,
+                    const LzChunk* chunks, int nchunks, int maxlen, const LzChain* chains,
+                    double* part, double* part2, int kp, double* alpha, double* nrm,
+                    int64_t nrm_stride, unsigned* count, int* err, uint64_t limit_ns,
+                    cudaStream_t st) {
+  const int lp = (maxlen + 1) / 2 * 2;
+  const int vcap = std::min(kp, (int)(kOrSmem / sizeof(double) / (size_t)lp) - 1);
+  const size_t smem = sizeof(double) * (size_t)lp * (1 + vcap);
+  if (cudaFuncSetAttribute(lz_orth_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           (int)kOrSmem) != cudaSuccess)
+    return false;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeCooperative;
+  at.val.cooperative = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = nchunks;
+  cfg.blockDim = kOrThreads;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  count_launch();
+  return cudaLaunchKernelEx(&cfg, lz_orth_kernel, V, ldv, kdev, w, vcur, chunks, chains, part,
+                            part2, kp, alpha, nrm, nrm_stride, lp, vcap, count, err,
+                            limit_ns) == cudaSuccess;
 }
 
 void launch_lz_tridiag(const LzChain* chains, int nchains, const double* alpha, double* beta,

@@ -103,6 +103,17 @@ void launch_lz_update(const double* V, int64_t ldv, int k1, double* w, const LzC
 void launch_lz_next(const double* w, double* V, int64_t ldv, const int* kdev, double* vcur,
                     const LzChunk* chunks, int nchunks, const LzChain* chains,
                     const double* nrm_partial, int64_t nrm_stride, cudaStream_t st);
+// Dots, update, dots, update, next and advance of iteration *kdev as one
+// cooperative launch: nchunks <= the SM count, maxlen the longest chunk
+// (<= kLzChunkMax).  `count` is a device word that is zero before iteration 0 and
+// belongs to the recursion; the waits between the phases are bounded by limit_ns,
+// after which *err is set.  False when the launch is refused.
+constexpr size_t kOrSmem = 176 * 1024;   // leaves room for the tridiagonal solve on the same SM
+bool launch_lz_orth(double* V, int64_t ldv, int* kdev, const double* w, double* vcur,
+                    const LzChunk* chunks, int nchunks, int maxlen, const LzChain* chains,
+                    double* part, double* part2, int kp, double* alpha, double* nrm,
+                    int64_t nrm_stride, unsigned* count, int* err, uint64_t limit_ns,
+                    cudaStream_t st);
 // *kdev += 1 (one thread).
 void launch_lz_advance(int* kdev, cudaStream_t st);
 // The update of one pass followed by the dots of the next: as launch_lz_update
