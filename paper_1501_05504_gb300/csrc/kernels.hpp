@@ -24,9 +24,9 @@ struct GemmTask {
   int32_t ldc, M, N, seg0, nseg, pad;
 };
 
-// One 64 x 64 output tile of a task.
+// One size x size output tile of a task (64, 32, 16 or 8).
 struct GemmTile {
-  int32_t task, tm, tn, pad;
+  int32_t task, tm, tn, size;
 };
 
 // Linear combination of blocks: out = sum_k coef_k in_k (rows x cols).

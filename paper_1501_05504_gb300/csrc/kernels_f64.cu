@@ -2,7 +2,7 @@
 //
 // The grouped GEMM computes every block product of one contraction step of
 // the order (((L M) W) R) of Sec. V of arXiv:1501.05504 in one launch: one CTA
-// per 64 x 64 output tile, summing all K-segments of its task.  The
+// per output tile, summing all K-segments of its task.  The
 // combination kernel applies the MPO step (T2 = sum W T1), which costs
 // O(m^2 d^2 w^2) and is bound by memory bandwidth.
 #include <atomic>
@@ -14,7 +14,118 @@ namespace dmrg3s {
 
 namespace {
 
-constexpr int BM = 64, BN = 64, BK = 16, NT = 256;
+constexpr int NT = 256;
+constexpr int kGemmSmem = 2 * 16 * 65;   // doubles: the chunks of A and B of a 64 x 64 tile
+
+// One SIZE x SIZE output tile: every thread sums R x R elements over the k of its
+// K-group (SIZE = 8: four groups of 64 threads, their sums added at the end).
+// Bound by the FP64 pipe (a warp's multiply-add takes ~64 cycles of a
+// sub-partition), so the work is what counts: rows and k beyond the block are
+// left out of the loops, and the next chunk's loads are in flight during the
+// current one's products.
+template <int SIZE, Trans TA, Trans TB>
+__device__ __forceinline__ void gemm_tile(const GemmTile& tile, const GemmTask& task,
+                                          const GemmSeg* __restrict__ segs, const double* A,
+                                          const double* B, double* C, double* sh) {
+  constexpr int KS = SIZE == 8 ? 4 : 1;                  // K-groups
+  constexpr int TX = SIZE == 8 ? 8 : 16, R = SIZE / TX;  // threads a side, elements a thread and side
+  constexpr int BK = SIZE == 8 ? 64 : SIZE == 16 ? 32 : 16;
+  constexpr int LD = SIZE + 1, E = SIZE * BK / NT;       // elements of a chunk a thread loads
+  static_assert(2 * BK * LD <= kGemmSmem, "shared memory");
+  double* As = sh;
+  double* Bs = sh + BK * LD;
+  const int tid = threadIdx.x;
+  const int grp = KS == 1 ? 0 : tid / (TX * TX), t = KS == 1 ? tid : tid % (TX * TX);
+  const int tx = t % TX, ty = t / TX;
+  const int m0 = tile.tm * SIZE, n0 = tile.tn * SIZE;
+  double acc[R][R];
+#pragma unroll
+  for (int i = 0; i < R; ++i)
+#pragma unroll
+    for (int j = 0; j < R; ++j) acc[i][j] = 0.0;
+  double ra[E], rb[E];
+  int sgi = 0, k0 = 0;
+  GemmSeg sg{};
+  if (task.nseg > 0) sg = segs[task.seg0];
+  while (sgi < task.nseg && sg.K <= 0)
+    if (++sgi < task.nseg) sg = segs[task.seg0 + sgi];
+  // the loads of chunk k0 of segment sg
+  auto load = [&]() {
+    const double* Ap = A + sg.offA;
+    const double* Bp = B + sg.offB;
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+      const int idx = tid + e * NT;
+      const int m = TA == Trans::N ? idx / BK : idx % SIZE, ka = TA == Trans::N ? idx % BK : idx / SIZE;
+      const int gm = m0 + m, gk = k0 + ka;
+      ra[e] = gm < task.M && gk < sg.K
+                  ? (TA == Trans::N ? Ap[(int64_t)gm * sg.lda + gk] : Ap[(int64_t)gk * sg.lda + gm])
+                  : 0.0;
+      const int n = TB == Trans::N ? idx % SIZE : idx / BK, kb = TB == Trans::N ? idx / SIZE : idx % BK;
+      const int gn = n0 + n, gb = k0 + kb;
+      rb[e] = gn < task.N && gb < sg.K
+                  ? (TB == Trans::N ? Bp[(int64_t)gb * sg.ldb + gn] : Bp[(int64_t)gn * sg.ldb + gb])
+                  : 0.0;
+    }
+  };
+  if (sgi < task.nseg) load();
+  while (sgi < task.nseg) {
+    const int kc = min(BK, sg.K - k0);
+    if (sg.scale != 1.0) {
+#pragma unroll
+      for (int e = 0; e < E; ++e) ra[e] *= sg.scale;
+    }
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+      const int idx = tid + e * NT;
+      As[TA == Trans::N ? (idx % BK) * LD + idx / BK : (idx / SIZE) * LD + idx % SIZE] = ra[e];
+      Bs[TB == Trans::N ? (idx / SIZE) * LD + idx % SIZE : (idx % BK) * LD + idx / BK] = rb[e];
+    }
+    __syncthreads();
+    k0 += BK;
+    while (sgi < task.nseg && k0 >= sg.K) {
+      k0 = 0;
+      if (++sgi < task.nseg) sg = segs[task.seg0 + sgi];
+    }
+    if (sgi < task.nseg) load();
+    const int kq = KS == 1 ? kc : (kc + KS - 1) / KS;
+    const int kend = min(kc, (grp + 1) * kq);
+    if (m0 + ty < task.M) {
+#pragma unroll 4
+      for (int k = grp * kq; k < kend; ++k) {
+        double a[R], b[R];
+#pragma unroll
+        for (int i = 0; i < R; ++i) a[i] = As[k * LD + ty + TX * i];
+#pragma unroll
+        for (int j = 0; j < R; ++j) b[j] = Bs[k * LD + tx + TX * j];
+#pragma unroll
+        for (int i = 0; i < R; ++i)
+#pragma unroll
+          for (int j = 0; j < R; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
+      }
+    }
+    __syncthreads();
+  }
+  if (KS > 1) {
+    sh[tid] = acc[0][0];
+    __syncthreads();
+    if (grp > 0) return;
+    double s = sh[t];
+#pragma unroll
+    for (int g = 1; g < KS; ++g) s += sh[g * TX * TX + t];
+    acc[0][0] = s;
+  }
+#pragma unroll
+  for (int i = 0; i < R; ++i) {
+    const int gm = m0 + ty + TX * i;
+    if (gm >= task.M) continue;
+#pragma unroll
+    for (int j = 0; j < R; ++j) {
+      const int gn = n0 + tx + TX * j;
+      if (gn < task.N) C[task.offC + (int64_t)gm * task.ldc + gn] = acc[i][j];
+    }
+  }
+}
 
 template <Trans TA, Trans TB>
 __global__ void __launch_bounds__(NT) gemm_f64_kernel(const GemmTile* __restrict__ tiles,
@@ -25,82 +136,13 @@ __global__ void __launch_bounds__(NT) gemm_f64_kernel(const GemmTile* __restrict
                                                       double* C) {
   grid_next();
   grid_wait();
-  __shared__ double As[BK][BM + 1];
-  __shared__ double Bs[BK][BN + 1];
+  __shared__ double sh[kGemmSmem];
   const GemmTile tile = tiles[blockIdx.x];
   const GemmTask task = tasks[tile.task];
-  const int tid = threadIdx.x;
-  const int tx = tid % 16, ty = tid / 16;
-  const int m0 = tile.tm * BM, n0 = tile.tn * BN;
-  double acc[4][4];
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = 0.0;
-
-  for (int sgi = 0; sgi < task.nseg; ++sgi) {
-    const GemmSeg sg = segs[task.seg0 + sgi];
-    const double* Ap = A + sg.offA;
-    const double* Bp = B + sg.offB;
-    for (int k0 = 0; k0 < sg.K; k0 += BK) {
-#pragma unroll
-      for (int r = 0; r < 4; ++r) {
-        int m, k;
-        if (TA == Trans::N) {
-          k = tid % 16;
-          m = tid / 16 + 16 * r;
-        } else {
-          m = tid % 64;
-          k = tid / 64 + 4 * r;
-        }
-        const int gm = m0 + m, gk = k0 + k;
-        double v = 0.0;
-        if (gm < task.M && gk < sg.K)
-          v = (TA == Trans::N) ? Ap[(int64_t)gm * sg.lda + gk] : Ap[(int64_t)gk * sg.lda + gm];
-        As[k][m] = v * sg.scale;
-      }
-#pragma unroll
-      for (int r = 0; r < 4; ++r) {
-        int n, k;
-        if (TB == Trans::N) {
-          n = tid % 64;
-          k = tid / 64 + 4 * r;
-        } else {
-          k = tid % 16;
-          n = tid / 16 + 16 * r;
-        }
-        const int gn = n0 + n, gk = k0 + k;
-        double v = 0.0;
-        if (gn < task.N && gk < sg.K)
-          v = (TB == Trans::N) ? Bp[(int64_t)gk * sg.ldb + gn] : Bp[(int64_t)gn * sg.ldb + gk];
-        Bs[k][n] = v;
-      }
-      __syncthreads();
-#pragma unroll
-      for (int k = 0; k < BK; ++k) {
-        double a[4], b[4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) a[i] = As[k][ty + 16 * i];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) b[j] = Bs[k][tx + 16 * j];
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-          for (int j = 0; j < 4; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
-      }
-      __syncthreads();
-    }
-  }
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int gm = m0 + ty + 16 * i;
-    if (gm >= task.M) continue;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int gn = n0 + tx + 16 * j;
-      if (gn < task.N) C[task.offC + (int64_t)gm * task.ldc + gn] = acc[i][j];
-    }
-  }
+  if (tile.size == 8) gemm_tile<8, TA, TB>(tile, task, segs, A, B, C, sh);
+  else if (tile.size == 16) gemm_tile<16, TA, TB>(tile, task, segs, A, B, C, sh);
+  else if (tile.size == 32) gemm_tile<32, TA, TB>(tile, task, segs, A, B, C, sh);
+  else gemm_tile<64, TA, TB>(tile, task, segs, A, B, C, sh);
 }
 
 __global__ void __launch_bounds__(256) combine_f64_kernel(const CombChunk* __restrict__ chunks,

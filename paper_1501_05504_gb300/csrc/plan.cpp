@@ -30,7 +30,51 @@ void GemmStage::add(int64_t offC, int ldc, int M, int N, const std::vector<GemmS
   }
   const int ntm = (M + 63) / 64, ntn = (N + 63) / 64;
   for (int a = 0; a < ntm; ++a)
-    for (int b = 0; b < ntn; ++b) tiles.push_back(GemmTile{id, a, b, 0});
+    for (int b = 0; b < ntn; ++b) tiles.push_back(GemmTile{id, a, b, 64});
+}
+
+// GB300's FP64 pipe (2 multiply-adds a cycle and SM) makes a k-step of a size x
+// size tile cost size^2 / 2 cycles of its SM whatever the operands' traffic, so
+// the largest tile is not the fastest one: a stage takes about its padded work
+// over the SMs plus its longest tile.  In 64 x 64 tiles the small calls ran a few
+// CTAs for a long time, mostly on padding: the prepared operator took 233 us on
+// the XXZ chain at m = 100, 165 on the Hubbard chain at m = 200 and 89 on one
+// 8 x 8 block; 15, 12 and 11 now.  A large stage is as good in any size (m = 512
+// XXZ 220 us, 80 % of the FP64 rate; 883 in 64 x 64 tiles, whose last wave and
+// ragged edges left the chip idle).
+std::vector<GemmTile> choose_tiles(const GemmStage& g) {
+  constexpr int64_t kMost = 32768;                    // tiles of a stage in a smaller size
+  constexpr double kTile = 300.0, kChunk = 600.0;     // cycles: a CTA's start, a chunk's latency
+  int best = 64;
+  double least = 0.0;
+  for (const int size : {64, 32, 16, 8}) {
+    const int bk = size == 8 ? 64 : size == 16 ? 32 : 16;
+    double sum = 0.0, most = 0.0;
+    int64_t n = 0;
+    for (const GemmTask& t : g.tasks) {
+      double cycles = 0.0, chunks = 0.0;
+      for (int k = 0; k < t.nseg; ++k) {
+        const int K = g.segs[t.seg0 + k].K;
+        cycles += 0.5 * size * size * K;
+        chunks += (K + bk - 1) / bk;
+      }
+      const int64_t tiles = (int64_t)((t.M + size - 1) / size) * ((t.N + size - 1) / size);
+      n += tiles;
+      sum += (double)tiles * (cycles + kTile);
+      most = std::max(most, cycles + kChunk * chunks);
+    }
+    const double time = sum / plan_ctas() + most;
+    if (size == 64 || (n <= kMost && time < least)) {
+      best = size;
+      least = time;
+    }
+  }
+  std::vector<GemmTile> tiles;
+  for (size_t id = 0; id < g.tasks.size(); ++id)
+    for (int a = 0; a < (g.tasks[id].M + best - 1) / best; ++a)
+      for (int b = 0; b < (g.tasks[id].N + best - 1) / best; ++b)
+        tiles.push_back(GemmTile{(int32_t)id, a, b, best});
+  return tiles;
 }
 
 void GemmStage::finalize_bytes(Trans, Trans) {
@@ -780,10 +824,15 @@ bool plan_t2(Plan* p, const std::vector<SlGroup>& groups, const std::vector<SlMe
   return true;
 }
 
-// Least algorithmic work of a contraction that takes the sliced form.
-constexpr double kSlicedMinFlops = 2e6;
+// Least algorithmic work of a contraction that takes the sliced form, whose time
+// hardly falls below 35 us.  Prepared operators, plain against sliced: XXZ m = 200
+// (10 Mflop) 31 and 37 us, m = 256 (22) 47 and 44, m = 512 (177) 220 and 67; one
+// block, m = 64 (9.5) 25 and 34, m = 96 (32) 53 and 46; Hubbard m = 400 (7) 23 and
+// 42, m = 700 (38) 65 and 53.  Gradients: 11 Mflop 38 and 36, 25 Mflop 59 and 44.
+constexpr double kSlicedMinFlops = 16e6;
 // Largest ratio of the fused stage's work to stage 1's: the sliced products
-// run ~15 times as fast as the plain ones; a model MPO has a ratio near 1.2.
+// run 3 (0.2 Gflop) to 16 (13 Gflop) times as fast as the plain ones; a model
+// MPO has a ratio near 1.2.  Below it, the least work grows with the ratio.
 constexpr double kSlicedMaxTerms = 6.0;
 
 // The sliced FP64 form, where there is enough work for it.
@@ -795,7 +844,8 @@ dmrg3s_status finish_sliced(Plan* p, int64_t nA1, int64_t nB1, int64_t nOut2, in
   double terms = 0.0, blocks = 0.0;
   for (const CombTask& t : p->c2.tasks) terms += (double)t.nt * t.rows * t.cols;
   for (const GemmTask& t : p->g1.tasks) blocks += (double)t.M * t.N;
-  if (terms > kSlicedMaxTerms * blocks) return DMRG3S_OK;
+  if (terms > kSlicedMaxTerms * blocks || p->flops() * blocks < kSlicedMinFlops * terms)
+    return DMRG3S_OK;
   const bool left = p->kind == Kind::Heff || p->kind == Kind::ExpandLR || p->kind == Kind::EnvLR;
   bool ok = fuse_f64(*p, &p->f12, err) && build_sliced(p->f12, left, &p->s12, err) &&
             sliced_ok(p->f12, p->s12, nA1, nB1, nOut2, err);
@@ -899,6 +949,8 @@ dmrg3s_status finish(Plan* p, int64_t nA1, int64_t nB1, int64_t nOut2, int64_t n
     *err = "internal planning error: " + *err;
     return DMRG3S_ERR_SHAPE;
   }
+  p->g1.tiles = choose_tiles(p->g1);
+  p->g3.tiles = choose_tiles(p->g3);
   rechunk(p->c2);
   rechunk(p->c3r);
   return finish_sliced(p, nA1, nB1, nOut2, nA3, nB3, nC3, err);
@@ -1223,6 +1275,8 @@ dmrg3s_status plan_mpo_grad(const EnvLayout& le, const MpoLayout& W, const EnvLa
         }
   p->g1.finalize_bytes(p->g1.ta, p->g1.tb);
   p->gy.finalize_bytes(p->gy.ta, p->gy.tb);
+  p->g1.tiles = choose_tiles(p->g1);
+  p->gy.tiles = choose_tiles(p->gy);
   const int64_t w1 = p->ws1 > 0 ? p->ws1 : 1, wy = p->wsy > 0 ? p->wsy : 1;
   if (!gemm_ok(p->g1.ta, p->g1.tb, p->g1.tasks, p->g1.segs, le.size, M.size, w1, err) ||
       !gemm_ok(p->gy.ta, p->gy.tb, p->gy.tasks, p->gy.segs, M.size, re.size, wy, err)) {

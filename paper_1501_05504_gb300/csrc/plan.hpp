@@ -71,13 +71,15 @@ struct GemmStage {
   Trans ta = Trans::N, tb = Trans::N;
   std::vector<GemmTask> tasks;
   std::vector<GemmSeg> segs;
-  std::vector<GemmTile> tiles;      // 64 x 64 tiles (FP64 kernel)
+  std::vector<GemmTile> tiles;      // of the FP64 kernel: 64 x 64 until choose_tiles
   TcStage tc;
   double flops = 0.0;
   double bytes = 0.0;     // algorithmic: distinct operand blocks read once + output written once
   void add(int64_t offC, int ldc, int M, int N, const std::vector<GemmSeg>& s);
   void finalize_bytes(Trans ta, Trans tb);
 };
+// The stage's output tiles in the size that should take the least time.
+std::vector<GemmTile> choose_tiles(const GemmStage& g);
 
 struct CombStage {
   std::vector<CombTask> tasks;

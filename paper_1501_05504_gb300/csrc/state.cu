@@ -149,11 +149,12 @@ dmrg3s_status run_gemm(Context* c, const GemmStage& g, const double* A, int64_t 
   GemmTask* dk;
   GemmSeg* ds;
   dmrg3s_status s;
-  if ((s = upload(c, g.tiles, &dt, st)) || (s = upload(c, g.tasks, &dk, st)) ||
+  const std::vector<GemmTile> tiles = choose_tiles(g);
+  if ((s = upload(c, tiles, &dt, st)) || (s = upload(c, g.tasks, &dk, st)) ||
       (s = upload(c, g.segs, &ds, st)))
     return s;
   const int id = c->prof.on ? c->prof.begin(kProfAuxGemm, g.flops, g.bytes, st) : -1;
-  launch_gemm_f64(g.ta, g.tb, dt, (int)g.tiles.size(), dk, ds, A, B, C, st);
+  launch_gemm_f64(g.ta, g.tb, dt, (int)tiles.size(), dk, ds, A, B, C, st);
   if (id >= 0) c->prof.end(id, st);
   cudaFreeAsync(dt, st);
   cudaFreeAsync(dk, st);
