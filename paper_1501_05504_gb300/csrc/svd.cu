@@ -64,7 +64,7 @@ struct JacPair {
   int64_t offY, offV;
   int32_t n, col0, k, N;
   int32_t job, staged;                // staged: the columns are held in shared memory
-  double tol2;                        // the square of the pair tolerance
+  float tol2;                         // the square of the pair tolerance
 };
 
 // Sum of v over the CTA (kJacThreads threads), returned to every thread.
@@ -144,19 +144,21 @@ __device__ __forceinline__ void jacobi_rotation(double d, double g, double* p, d
   float pf = 0.f;
   if (ed - eg > 20) {
     // |zeta| > 2^19: theta = gamma / (beta - alpha) to FP32 rounding
-    const float t = __fdiv_rn(float_of(g, eg - 1), float_of(d, ed));
+    const float t = __fdividef(float_of(g, eg - 1), float_of(d, ed));
     pp = double_of(t, eg - ed - 2);
     pp2 = double_of(t, eg - ed - 1);
   } else {
+    // tan(theta) = 2 g / (d +- sqrt(d^2 + 4 g^2)), tan(theta / 2) = t / (1 + sqrt(1 + t^2))
     const int e = max(ed, eg);
-    const float z = __fdiv_rn(float_of(d, e), float_of(g, e - 1));
-    const float t = copysignf(1.0f, z) / (fabsf(z) + sqrtf(fmaf(z, z, 1.0f)));
-    const float c = rsqrtf(fmaf(t, t, 1.0f));
-    pf = t * c / (1.0f + c);
+    const float df = float_of(d, e), gf = float_of(g, e - 1);
+    const float h2 = fmaf(df, df, gf * gf);
+    const float t = __fdividef(copysignf(1.0f, df) * gf, fabsf(df) + h2 * rsqrtf(h2));
+    const float u2 = fmaf(t, t, 1.0f);
+    pf = __fdividef(t, 1.0f + u2 * rsqrtf(u2));
     pp = double_of(pf, 0);
     pp2 = double_of(pf, 1);
   }
-  const double r0 = double_of(1.0f / fmaf(pf, pf, 1.0f), 0);
+  const double r0 = double_of(__fdividef(1.0f, fmaf(pf, pf, 1.0f)), 0);
   const double q = fma(pp, pp, 1.0);
   const double e1 = fma(-q, r0, 1.0);
   const double s0 = pp2 * r0;
@@ -173,6 +175,41 @@ __device__ __forceinline__ void shears(double p, double s, double& a, double& b)
   a = fma(-p, b, a);
   b = fma(s, a, b);
   a = fma(-p, b, a);
+}
+
+// gamma^2 > tol2 alpha beta, for positive alpha and beta, in FP32 on the mantissas
+// (the threshold moves by 1e-6 of itself at most).
+__device__ __forceinline__ bool needs_rotation(double alpha, double beta, double g, float tol2) {
+  const int ea = exponent_of(alpha), eb = exponent_of(beta), eg = exponent_of(g);
+  const float fg = float_of(g, eg), f = __fdividef(fg * fg, float_of(alpha, ea) * float_of(beta, eb));
+  const int e = 2 * eg - ea - eb;                    // gamma^2 / (alpha beta) = f 2^e, f in (1/4, 4)
+  if (eg == 0 || e < -120) return false;
+  return e > 100 || f * __uint_as_float((unsigned)(e + 127) << 23) > tol2;
+}
+
+// Sum of the lanes' x to FP64 rounding, in every lane, without FP64 additions: the
+// significands are shifted to a common exponent (63 bits with the carries of 32
+// lanes) and added as integers.  *finite is false when a lane holds Inf or NaN.
+__device__ __forceinline__ double warp_sum_fixed(double x, bool* finite) {
+  const unsigned long long u = (unsigned long long)__double_as_longlong(x);
+  const int e = exponent_of(x);
+  const int top = (int)__reduce_max_sync(0xffffffffu, (unsigned)e);
+  *finite = top < 0x7ff;
+  const int sh = top - e;
+  unsigned long long m = ((u & 0xfffffffffffffull) | (e > 0 ? 1ull << 52 : 0ull)) << 5;
+  m = sh < 64 ? m >> sh : 0ull;
+  const long long v = (long long)u < 0 ? -(long long)m : (long long)m;   // x 2^(1080 - top)
+  // limbs of 26 bits (the last signed)
+  const unsigned s0 = __reduce_add_sync(0xffffffffu, (unsigned)v & 0x3ffffffu);
+  const unsigned s1 = __reduce_add_sync(0xffffffffu, (unsigned)(v >> 26) & 0x3ffffffu);
+  const int s2 = __reduce_add_sync(0xffffffffu, (int)(v >> 52));
+  const long long s = (long long)s0 + ((long long)s1 << 26) + ((long long)s2 << 52);
+  const double r = (double)s;
+  // times 2^(top - 1080) on the exponent (0 below the normal range)
+  const int er = exponent_of(r) + top - 1080;
+  return s == 0 || er < 1 ? 0.0
+                          : __longlong_as_double((__double_as_longlong(r) & ~(0x7ffll << 52)) |
+                                                 (long long)er << 52);
 }
 
 // Starts a sweep: the squared norm of every column of every Y (one CTA per
@@ -202,14 +239,17 @@ jac_sweep_kernel(const JacJob* __restrict__ jobs, const int* __restrict__ col_jo
 // one dot product (the squared norms are kept through the sweep by the rotation's
 // own recurrence, |y_a'|^2 = alpha + s (s (beta - alpha) - 2 c gamma), and formed
 // anew at the next sweep's start, so the last sweep, which rotates nothing, tests
-// every pair with fresh norms), one reduction, ~15 for the rotation (every lane
-// computes the identical one: no exchange), and three shears per element: ~55 at
-// n = 245 where three dot products and the product form took ~80.  The columns
-// of a CTA stay in shared memory between the inner rounds where they fit, so
-// that only every kJacB-th round pays for a launch and for its loads.  Whole
-// factorisations, a launch per round of column pairs before: 762 x 245 18.1 ->
-// 13.3 ms, 900 x 600 74 -> 44, 1300 x 1100 (columns in global memory) 213 -> 124;
-// the local update of an m = 512 XXZ window 30.6 -> 24.9.
+// every pair with fresh norms), a reduction in integers, ~11 for the rotation (every
+// lane computes the identical one: no exchange) and the norms, and three shears per
+// element, four elements' chains interleaved: ~43 at n = 245, where three dot
+// products and the product form took ~80.  The columns of a CTA stay in shared
+// memory between the inner rounds where they fit, so that only every kJacB-th
+// round pays for a launch and for its loads.  ncu: the FP64 pipe 46 % busy on the
+// fullest SM, the rest is the chain of shared-memory loads, reduction and rotation.
+// Whole factorisations (a launch per round of column pairs / this / this with
+// the reduction, test and angle in FP64 and IEEE FP32): 762 x 245 18.1 / 11.9 / 13.2 ms,
+// 900 x 600 74 / 41 / 45, 1300 x 1100 (columns in global memory) 213 / 122 / 126;
+// the local update of an m = 512 XXZ window 30.6 / 22.7 / 24.3.
 constexpr int kJacB = 4;
 constexpr int kJacCache = 8;              // elements of a column that a lane keeps in registers
 constexpr size_t kJacStage = 64 * 1024;   // shared memory of a CTA: three fit an SM
@@ -253,6 +293,7 @@ jac_round_kernel(const JacPair* __restrict__ pairs, int njobs, int r, const int*
   if (before == 0) return;   // converged in the previous sweep (the same for the whole CTA)
   __syncthreads();
   const int M = 2 * kJacB - 1;
+  const int ne = (n + 31) / 32;
   const int inner = r == 0 ? M : kJacB;
   int nrot = 0;
   for (int q = 0; q < inner; ++q) {
@@ -270,40 +311,60 @@ jac_round_kernel(const JacPair* __restrict__ pairs, int njobs, int r, const int*
       double* yb = P.staged ? ys + b * n : yg + (int64_t)gb * n;
       const double alpha = s_nrm[a], beta = s_nrm[b];
       double ua[kJacCache], ub[kJacCache];
-      double g0 = 0.0, g1 = 0.0;
+      double gs[2] = {0.0, 0.0};
 #pragma unroll
       for (int e = 0; e < kJacCache; ++e) {
         const int i = lane + e * 32;
         ua[e] = i < n ? ya[i] : 0.0;
         ub[e] = i < n ? yb[i] : 0.0;
       }
+      // elements in fours (interleaved chains) while whole fours remain, then one
+      // by one
 #pragma unroll
-      for (int e = 0; e < kJacCache; ++e)
-        if (e * 32 < n) {
-          if (e & 1) g1 = fma(ua[e], ub[e], g1);
-          else g0 = fma(ua[e], ub[e], g0);
+      for (int e0 = 0; e0 < kJacCache; e0 += 4) {
+        if (ne >= e0 + 4) {
+#pragma unroll
+          for (int e = e0; e < e0 + 4; ++e) gs[e & 1] = fma(ua[e], ub[e], gs[e & 1]);
+        } else {
+#pragma unroll
+          for (int e = e0; e < e0 + 3; ++e)
+            if (e < ne) gs[e & 1] = fma(ua[e], ub[e], gs[e & 1]);
         }
-      for (int i = lane + kJacCache * 32; i < n; i += 32) g0 = fma(ya[i], yb[i], g0);
-      double g = g0 + g1;
-      for (int o = 16; o > 0; o >>= 1) g += __shfl_xor_sync(0xffffffffu, g, o);
-      // zero columns and NaN leave the pair unrotated (NaN reaches the singular
-      // values); a norm cancelled to nothing waits for the next sweep's
-      if (__double_as_longlong(alpha) > 0 && __double_as_longlong(beta) > 0 &&
-          g * g > P.tol2 * alpha * beta) {
+      }
+      for (int i = lane + kJacCache * 32; i < n; i += 32) gs[0] = fma(ya[i], yb[i], gs[0]);
+      bool finite;
+      const double g = warp_sum_fixed(gs[0] + gs[1], &finite);
+      // zero columns, Inf and NaN leave the pair unrotated (NaN reaches the
+      // singular values); a norm cancelled to nothing waits for the next sweep's
+      if (finite && __double_as_longlong(alpha) > 0 && __double_as_longlong(beta) > 0 &&
+          needs_rotation(alpha, beta, g, P.tol2)) {
         const double d = beta - alpha;
         double p, p2, s;
         jacobi_rotation(d, g, &p, &p2, &s);
         ++nrot;
 #pragma unroll
-        for (int e = 0; e < kJacCache; ++e)
-          if (e * 32 < n) {
-            shears(p, s, ua[e], ub[e]);
-            const int i = lane + e * 32;
-            if (i < n) {
-              ya[i] = ua[e];
-              yb[i] = ub[e];
-            }
+        for (int e0 = 0; e0 < kJacCache; e0 += 4) {
+          if (ne >= e0 + 4) {
+#pragma unroll
+            for (int e = e0; e < e0 + 4; ++e) ua[e] = fma(-p, ub[e], ua[e]);
+#pragma unroll
+            for (int e = e0; e < e0 + 4; ++e) ub[e] = fma(s, ua[e], ub[e]);
+#pragma unroll
+            for (int e = e0; e < e0 + 4; ++e) ua[e] = fma(-p, ub[e], ua[e]);
+          } else {
+#pragma unroll
+            for (int e = e0; e < e0 + 3; ++e)
+              if (e < ne) shears(p, s, ua[e], ub[e]);
           }
+        }
+#pragma unroll
+        for (int e = 0; e < kJacCache; ++e) {
+          const int i = lane + e * 32;
+          if (i < n) {
+            ya[i] = ua[e];
+            yb[i] = ub[e];
+          }
+        }
         for (int i = lane + kJacCache * 32; i < n; i += 32) {
           double u = ya[i], v = yb[i];
           shears(p, s, u, v);
@@ -478,7 +539,7 @@ dmrg3s_status svd_jacobi(Context* c, std::vector<SvdLane>& lanes, int nlanes,
     if (staged) smem = std::max(smem, bytes);
     maxr = std::max(maxr, nbpad - 1);
     for (int q = 0; q < nbpad / 2; ++q)
-      pairs.push_back(JacPair{t.offY, t.offV, t.n, t.col0, q, nbpad - 1, k, staged, tol * tol});
+      pairs.push_back(JacPair{t.offY, t.offV, t.n, t.col0, q, nbpad - 1, k, staged, (float)(tol * tol)});
   }
   const int ncta = (int)pairs.size(), ncol = (int)col_job.size();
   int64_t na = 0;   // extent of the A buffer used by the jobs
