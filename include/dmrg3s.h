@@ -71,7 +71,10 @@ typedef enum dmrg3s_status {
  * (FP32 pair) results, which the MPO combination (stage 2) and the split-K
  * sum combine in double-float arithmetic (~48 bits). */
 typedef enum dmrg3s_precision {
-  DMRG3S_FP64 = 0,    /* double precision on the CUDA cores                          */
+  DMRG3S_FP64 = 0,    /* double precision: contractions of 16 Mflop and more whose
+                         intermediates fit the workspace as exact FP16 slices on
+                         tcgen05 tensor cores (62-bit fixed-point rows, sums exact to
+                         the last digit kept, rounded once), others on the CUDA cores */
   DMRG3S_TF32X3 = 1,  /* 3xTF32 split products on tcgen05 tensor cores, FP32 accum.  */
   DMRG3S_TF32 = 2     /* single-pass TF32 on tcgen05 tensor cores, FP32 accumulate   */
 } dmrg3s_precision;
@@ -127,16 +130,17 @@ const char* dmrg3s_last_error(dmrg3s_ctx ctx);
 
 /* Synchronises `stream` and returns the device-side error latched by the
  * context's kernels since the last call: DMRG3S_ERR_TIMEOUT when a
- * tensor-core kernel gave up a bounded wait (its output is then invalid).
+ * kernel gave up a bounded wait (its output is then invalid; in any precision).
  * The latch is cleared.  Errors: ARG, CUDA, TIMEOUT. */
 dmrg3s_status dmrg3s_sync(dmrg3s_ctx ctx, dmrg3s_stream stream);
 
 /* Limit of every bounded wait inside this library's kernels (the tensor-core
- * kernel's waits for bulk copies, products and drains), in seconds of
+ * kernels' waits for bulk copies, products and drains, the device-wide barriers
+ * of the eigensolver and the waits between the CTAs of the QR), in seconds of
  * elapsed device time (%globaltimer); default 1.0.  A wait that runs out makes
  * its CTA stop (after the copies and products already in flight have
- * finished), latches DMRG3S_ERR_TIMEOUT for dmrg3s_sync and the eigensolver,
- * and leaves the context usable; the results of that launch are invalid.
+ * finished), latches DMRG3S_ERR_TIMEOUT for dmrg3s_sync and the eigensolver
+ * (the SVD returns it), and leaves the context usable; the results of that launch are invalid.
  * seconds = 0 makes every wait that does not succeed at once run out (for
  * testing the error path).  Errors: ARG (negative or not finite). */
 dmrg3s_status dmrg3s_set_wait_limit(dmrg3s_ctx ctx, double seconds);
@@ -206,17 +210,17 @@ dmrg3s_status dmrg3s_expanded_bond(int32_t nsym, const dmrg3s_bond* bond, int32_
  * Matrix k is A_k (m[k] x n[k], 1 <= n[k] <= m[k], n[k] <= 32768),
  * column-major with leading dimension m[k], stored back to back in `A`
  * (device; not modified).  With its columns in descending norm order (A P),
- * each is factorised A P = Q R (cuSOLVER Householder QR, on a copy) and R^T
- * is orthogonalised by one-sided Jacobi rotations (the parallel
- * round-robin order over column pairs, one warp per pair, every matrix in each
- * launch) until no pair has |<y_a, y_b>| > max(sqrt(n), 32) 2^-52 |y_a| |y_b|.
+ * each is factorised A P = Q R (Householder QR on a copy; by cuSOLVER where the
+ * columns do not fit the shared memory of the GPU) and R^T is orthogonalised
+ * by one-sided Jacobi rotations (the parallel round-robin order over blocks of
+ * four columns, one warp per pair, every matrix in each launch) until no pair has |<y_a, y_b>| > max(sqrt(n), 32) 2^-52 |y_a| |y_b|.
  * Outputs, back to back per matrix (device): S (n[k] singular values,
  * descending), VT (n[k] x n[k], ld n[k]; row c = right singular vector c,
  * zero for a zero singular value) and, when U is not NULL, U (m[k] x n[k],
- * ld m[k]; column c = left singular vector c).  Runs on `stream` and on a
- * cuSOLVER handle and stream created for the call (the local update reuses
- * its state's); synchronous (one host read per sweep).
- * Errors: ARG (shapes), CUDA, NOT_CONVERGED (a matrix still rotating after
+ * ld m[k]; column c = left singular vector c).  Runs on `stream` and, for left
+ * vectors, on a cuSOLVER handle and stream created for the call (the local
+ * update reuses its state's); synchronous (one host read per sweep).
+ * Errors: ARG (shapes), CUDA, TIMEOUT, NOT_CONVERGED (a matrix still rotating after
  * 40 sweeps, or after the number 1..40 in the environment variable
  * DMRG3S_JACOBI_SWEEPS; outputs then invalid). */
 dmrg3s_status dmrg3s_svd(dmrg3s_ctx ctx, int32_t nmat, const int64_t* m, const int64_t* n,
@@ -250,11 +254,11 @@ dmrg3s_status dmrg3s_apply_heff(dmrg3s_ctx ctx, const dmrg3s_env* L, const dmrg3
  * as in the Lanczos iteration of Sec. V step 1 (H_eff = L_{i-1} W_i . R_{i+1}
  * of Eq. es-iter, contracted as dmrg3s_apply_heff does).  dmrg3s_heff_create
  * plans the contraction for the structures of L, W, R and A (A->data is not
- * read) and, in the tensor-core modes, packs L and R once into device memory
- * owned by the handle (on `stream`); dmrg3s_heff_apply then computes
+ * read) and, in the tensor-core modes and in the sliced form of DMRG3S_FP64, packs
+ * L and R once into device memory owned by the handle (on `stream`); dmrg3s_heff_apply then computes
  * HA = H_eff A for a vector A (device, canonical layout of A's structure, and
  * HA likewise; both caller-owned) on `stream`, using the context's workspace.
- * In DMRG3S_FP64 the handle reads L->data and R->data at every application:
+ * In DMRG3S_FP64 the handle may read L->data and R->data at every application:
  * they must stay allocated and unchanged while the handle is used.  The
  * handle must not outlive its context; one host thread at a time.
  * Errors: as dmrg3s_apply_heff. */
@@ -335,7 +339,7 @@ dmrg3s_status dmrg3s_update_env(dmrg3s_ctx ctx, int32_t dir, const dmrg3s_env* e
  * [s'][s][bl][br]); overwritten, zero where the charge rule forbids an entry.
  * With L, R the environments of the current MPS and M its orthogonality
  * centre, sum_{entries} G * dW/dtheta / <M|M> is the Hellmann-Feynman
- * derivative of the energy.  FP64 on the CUDA cores; intermediates in the
+ * derivative of the energy.  FP64 (see DMRG3S_FP64); intermediates in the
  * context workspace.  Errors as dmrg3s_apply_heff. */
 dmrg3s_status dmrg3s_mpo_grad_site(dmrg3s_ctx ctx, const dmrg3s_env* L, const dmrg3s_mpo_site* W,
                                    const dmrg3s_env* R, const dmrg3s_site* M, double* G,
@@ -402,7 +406,7 @@ typedef struct dmrg3s_state_s* dmrg3s_state;
  * DMRG3S_SVD_AUTO is the Python binding's default. */
 typedef enum dmrg3s_svd_method {
   DMRG3S_SVD_GESVD = 0,   /* cuSOLVER gesvd per sector on concurrent streams      */
-  DMRG3S_SVD_JACOBI = 1,  /* cuSOLVER QR, then one-sided Jacobi on R^T in this
+  DMRG3S_SVD_JACOBI = 1,  /* QR, then one-sided Jacobi on R^T in this
                              library's kernels, every sector in each launch
                              (dmrg3s_svd); an update whose Jacobi sweeps do not
                              converge redoes its SVD with gesvd

@@ -43,5 +43,20 @@ __device__ __forceinline__ double recip(double x) {
   return fma(r0, fma(d, d, d), r0);
 }
 
+// sqrt(x) to about one unit in the last place (0 < x < 2^1000, normal): with x = m
+// 2^(2k), m in [1, 4), the FP32 rsqrt of m and Newton's coupled iteration for
+// sqrt(m) and 1 / (2 sqrt(m)).  Six dependent FP64 instructions.
+__device__ __forceinline__ double sqrt_of(double x) {
+  const int e = exponent_of(x), k = (e - 1023) >> 1;
+  const double m = __longlong_as_double(__double_as_longlong(x) - ((long long)(2 * k) << 52));
+  const double y = double_of(rsqrtf((float)m), 0);
+  double g = m * y, h = 0.5 * y;
+  const double r = fma(-g, h, 0.5);
+  g = fma(g, r, g);
+  h = fma(h, r, h);
+  g = fma(fma(-g, g, m), h, g);
+  return __longlong_as_double(__double_as_longlong(g) + ((long long)k << 52));
+}
+
 }  // namespace
 }  // namespace dmrg3s

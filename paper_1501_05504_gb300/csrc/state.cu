@@ -327,6 +327,12 @@ dmrg3s_status svd_sectors(State& S, const std::vector<Sector>& secs, double* X, 
                           double* Sv, int* info, cudaStream_t st) {
   Context* c = S.c;
   if (secs.empty()) return DMRG3S_OK;
+  const int lanes = (int)S.svd.size();
+  int nw = (int)secs.size() / 4;
+  if (nw < 4) nw = 4;
+  if (nw > lanes) nw = lanes;
+  for (int w = 0; w < nw; ++w)
+    if (dmrg3s_status s = lane_ready(c, &S.svd[w])) return s;
   size_t dmax = 1, hmax = 1;
   for (const Sector& sc : secs) {
     size_t wd = 0, wh = 0;
@@ -338,7 +344,8 @@ dmrg3s_status svd_sectors(State& S, const std::vector<Sector>& secs, double* X, 
     dmax = std::max(dmax, wd);
     hmax = std::max(hmax, wh);
   }
-  for (SvdWorker& w : S.svd) {
+  for (int k = 0; k < nw; ++k) {
+    SvdWorker& w = S.svd[k];
     if (w.dbytes < dmax) {
       if (w.dwork) cudaFree(w.dwork);
       w.dwork = nullptr;
@@ -355,10 +362,6 @@ dmrg3s_status svd_sectors(State& S, const std::vector<Sector>& secs, double* X, 
   std::sort(order.begin(), order.end(), [&](int a, int b) {
     return (double)secs[a].m * secs[a].n * secs[a].n > (double)secs[b].m * secs[b].n * secs[b].n;
   });
-  const int lanes = (int)S.svd.size();
-  int nw = (int)secs.size() / 4;
-  if (nw < 4) nw = 4;
-  if (nw > lanes) nw = lanes;
   std::vector<std::vector<int>> jobs(nw);
   std::vector<double> load(nw, 0.0);
   for (int k : order) {
@@ -1506,8 +1509,6 @@ dmrg3s_status dmrg3s_state_create(dmrg3s_ctx ctx, int32_t nsites, const dmrg3s_m
                     cudaMemcpyDeviceToDevice, st);
   }
   S->svd.resize(svd_lanes());
-  for (SvdWorker& w : S->svd)
-    if ((s = lane_create(c, &w))) return s;
   if (cudaEventCreateWithFlags(&S->svd_in, cudaEventDisableTiming) != cudaSuccess)
     return fail(c, DMRG3S_ERR_CUDA, "SVD event");
   if ((s = boundary_env(*S, left_env, true, st)) || (s = boundary_env(*S, right_env, false, st)))

@@ -1,5 +1,6 @@
-// FP64 SVD of the truncation step (Sec. IV A, Sec. V step 4): cuSOLVER QR,
-// then the one-sided Jacobi method on R^T in this library's kernels.
+// FP64 SVD of the truncation step (Sec. IV A, Sec. V step 4): Householder QR, then
+// the one-sided Jacobi method on R^T, in this library's kernels (cuSOLVER factorises
+// the matrices too large for the shared memory of the GPU's SMs).
 //
 // One-sided Jacobi (Hestenes): plane rotations of column pairs (a, b) of a
 // matrix Y, each chosen so that the rotated pair is orthogonal; repeated over
@@ -124,6 +125,303 @@ jac_permute_kernel(const JacJob* __restrict__ jobs, const int* __restrict__ col_
   const double* x = A + J.offA + (int64_t)perm[blockIdx.x] * J.m;
   double* t = T + J.offA + (int64_t)j * J.m;
   for (int i = threadIdx.x; i < J.m; i += kJacThreads) t[i] = x[i];
+}
+
+// ---- Householder QR of every matrix of the batch ----
+
+// A matrix's columns are dealt round-robin to G CTAs, which hold them in shared
+// memory.  Step j: the owner of column j forms its reflector (LAPACK's
+// convention: v below the diagonal with v_j = 1 implied, beta on it, H = I - tau v
+// v^T) and publishes it in place; every CTA applies it to its later columns,
+// the owner of column j + 1 to that one first, so that the next reflector is on
+// its way while the others still update (a step waits for one flag, not for a
+// barrier).  CTAs of one matrix wait for each other: cooperative launch, a CTA takes
+// its share of one divided matrix first and then whole small matrices.
+// Bound by the FP64 pipe of the matrix's SMs (two multiply-adds per element of
+// the trailing columns and step) and, per step, by ~2 us of the chain norm, square
+// root, publication.  Whole SVDs with cuSOLVER's QR before: the 14 sectors (up to 762 x
+// 245) of an m = 512 XXZ truncation 22.1 -> 10.9 ms, 60 matrices of 60 x 40 31.0 ->
+// 3.5, 762 x 245 alone 11.9 -> 10.1, 1300 x 1100 121 -> 110, 16 x 8 1.09 -> 0.55.
+struct QrItem {
+  int64_t offA, offTau;
+  int32_t m, n, rank, G, job, pad;   // G CTAs, this one has the columns rank, rank + G, ..
+};
+constexpr int kQrThreads = 512, kQrWarps = kQrThreads / 32;
+constexpr size_t kQrSmem = 200 * 1024;
+constexpr int kQrUnits = 64;         // partial dot products of a round
+
+// The chain of a step runs on the first four warps, one per sub-partition: with
+// more, the reductions' FP64 additions would cost more than the split saves.
+constexpr int kQrChain = 128;
+__device__ __forceinline__ void chain_sync() { asm volatile("bar.sync 1, 128;" ::: "memory"); }
+
+// Sum over the chain's warps, the same in every thread of it.
+__device__ __forceinline__ double chain_sum4(double v, double* red) {
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+  chain_sync();
+  return (red[0] + red[1]) + (red[2] + red[3]);
+}
+
+// By the chain's threads: the reflector of column a (rows j .. m - 1, in shared
+// memory) into v (v[j] = 1) and, with beta on the diagonal, into the matrix; tau
+// into *tau and red[6].
+__device__ __forceinline__ void qr_reflector(double* a, double* v, int j, int m, double* T,
+                                             double* tau, double* red) {
+  double s = 0.0;
+  for (int i = j + 1 + threadIdx.x; i < m; i += kQrChain) s = fma(a[i], a[i], s);
+  s = chain_sum4(s, red);
+  const double alpha = a[j];
+  double beta = alpha, tv = 0.0, sc = 0.0;
+  if (s != 0.0) {                       // (NaN: every result is NaN)
+    const double n2 = fma(alpha, alpha, s);
+    if (n2 > 1e-290 && n2 < 1e290) {
+      const double nr = sqrt_of(n2);
+      beta = alpha >= 0.0 ? -nr : nr;
+      sc = recip(alpha - beta);         // |alpha - beta| >= |beta|
+      tv = (beta - alpha) * recip(beta);
+    } else {
+      const double nr = sqrt(n2);
+      beta = alpha >= 0.0 ? -nr : nr;
+      sc = 1.0 / (alpha - beta);
+      tv = (beta - alpha) / beta;
+    }
+  }
+  for (int i = j + threadIdx.x; i < m; i += kQrChain) {
+    const double x = i == j ? 1.0 : a[i] * sc;
+    v[i] = x;
+    T[i] = i == j ? beta : x;
+  }
+  if (threadIdx.x == 0) {
+    *tau = tv;
+    red[6] = tv;
+  }
+}
+
+__global__ void __launch_bounds__(kQrThreads, 1)
+qr_kernel(const QrItem* __restrict__ items, const int* __restrict__ cta_item, double* A, double* tau,
+          int* ready, int* err, uint64_t limit_ns) {
+  extern __shared__ double sh[];
+  __shared__ double red[8];              // two sums' partials, tau
+  __shared__ double part[kQrUnits * kQrWarps];
+  __shared__ int s_ok;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  for (int it = cta_item[blockIdx.x]; it < cta_item[blockIdx.x + 1]; ++it) {
+    const QrItem Q = items[it];
+    const int m = Q.m, n = Q.n, G = Q.G;
+    const int nc = Q.rank < n ? (n - Q.rank + G - 1) / G : 0;   // own columns
+    double* vb = sh;                                 // two reflectors, then the columns
+    double* cols = sh + 2 * m;
+    double* T = A + Q.offA;
+    for (int q = 0; q < nc; ++q) {
+      const double* src = T + (int64_t)(Q.rank + q * G) * m;
+      for (int i = tid; i < m; i += kQrThreads) cols[(int64_t)q * m + i] = src[i];
+    }
+    __syncthreads();
+    double t_next = 0.0;
+    bool have = false;                               // the next reflector is in place
+    const int steps = min(n, m);
+    for (int j = 0; j < steps; ++j) {
+      double* v = vb + (j & 1) * m;
+      double tv;
+      if (have) {
+        tv = t_next;
+      } else if (j % G == Q.rank) {                  // (step 0 only)
+        if (tid < kQrChain)
+          qr_reflector(cols + (int64_t)(j / G) * m, v, j, m, T + (int64_t)j * m,
+                       tau + Q.offTau + j, red);
+        __syncthreads();
+        tv = red[6];
+        if (G > 1 && tid == 0) {
+          __threadfence();
+          asm volatile("st.release.gpu.global.s32 [%0], %1;" ::"l"(ready + Q.job), "r"(j + 1) : "memory");
+        }
+      } else {
+        if (j >= Q.rank + (nc - 1) * G) break;       // no column of this CTA is left
+        if (tid == 0) {
+          int ok = 1, r;
+          uint64_t t0, t;
+          asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t0));
+          for (;;) {
+            asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(r) : "l"(ready + Q.job) : "memory");
+            if (r > j) break;
+            asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+            if (t - t0 > limit_ns) {
+              atomicExch(err, 1);
+              ok = 0;
+              break;
+            }
+          }
+          s_ok = ok;
+        }
+        __syncthreads();
+        if (!s_ok) return;
+        const double* src = T + (int64_t)j * m;
+        for (int i = j + tid; i < m; i += kQrThreads) v[i] = i == j ? 1.0 : __ldcg(src + i);
+        tv = __ldcg(tau + Q.offTau + j);
+        __syncthreads();
+      }
+      // the next column first, by the whole CTA, and its reflector
+      have = j + 1 < steps && (j + 1) % G == Q.rank;
+      int q0 = j < Q.rank ? 0 : (j - Q.rank) / G + 1;   // first own column > j
+      if (have) {
+        if (tid < kQrChain) {
+          double* a = cols + (int64_t)q0 * m;
+          double s = 0.0;
+          for (int i = j + tid; i < m; i += kQrChain) s = fma(v[i], a[i], s);
+          s = -tv * chain_sum4(s, red);
+          for (int i = j + tid; i < m; i += kQrChain) a[i] = fma(s, v[i], a[i]);
+          chain_sync();
+          qr_reflector(a, vb + ((j + 1) & 1) * m, j + 1, m, T + (int64_t)(j + 1) * m,
+                       tau + Q.offTau + j + 1, red);
+        }
+        __syncthreads();
+        t_next = red[6];
+        if (G > 1 && tid == 0) {
+          __threadfence();
+          asm volatile("st.release.gpu.global.s32 [%0], %1;" ::"l"(ready + Q.job), "r"(j + 2) : "memory");
+        }
+        ++q0;
+      }
+      // the others: w warps a column, in rounds of kQrUnits columns
+      for (int qb = q0; qb < nc; qb += kQrUnits) {
+        const int k = min(kQrUnits, nc - qb);
+        int w = 1;
+        while (2 * w * k <= kQrWarps) w *= 2;
+        const int len = (((m - j + w - 1) / w) + 31) & ~31;   // rows of a warp
+        for (int u = warp; u < k * w; u += kQrWarps) {
+          const int c = u / w, part_i = u % w;
+          const double* a = cols + (int64_t)(qb + c) * m;
+          const int i0 = j + part_i * len, i1 = min(m, i0 + len);
+          double s0 = 0.0, s1 = 0.0;
+          int i = i0 + lane;
+          for (; i + 32 < i1; i += 64) {
+            s0 = fma(v[i], a[i], s0);
+            s1 = fma(v[i + 32], a[i + 32], s1);
+          }
+          if (i < i1) s0 = fma(v[i], a[i], s0);
+          s0 += s1;
+          for (int o = 16; o > 0; o >>= 1) s0 += __shfl_xor_sync(0xffffffffu, s0, o);
+          if (w == 1) {
+            const double f = -tv * s0;
+            double* aw = cols + (int64_t)(qb + c) * m;
+            for (i = i0 + lane; i < i1; i += 32) aw[i] = fma(f, v[i], aw[i]);
+          } else if (lane == 0) {
+            part[c * kQrWarps + part_i] = s0;
+          }
+        }
+        if (w > 1) {
+          __syncthreads();
+          for (int u = warp; u < k * w; u += kQrWarps) {
+            const int c = u / w, part_i = u % w;
+            double s = part[c * kQrWarps];
+            for (int x = 1; x < w; ++x) s += part[c * kQrWarps + x];
+            const double f = -tv * s;
+            double* a = cols + (int64_t)(qb + c) * m;
+            const int i0 = j + part_i * len, i1 = min(m, i0 + len);
+            for (int i = i0 + lane; i < i1; i += 32) a[i] = fma(f, v[i], a[i]);
+          }
+        }
+      }
+      __syncthreads();
+    }
+    // R above the diagonal (the rest is in place)
+    for (int q = 0; q < nc; ++q) {
+      const int c = Q.rank + q * G;
+      for (int i = tid; i < min(c, m); i += kQrThreads) T[(int64_t)c * m + i] = cols[(int64_t)q * m + i];
+    }
+    __syncthreads();
+  }
+}
+
+// The batch's matrices dealt to at most `ctas` CTAs so that the longest takes about
+// the least time by a model of the kernel (microseconds): FP64 work over the
+// matrix's SMs plus a step's chain.  `lib` receives the matrices whose columns do
+// not fit the shared memory of the CTAs (cuSOLVER factorises those).
+struct QrPlan {
+  std::vector<QrItem> items;
+  std::vector<int> cta_item{0};
+  size_t smem = 0;
+};
+void plan_qr(const std::vector<JacJob>& tab, int ctas, QrPlan* plan, std::vector<int>* lib) {
+  const auto time = [](double m, double n, int G) {
+    return n * (G > 1 ? 3.0 : 2.0) + (m * n * n - n * n * n / 3.0) / (3800.0 * G);
+  };
+  const auto least = [](int64_t m, int64_t n) {       // CTAs whose shared memory holds the columns
+    const int64_t fit = (int64_t)(kQrSmem / sizeof(double)) / m - 2;
+    return fit < 1 ? (int64_t)0 : (n + fit - 1) / fit;
+  };
+  std::vector<int> jobs;
+  lib->clear();
+  int64_t need = 0;
+  for (int k = 0; k < (int)tab.size(); ++k) {
+    const int64_t g = least(tab[k].m, tab[k].n);
+    if (g < 1 || (g > 1 && need + g > ctas - 2)) {
+      lib->push_back(k);
+    } else {
+      if (g > 1) need += g;
+      jobs.push_back(k);
+    }
+  }
+  if (jobs.empty()) return;
+  // the CTAs of every matrix for a makespan t: the fewest that keep to it
+  std::vector<int> G(tab.size(), 1);
+  const auto fits = [&](double t) {
+    int64_t many = 0;
+    double rest = 0.0;
+    for (int k : jobs) {
+      const double m = tab[k].m, n = tab[k].n;
+      int64_t g = least(tab[k].m, tab[k].n);
+      if (g == 1 && time(m, n, 1) <= t) {
+        rest += time(m, n, 1);
+      } else {
+        g = std::max<int64_t>(g, 2);
+        while (g < tab[k].n && time(m, n, (int)g) > t) ++g;
+        many += g;
+      }
+      G[k] = (int)g;
+    }
+    return many + (int64_t)std::ceil(rest / t) + (rest > 0.0 ? 1 : 0) <= ctas;
+  };
+  double t = 20.0;
+  while (!fits(t) && t < 1e9) t *= 1.1;
+  if (t >= 1e9) {                                    // (the CTAs are few: everything to the library)
+    lib->insert(lib->end(), jobs.begin(), jobs.end());
+    return;
+  }
+  std::vector<std::vector<QrItem>> queue;
+  std::vector<double> load;
+  std::sort(jobs.begin(), jobs.end(), [&](int a, int b) {
+    if ((G[a] > 1) != (G[b] > 1)) return G[a] > 1;
+    return time(tab[a].m, tab[a].n, 1) > time(tab[b].m, tab[b].n, 1);
+  });
+  for (int k : jobs) {
+    const JacJob& J = tab[k];
+    const QrItem q{J.offA, J.offTau, J.m, J.n, 0, G[k], k, 0};
+    const size_t own = (size_t)((J.n + G[k] - 1) / G[k]);
+    plan->smem = std::max(plan->smem, (2 + own) * J.m * sizeof(double));
+    if (G[k] > 1) {
+      for (int r = 0; r < G[k]; ++r) {
+        queue.push_back({q});
+        queue.back()[0].rank = r;
+        load.push_back(time(J.m, J.n, G[k]));
+      }
+      continue;
+    }
+    // whole matrices: to the least loaded CTA, a new one while there are any
+    size_t w = std::min_element(load.begin(), load.end()) - load.begin();
+    if ((int)queue.size() < ctas) {
+      w = queue.size();
+      queue.emplace_back();
+      load.push_back(0.0);
+    }
+    queue[w].push_back(q);
+    load[w] += time(J.m, J.n, 1);
+  }
+  for (const auto& v : queue) {
+    plan->items.insert(plan->items.end(), v.begin(), v.end());
+    plan->cta_item.push_back((int)plan->items.size());
+  }
 }
 
 // The rotation of a pair with d = beta - alpha and gamma = g, as p = tan(theta / 2)
@@ -471,12 +769,15 @@ dmrg3s_status cuda_ok(Context* c, cudaError_t e, const char* what) {
 
 }  // namespace
 
-dmrg3s_status lane_create(Context* c, SvdLane* w) {
+dmrg3s_status lane_ready(Context* c, SvdLane* w) {
+  if (w->ev) return DMRG3S_OK;
   if (cusolverDnCreate(&w->h) != CUSOLVER_STATUS_SUCCESS ||
       cusolverDnCreateParams(&w->p) != CUSOLVER_STATUS_SUCCESS ||
       cudaStreamCreateWithFlags(&w->s, cudaStreamNonBlocking) != cudaSuccess ||
-      cudaEventCreateWithFlags(&w->ev, cudaEventDisableTiming) != cudaSuccess)
+      cudaEventCreateWithFlags(&w->ev, cudaEventDisableTiming) != cudaSuccess) {
+    lane_destroy(w);
     return fail(c, DMRG3S_ERR_CUDA, "SVD lane set-up");
+  }
   return DMRG3S_OK;
 }
 
@@ -544,19 +845,28 @@ dmrg3s_status svd_jacobi(Context* c, std::vector<SvdLane>& lanes, int nlanes,
   const int ncta = (int)pairs.size(), ncol = (int)col_job.size();
   int64_t na = 0;   // extent of the A buffer used by the jobs
   for (const JacJob& t : tab) na = std::max(na, t.offA + (int64_t)t.m * t.n);
+  QrPlan qr;
+  std::vector<int> by_lib;       // matrices left to cuSOLVER's QR
+  plan_qr(tab, plan_ctas(), &qr, &by_lib);
   // ---- device buffers: doubles [tau | Y | V1 | sigma | column norms | T = A P],
-  //      ints [col_job | perm | rot | sweep | qinfo]
+  //      ints [col_job | perm | rot | sweep | qinfo | QR flags | QR error]
   const int64_t nd = ntau + ny + nv + 2 * (int64_t)ncol + na;
-  const int64_t ni = 2 * (int64_t)ncol + (int64_t)kJacobiMaxSweeps * nj + 1 + nj;
+  const int64_t ni = 2 * (int64_t)ncol + (int64_t)kJacobiMaxSweeps * nj + 1 + 2 * nj + 1 +
+                     (int64_t)qr.cta_item.size();
   double* dd = nullptr;
   int* di = nullptr;
   JacJob* dt = nullptr;
   JacPair* dp = nullptr;
+  QrItem* dq = nullptr;
   dmrg3s_status s = DMRG3S_OK;
   if ((s = cuda_ok(c, cudaMallocAsync((void**)&dd, (size_t)nd * sizeof(double), st), "SVD buffers")) ||
       (s = cuda_ok(c, cudaMallocAsync((void**)&di, (size_t)ni * sizeof(int), st), "SVD buffers")) ||
       (s = cuda_ok(c, cudaMallocAsync((void**)&dt, tab.size() * sizeof(JacJob), st), "SVD buffers")) ||
       (s = cuda_ok(c, cudaMallocAsync((void**)&dp, pairs.size() * sizeof(JacPair), st), "SVD buffers")) ||
+      (!qr.items.empty() &&
+       (s = cuda_ok(c, cudaMallocAsync((void**)&dq, qr.items.size() * sizeof(QrItem), st), "SVD buffers"))) ||
+      (s = cuda_ok(c, cudaFuncSetAttribute(qr_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                           (int)kQrSmem), "QR shared memory")) ||
       (s = cuda_ok(c, cudaFuncSetAttribute(jac_round_kernel,
                                            cudaFuncAttributeMaxDynamicSharedMemorySize,
                                            (int)kJacStage), "Jacobi shared memory"))) {
@@ -564,6 +874,7 @@ dmrg3s_status svd_jacobi(Context* c, std::vector<SvdLane>& lanes, int nlanes,
     if (di) cudaFreeAsync(di, st);
     if (dt) cudaFreeAsync(dt, st);
     if (dp) cudaFreeAsync(dp, st);
+    if (dq) cudaFreeAsync(dq, st);
     return s;
   }
   double* tau = dd;
@@ -577,9 +888,17 @@ dmrg3s_status svd_jacobi(Context* c, std::vector<SvdLane>& lanes, int nlanes,
   int* rot = d_perm + ncol;
   int* d_sweep = rot + (int64_t)kJacobiMaxSweeps * nj;
   int* qinfo = d_sweep + 1;
+  int* qr_ready = qinfo + nj;
+  int* qr_err = qr_ready + nj;
+  int* qr_cta = qr_err + 1;
   cudaMemcpyAsync(dt, tab.data(), tab.size() * sizeof(JacJob), cudaMemcpyHostToDevice, st);
   cudaMemcpyAsync(dp, pairs.data(), pairs.size() * sizeof(JacPair), cudaMemcpyHostToDevice, st);
   cudaMemcpyAsync(d_col, col_job.data(), col_job.size() * sizeof(int), cudaMemcpyHostToDevice, st);
+  cudaMemsetAsync(qr_ready, 0, (size_t)(nj + 1) * sizeof(int), st);
+  if (!qr.items.empty()) {
+    cudaMemcpyAsync(dq, qr.items.data(), qr.items.size() * sizeof(QrItem), cudaMemcpyHostToDevice, st);
+    cudaMemcpyAsync(qr_cta, qr.cta_item.data(), qr.cta_item.size() * sizeof(int), cudaMemcpyHostToDevice, st);
+  }
   cudaMemsetAsync(rot, 0, (size_t)kJacobiMaxSweeps * nj * sizeof(int), st);
   cudaMemsetAsync(d_sweep, 0xff, sizeof(int), st);   // -1: the first sweep advances it to 0
   s = cuda_ok(c, cudaGetLastError(), "SVD tables");
@@ -605,12 +924,32 @@ dmrg3s_status svd_jacobi(Context* c, std::vector<SvdLane>& lanes, int nlanes,
       s = cuda_ok(c, cudaGetLastError(), "column order");
     }
   }
-  // ---- lane workspaces (QR, and Q V1 for the left vectors)
+  // ---- lanes for the matrices that need cuSOLVER (a QR too large for qr_kernel, Q V1
+  // for the left vectors), by QR cost m n^2, largest first; created when first used
+  std::vector<char> lib_qr(nj, 0);
+  for (int k : by_lib) lib_qr[k] = 1;
+  std::vector<int> order;
+  for (int k = 0; k < nj; ++k)
+    if (lib_qr[k] || tab[k].offU >= 0) order.push_back(k);
+  std::sort(order.begin(), order.end(), [&](int a, int b) {
+    return (double)tab[a].m * tab[a].n * tab[a].n > (double)tab[b].m * tab[b].n * tab[b].n;
+  });
+  nlanes = std::min(nlanes, (int)order.size());
+  std::vector<std::vector<int>> part(nlanes);
+  std::vector<double> load(nlanes, 0.0);
+  for (int k : order) {
+    const int w = (int)(std::min_element(load.begin(), load.end()) - load.begin());
+    part[w].push_back(k);
+    load[w] += (double)tab[k].m * tab[k].n * tab[k].n + 1e5;
+  }
+  for (int w = 0; !s && w < nlanes; ++w) s = lane_ready(c, &lanes[w]);
   size_t dmax = 1, hmax = 1;
-  for (const JacJob& t : tab) {
+  for (int k : order) {
     if (s) break;
+    const JacJob& t = tab[k];
     size_t wd = 0, wh = 0;
-    if (cusolverDnXgeqrf_bufferSize(lanes[0].h, lanes[0].p, t.m, t.n, CUDA_R_64F, T + t.offA, t.m,
+    if (lib_qr[k] &&
+        cusolverDnXgeqrf_bufferSize(lanes[0].h, lanes[0].p, t.m, t.n, CUDA_R_64F, T + t.offA, t.m,
                                     CUDA_R_64F, tau + t.offTau, CUDA_R_64F, &wd,
                                     &wh) != CUSOLVER_STATUS_SUCCESS)
       s = fail(c, DMRG3S_ERR_CUDA, "QR buffer size");
@@ -639,19 +978,6 @@ dmrg3s_status svd_jacobi(Context* c, std::vector<SvdLane>& lanes, int nlanes,
     }
     if (l.hwork.size() < hmax) l.hwork.resize(hmax);
   }
-  // greedy assignment to lanes by QR cost m n^2, largest first
-  std::vector<int> order(nj);
-  for (int k = 0; k < nj; ++k) order[k] = k;
-  std::sort(order.begin(), order.end(), [&](int a, int b) {
-    return (double)tab[a].m * tab[a].n * tab[a].n > (double)tab[b].m * tab[b].n * tab[b].n;
-  });
-  std::vector<std::vector<int>> part(nlanes);
-  std::vector<double> load(nlanes, 0.0);
-  for (int k : order) {
-    const int w = (int)(std::min_element(load.begin(), load.end()) - load.begin());
-    part[w].push_back(k);
-    load[w] += (double)tab[k].m * tab[k].n * tab[k].n + 1e5;
-  }
   cudaEvent_t ev_in = nullptr;
   if (!s && cudaEventCreateWithFlags(&ev_in, cudaEventDisableTiming) != cudaSuccess)
     s = fail(c, DMRG3S_ERR_CUDA, "SVD event");
@@ -672,7 +998,7 @@ dmrg3s_status svd_jacobi(Context* c, std::vector<SvdLane>& lanes, int nlanes,
     std::vector<std::thread> th;
     for (int w = 1; w < nlanes; ++w)
       if (!part[w].empty()) th.emplace_back(run, w);
-    if (!part[0].empty()) run(0);
+    if (nlanes > 0 && !part[0].empty()) run(0);
     for (auto& t : th) t.join();
     bool ok = true;
     for (int w = 0; w < nlanes; ++w) {
@@ -681,16 +1007,30 @@ dmrg3s_status svd_jacobi(Context* c, std::vector<SvdLane>& lanes, int nlanes,
     }
     return ok;
   };
-  auto all = [](int) { return true; };
   // ---- 1. A = Q R
-  const bool qr_ok = s || on_lanes(
+  if (!s && !qr.items.empty()) {
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeCooperative;
+    at.val.cooperative = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = (unsigned)qr.cta_item.size() - 1;
+    cfg.blockDim = kQrThreads;
+    cfg.dynamicSmemBytes = qr.smem;
+    cfg.stream = st;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    s = cuda_ok(c, cudaLaunchKernelEx(&cfg, qr_kernel, (const QrItem*)dq, (const int*)qr_cta, T, tau,
+                                      qr_ready, qr_err, c->wait_ns), "QR factorisation");
+    count_launch();
+  }
+  const bool qr_ok = s || by_lib.empty() || on_lanes(
       [&](SvdLane& l, int k) {
         const JacJob& t = tab[k];
         return cusolverDnXgeqrf(l.h, l.p, t.m, t.n, CUDA_R_64F, T + t.offA, t.m, CUDA_R_64F,
                                 tau + t.offTau, CUDA_R_64F, l.dwork, l.dbytes, l.hwork.data(),
                                 l.hwork.size(), qinfo + k) == CUSOLVER_STATUS_SUCCESS;
       },
-      all);
+      [&](int k) { return lib_qr[k] != 0; });
   if (!s && !qr_ok) s = fail(c, DMRG3S_ERR_CUDA, "QR factorisation");
   // ---- 2. Y = R^T, V1 = I
   if (!s) {
@@ -714,6 +1054,7 @@ dmrg3s_status svd_jacobi(Context* c, std::vector<SvdLane>& lanes, int nlanes,
   }
   cudaGetLastError();   // a failed capture leaves the plain launches below
   std::vector<int> hrot(nj), active(nj, 1);
+  int herr = 0;
   std::vector<int> conv(nj, 0);
   Profiler& pr = c->prof;
   const int max_sweeps = jacobi_max_sweeps();
@@ -734,8 +1075,14 @@ dmrg3s_status svd_jacobi(Context* c, std::vector<SvdLane>& lanes, int nlanes,
     if (s) break;
     if ((s = cuda_ok(c, cudaMemcpyAsync(hrot.data(), rot + (int64_t)sw * nj, nj * sizeof(int),
                                         cudaMemcpyDeviceToHost, st), "Jacobi rotations")) ||
+        (sw == 0 && (s = cuda_ok(c, cudaMemcpyAsync(&herr, qr_err, sizeof(int), cudaMemcpyDeviceToHost,
+                                                    st), "QR status"))) ||
         (s = cuda_ok(c, cudaStreamSynchronize(st), "Jacobi sweep")))
       break;
+    if (herr) {
+      s = fail(c, DMRG3S_ERR_TIMEOUT, "the QR factorisation gave up a bounded wait");
+      break;
+    }
     // algorithmic cost of the sweep: a pair test reads two columns (16n bytes)
     // for three dot products (6n flops); a rotation of a column pair of Y and
     // of V1 takes 6n flops each and writes 16n bytes each (V1 also read)
@@ -795,6 +1142,7 @@ dmrg3s_status svd_jacobi(Context* c, std::vector<SvdLane>& lanes, int nlanes,
   cudaFreeAsync(di, st);
   cudaFreeAsync(dt, st);
   cudaFreeAsync(dp, st);
+  if (dq) cudaFreeAsync(dq, st);
   if (ev_in) cudaEventDestroy(ev_in);
   return s;
 }
@@ -830,11 +1178,9 @@ extern "C" dmrg3s_status dmrg3s_svd(dmrg3s_ctx ctx, int32_t nmat, const int64_t*
   std::vector<SvdLane> lanes(1);
   std::vector<int> info(nmat, 0);
   std::string diag;
-  if (!(s = lane_create(c, &lanes[0]))) {
-    s = svd_jacobi(c, lanes, 1, jobs, A, S, VT, U, info.data(), st, &diag);
-    if (!s && cudaStreamSynchronize(st) != cudaSuccess)
-      s = fail(c, DMRG3S_ERR_CUDA, "dmrg3s_svd: stream synchronisation");
-  }
+  s = svd_jacobi(c, lanes, 1, jobs, A, S, VT, U, info.data(), st, &diag);
+  if (!s && cudaStreamSynchronize(st) != cudaSuccess)
+    s = fail(c, DMRG3S_ERR_CUDA, "dmrg3s_svd: stream synchronisation");
   lane_destroy(&lanes[0]);
   for (int k = 0; !s && k < nmat; ++k)
     if (info[k]) s = fail(c, DMRG3S_ERR_NOT_CONVERGED, "dmrg3s_svd: " + diag);

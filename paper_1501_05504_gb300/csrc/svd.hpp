@@ -31,7 +31,7 @@ struct SvdLane {
   size_t dbytes = 0;
   std::vector<char> hwork;
 };
-dmrg3s_status lane_create(Context* c, SvdLane* w);
+dmrg3s_status lane_ready(Context* c, SvdLane* w);   // created on first use
 void lane_destroy(SvdLane* w);
 
 // One matrix of a batch.  A (m x n, ld m, m >= n >= 1) at element offset offA
