@@ -334,6 +334,61 @@ qr_kernel(const QrItem* __restrict__ items, const int* __restrict__ cta_item, do
   }
 }
 
+// U <- Q U for the left vectors: the reflectors in reverse order on every column, a
+// warp per column with the column in shared memory (m <= kQrApplyRows) and the
+// same rows in the same lanes throughout, so a warp needs nothing from another.
+// Bound by the FP64 pipe.  Whole SVDs with left vectors, cuSOLVER's ormqr before: 60
+// matrices of 60 x 40 34 -> 4.1 ms, 14 sectors up to 762 x 245 24.1 -> 16.7, 200 x 100
+// 6.6 -> 5.2, 762 x 245 alone 16.6 -> 16.2.
+struct QrColumns {
+  int32_t job, col0;
+};
+constexpr int kQrApplyWarps = 4;
+constexpr int kQrApplyRows = 6400;
+__global__ void __launch_bounds__(32 * kQrApplyWarps)
+qr_apply_kernel(const JacJob* __restrict__ jobs, const QrColumns* __restrict__ items, const double* A,
+                const double* tau, double* U, int stride) {
+  grid_next();
+  grid_wait();
+  extern __shared__ double sh[];
+  const QrColumns I = items[blockIdx.x];
+  const JacJob J = jobs[I.job];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int c = I.col0 + warp, m = J.m, n = J.n;
+  if (c >= n) return;
+  double* ug = U + J.offU + (int64_t)c * m;
+  const bool staged = m <= stride;
+  double* u = staged ? sh + (int64_t)warp * stride : ug;
+  if (staged)
+    for (int i = lane; i < m; i += 32) u[i] = ug[i];
+  const double* T = A + J.offA;
+  double t_next = tau[J.offTau + n - 1];
+  for (int j = n - 1; j >= 0; --j) {
+    const double t = t_next;
+    if (j > 0) t_next = tau[J.offTau + j - 1];
+    if (t == 0.0) continue;
+    const double* v = T + (int64_t)j * m;
+    const int i0 = (j & ~31) + lane;                 // v is 0 above row j, 1 on it
+    const double vd = i0 > j ? (i0 < m ? v[i0] : 0.0) : i0 == j ? 1.0 : 0.0;
+    double s0 = i0 < m ? vd * u[i0] : 0.0, s1 = 0.0;
+    int i = i0 + 32;
+#pragma unroll 2
+    for (; i + 32 < m; i += 64) {
+      s0 = fma(v[i], u[i], s0);
+      s1 = fma(v[i + 32], u[i + 32], s1);
+    }
+    if (i < m) s0 = fma(v[i], u[i], s0);
+    s0 += s1;
+    for (int o = 16; o > 0; o >>= 1) s0 += __shfl_xor_sync(0xffffffffu, s0, o);
+    const double f = -t * s0;
+    if (i0 < m) u[i0] = fma(f, vd, u[i0]);
+#pragma unroll 4
+    for (i = i0 + 32; i < m; i += 32) u[i] = fma(f, v[i], u[i]);
+  }
+  if (staged)
+    for (int i = lane; i < m; i += 32) ug[i] = u[i];
+}
+
 // The batch's matrices dealt to at most `ctas` CTAs so that the longest takes about
 // the least time by a model of the kernel (microseconds): FP64 work over the
 // matrix's SMs plus a step's chain.  `lib` receives the matrices whose columns do
@@ -845,14 +900,21 @@ dmrg3s_status svd_jacobi(Context* c, std::vector<SvdLane>& lanes, int nlanes,
   const int ncta = (int)pairs.size(), ncol = (int)col_job.size();
   int64_t na = 0;   // extent of the A buffer used by the jobs
   for (const JacJob& t : tab) na = std::max(na, t.offA + (int64_t)t.m * t.n);
+  std::vector<QrColumns> qcols;  // the left vectors' columns by CTA
+  int umax = 0;                  // their longest
+  for (int k = 0; k < nj; ++k)
+    if (tab[k].offU >= 0) {
+      for (int q = 0; q < tab[k].n; q += kQrApplyWarps) qcols.push_back(QrColumns{k, q});
+      umax = std::max(umax, (int)tab[k].m);
+    }
   QrPlan qr;
   std::vector<int> by_lib;       // matrices left to cuSOLVER's QR
   plan_qr(tab, plan_ctas(), &qr, &by_lib);
   // ---- device buffers: doubles [tau | Y | V1 | sigma | column norms | T = A P],
-  //      ints [col_job | perm | rot | sweep | qinfo | QR flags | QR error]
+  //      ints [col_job | perm | rot | sweep | qinfo | QR flags | QR error | QR items | left columns]
   const int64_t nd = ntau + ny + nv + 2 * (int64_t)ncol + na;
   const int64_t ni = 2 * (int64_t)ncol + (int64_t)kJacobiMaxSweeps * nj + 1 + 2 * nj + 1 +
-                     (int64_t)qr.cta_item.size();
+                     (int64_t)qr.cta_item.size() + 2 * (int64_t)qcols.size();
   double* dd = nullptr;
   int* di = nullptr;
   JacJob* dt = nullptr;
@@ -891,10 +953,13 @@ dmrg3s_status svd_jacobi(Context* c, std::vector<SvdLane>& lanes, int nlanes,
   int* qr_ready = qinfo + nj;
   int* qr_err = qr_ready + nj;
   int* qr_cta = qr_err + 1;
+  QrColumns* d_qcols = reinterpret_cast<QrColumns*>(qr_cta + qr.cta_item.size());
   cudaMemcpyAsync(dt, tab.data(), tab.size() * sizeof(JacJob), cudaMemcpyHostToDevice, st);
   cudaMemcpyAsync(dp, pairs.data(), pairs.size() * sizeof(JacPair), cudaMemcpyHostToDevice, st);
   cudaMemcpyAsync(d_col, col_job.data(), col_job.size() * sizeof(int), cudaMemcpyHostToDevice, st);
   cudaMemsetAsync(qr_ready, 0, (size_t)(nj + 1) * sizeof(int), st);
+  if (!qcols.empty())
+    cudaMemcpyAsync(d_qcols, qcols.data(), qcols.size() * sizeof(QrColumns), cudaMemcpyHostToDevice, st);
   if (!qr.items.empty()) {
     cudaMemcpyAsync(dq, qr.items.data(), qr.items.size() * sizeof(QrItem), cudaMemcpyHostToDevice, st);
     cudaMemcpyAsync(qr_cta, qr.cta_item.data(), qr.cta_item.size() * sizeof(int), cudaMemcpyHostToDevice, st);
@@ -924,13 +989,9 @@ dmrg3s_status svd_jacobi(Context* c, std::vector<SvdLane>& lanes, int nlanes,
       s = cuda_ok(c, cudaGetLastError(), "column order");
     }
   }
-  // ---- lanes for the matrices that need cuSOLVER (a QR too large for qr_kernel, Q V1
-  // for the left vectors), by QR cost m n^2, largest first; created when first used
-  std::vector<char> lib_qr(nj, 0);
-  for (int k : by_lib) lib_qr[k] = 1;
-  std::vector<int> order;
-  for (int k = 0; k < nj; ++k)
-    if (lib_qr[k] || tab[k].offU >= 0) order.push_back(k);
+  // ---- lanes for the matrices whose QR is too large for qr_kernel, by its cost m n^2,
+  // largest first; created when first used
+  std::vector<int> order(by_lib);
   std::sort(order.begin(), order.end(), [&](int a, int b) {
     return (double)tab[a].m * tab[a].n * tab[a].n > (double)tab[b].m * tab[b].n * tab[b].n;
   });
@@ -948,21 +1009,12 @@ dmrg3s_status svd_jacobi(Context* c, std::vector<SvdLane>& lanes, int nlanes,
     if (s) break;
     const JacJob& t = tab[k];
     size_t wd = 0, wh = 0;
-    if (lib_qr[k] &&
-        cusolverDnXgeqrf_bufferSize(lanes[0].h, lanes[0].p, t.m, t.n, CUDA_R_64F, T + t.offA, t.m,
+    if (cusolverDnXgeqrf_bufferSize(lanes[0].h, lanes[0].p, t.m, t.n, CUDA_R_64F, T + t.offA, t.m,
                                     CUDA_R_64F, tau + t.offTau, CUDA_R_64F, &wd,
                                     &wh) != CUSOLVER_STATUS_SUCCESS)
       s = fail(c, DMRG3S_ERR_CUDA, "QR buffer size");
     dmax = std::max(dmax, wd);
     hmax = std::max(hmax, wh);
-    if (!s && t.offU >= 0) {
-      int lw = 0;
-      if (cusolverDnDormqr_bufferSize(lanes[0].h, CUBLAS_SIDE_LEFT, CUBLAS_OP_N, t.m, t.n, t.n,
-                                      T + t.offA, t.m, tau + t.offTau, U + t.offU, t.m,
-                                      &lw) != CUSOLVER_STATUS_SUCCESS)
-        s = fail(c, DMRG3S_ERR_CUDA, "ormqr buffer size");
-      dmax = std::max(dmax, (size_t)lw * sizeof(double));
-    }
   }
   for (int w = 0; !s && w < nlanes; ++w) {
     SvdLane& l = lanes[w];
@@ -981,32 +1033,6 @@ dmrg3s_status svd_jacobi(Context* c, std::vector<SvdLane>& lanes, int nlanes,
   cudaEvent_t ev_in = nullptr;
   if (!s && cudaEventCreateWithFlags(&ev_in, cudaEventDisableTiming) != cudaSuccess)
     s = fail(c, DMRG3S_ERR_CUDA, "SVD event");
-  // runs fn(lane, job) for every wanted job on its lane after the work queued
-  // on st; st waits for the lanes
-  auto on_lanes = [&](auto fn, auto wanted) -> bool {
-    cudaEventRecord(ev_in, st);
-    std::vector<int> bad(nlanes, 0);
-    auto run = [&](int w) {
-      SvdLane& l = lanes[w];
-      cudaSetDevice(c->device);
-      cudaStreamWaitEvent(l.s, ev_in, 0);
-      cusolverDnSetStream(l.h, l.s);
-      for (int k : part[w])
-        if (wanted(k) && !fn(l, k)) bad[w] = 1;
-      cudaEventRecord(l.ev, l.s);
-    };
-    std::vector<std::thread> th;
-    for (int w = 1; w < nlanes; ++w)
-      if (!part[w].empty()) th.emplace_back(run, w);
-    if (nlanes > 0 && !part[0].empty()) run(0);
-    for (auto& t : th) t.join();
-    bool ok = true;
-    for (int w = 0; w < nlanes; ++w) {
-      ok = ok && !bad[w];
-      if (!part[w].empty()) cudaStreamWaitEvent(st, lanes[w].ev, 0);
-    }
-    return ok;
-  };
   // ---- 1. A = Q R
   if (!s && !qr.items.empty()) {
     cudaLaunchAttribute at{};
@@ -1023,15 +1049,33 @@ dmrg3s_status svd_jacobi(Context* c, std::vector<SvdLane>& lanes, int nlanes,
                                       qr_ready, qr_err, c->wait_ns), "QR factorisation");
     count_launch();
   }
-  const bool qr_ok = s || by_lib.empty() || on_lanes(
-      [&](SvdLane& l, int k) {
+  if (!s && nlanes > 0) {
+    // on the lanes after the work queued on st, which waits for them
+    cudaEventRecord(ev_in, st);
+    std::vector<int> bad(nlanes, 0);
+    auto run = [&](int w) {
+      SvdLane& l = lanes[w];
+      cudaSetDevice(c->device);
+      cudaStreamWaitEvent(l.s, ev_in, 0);
+      cusolverDnSetStream(l.h, l.s);
+      for (int k : part[w]) {
         const JacJob& t = tab[k];
-        return cusolverDnXgeqrf(l.h, l.p, t.m, t.n, CUDA_R_64F, T + t.offA, t.m, CUDA_R_64F,
-                                tau + t.offTau, CUDA_R_64F, l.dwork, l.dbytes, l.hwork.data(),
-                                l.hwork.size(), qinfo + k) == CUSOLVER_STATUS_SUCCESS;
-      },
-      [&](int k) { return lib_qr[k] != 0; });
-  if (!s && !qr_ok) s = fail(c, DMRG3S_ERR_CUDA, "QR factorisation");
+        if (cusolverDnXgeqrf(l.h, l.p, t.m, t.n, CUDA_R_64F, T + t.offA, t.m, CUDA_R_64F,
+                             tau + t.offTau, CUDA_R_64F, l.dwork, l.dbytes, l.hwork.data(),
+                             l.hwork.size(), qinfo + k) != CUSOLVER_STATUS_SUCCESS)
+          bad[w] = 1;
+      }
+      cudaEventRecord(l.ev, l.s);
+    };
+    std::vector<std::thread> th;
+    for (int w = 1; w < nlanes; ++w) th.emplace_back(run, w);
+    run(0);
+    for (auto& t : th) t.join();
+    for (int w = 0; w < nlanes; ++w) {
+      if (bad[w] && !s) s = fail(c, DMRG3S_ERR_CUDA, "QR factorisation");
+      cudaStreamWaitEvent(st, lanes[w].ev, 0);
+    }
+  }
   // ---- 2. Y = R^T, V1 = I
   if (!s) {
     launch_chain(jac_init_kernel, ncol, kJacThreads, 0, st, dt, d_col, T, Y, V1);
@@ -1119,17 +1163,15 @@ dmrg3s_status svd_jacobi(Context* c, std::vector<SvdLane>& lanes, int nlanes,
     s = cuda_ok(c, cudaGetLastError(), "singular vectors");
   }
   // ---- 5. U = Q (V1; 0)
-  if (!s && nv > 0) {
-    const bool ok = on_lanes(
-        [&](SvdLane& l, int k) {
-          const JacJob& t = tab[k];
-          return cusolverDnDormqr(l.h, CUBLAS_SIDE_LEFT, CUBLAS_OP_N, t.m, t.n, t.n, T + t.offA,
-                                  t.m, tau + t.offTau, U + t.offU, t.m, (double*)l.dwork,
-                                  (int)(l.dbytes / sizeof(double)),
-                                  qinfo + k) == CUSOLVER_STATUS_SUCCESS;
-        },
-        [&](int k) { return tab[k].offV >= 0; });
-    if (!ok) s = fail(c, DMRG3S_ERR_CUDA, "left singular vectors (ormqr)");
+  if (!s && !qcols.empty()) {
+    const int stride = std::min(umax, kQrApplyRows);
+    const size_t bytes = (size_t)kQrApplyWarps * stride * sizeof(double);
+    if (!(s = cuda_ok(c, cudaFuncSetAttribute(qr_apply_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                              (int)bytes), "left vectors")))
+      launch_chain(qr_apply_kernel, (int)qcols.size(), 32 * kQrApplyWarps, bytes, st, dt, d_qcols, T, tau, U,
+                   stride);
+    count_launch();
+    if (!s) s = cuda_ok(c, cudaGetLastError(), "left vectors");
   }
   for (int k = 0; k < nj; ++k) {
     info[k] = conv[k] ? 0 : 1;
