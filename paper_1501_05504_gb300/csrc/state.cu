@@ -422,13 +422,8 @@ struct Trunc {
   dmrg3s_svd_method method = DMRG3S_SVD_GESVD;   // the factorisation used (AUTO resolved)
 };
 
-// Smaller side of the largest sector from which DMRG3S_SVD_AUTO takes the
-// Jacobi SVD.
-constexpr int64_t kSvdAutoJacobiN = 192;
-
 void prepare_truncation(const SiteLayout& ml, int dir, bool expand, const FusedBond& fp,
-                        const SiteLayout& pl, dmrg3s_svd_method svd, dmrg3s_precision prec,
-                        Trunc* t) {
+                        const SiteLayout& pl, dmrg3s_svd_method svd, Trunc* t) {
   const Bond& old = dir == 1 ? ml.right : ml.left;
   // Sector k of M~ is a rows x cols matrix X (rows: (s, a_l) for L->R, the
   // expanded left states for R->L).  It is gathered column-major in the tall
@@ -533,14 +528,12 @@ void prepare_truncation(const SiteLayout& ml, int dir, bool expand, const FusedB
   }
   t->foff = foff;
   t->soff = soff;
-  if (svd == DMRG3S_SVD_AUTO) {
-    // the Jacobi rounds win on large sectors of FP64 updates; after a 3xTF32
-    // or TF32 eigensolver the kept vector carries ~1e-7 noise, whose cluster of
-    // small singular values takes the Jacobi sweeps longer than gesvd
-    int64_t nmax = 0;
-    for (const Sector& sc : secs) nmax = std::max(nmax, sc.n);
-    svd = prec == DMRG3S_FP64 && nmax >= kSvdAutoJacobiN ? DMRG3S_SVD_JACOBI : DMRG3S_SVD_GESVD;
-  }
+  // AUTO: the Jacobi SVD, since its QR and left vectors run in this library's
+  // kernels.  Whole updates, gesvd against it (ms): XXZ FP64 m = 16 2.8 and 1.7, 128
+  // 7.9 and 5.7, 512 39.9 and 14.2, 1024 97 and 52; 3xTF32 m = 64 3.5 and 2.3, 512 37.8
+  // and 12.6; Hubbard FP64 m = 128 9.3 and 3.9, 1024 97 and 24.  Eight sweeps of the
+  // L = 40 chain at m = 128, 3xTF32 (whose noise costs Jacobi sweeps): 3.3 and 1.5 s.
+  if (svd == DMRG3S_SVD_AUTO) svd = DMRG3S_SVD_JACOBI;
   t->method = svd;
   bool any_proj = svd == DMRG3S_SVD_JACOBI;
   for (const Sector& sc : secs) any_proj = any_proj || (sc.vt_only && sc.base > 0);
@@ -887,7 +880,7 @@ dmrg3s_status local_update(State& S, int dir, double alpha, const Opts& o, Info*
   ph = phase(kProfSvd);
   // ---- 3. sectors of M~ = [M* P] (L->R) or [M*; P] (R->L), gathered
   Trunc t;
-  prepare_truncation(m.lay, dir, expand, fp, pl, o.svd, o.prec, &t);
+  prepare_truncation(m.lay, dir, expand, fp, pl, o.svd, &t);
   double* X;
   if ((s = scr.get(&X, t.xoff))) return s;
   cudaMemsetAsync(X, 0, (size_t)std::max<int64_t>(t.xoff, 1) * sizeof(double), st);
@@ -1142,12 +1135,10 @@ dmrg3s_status batch_truncate(Context* c, std::vector<BItem>& items, dmrg3s_svd_m
   int64_t nX = 0, nF = 0, nS = 0;
   size_t nsec = 0;
   bool any_proj = false;
-  dmrg3s_svd_method resolved = method == DMRG3S_SVD_AUTO ? DMRG3S_SVD_GESVD : method;
+  if (method == DMRG3S_SVD_AUTO) method = DMRG3S_SVD_JACOBI;   // (prepare_truncation)
   for (BItem& it : items) {
     State& S = *it.S;
-    prepare_truncation(S.M[S.centre].lay, it.dir, it.expand, it.fp, it.pl, method, it.o.prec,
-                       &it.t);
-    if (it.t.method == DMRG3S_SVD_JACOBI) resolved = DMRG3S_SVD_JACOBI;   // one call for all
+    prepare_truncation(S.M[S.centre].lay, it.dir, it.expand, it.fp, it.pl, method, &it.t);
     it.xb = nX;
     it.fb = nF;
     it.sb = nS;
@@ -1157,7 +1148,6 @@ dmrg3s_status batch_truncate(Context* c, std::vector<BItem>& items, dmrg3s_svd_m
     nsec += it.t.secs.size();
     any_proj = any_proj || it.t.any_proj;
   }
-  method = resolved;
   any_proj = any_proj || method == DMRG3S_SVD_JACOBI;
   Scratch scr(c, st);
   double *X, *F, *Sv, *dinfo_d, *X0 = nullptr;
