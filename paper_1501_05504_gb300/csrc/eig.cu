@@ -66,10 +66,10 @@ dmrg3s_status lanczos_batch(Context* c, const DevicePlan& heff, const double* Ld
   for (int i = 0; i < np; ++i) ranges[i] = {probs[i].off, probs[i].n};
   std::vector<LzChunk> hch;
   std::vector<LzChain> hcn;
-  // at most one chunk per SM where the sizes allow: few partials per problem to
-  // finish the sums from, and an iteration's orthogonalisation in one cooperative
-  // launch (the longest chunk is kLzChunkMax: 0.6 M elements in all)
-  lz_layout(ranges, std::max(1, plan_ctas() - np), &hch, &hcn);
+  // about one chunk per SM: few partials per problem to finish the sums from; with
+  // no more than that (always for one problem of up to 0.6 M elements) an
+  // iteration's orthogonalisation is one cooperative launch
+  lz_layout(ranges, plan_ctas(), &hch, &hcn);
   const int nchunks = (int)hch.size();
   const bool one_launch = nchunks <= plan_ctas();
   int maxlen = 0;
@@ -197,8 +197,9 @@ dmrg3s_status lanczos_batch(Context* c, const DevicePlan& heff, const double* Ld
   // (launch.hpp) keep the device busier than replays of a captured iteration, in
   // which the products cannot be chained (3387 us against 3505 for 40 iterations
   // of the m = 512 XXZ chain in 3xTF32; 72 us an iteration against 73 at m = 32,
-  // where the host's share is largest).  In all, with the tridiagonal solve beside
-  // the product: 4745 -> 3284 us (3xTF32) and 5288 -> 4371 us (FP64).
+  // where the host's share is largest).  In all, with the one-launch
+  // orthogonalisation and the tridiagonal solve beside the product: 4745 -> 3469 us
+  // (3xTF32) and 5288 -> 4590 us (FP64).
   auto orthogonalise = [&]() -> dmrg3s_status {
     if (one_launch) {
       if (!launch_lz_orth(V, ldv, kdev, w, vcur, dch, nchunks, maxlen, dcn, part, part2, kp, alpha,

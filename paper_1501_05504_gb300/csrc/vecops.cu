@@ -566,7 +566,6 @@ __global__ void lz_advance_kernel(int* kdev) {
 
 constexpr int kOrThreads = 512;
 constexpr int kOrWarps = kOrThreads / 32;
-constexpr int kOrSegs = 4;          // element ranges a chunk's dot products are split into
 
 // Barrier of all CTAs of a cooperative launch: `count` counts arrivals and is
 // never reset, `target` is its value once all have arrived.  Bounded: false (in
@@ -598,105 +597,128 @@ __device__ __forceinline__ bool grid_sync(unsigned* count, unsigned target, int*
   return *s_ok != 0;
 }
 
-// h[j] = the sum of partial[., j] over the chain's chunks, j < k1, in a fixed order: a
-// group of warps per eight columns, four chunks at a time side by side in a warp.
+// The kernel's sums have the order of the separate launches (warp_dot, chain_sum,
+// block_sum: the same partial sums in the same trees), so both forms give the
+// same bits: 3xTF32 products round their operands, and a last bit of v_k that
+// differs can come back as 1e-8 of the eigenvector.  Sums of several values share a
+// tree: the values' halves are exchanged first, which pairs the same lanes.
+__device__ __forceinline__ double warp_sum4(const double (&a)[4], int lane) {   // value lane / 8
+  const bool h16 = (lane & 16) != 0, h8 = (lane & 8) != 0;
+  const double b0 = (h16 ? a[2] : a[0]) + __shfl_xor_sync(0xffffffffu, h16 ? a[0] : a[2], 16);
+  const double b1 = (h16 ? a[3] : a[1]) + __shfl_xor_sync(0xffffffffu, h16 ? a[1] : a[3], 16);
+  double c = (h8 ? b1 : b0) + __shfl_xor_sync(0xffffffffu, h8 ? b0 : b1, 8);
+  for (int o = 4; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
+  return c;
+}
+
+// h[j] = the sum of partial[., j] over the chain's chunks, j < k1: four columns a
+// warp, all their loads in flight.
 __device__ __forceinline__ void chain_sums(const double* partial, int kp, const LzChain& cn, int k1,
-                                           double* red, double* h) {
+                                           double* h) {
   const int lane = threadIdx.x & 31, q = threadIdx.x >> 5;
-  const int nb = (k1 + 7) / 8;                       // column blocks: at most 17
-  const int ways = nb < kOrWarps ? kOrWarps / nb : 1;   // warps per block
-  for (int u = q; u < nb * ways; u += kOrWarps) {
-    const int jb = u % nb, way = u / nb;
-    const int j = jb * 8 + (lane & 7);
-    const int step = 4 * ways;
-    double a0 = 0.0, a1 = 0.0;
-    if (j < k1) {
-      const double* p = partial + (int64_t)cn.c0 * kp + j;
-      int b = way * 4 + (lane >> 3);
-      for (; b + 3 * step < cn.nc; b += 4 * step) {   // four loads in flight per lane
-        const double x0 = __ldcg(p + (int64_t)b * kp), x1 = __ldcg(p + (int64_t)(b + step) * kp);
-        const double x2 = __ldcg(p + (int64_t)(b + 2 * step) * kp);
-        const double x3 = __ldcg(p + (int64_t)(b + 3 * step) * kp);
-        a0 += x0;
-        a1 += x1;
-        a0 += x2;
-        a1 += x3;
-      }
-      for (; b < cn.nc; b += step) a0 += __ldcg(p + (int64_t)b * kp);
-    }
-    a0 += a1;
-    a0 += __shfl_xor_sync(0xffffffffu, a0, 8);
-    a0 += __shfl_xor_sync(0xffffffffu, a0, 16);
-    if (lane < 8) red[way * (kLzMaxK + 7) + jb * 8 + lane] = a0;
-  }
-  __syncthreads();
-  for (int j = threadIdx.x; j < k1; j += kOrThreads) {
-    double s = red[j];
-    for (int w = 1; w < ways; ++w) s += red[w * (kLzMaxK + 7) + j];
-    h[j] = s;
+  for (int g = q; 4 * g < k1; g += kOrWarps) {
+    const double* p = partial + (int64_t)cn.c0 * kp + 4 * g;
+    const int nj = min(4, k1 - 4 * g);
+    double a0[4] = {0.0, 0.0, 0.0, 0.0}, a1[4] = {0.0, 0.0, 0.0, 0.0};
+    int b = lane;
+#pragma unroll 3
+    for (; b + 32 < cn.nc; b += 64)
+#pragma unroll
+      for (int t = 0; t < 4; ++t)
+        if (t < nj) {
+          a0[t] += __ldcg(p + (int64_t)b * kp + t);
+          a1[t] += __ldcg(p + (int64_t)(b + 32) * kp + t);
+        }
+    if (b < cn.nc)
+#pragma unroll
+      for (int t = 0; t < 4; ++t)
+        if (t < nj) a0[t] += __ldcg(p + (int64_t)b * kp + t);
+#pragma unroll
+    for (int t = 0; t < 4; ++t) a0[t] += a1[t];
+    const double c = warp_sum4(a0, lane);
+    if ((lane & 7) == 0 && (lane >> 3) < nj) h[4 * g + (lane >> 3)] = c;
   }
   __syncthreads();
 }
 
-// partial_b[j] = <V_j, x> over the chunk, j < k1: a warp takes four vectors over one of
-// kOrSegs element ranges (four vectors share the reads of x and one reduction:
-// 22 FP64 instructions per 16 multiply-adds at four elements a lane).  Vectors below
-// `have` are read from Vs (stride lp); FILL stores the others there while they fit.
+// out[j] = <V_j, x> over the chunk, j < k1: two vectors a warp (they share the reads
+// of x and a tree), 16 loads in flight.  Vectors below vcap are read from Vs (stride
+// lp); FILL stores them there.
 template <bool FILL>
 __device__ __forceinline__ void chunk_dots(const double* V, int64_t ldv, double* Vs, int lp,
-                                           int vcap, const double* x, int len, int k1, double* red,
-                                           double* out) {
+                                           int vcap, const double* x, int len, int k1, double* out) {
   const int lane = threadIdx.x & 31, q = threadIdx.x >> 5;
-  const int ng = (k1 + 3) / 4;
-  const int seg = ((len + kOrSegs - 1) / kOrSegs + 31) & ~31;
-  for (int u = q; u < ng * kOrSegs; u += kOrWarps) {
-    const int g = u / kOrSegs, sg = u % kOrSegs;
-    const int i0 = sg * seg, i1 = min(len, i0 + seg);
-    const int nj = min(4, k1 - 4 * g);
-    double a[4] = {0.0, 0.0, 0.0, 0.0};
-    const double* src[4];
+  const int full = len / 128;          // blocks of 128 elements, four per lane
+  for (int g = q; 2 * g < k1; g += kOrWarps) {
+    const bool two = 2 * g + 1 < k1;
+    const double* src[2];
+    double* dst[2];
 #pragma unroll
-    for (int t = 0; t < 4; ++t) {
-      const int j = 4 * g + (t < nj ? t : 0);
+    for (int t = 0; t < 2; ++t) {
+      const int j = 2 * g + (two ? t : 0);
       src[t] = !FILL && j < vcap ? Vs + (int64_t)j * lp : V + (int64_t)j * ldv;
+      dst[t] = FILL && j < vcap ? Vs + (int64_t)j * lp : nullptr;
     }
-    for (int ib = i0; ib < i1; ib += 128) {        // 16 loads of V in flight per lane
-      double v[4][4];
+    double a[2][4];
+#pragma unroll
+    for (int t = 0; t < 2; ++t)
+#pragma unroll
+      for (int m = 0; m < 4; ++m) a[t][m] = 0.0;
+    for (int b0 = 0; b0 < full; b0 += 2) {
+      double v[2][2][4];
+#pragma unroll
+      for (int u = 0; u < 2; ++u)
+        if (b0 + u < full)
+#pragma unroll
+          for (int t = 0; t < 2; ++t)
+#pragma unroll
+            for (int m = 0; m < 4; ++m) v[u][t][m] = src[t][(b0 + u) * 128 + m * 32 + lane];
+#pragma unroll
+      for (int u = 0; u < 2; ++u)
+        if (b0 + u < full)
+#pragma unroll
+          for (int m = 0; m < 4; ++m) {
+            const int i = (b0 + u) * 128 + m * 32 + lane;
+            const double xi = x[i];
+#pragma unroll
+            for (int t = 0; t < 2; ++t) {
+              if (FILL && dst[t]) dst[t][i] = v[u][t][m];
+              a[t][m] = fma(v[u][t][m], xi, a[t][m]);
+            }
+          }
+    }
+    if (full * 128 < len) {
+      // the last elements: a lane with all four of them adds them to its four sums, a
+      // lane with fewer to its first
+      const int i = full * 128 + lane;
+      const bool all = i + 96 < len;
+      double v[2][4];
+#pragma unroll
+      for (int t = 0; t < 2; ++t)
+#pragma unroll
+        for (int m = 0; m < 4; ++m) v[t][m] = i + 32 * m < len ? src[t][i + 32 * m] : 0.0;
 #pragma unroll
       for (int m = 0; m < 4; ++m) {
-        const int i = ib + 32 * m + lane;
+        const bool in = i + 32 * m < len;
+        const double xi = in ? x[i + 32 * m] : 0.0;
 #pragma unroll
-        for (int t = 0; t < 4; ++t) v[m][t] = i < i1 ? src[t][i] : 0.0;
-      }
-#pragma unroll
-      for (int m = 0; m < 4; ++m) {
-        const int i = ib + 32 * m + lane;
-        if (ib + 32 * m >= i1) break;
-        const double xi = i < i1 ? x[i] : 0.0;
-#pragma unroll
-        for (int t = 0; t < 4; ++t) {
-          if (FILL && i < i1 && t < nj && 4 * g + t < vcap)
-            Vs[(int64_t)(4 * g + t) * lp + i] = v[m][t];
-          a[t] = fma(v[m][t], xi, a[t]);
+        for (int t = 0; t < 2; ++t) {
+          if (FILL && in && dst[t]) dst[t][i + 32 * m] = v[t][m];
+          const double s = fma(v[t][m], xi, m == 0 || !all ? a[t][0] : a[t][m]);
+          if (m == 0 || !all) {
+            if (in) a[t][0] = s;
+          } else {
+            a[t][m] = s;
+          }
         }
       }
     }
-    // the four sums over the lanes: halves exchanged twice, then a butterfly
-    const bool h16 = (lane & 16) != 0, h8 = (lane & 8) != 0;
-    double b0 = (h16 ? a[2] : a[0]) + __shfl_xor_sync(0xffffffffu, h16 ? a[0] : a[2], 16);
-    double b1 = (h16 ? a[3] : a[1]) + __shfl_xor_sync(0xffffffffu, h16 ? a[1] : a[3], 16);
-    double c = (h8 ? b1 : b0) + __shfl_xor_sync(0xffffffffu, h8 ? b0 : b1, 8);
-    for (int o = 4; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
-    if ((lane & 7) == 0) {
-      const int t = (h16 ? 2 : 0) + (h8 ? 1 : 0);
-      if (t < nj) red[sg * (kLzMaxK + 7) + 4 * g + t] = c;
-    }
-  }
-  __syncthreads();
-  for (int j = threadIdx.x; j < k1; j += kOrThreads) {
-    double s = red[j];
-    for (int w = 1; w < kOrSegs; ++w) s += red[w * (kLzMaxK + 7) + j];
-    out[j] = s;
+    const double s0 = (a[0][0] + a[0][1]) + (a[0][2] + a[0][3]);
+    const double s1 = (a[1][0] + a[1][1]) + (a[1][2] + a[1][3]);
+    const bool h16 = (lane & 16) != 0;
+    double c = (h16 ? s1 : s0) + __shfl_xor_sync(0xffffffffu, h16 ? s0 : s1, 16);
+    for (int o = 8; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
+    if ((lane & 15) == 0 && (lane == 0 || two)) out[2 * g + (lane >> 4)] = c;
   }
 }
 
@@ -707,16 +729,17 @@ __device__ __forceinline__ void chunk_dots(const double* V, int64_t ldv, double*
 // separated by device-wide barriers instead of launches.  Bound by the FP64
 // pipe: 4 k multiply-adds per element are 19 us at k = 37 for the 75 k elements
 // of an m = 512 XXZ tensor, beside three barriers and the sums over the chunks'
-// partials.  At k = 32 to 37 (cold caches) 52 us; as five launches (dots, update
-// and dots, update, next, advance) 107 us.
+// partials.  40 iterations with 3xTF32 products: 3.47 ms; as five launches an
+// iteration (dots, update and dots, update, next, advance: 107 us at k = 32 to 37, cold
+// caches) 4.75 ms.
 __global__ void __launch_bounds__(kOrThreads, 1) lz_orth_kernel(
     double* V, int64_t ldv, int* kdev, const double* w, double* vcur,
     const LzChunk* __restrict__ chunks, const LzChain* __restrict__ chains, double* part,
     double* part2, int kp, double* alpha, double* nrm, int64_t nrm_stride, int lp, int vcap,
     unsigned* count, int* err, uint64_t limit_ns) {
   extern __shared__ double osh[];
-  __shared__ double h[kLzMaxK + 7];
-  __shared__ double red[kOrWarps * (kLzMaxK + 7)];
+  __shared__ double h[kLzMaxK];
+  __shared__ double red[32];
   __shared__ double s_scale;
   __shared__ int s_ok;
   const int k = *kdev, k1 = k + 1;
@@ -730,15 +753,14 @@ __global__ void __launch_bounds__(kOrThreads, 1) lz_orth_kernel(
   const double* Vc = V + ch.e0;
   for (int i = threadIdx.x; i < len; i += kOrThreads) x[i] = w[ch.e0 + i];
   __syncthreads();
-  double nacc = 0.0;
   for (int pass = 0; pass < 2; ++pass) {
     double* pp = pass == 0 ? part : part2;
     if (pass == 0)
-      chunk_dots<true>(Vc, ldv, Vs, lp, vcap, x, len, k1, red, pp + (int64_t)blockIdx.x * kp);
+      chunk_dots<true>(Vc, ldv, Vs, lp, vcap, x, len, k1, pp + (int64_t)blockIdx.x * kp);
     else
-      chunk_dots<false>(Vc, ldv, Vs, lp, vcap, x, len, k1, red, pp + (int64_t)blockIdx.x * kp);
+      chunk_dots<false>(Vc, ldv, Vs, lp, vcap, x, len, k1, pp + (int64_t)blockIdx.x * kp);
     if (!grid_sync(count, base + (unsigned)(pass + 1) * G, err, limit_ns, &s_ok)) return;
-    chain_sums(pp, kp, cn, k1, red, h);
+    chain_sums(pp, kp, cn, k1, h);
     if (pass == 0 && threadIdx.x == 0 && (int)blockIdx.x == cn.c0)
       alpha[(int64_t)ch.chain * kp + k] = h[k];
     for (int i = threadIdx.x; i < len; i += kOrThreads) {
@@ -749,18 +771,18 @@ __global__ void __launch_bounds__(kOrThreads, 1) lz_orth_kernel(
 #pragma unroll 4
       for (; j < k1; ++j) acc = fma(-h[j], Vc[(int64_t)j * ldv + i], acc);
       x[i] = acc;
-      if (pass == 1) nacc = fma(acc, acc, nacc);
     }
     __syncthreads();
   }
   double* np = nrm + (int64_t)(k % kLzLag) * nrm_stride;
-  nacc = block_sum(nacc, red);
+  double nacc = 0.0;
+  if (threadIdx.x < kLzThreads)
+    for (int i = threadIdx.x; i < len; i += kLzThreads) nacc = fma(x[i], x[i], nacc);
+  nacc = block_sum(nacc, red);         // (the upper half's zeros change nothing)
   if (threadIdx.x == 0) np[blockIdx.x] = nacc;
   if (!grid_sync(count, base + 3u * G, err, limit_ns, &s_ok)) return;
   if (threadIdx.x < 32) {
-    double a = 0.0;
-    for (int b = threadIdx.x; b < cn.nc; b += 32) a += __ldcg(np + cn.c0 + b);
-    a = warp_sum(a);
+    const double a = chain_sum(np, 1, cn.c0, cn.nc, 0, threadIdx.x);
     if (threadIdx.x == 0) s_scale = (a > 0.0 && a < 1e308) ? 1.0 / sqrt(a) : 0.0;
   }
   __syncthreads();
