@@ -165,7 +165,8 @@ __device__ __forceinline__ double chain_sum4(double v, double* red) {
 
 // By the chain's threads: the reflector of column a (rows j .. m - 1, in shared
 // memory) into v (v[j] = 1) and, with beta on the diagonal, into the matrix; tau
-// into *tau and red[6].
+// into *tau and red[6 + (j & 1)] (a CTA of a matrix of its own forms reflector j + 1
+// while its other warps still read tau_j).
 __device__ __forceinline__ void qr_reflector(double* a, double* v, int j, int m, double* T,
                                              double* tau, double* red) {
   double s = 0.0;
@@ -194,7 +195,7 @@ __device__ __forceinline__ void qr_reflector(double* a, double* v, int j, int m,
   }
   if (threadIdx.x == 0) {
     *tau = tv;
-    red[6] = tv;
+    red[6 + (j & 1)] = tv;
   }
 }
 
@@ -202,7 +203,7 @@ __global__ void __launch_bounds__(kQrThreads, 1)
 qr_kernel(const QrItem* __restrict__ items, const int* __restrict__ cta_item, double* A, double* tau,
           int* ready, int* err, uint64_t limit_ns) {
   extern __shared__ double sh[];
-  __shared__ double red[8];              // two sums' partials, tau
+  __shared__ double red[8];              // a sum's partials, two taus
   __shared__ double part[kQrUnits * kQrWarps];
   __shared__ int s_ok;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -231,7 +232,7 @@ qr_kernel(const QrItem* __restrict__ items, const int* __restrict__ cta_item, do
           qr_reflector(cols + (int64_t)(j / G) * m, v, j, m, T + (int64_t)j * m,
                        tau + Q.offTau + j, red);
         __syncthreads();
-        tv = red[6];
+        tv = red[6 + (j & 1)];
         if (G > 1 && tid == 0) {
           __threadfence();
           asm volatile("st.release.gpu.global.s32 [%0], %1;" ::"l"(ready + Q.job), "r"(j + 1) : "memory");
@@ -276,7 +277,7 @@ qr_kernel(const QrItem* __restrict__ items, const int* __restrict__ cta_item, do
                        tau + Q.offTau + j + 1, red);
         }
         __syncthreads();
-        t_next = red[6];
+        t_next = red[6 + ((j + 1) & 1)];
         if (G > 1 && tid == 0) {
           __threadfence();
           asm volatile("st.release.gpu.global.s32 [%0], %1;" ::"l"(ready + Q.job), "r"(j + 2) : "memory");
