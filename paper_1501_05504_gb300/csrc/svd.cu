@@ -163,6 +163,13 @@ __device__ __forceinline__ double chain_sum4(double v, double* red) {
   return (red[0] + red[1]) + (red[2] + red[3]);
 }
 
+__device__ __forceinline__ double chain_max4(double v, double* red) {
+  for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+  chain_sync();
+  return fmax(fmax(red[0], red[1]), fmax(red[2], red[3]));
+}
+
 // By the chain's threads: the reflector of column a (rows j .. m - 1, in shared
 // memory) into v (v[j] = 1) and, with beta on the diagonal, into the matrix; tau
 // into *tau and red[6 + (j & 1)] (a CTA of a matrix of its own forms reflector j + 1
@@ -174,18 +181,37 @@ __device__ __forceinline__ void qr_reflector(double* a, double* v, int j, int m,
   s = chain_sum4(s, red);
   const double alpha = a[j];
   double beta = alpha, tv = 0.0, sc = 0.0;
-  if (s != 0.0) {                       // (NaN: every result is NaN)
-    const double n2 = fma(alpha, alpha, s);
-    if (n2 > 1e-290 && n2 < 1e290) {
+  const double n2 = fma(alpha, alpha, s);
+  if (n2 > 1e-290 && n2 < 1e290) {
+    if (s != 0.0) {
       const double nr = sqrt_of(n2);
       beta = alpha >= 0.0 ? -nr : nr;
       sc = recip(alpha - beta);         // |alpha - beta| >= |beta|
       tv = (beta - alpha) * recip(beta);
-    } else {
-      const double nr = sqrt(n2);
-      beta = alpha >= 0.0 ? -nr : nr;
-      sc = 1.0 / (alpha - beta);
-      tv = (beta - alpha) / beta;
+    }
+  } else {
+    // squares outside the FP64 range (a norm with few digits would give a reflection
+    // that is not orthogonal): the column scaled by a power of two of its largest
+    // element (Inf and NaN pass through)
+    double mx = 0.0;
+    for (int i = j + threadIdx.x; i < m; i += kQrChain) mx = fmax(mx, fabs(a[i]));
+    chain_sync();
+    mx = chain_max4(mx, red);
+    if (!(n2 == n2)) mx = n2;
+    if (mx != 0.0) {
+      const double up = inverse_scale(mx);
+      for (int i = j + threadIdx.x; i < m; i += kQrChain) a[i] *= up;
+      chain_sync();
+      double s1 = 0.0;
+      for (int i = j + 1 + threadIdx.x; i < m; i += kQrChain) s1 = fma(a[i], a[i], s1);
+      s1 = chain_sum4(s1, red);
+      if (s1 != 0.0) {                  // (NaN: every result is NaN)
+        const double al = up * alpha, nr = sqrt(fma(al, al, s1));
+        const double b = al >= 0.0 ? -nr : nr;
+        beta = b / up;
+        sc = 1.0 / (al - b);
+        tv = (b - al) / b;
+      }
     }
   }
   for (int i = j + threadIdx.x; i < m; i += kQrChain) {
