@@ -372,6 +372,7 @@ struct QrColumns {
 };
 constexpr int kQrApplyWarps = 4;
 constexpr int kQrApplyRows = 6400;
+constexpr size_t kQrApplySmem = sizeof(double) * kQrApplyWarps * kQrApplyRows;
 __global__ void __launch_bounds__(32 * kQrApplyWarps)
 qr_apply_kernel(const JacJob* __restrict__ jobs, const QrColumns* __restrict__ items, const double* A,
                 const double* tau, double* U, int stride) {
@@ -1193,8 +1194,10 @@ dmrg3s_status svd_jacobi(Context* c, std::vector<SvdLane>& lanes, int nlanes,
   if (!s && !qcols.empty()) {
     const int stride = std::min(umax, kQrApplyRows);
     const size_t bytes = (size_t)kQrApplyWarps * stride * sizeof(double);
+    // (the limit belongs to the kernel, not to the call: always the same value, or
+    // another thread's smaller one could come between it and the launch)
     if (!(s = cuda_ok(c, cudaFuncSetAttribute(qr_apply_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                              (int)bytes), "left vectors")))
+                                              (int)kQrApplySmem), "left vectors")))
       launch_chain(qr_apply_kernel, (int)qcols.size(), 32 * kQrApplyWarps, bytes, st, dt, d_qcols, T, tau, U,
                    stride);
     count_launch();
