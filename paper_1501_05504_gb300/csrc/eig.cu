@@ -71,7 +71,7 @@ dmrg3s_status lanczos_batch(Context* c, const DevicePlan& heff, const double* Ld
   // iteration's orthogonalisation is one cooperative launch
   lz_layout(ranges, plan_ctas(), &hch, &hcn);
   const int nchunks = (int)hch.size();
-  const bool one_launch = nchunks <= plan_ctas();
+  bool one_launch = nchunks <= plan_ctas();
   int maxlen = 0;
   for (const LzChunk& ch : hch) maxlen = std::max(maxlen, (int)(ch.e1 - ch.e0));
   // FP64 products in the sliced form when the Krylov basis fits behind its
@@ -200,19 +200,20 @@ dmrg3s_status lanczos_batch(Context* c, const DevicePlan& heff, const double* Ld
   // where the host's share is largest).  In all, with the one-launch
   // orthogonalisation and the tridiagonal solve beside the product: 4745 -> 3469 us
   // (3xTF32) and 5288 -> 4590 us (FP64).
-  auto orthogonalise = [&]() -> dmrg3s_status {
+  // A stream with fewer SMs than chunks (of a green context, say) refuses the
+  // cooperative launch: then the separate launches, which add in the same order.
+  auto orthogonalise = [&]() {
     if (one_launch) {
-      if (!launch_lz_orth(V, ldv, kdev, w, vcur, dch, nchunks, maxlen, dcn, part, part2, kp, alpha,
-                          nrm, nchunks, arrivals, c->d_err, c->wait_ns, st))
-        return fail(c, DMRG3S_ERR_CUDA, "Lanczos orthogonalisation launch");
-    } else {
-      launch_lz_dots(V, ldv, 0, w, dch, nchunks, part, kp, st, kdev);
-      launch_lz_update_dots(V, ldv, 0, w, dch, nchunks, dcn, part, kp, alpha, part2, st, kdev);
-      launch_lz_update(V, ldv, 0, w, dch, nchunks, dcn, part2, kp, nullptr, nrm, st, kdev, nchunks);
-      launch_lz_next(w, V, ldv, kdev, vcur, dch, nchunks, dcn, nrm, nchunks, st);
-      launch_lz_advance(kdev, st);
+      one_launch = launch_lz_orth(V, ldv, kdev, w, vcur, dch, nchunks, maxlen, dcn, part, part2, kp,
+                                  alpha, nrm, nchunks, arrivals, c->d_err, c->wait_ns, st);
+      if (one_launch) return;
+      cudaGetLastError();
     }
-    return DMRG3S_OK;
+    launch_lz_dots(V, ldv, 0, w, dch, nchunks, part, kp, st, kdev);
+    launch_lz_update_dots(V, ldv, 0, w, dch, nchunks, dcn, part, kp, alpha, part2, st, kdev);
+    launch_lz_update(V, ldv, 0, w, dch, nchunks, dcn, part2, kp, nullptr, nrm, st, kdev, nchunks);
+    launch_lz_next(w, V, ldv, kdev, vcur, dch, nchunks, dcn, nrm, nchunks, st);
+    launch_lz_advance(kdev, st);
   };
   if ((s = product(0))) return bail(s);
   // the host's reading of iteration k
@@ -251,7 +252,7 @@ dmrg3s_status lanczos_batch(Context* c, const DevicePlan& heff, const double* Ld
   int last = -1;   // the last iteration enqueued
   int next_read = 0;
   for (int k = 0; k < kmax; ++k) {
-    if ((s = orthogonalise())) return bail(s);
+    orthogonalise();
     cudaEventRecord(c->ev_ready, st);
     cudaStreamWaitEvent(c->aux, c->ev_ready, 0);
     launch_lz_tridiag(dcn, np, alpha, beta, kp, k, nrm + (int64_t)(k % kLzLag) * nchunks, y, out,

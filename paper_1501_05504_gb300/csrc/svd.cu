@@ -1017,8 +1017,31 @@ dmrg3s_status svd_jacobi(Context* c, std::vector<SvdLane>& lanes, int nlanes,
       s = cuda_ok(c, cudaGetLastError(), "column order");
     }
   }
-  // ---- lanes for the matrices whose QR is too large for qr_kernel, by its cost m n^2,
-  // largest first; created when first used
+  // ---- 1. A = Q R: qr_kernel, and cuSOLVER for the matrices too large for it.  A
+  // stream with fewer SMs than the plan's CTAs (of a green context, say) refuses the
+  // cooperative launch: then cuSOLVER factorises every matrix.
+  if (!s && !qr.items.empty()) {
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeCooperative;
+    at.val.cooperative = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = (unsigned)qr.cta_item.size() - 1;
+    cfg.blockDim = kQrThreads;
+    cfg.dynamicSmemBytes = qr.smem;
+    cfg.stream = st;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    if (cudaLaunchKernelEx(&cfg, qr_kernel, (const QrItem*)dq, (const int*)qr_cta, T, tau, qr_ready, qr_err,
+                           c->wait_ns) == cudaSuccess) {
+      count_launch();
+    } else {
+      cudaGetLastError();
+      by_lib.resize(nj);
+      for (int k = 0; k < nj; ++k) by_lib[k] = k;
+    }
+  }
+  // ---- lanes for cuSOLVER's matrices, by the cost m n^2, largest first; created when
+  // first used
   std::vector<int> order(by_lib);
   std::sort(order.begin(), order.end(), [&](int a, int b) {
     return (double)tab[a].m * tab[a].n * tab[a].n > (double)tab[b].m * tab[b].n * tab[b].n;
@@ -1061,22 +1084,6 @@ dmrg3s_status svd_jacobi(Context* c, std::vector<SvdLane>& lanes, int nlanes,
   cudaEvent_t ev_in = nullptr;
   if (!s && cudaEventCreateWithFlags(&ev_in, cudaEventDisableTiming) != cudaSuccess)
     s = fail(c, DMRG3S_ERR_CUDA, "SVD event");
-  // ---- 1. A = Q R
-  if (!s && !qr.items.empty()) {
-    cudaLaunchAttribute at{};
-    at.id = cudaLaunchAttributeCooperative;
-    at.val.cooperative = 1;
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = (unsigned)qr.cta_item.size() - 1;
-    cfg.blockDim = kQrThreads;
-    cfg.dynamicSmemBytes = qr.smem;
-    cfg.stream = st;
-    cfg.attrs = &at;
-    cfg.numAttrs = 1;
-    s = cuda_ok(c, cudaLaunchKernelEx(&cfg, qr_kernel, (const QrItem*)dq, (const int*)qr_cta, T, tau,
-                                      qr_ready, qr_err, c->wait_ns), "QR factorisation");
-    count_launch();
-  }
   if (!s && nlanes > 0) {
     // on the lanes after the work queued on st, which waits for them
     cudaEventRecord(ev_in, st);

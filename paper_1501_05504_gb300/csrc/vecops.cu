@@ -915,10 +915,11 @@ bool launch_lz_orth(double* V, int64_t ldv, int* kdev, const double* w, double* 
   cfg.stream = st;
   cfg.attrs = &at;
   cfg.numAttrs = 1;
+  if (cudaLaunchKernelEx(&cfg, lz_orth_kernel, V, ldv, kdev, w, vcur, chunks, chains, part, part2, kp,
+                         alpha, nrm, nrm_stride, lp, vcap, count, err, limit_ns) != cudaSuccess)
+    return false;
   count_launch();
-  return cudaLaunchKernelEx(&cfg, lz_orth_kernel, V, ldv, kdev, w, vcur, chunks, chains, part,
-                            part2, kp, alpha, nrm, nrm_stride, lp, vcap, count, err,
-                            limit_ns) == cudaSuccess;
+  return true;
 }
 
 void launch_lz_tridiag(const LzChain* chains, int nchains, const double* alpha, double* beta,
