@@ -71,10 +71,15 @@ typedef enum dmrg3s_status {
  * (FP32 pair) results, which the MPO combination (stage 2) and the split-K
  * sum combine in double-float arithmetic (~48 bits). */
 typedef enum dmrg3s_precision {
-  DMRG3S_FP64 = 0,    /* double precision: contractions of 16 Mflop and more whose
-                         intermediates fit the workspace as exact FP16 slices on
-                         tcgen05 tensor cores (62-bit fixed-point rows, sums exact to
-                         the last digit kept, rounded once), others on the CUDA cores */
+  DMRG3S_FP64 = 0,    /* double precision.  Every element of a sum of n terms keeps the
+                         componentwise bound of FP64 arithmetic, n 2^-53 of the sum
+                         of the terms' magnitudes, however graded the tensors.  Large
+                         contractions (11 Mflop that fill 128 x 16 tiles) whose
+                         intermediates fit the workspace run as exact FP16 slices on
+                         tcgen05 tensor cores (71-bit fixed-point rows, sums exact to the
+                         last digit kept, rounded once; elements that this holds with
+                         fewer digits than FP64 are formed from the FP64 operands),
+                         others on the CUDA cores                                    */
   DMRG3S_TF32X3 = 1,  /* 3xTF32 split products on tcgen05 tensor cores, FP32 accum.  */
   DMRG3S_TF32 = 2     /* single-pass TF32 on tcgen05 tensor cores, FP32 accumulate   */
 } dmrg3s_precision;
@@ -254,11 +259,11 @@ dmrg3s_status dmrg3s_apply_heff(dmrg3s_ctx ctx, const dmrg3s_env* L, const dmrg3
  * as in the Lanczos iteration of Sec. V step 1 (H_eff = L_{i-1} W_i . R_{i+1}
  * of Eq. es-iter, contracted as dmrg3s_apply_heff does).  dmrg3s_heff_create
  * plans the contraction for the structures of L, W, R and A (A->data is not
- * read) and, in the tensor-core modes and in the sliced form of DMRG3S_FP64, packs
- * L and R once into device memory owned by the handle (on `stream`); dmrg3s_heff_apply then computes
+ * read) and, in the tensor-core modes, packs L and R once into device memory
+ * owned by the handle (on `stream`); dmrg3s_heff_apply then computes
  * HA = H_eff A for a vector A (device, canonical layout of A's structure, and
  * HA likewise; both caller-owned) on `stream`, using the context's workspace.
- * In DMRG3S_FP64 the handle may read L->data and R->data at every application:
+ * In DMRG3S_FP64 the handle reads L->data and R->data at every application:
  * they must stay allocated and unchanged while the handle is used.  The
  * handle must not outlive its context; one host thread at a time.
  * Errors: as dmrg3s_apply_heff. */

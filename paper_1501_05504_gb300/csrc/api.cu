@@ -48,7 +48,7 @@ DeviceGradPlan::~DeviceGradPlan() {
 
 SlTables sliced_tables(const DeviceSliced& d, const SlStage& s) {
   return SlTables{d.units,    d.chunks, d.words, d.cta_unit, d.cta_chunk, d.segs,
-                  s.cta_unit.empty() ? 0 : (int)s.cta_unit.size() - 1,
+                  s.cta_unit.empty() ? 0 : (int)s.cta_unit.size() - 1, (int)s.units.size(),
                   s.chunks.size() <= (size_t)kChainChunks * s.cta_unit.size()};
 }
 
@@ -96,7 +96,8 @@ dmrg3s_status upload_plan(Plan&& host, std::unique_ptr<DevicePlan>* out) {
                  bytes_of(h.g12.tc.cta_start);
   total += bytes_of(h.s12) + bytes_of(h.s3);
   total += bytes_of(h.slices.groups) + bytes_of(h.slices.members) +
-           bytes_of(h.slices.cta_group) + bytes_of(h.t2) + bytes_of(h.t2_first);
+           bytes_of(h.slices.cta_group) + bytes_of(h.grades) + bytes_of(h.views) + bytes_of(h.t2) +
+           bytes_of(h.t2_first);
   total += bytes_of(h.s3r.chunks) + bytes_of(h.s3r.tasks) + bytes_of(h.s3r.terms);
   if (total == 0) total = 256;
   if (cudaMalloc(&dp->mem, total) != cudaSuccess) return DMRG3S_ERR_CUDA;
@@ -138,6 +139,8 @@ dmrg3s_status upload_plan(Plan&& host, std::unique_ptr<DevicePlan>* out) {
   dp->sl_groups = place(base, &off, h.slices.groups, &staging);
   dp->sl_members = place(base, &off, h.slices.members, &staging);
   dp->sl_cta_group = place(base, &off, h.slices.cta_group, &staging);
+  dp->grades = place(base, &off, h.grades, &staging);
+  dp->views = place(base, &off, h.views, &staging);
   dp->t2 = place(base, &off, h.t2, &staging);
   dp->t2_first = place(base, &off, h.t2_first, &staging);
   dp->s3r_chunks = place(base, &off, h.s3r.chunks, &staging);
@@ -168,39 +171,43 @@ dmrg3s_status run_sliced(Context* c, const DevicePlan& p, const double* g1A, con
   int32_t* e1B = e1A + h.s12.neA;
   int32_t* e3A = e1B + h.s12.neB;
   int32_t* e3B = e3A + h.s3.neA;
+  int32_t* d = e3B + h.s3.neB;
+  int32_t* fix = d + h.ngrade;
+  const size_t fix_units = std::max(h.s12.units.size(), h.s3.units.size());
   const bool left = h.kind == Kind::Heff || h.kind == Kind::ExpandLR || h.kind == Kind::EnvLR;
   double* t2 = h.has_g3 ? base + sl.t2 : out2;
   const bool t2_is_a = h.kind == Kind::Heff;
   SlOperands ops{};
-  ops.op[0] = left ? SlOperand{g1A, pk(sl.a1), e1A, scale} : SlOperand{g1B, pk(sl.b1), e1B, scale};
-  ops.op[1] = t2_is_a ? SlOperand{g3B, pk(sl.b3), e3B, 1.0} : SlOperand{g3A, pk(sl.a3), e3A, 1.0};
-  ops.op[2] = left ? SlOperand{g1B, pk(sl.b1), e1B, 1.0} : SlOperand{g1A, pk(sl.a1), e1A, 1.0};
+  ops.op[1] = left ? SlOperand{g1A, pk(sl.a1), e1A, scale, d, 1} : SlOperand{g1B, pk(sl.b1), e1B, scale, d, 1};
+  ops.op[0] = t2_is_a ? SlOperand{g3B, pk(sl.b3), e3B, 1.0, d, 1}
+                      : SlOperand{g3A, pk(sl.a3), e3A, 1.0, nullptr, 0};
+  ops.op[2] = left ? SlOperand{g1B, pk(sl.b1), e1B, 1.0, d, -1} : SlOperand{g1A, pk(sl.a1), e1A, 1.0, d, -1};
   int32_t* et2 = t2_is_a ? e3A : e3B;        // row scales of T2, collected by stage 2
   if (h.has_g3) {
     ops.clear = et2;
     ops.nclear = t2_is_a ? h.s3.neA : h.s3.neB;
   }
-  // (a caller that has sliced the environments does so for both)
-  slice_operands(p, hn.sliced_env ? 2 : 0, 2, ops, st);
+  ops.fix = fix;
+  ops.nfix = 2;
+  launch_grade(p.grades, (int)h.grades.size(), p.views, left ? g1B : g1A, d, st);
+  launch_slice(p.sl_groups, p.sl_cta_group, h.slices.cta.back(), p.sl_members, ops, st);
   if (!h.s12.units.empty()) {
     const int id = pr.on ? pr.begin(kProfGemm, h.f12.flops, h.f12.bytes, st) : -1;
-    launch_gemm_sliced(sliced_tables(p.s12, h.s12), hn.s1A ? hn.s1A : pk(sl.a1), pk(sl.b1),
-                       hn.s1A ? hn.e1A : e1A, e1B, source(h.f12, g1A, g1B, scale), t2, et2,
-                       h.kind == Kind::EnvLR, c->d_err, c->wait_ns, st);
+    launch_gemm_sliced(sliced_tables(p.s12, h.s12), pk(sl.a1), pk(sl.b1), e1A, e1B, source(h.f12, g1A, g1B, scale), t2, et2,
+                       h.kind == Kind::EnvLR, d, sl_fix(fix, 0, 2, fix_units), c->d_err, c->wait_ns, st);
     if (id >= 0) pr.end(id, st);
   }
   if (h.has_g3) {
     const double* a3 = t2_is_a ? t2 : g3A;
     const double* b3 = t2_is_a ? g3B : t2;
     launch_slice_known(p.t2, (int)h.t2.size(), p.t2_first, h.t2_tiles, t2, pk(t2_is_a ? sl.a3 : sl.b3),
-                       et2, st);
+                       et2, d, st);
     const bool split = !h.s3r.chunks.empty();
     double* c3 = split ? base + sl.p3 : g3C;
     if (!h.s3.units.empty()) {
       const int id = pr.on ? pr.begin(kProfGemm, h.g3.flops, h.g3.bytes, st) : -1;
-      launch_gemm_sliced(sliced_tables(p.s3, h.s3), pk(sl.a3), hn.s3B ? hn.s3B : pk(sl.b3), e3A,
-                         hn.s3B ? hn.e3B : e3B, source(h.f3, a3, b3, 1.0), c3, nullptr, false,
-                         c->d_err, c->wait_ns, st);
+      launch_gemm_sliced(sliced_tables(p.s3, h.s3), pk(sl.a3), pk(sl.b3), e3A, e3B, source(h.f3, a3, b3, 1.0), c3, nullptr, false, d,
+                         sl_fix(fix, 1, 2, fix_units), c->d_err, c->wait_ns, st);
       if (id >= 0) pr.end(id, st);
     }
     if (split) {

@@ -3,6 +3,7 @@
 
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstdint>
 #include <cstring>
 #include <memory>
@@ -85,6 +86,8 @@ struct DevicePlan {
   SlGroup* sl_groups = nullptr;
   SlMember* sl_members = nullptr;
   int32_t* sl_cta_group = nullptr;
+  SlGrade* grades = nullptr;
+  SlView* views = nullptr;
   SlPiece* t2 = nullptr;
   int32_t* t2_first = nullptr;
   CombChunk* s3r_chunks = nullptr;
@@ -351,12 +354,8 @@ struct SplitHints {
   // workspace (a prepared operator); when set they replace those slots
   const float *g1A_hi = nullptr, *g1A_lo = nullptr, *g3B_hi = nullptr, *g3B_lo = nullptr;
   // FP64: which form runs (kF64Auto: sliced when the plan has it and its
-  // intermediates fit the workspace), and, H_eff only, sliced L and R held
-  // outside the workspace with their row scales
+  // intermediates fit the workspace)
   int f64 = 0;
-  bool sliced_env = false;   // L and R are sliced already (in the workspace slots or below)
-  const uint16_t *s1A = nullptr, *s3B = nullptr;
-  const int32_t *e1A = nullptr, *e3B = nullptr;
 };
 constexpr int kF64Auto = 0, kF64Plain = 1, kF64Sliced = 2;
 struct TcSlots {
@@ -377,11 +376,17 @@ inline TcSlots tc_slots(const Plan& p) {
   return s;
 }
 // Sliced FP64 mode:
-//   [T2][s12 A][s12 B][s3 A][s3 B][row scales: s12 A, s12 B, s3 A, s3 B][stage-3 partials]
+//   [T2][s12 A][s12 B][s3 A][s3 B][row scales: s12 A, s12 B, s3 A, s3 B; grading;
+//   counters, list and masks of listed elements][stage-3 partials]
 // (offsets in doubles, 1 KB aligned; without stage 3 the output is not here).
 struct SlSlots {
   int64_t t2, a1, b1, a3, b3, e, p3, end;
 };
+// The list of listed elements from `at` on (counter i of the launch's `n`).
+inline SlFix sl_fix(int32_t* at, int i, int n, size_t units) {
+  int32_t* list = at + n;
+  return SlFix{at + i, list, reinterpret_cast<uint32_t*>(list + kSlParts * units)};
+}
 inline SlSlots sl_slots(const Plan& p) {
   SlSlots s;
   s.t2 = 0;
@@ -390,17 +395,11 @@ inline SlSlots sl_slots(const Plan& p) {
   s.a3 = s.b1 + slot_round((p.s12.nB + 3) / 4);
   s.b3 = s.a3 + slot_round((p.s3.nA + 3) / 4);
   s.e = s.b3 + slot_round((p.s3.nB + 3) / 4);
-  s.p3 = s.e + slot_round(((int64_t)p.s12.neA + p.s12.neB + p.s3.neA + p.s3.neB + 1) / 2);
+  const int64_t parts = kSlParts * (int64_t)std::max(p.s12.units.size(), p.s3.units.size());
+  s.p3 = s.e + slot_round(((int64_t)p.s12.neA + p.s12.neB + p.s3.neA + p.s3.neB + p.ngrade + 2 +
+                           kSlFixInts * parts + 1) / 2);
   s.end = s.p3 + slot_round(p.ws3s);
   return s;
-}
-// Slices operands [first, last] of a plan (Plan::slices); ops[i] describes
-// operand i.
-inline void slice_operands(const DevicePlan& p, int first, int last, const SlOperands& ops,
-                           cudaStream_t st) {
-  const SliceTable& t = p.host.slices;
-  launch_slice(p.sl_groups, p.sl_cta_group, t.cta[first], t.cta[last + 1] - t.cta[first],
-               p.sl_members, ops, st);
 }
 inline bool sliced_fits(const Plan& p, size_t ws_bytes) {
   return p.sliced && (size_t)sl_slots(p).end * sizeof(double) <= ws_bytes;
@@ -411,8 +410,8 @@ inline int64_t plan_ws_doubles(const Plan& p, dmrg3s_precision prec) {
   return prec == DMRG3S_FP64 ? p.ws1 + p.ws2 : tc_slots(p).end;
 }
 
-// `prec` selects the grouped-GEMM kernel of stages 1 and 3 (the combination
-// of stage 2 is always FP64).
+// `prec` selects the form: plain or sliced FP64 (the sliced one forms stage 2 within
+// stage 1's products), or the tensor-core one.
 dmrg3s_status run_plan(Context* c, const DevicePlan& p, const double* g1A, const double* g1B,
                        double* ws1, double* c2out, double c2scale, const double* g3A,
                        const double* g3B, double* g3C, cudaStream_t st,

@@ -131,17 +131,6 @@ dmrg3s_status lanczos_batch(Context* c, const DevicePlan& heff, const double* Ld
   double* ws1 = reinterpret_cast<double*>(c->ws);
   double* ws2 = ws1 + heff.host.ws1;
   // tensor-core products: pack the environments once for the whole run
-  if (hints.f64 == kF64Sliced) {
-    const Plan& hp = heff.host;
-    const SlSlots sl = sl_slots(hp);
-    int32_t* e = reinterpret_cast<int32_t*>(ws1 + sl.e);
-    SlOperands ops{};
-    ops.op[0] = SlOperand{Ldata, reinterpret_cast<uint16_t*>(ws1 + sl.a1), e, 1.0};
-    ops.op[1] = SlOperand{Rdata, reinterpret_cast<uint16_t*>(ws1 + sl.b3),
-                          e + hp.s12.neA + hp.s12.neB + hp.s3.neA, 1.0};
-    slice_operands(heff, 0, 1, ops, st);
-    hints.sliced_env = true;
-  }
   if (prec != DMRG3S_FP64) {
     const Plan& hp = heff.host;
     const TcSlots sl = tc_slots(hp);

@@ -32,21 +32,24 @@ dmrg3s_status run_mpo_grad(Context* c, const DeviceGradPlan& dp, const double* L
   Profiler& pr = c->prof;
   const int64_t a = slot_round(w1 + wy), b = a + slot_round((p.s.nA + 3) / 4),
                 e = b + slot_round((p.s.nB + 3) / 4),
-                end = e + slot_round(((int64_t)p.s.neA + p.s.neB + 1) / 2);
+                parts = kSlParts * (int64_t)p.s.units.size(),
+                end = e + slot_round(((int64_t)p.s.neA + p.s.neB + 1 + kSlFixInts * parts + 1) / 2);
   if (p.sliced && (size_t)end * sizeof(double) <= c->ws_bytes) {
     uint16_t* pA = reinterpret_cast<uint16_t*>(ws1 + a);
     uint16_t* pB = reinterpret_cast<uint16_t*>(ws1 + b);
     int32_t* eA = reinterpret_cast<int32_t*>(ws1 + e);
     int32_t* eB = eA + p.s.neA;
     SlOperands ops{};
-    ops.op[0] = SlOperand{L, pA, eA, 1.0};
-    ops.op[1] = SlOperand{M, pA, eA, 1.0};
-    ops.op[2] = SlOperand{M, pB, eB, 1.0};
-    ops.op[3] = SlOperand{R, pB, eB, 1.0};
-    launch_slice(dp.sl_groups, dp.sl_cta_group, 0, p.slices.cta.back(), dp.sl_members, ops, st);
+    ops.op[0] = SlOperand{L, pA, eA, 1.0, nullptr, 0};
+    ops.op[1] = SlOperand{M, pA, eA, 1.0, nullptr, 0};
+    ops.op[2] = SlOperand{M, pB, eB, 1.0, nullptr, 0};
+    ops.op[3] = SlOperand{R, pB, eB, 1.0, nullptr, 0};
+    ops.fix = eB + p.s.neB;
+    ops.nfix = 1;
+    launch_slice(dp.sl_groups, dp.sl_cta_group, p.slices.cta.back(), dp.sl_members, ops, st);
     const int id = pr.on ? pr.begin(kProfAuxGemm, p.g1.flops + p.gy.flops, p.g1.bytes + p.gy.bytes, st) : -1;
     launch_gemm_sliced(sliced_tables(dp.s, p.s), pA, pB, eA, eB, SlSource{L, M, M, R, 0, 0, 1.0}, ws1,
-                       nullptr, false, c->d_err, c->wait_ns, st);
+                       nullptr, false, nullptr, sl_fix(ops.fix, 0, 1, p.s.units.size()), c->d_err, c->wait_ns, st);
     if (id >= 0) pr.end(id, st);
   } else {
     wsy = ws1 + p.ws1;

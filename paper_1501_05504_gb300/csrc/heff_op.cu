@@ -23,14 +23,8 @@ struct HeffOp {
   const double* R = nullptr;
   float* packL = nullptr;      // tensor-core modes: packed copies (hi then lo)
   float* packR = nullptr;
-  uint16_t* sliceL = nullptr;  // sliced FP64: L and R, with their row scales behind them
-  uint16_t* sliceR = nullptr;
   int64_t nA = 0;              // elements of A and HA
 };
-namespace {
-size_t sliced_bytes(int64_t n, int32_t ne) { return (size_t)(n + 1) / 2 * 4 + (size_t)ne * 4 + 4; }
-int32_t* row_scales(uint16_t* p, int64_t n) { return reinterpret_cast<int32_t*>(p + (n + 1) / 2 * 2); }
-}  // namespace
 }  // namespace dmrg3s
 
 extern "C" {
@@ -93,29 +87,6 @@ dmrg3s_status dmrg3s_heff_create(dmrg3s_ctx ctx, const dmrg3s_env* L, const dmrg
       return fail(c, DMRG3S_ERR_CUDA, "H_eff handle: packing launch");
     }
   }
-  // FP64: L and R sliced once; without the memory for them the products run
-  // in the plain form, which needs none
-  if (prec == DMRG3S_FP64 && sliced_fits(p->host, c->ws_bytes)) {
-    const SlStage& s1 = p->host.s12;
-    const SlStage& s3 = p->host.s3;
-    if (cudaMalloc(&h->sliceL, sliced_bytes(s1.nA, s1.neA)) == cudaSuccess &&
-        cudaMalloc(&h->sliceR, sliced_bytes(s3.nB, s3.neB)) == cudaSuccess) {
-      SlOperands ops{};
-      ops.op[0] = SlOperand{L->data, h->sliceL, row_scales(h->sliceL, s1.nA), 1.0};
-      ops.op[1] = SlOperand{R->data, h->sliceR, row_scales(h->sliceR, s3.nB), 1.0};
-      slice_operands(*p, 0, 1, ops, s);
-      if (cudaGetLastError() != cudaSuccess) {
-        cudaFree(h->sliceL);
-        cudaFree(h->sliceR);
-        delete h;
-        return fail(c, DMRG3S_ERR_CUDA, "H_eff handle: slicing launch");
-      }
-    } else {
-      cudaGetLastError();
-      if (h->sliceL) cudaFree(h->sliceL);
-      h->sliceL = h->sliceR = nullptr;
-    }
-  }
   *out = reinterpret_cast<dmrg3s_heff>(h);
   return DMRG3S_OK;
 }
@@ -143,17 +114,6 @@ dmrg3s_status dmrg3s_heff_apply(dmrg3s_heff op, const double* A, double* HA,
     hints.g3B_hi = h->packR;
     hints.g3B_lo = x3 ? h->packR + pl.g3s.tc.nB : nullptr;
     hp = &hints;
-  } else {
-    const Plan& pl = h->plan->host;
-    hints.f64 = h->sliceL ? kF64Sliced : kF64Plain;
-    if (h->sliceL) {
-      hints.sliced_env = true;
-      hints.s1A = h->sliceL;
-      hints.e1A = row_scales(h->sliceL, pl.s12.nA);
-      hints.s3B = h->sliceR;
-      hints.e3B = row_scales(h->sliceR, pl.s3.nB);
-    }
-    hp = &hints;
   }
   st = run_plan(c, *h->plan, h->L, A, ws1, ws2, 1.0, ws2, h->R, HA, s, h->prec, hp);
   return st == DMRG3S_OK ? DMRG3S_OK : fail(c, st, "H_eff launch failed");
@@ -163,11 +123,9 @@ dmrg3s_status dmrg3s_heff_destroy(dmrg3s_heff op) {
   HeffOp* h = reinterpret_cast<HeffOp*>(op);
   if (!h) return DMRG3S_ERR_ARG;
   use_device(h->c);
-  if (h->packL || h->packR || h->sliceL) cudaDeviceSynchronize();
+  if (h->packL || h->packR) cudaDeviceSynchronize();
   if (h->packL) cudaFree(h->packL);
   if (h->packR) cudaFree(h->packR);
-  if (h->sliceL) cudaFree(h->sliceL);
-  if (h->sliceR) cudaFree(h->sliceR);
   delete h;
   return DMRG3S_OK;
 }

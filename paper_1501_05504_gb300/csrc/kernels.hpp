@@ -96,16 +96,30 @@ struct PackOut {
 // 16 columns of an MMA).  A tile is one 1 KB atom of the K-major 128-byte
 // swizzled layout: row r % 8 is a 128-byte line (64 k), its 16-byte piece j =
 // (k % 64) / 8 at position j ^ (r % 8).
-constexpr int kSlices = 7;
+constexpr int kSlices = 8;
 constexpr int kSlTile = 512;               // FP16 elements of a tile
-constexpr int32_t kSlSpecial = 0x40000000; // row scale of a row with Inf or NaN
+// A row scale: the exponent field F of the row's largest element (below 2^(F - 1022);
+// possibly outside an FP64 number's range) + kSlBias; 0 for a zero row, kSlSpecial
+// for one with Inf or NaN.
+constexpr int32_t kSlSpecial = 0x40000000, kSlBias = 4096;
 // One block of a scale group: element (r, k) is coef * src[src + r ld + k]
 // (trans = 0) or coef * src[src + k ld + r] (trans = 1).
-// t0: its first 64-wide chunk among the chunks of its group.
+// t0: its first 64-wide chunk among the chunks of its group.  d0: its first entry of
+// the operand's grading (SlOperand), or -1.
 struct SlMember {
   int64_t src, dst;
   double coef;
-  int32_t ld, K, KC, trans, t0, pad;
+  int32_t ld, K, KC, trans, t0, d0;
+};
+// Up to 32 consecutive k of blocks that share a grading: d[d0 + k] (k < nk) = the
+// exponent of the largest element at that k of the views [v0, v0 + nv), so that
+// |element| 2^-d < 1 (0 for none, or with Inf or NaN).
+struct SlGrade {
+  int32_t d0, nk, v0, nv;
+};
+struct SlView {
+  int64_t src;             // of the first k
+  int32_t ld, R, trans, pad;
 };
 // Blocks with the same rows whose rows share scales: scales[e0 + r]; one CTA
 // of the slicing kernel per row group, from cta0 on.
@@ -134,12 +148,14 @@ struct SlUnit {
   int32_t shift;    // of A's row scales (SlGroup.shift)
   int32_t em;       // first row scale of the output as a later operand, or -1
   int32_t sel;      // which pair of FP64 operands (SlSource) its segments read
+  uint32_t least;   // least |sum| that is taken without a look at its terms, in 2^32 of H
+  int32_t d0;       // first grading entry of its columns for the collected scales, or -1
 };
 // The units' 64-wide k-chunks in the order a CTA runs them.  The copies: slice
 // i of A is `ga` tiles at a + i sa, slice j of B `gb` tiles at b + j sb (FP16
 // elements); `word` is the MMA issuer's view: kSlSteps = its k16 steps (1-4),
 // kSlFirst / kSlLast = first / last chunk of a span (at most 64 k),
-// kSlLongFirst / kSlLongLast = of a long span (four spans, levels 4-6), kSlMove
+// kSlLongFirst / kSlLongLast = of a long span (four spans, levels 4-7), kSlMove
 // = the accumulators' columns move (another nw than the chunk before), and nw
 // from bit kSlNw on.
 struct SlChunk {
@@ -151,34 +167,53 @@ constexpr uint32_t kSlSteps = 7, kSlFirst = 8, kSlLast = 16, kSlLongFirst = 32, 
                    kSlMove = 128, kSlNw = 8;
 constexpr int kSlLongSpan = 4;
 // An operand: its FP64 array, its packed array, its row scales; `scale`
-// multiplies every coefficient.
+// multiplies every coefficient; element (r, k) also takes the factor 2^(sign d[d0 + k]).
 struct SlOperand {
   const double* src;
   uint16_t* out;
   int32_t* scales;
   double scale;
+  const int32_t* d;
+  int32_t sign, pad;
 };
-// The launch also clears `nclear` scales (which a later launch collects).
+// The launch also clears `nclear` scales (which a later launch collects) and the
+// `nfix` counters of the SlFix lists.
 struct SlOperands {
   SlOperand op[4];
   int32_t* clear;
-  int32_t nclear;
+  int32_t* fix;
+  int32_t nclear, nfix;
 };
+// The elements of a product that its slices may hold with fewer digits than FP64
+// would: `count` parts of units (a drain warp's 32 rows x 16 columns; part w of
+// unit u is 16 u + w) listed in `list`, with a word of 32 rows for each column in
+// mask[16 (16 u + w) ..].
+struct SlFix {
+  int32_t* count;
+  int32_t* list;
+  uint32_t* mask;
+};
+constexpr int kSlParts = 16;
+constexpr int64_t kSlFixInts = 17;         // of list and mask, for a part
+constexpr int32_t kSlForce = 1 << 30;      // on a list entry: form the elements whatever their terms' size
 // A block of an operand whose row scales are known (collected by the launch
 // that wrote it): tiles [tile0, tile0 + R8 KC), tile t = (chunk, row group) with
 // t = chunk R8 + group.
 struct SlPiece {
   int64_t src, dst;
-  int32_t ld, K, KC, trans, R, R8, e0, shift, tile0, pad;
+  int32_t ld, K, KC, trans, R, R8, e0, shift, tile0, d0;   // d0: as in SlMember (sign -1)
 };
-// Row scales and slices of every block of the groups whose CTAs are
-// [cta0, cta0 + nctas) (a group has R8 CTAs from its cta0 on; cta_group[c] = the
-// group of CTA c).
-void launch_slice(const SlGroup* groups, const int32_t* cta_group, int cta0, int nctas,
+// Row scales and slices of every block of every group (a group has R8 CTAs from its
+// cta0 on; cta_group[c] = the group of CTA c).
+void launch_slice(const SlGroup* groups, const int32_t* cta_group, int nctas,
                   const SlMember* members, const SlOperands& ops, cudaStream_t st);
+// The gradings of a site tensor (kernels_sliced.cu).
+void launch_grade(const SlGrade* items, int nitems, const SlView* views, const double* src, int32_t* d,
+                  cudaStream_t st);
 // Slices of the pieces, a warp per tile; first[c] = the piece of tile 8 c.
 void launch_slice_known(const SlPiece* pieces, int npieces, const int32_t* first, int ntiles,
-                        const double* src, uint16_t* out, const int32_t* scales, cudaStream_t st);
+                        const double* src, uint16_t* out, const int32_t* scales, const int32_t* d,
+                        cudaStream_t st);
 
 // C = sum over the task's segments of op(A) op(B), one rounding to FP64 (see
 // kernels_sliced.cu).  CTA b runs units [cta_unit[b], cta_unit[b + 1]) and
@@ -191,7 +226,7 @@ struct SlTables {
   const uint32_t* words;
   const int32_t *cta_unit, *cta_chunk;
   const SlSeg* segs;
-  int ncta;
+  int ncta, nunits;
   bool chain;       // short enough for a chained launch (launch.hpp)
 };
 struct SlSource {
@@ -199,10 +234,13 @@ struct SlSource {
   int32_t ta, tb;                    // stored transposed (as in launch_gemm_f64)
   double scale;
 };
+// d: the gradings (SlUnit.d0; the scales of column c are collected as those of the
+// elements times 2^-d).  fix (its count cleared before): receives the elements to form from the FP64
+// operands, which a second launch does.
 void launch_gemm_sliced(const SlTables& t, const uint16_t* pA, const uint16_t* pB,
                         const int32_t* eA, const int32_t* eB, const SlSource& src, double* C,
-                        int32_t* collect, bool collect_cols, int* err, uint64_t wait_ns,
-                        cudaStream_t st);
+                        int32_t* collect, bool collect_cols, const int32_t* d, const SlFix& fix, int* err,
+                        uint64_t wait_ns, cudaStream_t st);
 
 // Blockwise inner products: out[task.out] = sum over the task's segments of
 // <A[offA .. offA+len), B[offB .. offB+len)> (FP64, fixed summation order).

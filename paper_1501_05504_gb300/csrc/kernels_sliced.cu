@@ -4,35 +4,46 @@
 //
 // Every row of a packed operand (an output row of A, an output column of B)
 // carries one power-of-two scale over the whole contracted index; relative to
-// it an element is a 62-bit fixed-point number v (|v| <= 2^62, rounded to
-// nearest), written in seven balanced digits of 9 bits,
-//   v = sum_i q_i 2^(54 - 9 i),   -256 <= q_i <= 256,
+// it an element is a 71-bit fixed-point number v (|v| <= 2^71, rounded to
+// nearest), written in eight balanced digits of 9 bits,
+//   v = sum_i q_i 2^(63 - 9 i),   -256 <= q_i <= 256,
 // each exact in FP16.  With both operands sliced,
-//   C = 2^(scales) sum_l 2^(108 - 9 l) S_l,   S_l = sum_{i + j = l} A_i B_j,
-// and the 28 digit products of the levels l = 0 .. 6 are formed (levels >= 7
-// lie below 2^-62 of the row scales).  One S_l collects at most 64 k before
-// it is drained, so |S_l| <= (l + 1) 64 2^16: levels 0-3 are exact integers in
-// the FP32 accumulators (<= 2^24), levels 4-6 carry weights below 2^-36.  The
-// drained levels 0-3 are summed exactly in a 64-bit integer (H; the row scales
-// leave it room for the task's spans); levels 4-6 run on for 256 k, level 4 then
-// joins H and levels 5-6 are summed in FP32 (L: 2^-24 of weights below 2^-45),
-// and the output is H 2^18 + L rounded once to FP64 with integer instructions.
-// Besides that rounding only the slices' own (2^-63 of the row scale) enters an
-// output element, however long its contraction.
+//   C = 2^(scales) sum_l 2^(126 - 9 l) S_l,   S_l = sum_{i + j = l} A_i B_j,
+// and the 36 digit products of the levels l = 0 .. 7 are formed (levels >= 8
+// lie below 2^-72 of the row scales).  One S_l collects at most 64 k before
+// it is drained for l <= 3, 256 k for l >= 4.  Levels 0-3 are exact integers in
+// the FP32 accumulators (|S_l| <= (l + 1) 64 2^16 <= 2^24); levels 4-7 are while
+// their sums stay below 2^24 (17 sigma of rounding digits), and rows with one near 2^24
+// or above (digits that repeat along k) are listed (below).
+// The drained levels are summed exactly in integers: H (64 bits, in units of level
+// 4; the row scales leave it room for the task's spans) and L (27 bits below it),
+// and the output is H 2^27 + L rounded once to FP64 with integer instructions.
+//
+// Precision: an FP64 product keeps 53 bits of every term, however small beside the
+// others of its row; here a term is held to 2^-72 of the row scales.  Over K
+// terms the rounding of the slices and the missing levels amount to about E =
+// sqrt(K) 2^-72 of the scales (0.95 rms a term), so an output element with
+// S = sum |a| |b| >= 3 2^54 E loses less by them than by the roundings of an FP64
+// sum (2^-53 of S each), and is stored: |C| >= that bound shows it, or the sum of any
+// one span (levels 0 and 1; the lower ones reach 25000 units of level 1).  Any
+// other element (small terms of a graded row, cancelling terms) is listed, and a second
+// launch (fix_kernel) looks at it: it computes S of the part, and what stays below the
+// bound is formed from the FP64 operands, term by term (rows with large levels always,
+// in compensated sums).  So no element is further from the exact sum than the plain
+// form's bound, whatever the grading.
 //
 // Why: GB300 multiplies FP64 at 2 multiply-adds per SM and clock (1.1 TFLOP/s
-// measured) and FP16 with FP32 accumulation at ~1700 times that, so 28 exact
-// products cost less than a sixtieth of one FP64 product.
+// measured) and FP16 with FP32 accumulation at ~1700 times that, so 36 exact
+// products cost less than a fortieth of one FP64 product.
 //
 // Kernel: persistent CTAs (one per SM, 576 threads) over output tiles of
-// 128 x 64.  The seven levels are seven accumulators of nw <= 64 columns side
-// by side in tensor memory, and the B slices lie back to back in shared
-// memory, so digit A_i meets the slices B_0 .. B_(6-i) in MMAs of up to 256
-// columns (one issue serves up to four digit products, and the A digit is read
-// from shared memory once for all of them).  A tile of 128 x 128 would need 896
-// tensor-memory columns of the 512.
-//   warp 0     one lane issues the bulk copies: the seven B slices of a 64-wide
-//              k-chunk in one of two 56 KB buffers, the A slices through a ring
+// 128 x 64.  The eight levels are eight accumulators of nw <= 64 columns side
+// by side in tensor memory (all 512 of its columns), and the B slices lie back to
+// back in shared memory, so digit A_i meets the slices B_0 .. B_(7-i) in MMAs of up
+// to 256 columns (one issue serves up to four digit products, and the A digit is read
+// from shared memory once for all of them).
+//   warp 0     one lane issues the bulk copies: the eight B slices of a 64-wide
+//              k-chunk in one of two 64 KB buffers, the A slices through a ring
 //              of 16 KB slabs
 //   warp 1     one lane issues tcgen05.mma (kind::f16); level l is committed to
 //              its own barrier right after digit A_l, while the later digits
@@ -40,15 +51,18 @@
 //   warps 2-17 drain: 32 rows x 16 columns each, H and L in registers
 // Every wait is bounded as in the other tensor-core kernel.
 //
-// Inside a tile it is bound by shared-memory bandwidth: the 28 products of 16 k read
-// 138 KB of slices, 1078 cycles, where the MMAs alone would take 896.  Measured
-// (the plain form in 64 x 64 tiles / this): the m = 2048 cylinder's environment update,
-// 13 Gflop, 14.1 / 0.75 ms; the m = 512 XXZ operator, 0.18 Gflop, 884 / 71 us, where
-// the launches, the slicing and short units (2 to 4 spans) count as much.
+// Inside a tile it is bound by the MMAs and by shared-memory bandwidth: the 36 products
+// of 16 k take 1312 cycles for 64 columns.  Measured (the plain form / this): the m = 2048
+// cylinder's environment update, 13 Gflop, 12.1 / 0.93 ms; the m = 512 XXZ operator, 0.18
+// Gflop, 219 / 120 us, where eight launches, the slicing and short units (2 to 4 spans)
+// count as much.  (With seven slices, no gradings and no fix launches, and so with
+// small terms held to 2^-63 of the scales only: 0.75 ms and 71 us.)
+#include <algorithm>
 #include <atomic>
 #include <cstdint>
 
 #include "kernels.hpp"
+#include "fp64.cuh"
 #include "launch.hpp"
 #include "tc_common.cuh"
 
@@ -59,7 +73,7 @@ namespace {
 constexpr int kFirstDrainWarp = 2, kDrainWarps = 16;
 constexpr int kThreads = 32 * (kFirstDrainWarp + kDrainWarps);
 constexpr int kSlabA = 16384;                          // 128 rows x 64 k of one slice
-constexpr int kSlots = 5;                              // A ring
+constexpr int kSlots = 4;                              // A ring
 constexpr int kBufB = kSlices * 8192;                  // 64 columns x 64 k of all slices
 constexpr int kOffA = 2 * kBufB;
 constexpr int kOffStage = kOffA + kSlots * kSlabA;
@@ -71,11 +85,13 @@ constexpr uint32_t kTmemCols = 512;
 // of x + 1.5 2^23 are x + 2^22; a conversion instruction takes 8 cycles a warp
 // and sub-partition, the addition one).  Two levels of at most 2^21 make one
 // unsigned 32-bit word, (a + 2^21) 512 + b + (the bits of 1.5 2^23), so H grows
-// by kBiasH per span, and by kBiasOne per long span, besides the levels; larger
-// levels (possible, but far outside what rounding digits give) take the
-// conversion.
-constexpr unsigned long long kBiasOne = 0x4B400000ull;
+// by kBiasH per span besides the levels, and by kBiasOne and kBiasLow (27 bits below it)
+// per long span; larger levels (possible, but far outside what rounding digits give)
+// take the conversion.
+constexpr uint32_t kBiasOne = 0x4B400000u;
 constexpr unsigned long long kBiasPair = (2097152ull << 9) + kBiasOne;
+constexpr uint32_t kLowMask = (1u << 27) - 1;
+constexpr unsigned long long kBiasLow = (unsigned long long)kBiasOne * ((1u << 18) + (1u << 9) + 1u);
 constexpr unsigned long long kBiasH = (kBiasPair << 27) + (kBiasPair << 9);
 
 // Instruction descriptor of kind::f16: D = F32, A = B = F16, both K-major.
@@ -118,6 +134,11 @@ __device__ __forceinline__ void tmem_ld8_async(uint32_t taddr, uint32_t* v) {
                  "=r"(v[6]), "=r"(v[7])
                : "r"(taddr));
 }
+__device__ __forceinline__ void tmem_wait_ld8(uint32_t (&v)[16]) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;"
+               : "+r"(v[0]), "+r"(v[1]), "+r"(v[2]), "+r"(v[3]), "+r"(v[4]), "+r"(v[5]),
+                 "+r"(v[6]), "+r"(v[7])::"memory");
+}
 // Waits for the loads; v passes through it, so that no use moves before it.
 __device__ __forceinline__ void tmem_wait_ld(uint32_t (&v)[16]) {
   asm volatile("tcgen05.wait::ld.sync.aligned;"
@@ -126,19 +147,16 @@ __device__ __forceinline__ void tmem_wait_ld(uint32_t (&v)[16]) {
                  "+r"(v[12]), "+r"(v[13]), "+r"(v[14]), "+r"(v[15])::"memory");
 }
 
-// (H 2^14 + L) 2^(ex + 4) rounded to the nearest FP64 value: 32-bit integer
+// (H 2^27 + L) 2^ex (L < 2^27) rounded to the nearest FP64 value: 32-bit integer
 // instructions on the 96-bit sum (an FP64 conversion or addition holds GB300's
 // FP64 unit for 64 cycles a warp), without branches, so that several elements
 // are in flight.  (A negative sum is complemented, one unit below its
-// magnitude: 2^-66 of the scales.)  Sets `out` when the result needs the
+// magnitude: 2^-79 of the scales.)  Sets `out` when the result needs the
 // general form below: exponent outside the normal range, or no bit above the
 // last 32 of the 96.
-__device__ __forceinline__ double fixed_to_f64(long long H, int L, int ex, bool* out) {
+__device__ __forceinline__ double fixed_to_f64(long long H, uint32_t L, int ex, bool* out) {
   const uint32_t h0 = (uint32_t)H, h1 = (uint32_t)((unsigned long long)H >> 32);
-  uint32_t x0 = h0 << 14, x1 = __funnelshift_l(h0, h1, 14), x2 = (uint32_t)((int32_t)h1 >> 18);
-  asm("add.cc.u32 %0, %0, %3;\n\taddc.cc.u32 %1, %1, %4;\n\taddc.u32 %2, %2, %4;"
-      : "+r"(x0), "+r"(x1), "+r"(x2)
-      : "r"(L), "r"(L >> 31));
+  uint32_t x0 = (h0 << 27) | L, x1 = __funnelshift_l(h0, h1, 27), x2 = (uint32_t)((int32_t)h1 >> 5);
   const uint32_t s = (uint32_t)((int32_t)x2 >> 31);
   x0 ^= s;
   x1 ^= s;
@@ -154,46 +172,33 @@ __device__ __forceinline__ double fixed_to_f64(long long H, int L, int ex, bool*
       : "r"(w0), "r"(w1));
   // exponent field less one: the leading bit of r1 >> 11 adds it (it is gone
   // when the rounding carried out)
-  const int f = ex + (4 + 95 + 1022) - (z ? 32 : 0) - (int)lz + 2 * (int)c;
+  const int f = ex + (95 + 1022) - (z ? 32 : 0) - (int)lz + 2 * (int)c;
   const bool zero = (y2 | y1) == 0;
   *out = *out || (!zero && ((uint32_t)f >= 2045u || y2 == 0));
   const uint32_t hi = ((r1 >> 11) + ((uint32_t)f << 20)) | (s & 0x80000000u);
   return __hiloint2double((int)(zero ? 0u : hi), (int)(zero ? 0u : __funnelshift_r(r0, r1, 11)));
 }
 
-// The same sum, (H 2^18 + L) 2^ex, for any range, in FP64 arithmetic.
-__device__ __noinline__ double fixed_to_f64_any(long long H, float L, int ex) {
-  const long long l = __float2ll_rn(L);
-  const long long h = H + (l >> 18);
-  const double top = (double)(h >> 32) * 4294967296.0, low = (double)(h & 0xFFFFFFFFll);
-  return ldexp(fma(top + low, 262144.0, (double)(l & 0x3FFFF)), ex);
+// The same for any range, in FP64 arithmetic.
+__device__ __noinline__ double fixed_to_f64_any(long long H, uint32_t L, int ex) {
+  const double top = (double)(H >> 32) * 4294967296.0, low = (double)(H & 0xFFFFFFFFll);
+  return ldexp(fma(top + low, 134217728.0, (double)L), ex);
 }
 
-// One output element the plain way (rows or columns with Inf or NaN).
-__device__ __noinline__ double element_f64(const SlSeg* __restrict__ segs, int nseg,
-                                           const double* A,
-                                           const double* B, int ta, int tb, int m,
-                                           int n, double scale) {
-  double acc = 0.0;
-  for (int k = 0; k < nseg; ++k) {
-    const SlSeg s = segs[k];
-    double part = 0.0;
-    for (int q = 0; q < s.K; ++q) {
-      const double a = ta ? A[s.offA + (int64_t)q * s.lda + m] : A[s.offA + (int64_t)m * s.lda + q];
-      const double b = tb ? B[s.offB + (int64_t)n * s.ldb + q] : B[s.offB + (int64_t)q * s.ldb + n];
-      part = fma(a, b, part);
-    }
-    acc = fma(s.scale, part, acc);
-  }
-  return scale * acc;
+// The row scale that x 2^-d asks for (a subnormal counts as the smallest exponent).
+__device__ __forceinline__ int scale_of(double x, int d) {
+  const uint32_t hi = (uint32_t)__double2hiint(x) & 0x7FFFFFFFu;
+  const int f = (int)(hi >> 20);
+  if (f == 0x7FF) return kSlSpecial;
+  return (hi | (uint32_t)__double2loint(x)) == 0u ? 0 : max(f, 1) - d + kSlBias;
 }
 
 __global__ void __launch_bounds__(kThreads, 1)
     gemm_sliced_kernel(const SlTables tab, const uint16_t* pA,
                        const uint16_t* pB, const int32_t* eA,
-                       const int32_t* eB, const __grid_constant__ SlSource src,
-                       double* C, int32_t* collect, int collect_cols,
-                       int* err, uint64_t wait_ns) {
+                       const int32_t* eB,
+                       double* C, int32_t* collect, int collect_cols, const int32_t* d,
+                       const SlFix fix, int* err, uint64_t wait_ns) {
   extern __shared__ __align__(1024) unsigned char smem[];
   __shared__ __align__(8) uint64_t afull[kSlots], aempty[kSlots], bfull[2], bempty[2];
   __shared__ __align__(8) uint64_t lfull[kSlices], lempty[kSlices], done;
@@ -289,7 +294,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int c_end = tab.cta_chunk[blockIdx.x + 1];
     int ci = tab.cta_chunk[blockIdx.x];
     uint32_t slot = 0, aph = 0, bs = 0, bph = 0;
-    uint32_t ph = 0, pl = 0;             // spans (levels 0-3), long spans (levels 4-6)
+    uint32_t ph = 0, pl = 0;             // spans (levels 0-3), long spans (levels 4-7)
     uint32_t next = ci < c_end ? tab.words[ci] : 0u;
     const uint32_t s0 = smem_u32(smem);
     const uint32_t tmem_u = __reduce_or_sync(0xffffffffu, tmem);
@@ -330,11 +335,11 @@ __global__ void __launch_bounds__(kThreads, 1)
           aph ^= 1;
         }
         a_ready = mbar_test(&afull[slot], aph);
-        // B slices 0 .. 6 - i in one MMA, or in two when they are more than 256
-        // columns (the first digit always: its levels 4-6 are drained later)
-        const uint32_t all = (uint32_t)(7 - i);
-        const uint32_t n1 = i == 0 ? 4u : (i < 3 && all * nw > 256u) ? 3u : all;
-        const bool two = i < 3 && n1 < all;
+        // B slices 0 .. 7 - i in one MMA, or in two when they are more than 256
+        // columns (the first digit always: its levels 4-7 are drained later)
+        const uint32_t all = (uint32_t)(kSlices - i);
+        const uint32_t n1 = i == 0 ? 4u : (i < 4 && all * nw > 256u) ? 3u : all;
+        const bool two = i < 4 && n1 < all;
         const bool wait2 = i == 0 && (w & kSlLongFirst) && pl > 0;
         if (wait2) {
           if (one)
@@ -391,17 +396,20 @@ __global__ void __launch_bounds__(kThreads, 1)
       const int spans = un.spans;
       // (a warp beyond the tile only arrives)
       const bool mine = (uint32_t)(part * 16) < nw && quarter * 32 < un.rows;
-      unsigned long long H[16];                          // levels 0-4, biased
-      float L[16];                                       // levels 5-6, FP32
+      unsigned long long H[16];                          // units of level 4 (levels 0-3 biased)
+      uint32_t L[16];                                    // below them, units of level 7
+      bool large = false;                                // a level 4-7 near 2^24 or above
+      uint32_t sized = 0;                                // columns with a span of enough size
+      const uint32_t enough = min(32u * un.least + 25000u, 1u << 30);
 #pragma unroll
       for (int j = 0; j < 16; ++j) {
         H[j] = 0;
-        L[j] = 0.f;
+        L[j] = 0;
       }
       const int row0 = quarter * 32, row = row0 + lane, n0 = part * 16;
       // (rows and columns of the padding get a scale in the normal range)
-      const int fa = row < un.rows && spans > 0 ? eA[un.ea + row] : 1057;
-      const int fb_lane = lane < 16 && n0 + lane < un.cols && spans > 0 ? eB[un.eb + n0 + lane] : 1057;
+      const int fa = row < un.rows && spans > 0 ? eA[un.ea + row] : kSlBias + 1057;
+      const int fb_lane = lane < 16 && n0 + lane < un.cols && spans > 0 ? eB[un.eb + n0 + lane] : kSlBias + 1057;
       for (int sp = 0; sp < spans && ok; ++sp, ++ph) {
         const bool longer = sp % kSlLongSpan == kSlLongSpan - 1 || sp == spans - 1;
 #pragma unroll
@@ -430,6 +438,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                       __float_as_uint(__fadd_rn(__uint_as_float(v[j]), 10485760.f)) * 512u +
                       __float_as_uint(__fadd_rn(__uint_as_float(v[8 + j]), 12582912.f));
                   H[h + j] += (unsigned long long)w * (l == 0 ? 134217728u : 512u);
+                  if (l == 0 && w - (uint32_t)kBiasPair + enough > 2u * enough) sized |= 1u << (h + j);
                 }
               } else {
 #pragma unroll
@@ -437,6 +446,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                   const long long a = (long long)__float2int_rn(__uint_as_float(v[j])) * 512 +
                                       __float2int_rn(__uint_as_float(v[8 + j]));
                   H[h + j] += ((unsigned long long)a + kBiasPair) * (l == 0 ? 134217728u : 512u);
+                  if (l == 0 && llabs(a) > (long long)enough) sized |= 1u << (h + j);
                 }
               }
             }
@@ -449,57 +459,98 @@ __global__ void __launch_bounds__(kThreads, 1)
           }
         }
         if (!ok || !longer) continue;
+        // level 4 into H, then levels 5-7 together: t = S_5 2^18 + S_6 2^9 + S_7 + L is at most
+        // 63 bits, its upper part belongs to H
 #pragma unroll
-        for (int l = 4; l < kSlices; ++l) {
-          if (!__all_sync(0xffffffffu, mbar_wait(&lfull[l], pl & 1, wc))) {
-            ok = false;
-            break;
-          }
+        for (int g = 0; g < 2; ++g) {
+          const int l = g == 0 ? 4 : kSlices - 1;
+          for (int w = g == 0 ? 4 : 5; w <= l && ok; ++w)
+            if (!__all_sync(0xffffffffu, mbar_wait(&lfull[w], pl & 1, wc))) ok = false;
+          if (!ok) break;
           asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-          if (mine) {
+          if (mine && g == 0) {
             uint32_t v[16];
-            tmem_ld8_async(tcol + (uint32_t)l * nw, v);
-            tmem_ld8_async(tcol + (uint32_t)l * nw + 8, v + 8);
+            tmem_ld8_async(tcol + 4u * nw, v);
+            tmem_ld8_async(tcol + 4u * nw + 8, v + 8);
             tmem_wait_ld(v);
-            if (l == 4) {
-              float m = 0.f;
+            float m = 0.f;
 #pragma unroll
-              for (int j = 0; j < 16; ++j) m = fmaxf(m, fabsf(__uint_as_float(v[j])));
-              if (!__any_sync(0xffffffffu, !(m < 4194304.f))) {
+            for (int j = 0; j < 16; ++j) m = fmaxf(m, fabsf(__uint_as_float(v[j])));
+            if (!__any_sync(0xffffffffu, !(m < 4194304.f))) {
 #pragma unroll
-                for (int j = 0; j < 16; ++j)
-                  H[j] += __float_as_uint(__fadd_rn(__uint_as_float(v[j]), 12582912.f));
-              } else {
-#pragma unroll
-                for (int j = 0; j < 16; ++j)
-                  H[j] += (unsigned long long)(long long)__float2int_rn(__uint_as_float(v[j])) + kBiasOne;
-              }
+              for (int j = 0; j < 16; ++j) H[j] += __float_as_uint(__fadd_rn(__uint_as_float(v[j]), 12582912.f));
             } else {
+              large = large || (row < un.rows && !(m < 16000000.f));   // (lanes beyond hold garbage)
 #pragma unroll
               for (int j = 0; j < 16; ++j)
-                L[j] = __fmaf_rn(__uint_as_float(v[j]), l == 5 ? 512.f : 1.f, L[j]);
+                H[j] += (unsigned long long)(long long)__float2int_rn(__uint_as_float(v[j])) + kBiasOne;
+            }
+          } else if (mine) {
+#pragma unroll
+            for (int h = 0; h < 16; h += 8) {
+              uint32_t v[16], u[16];
+              tmem_ld8_async(tcol + 5u * nw + h, v);
+              tmem_ld8_async(tcol + 6u * nw + h, v + 8);
+              tmem_ld8_async(tcol + 7u * nw + h, u);
+              tmem_wait_ld(v);
+              tmem_wait_ld8(u);
+              float m = 0.f;
+#pragma unroll
+              for (int j = 0; j < 8; ++j)
+                m = fmaxf(m, fmaxf(fmaxf(fabsf(__uint_as_float(v[j])), fabsf(__uint_as_float(v[8 + j]))),
+                                   fabsf(__uint_as_float(u[j]))));
+              if (!__any_sync(0xffffffffu, !(m < 4194304.f))) {
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                  const uint32_t a = __float_as_uint(__fadd_rn(__uint_as_float(v[j]), 12582912.f));
+                  const uint32_t b = __float_as_uint(__fadd_rn(__uint_as_float(v[8 + j]), 12582912.f));
+                  const uint32_t c = __float_as_uint(__fadd_rn(__uint_as_float(u[j]), 12582912.f)) + L[h + j];
+                  const unsigned long long t = (unsigned long long)a * 262144u + ((unsigned long long)b * 512u + c);
+                  H[h + j] += t >> 27;
+                  L[h + j] = (uint32_t)t & kLowMask;
+                }
+              } else {
+                large = large || (row < un.rows && !(m < 16000000.f));
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                  const long long t = (long long)__float2int_rn(__uint_as_float(v[j])) * 262144 +
+                                      (long long)__float2int_rn(__uint_as_float(v[8 + j])) * 512 +
+                                      __float2int_rn(__uint_as_float(u[j])) + (long long)(kBiasLow + L[h + j]);
+                  H[h + j] += (unsigned long long)(t >> 27);
+                  L[h + j] = (uint32_t)t & kLowMask;
+                }
+              }
             }
           }
           asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
           __syncwarp();
-          if (lane == 0) mbar_arrive(&lempty[l]);
+          if (lane == 0)
+            for (int w = g == 0 ? 4 : 5; w <= l; ++w) mbar_arrive(&lempty[w]);
         }
+        if (!ok) break;
         ++pl;
       }
       if (!ok) break;
       if (!mine) continue;
       // rows of 4 consecutive doubles through the warp's staging rows
-      const unsigned long long bh =
-          (unsigned long long)spans * kBiasH +
-          (unsigned long long)((spans + kSlLongSpan - 1) / kSlLongSpan) * kBiasOne;
+      // the biases: X = H 2^27 + L less `longs` kBiasLow
+      const unsigned long long longs = (unsigned long long)((spans + kSlLongSpan - 1) / kSlLongSpan);
+      const unsigned long long low = longs * kBiasLow;
+      const unsigned long long bh = (unsigned long long)spans * kBiasH + longs * kBiasOne + (low >> 27);
+      const uint32_t bl = (uint32_t)low & kLowMask;
       const int rows = un.rows, cols = un.cols;
       double* Cu = C + un.offC + n0;
       const int64_t ldc = un.ldc;
       const int em = un.em, shift = un.shift;
-      uint32_t hmax = 0;                       // largest |high word| of the row (column `lane`)
-      // (the vote first: every lane takes part in it)
-      const bool special_col = __any_sync(0xffffffffu, fb_lane == kSlSpecial);
-      const bool special = special_col || fa == kSlSpecial;
+      // largest scale of the row (of column `lane`), and this lane's column's grading
+      int fmax = 0;
+      const int d_lane = em >= 0 && un.d0 >= 0 && lane < 16 && n0 + lane < cols ? d[un.d0 + n0 + lane] : 0;
+      // a zero row or column has no error; elements of rows and columns with Inf or
+      // NaN (their slices are zero) are listed
+      const uint32_t zero_col = __ballot_sync(0xffffffffu, lane < 16 && fb_lane == 0);
+      const uint32_t bad_col = __ballot_sync(0xffffffffu, lane < 16 && fb_lane == kSlSpecial);
+      const uint32_t least = fa == 0 ? 0u : un.least;
+      uint32_t listed = fa == kSlSpecial || large ? 0xffffu : bad_col;   // this lane's columns
 #pragma unroll
       for (int c4 = 0; c4 < 16; c4 += 4) {
         if (n0 + c4 >= cols) break;
@@ -508,30 +559,34 @@ __global__ void __launch_bounds__(kThreads, 1)
         double val[4];
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-          const float lf = L[c4 + i];
-          bool o = !(fabsf(lf) < 17179869184.f);           // 2^34: the range of the conversion
-          ex[i] = fa + shift + __shfl_sync(0xffffffffu, fb_lane, c4 + i) - 2114;
-          val[i] = fixed_to_f64((long long)(H[c4 + i] - bh), __float2int_rn(lf * 0.0625f), ex[i], &o);
+          const uint32_t lo = L[c4 + i] - bl;                  // (a borrow leaves the sign bit)
+          const long long h = (long long)(H[c4 + i] - bh) - (long long)(lo >> 31);
+          const int hs = (int)(h >> 32);
+          if ((uint32_t)(hs ^ (hs >> 31)) < least) listed |= 1u << (c4 + i) & ~(zero_col | sized);
+          bool o = false;
+          ex[i] = fa + shift + __shfl_sync(0xffffffffu, fb_lane, c4 + i) - (2123 + 2 * kSlBias);
+          val[i] = fixed_to_f64(h, lo & kLowMask, ex[i], &o);
           out = out || (o && row < rows && n0 + c4 + i < cols);
         }
         if (out)
 #pragma unroll
-          for (int i = 0; i < 4; ++i)
-            val[i] = fixed_to_f64_any((long long)(H[c4 + i] - bh), L[c4 + i], ex[i]);
+          for (int i = 0; i < 4; ++i) {
+            const uint32_t lo = L[c4 + i] - bl;
+            val[i] = fixed_to_f64_any((long long)(H[c4 + i] - bh) - (long long)(lo >> 31), lo & kLowMask, ex[i]);
+          }
 #pragma unroll
         for (int i = 0; i < 4; ++i) stage[lane * kStageRow + i] = val[i];
         if (em >= 0) {
 #pragma unroll
           for (int i = 0; i < 4; ++i) {
-            // (a nonzero low word alone still counts as a smallest exponent)
-            uint32_t hw = (uint32_t)__double2hiint(val[i]) & 0x7FFFFFFFu;
-            hw |= __double2loint(val[i]) != 0 ? 1u : 0u;
-            if (row >= rows || n0 + c4 + i >= cols) hw = 0;
+            const int dc = un.d0 >= 0 ? __shfl_sync(0xffffffffu, d_lane, c4 + i) : 0;
+            int f = scale_of(val[i], dc);
+            if (row >= rows || n0 + c4 + i >= cols || (listed >> (c4 + i) & 1u)) f = 0;
             if (collect_cols) {
-              hw = __reduce_max_sync(0xffffffffu, hw);
-              hmax = lane == c4 + i ? hw : hmax;
+              f = __reduce_max_sync(0xffffffffu, f);
+              fmax = lane == c4 + i ? f : fmax;
             } else {
-              hmax = max(hmax, hw);
+              fmax = max(fmax, f);
             }
           }
         }
@@ -545,21 +600,22 @@ __global__ void __launch_bounds__(kThreads, 1)
         __syncwarp();
       }
       if (em >= 0) {
-        // exponent field of the largest element (0: all zero); rows (columns)
-        // that meet Inf or NaN have no scale
         const bool inside = collect_cols ? lane < 16 && n0 + lane < cols : row < rows;
-        int f = hmax == 0 ? 0 : max((int)(hmax >> 20), 1);
-        const bool any = __any_sync(0xffffffffu, special && row < rows);
-        if (f >= 0x7FF || (collect_cols ? any : special)) f = kSlSpecial;
-        if (inside && f) atomicMax(collect + em + (collect_cols ? n0 + lane : row), f);
+        if (inside && fmax) atomicMax(collect + em + (collect_cols ? n0 + lane : row), fmax);
       }
-      // rows and columns with Inf or NaN (their slices are zero): the FP64 sum
-      if (special && row < rows) {
-        for (int j = 0; j < 16 && n0 + j < cols; ++j)
-          if (fa == kSlSpecial || eB[un.eb + n0 + j] == kSlSpecial)
-            Cu[row * ldc + j] =
-                element_f64(tab.segs + un.seg0, un.nseg, un.sel ? src.A1 : src.A,
-                            un.sel ? src.B1 : src.B, src.ta, src.tb, un.m0 + row, un.n0 + n0 + j, src.scale);
+      if (row >= rows) listed = 0;
+      if (cols - n0 < 16) listed &= (1u << (cols - n0)) - 1u;
+      if (__any_sync(0xffffffffu, listed != 0)) {
+        const int p = u * kSlParts + warp - kFirstDrainWarp;
+        uint32_t w = 0;
+#pragma unroll
+        for (int c = 0; c < 16; ++c) {
+          const uint32_t x = __ballot_sync(0xffffffffu, listed >> c & 1u);
+          w = lane == c ? x : w;
+        }
+        if (lane < 16) fix.mask[p * 16 + lane] = w;
+        const bool force = __any_sync(0xffffffffu, large);
+        if (lane == 0) fix.list[atomicAdd(fix.count, 1)] = force ? p | kSlForce : p;
       }
       __syncwarp();
     }
@@ -574,6 +630,171 @@ __global__ void __launch_bounds__(kThreads, 1)
                  : "memory");
 }
 
+// ---- listed elements ---------------------------------------------------------------
+// One CTA per listed part (32 rows x 16 columns) at a time.  More than a few elements:
+// a first pass forms S = sum |a| |b| of the whole part relative to the scales, on the
+// FP32 pipe (truncated operands: a lower bound to K 2^-24), and those whose S reaches
+// the bound are done.  The others are formed by a warp each, or by several, its lanes
+// over k.  Empty lists cost the launch.
+constexpr int kFixThreads = 256, kFixWarps = kFixThreads / 32;
+constexpr int kFixFew = 16;
+constexpr int kFixK = 32;
+constexpr int kFixCtas = 4 * 152;
+
+// |x| / 2^(e - 1023) truncated (0 for a subnormal; Inf beyond the range)
+__device__ __forceinline__ float part_of(double x, int e) {
+  const int f = exponent_of(x);
+  return f == 0 ? 0.f : f - e > 127 ? INFINITY : fabsf(float_of(x, e));
+}
+
+// acc + a b, with what its roundings leave added to lo (Ogita, Rump and Oishi, 2005).
+__device__ __forceinline__ double dot2(double a, double b, double acc, double& lo) {
+  const double p = __dmul_rn(a, b), e = fma(a, b, -p);
+  const double s = __dadd_rn(acc, p), z = __dadd_rn(s, -acc);
+  lo += __dadd_rn(__dadd_rn(acc, -__dadd_rn(s, -z)), __dadd_rn(p, -z)) + e;
+  return s;
+}
+
+__global__ void __launch_bounds__(kFixThreads, 4)
+    fix_kernel(const SlUnit* __restrict__ units, const SlSeg* __restrict__ segs, const SlFix fix,
+               const int32_t* eA, const int32_t* eB, const __grid_constant__ SlSource src, double* C,
+               int32_t* collect, int collect_cols, const int32_t* d) {
+  grid_next();
+  grid_wait();
+  __shared__ float sa[kFixK][33], sb[kFixK][16];
+  __shared__ uint32_t mask[16];
+  __shared__ int s_fa[32], s_fb[16];
+  __shared__ double s_sum[kFixWarps];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int count = *fix.count, mine = fix.list[blockIdx.x];   // (the list has an entry for every CTA)
+  for (int it = blockIdx.x; it < count; it += gridDim.x) {
+    const int entry = it == (int)blockIdx.x ? mine : fix.list[it], p = entry & ~kSlForce;
+    const bool force = (entry & kSlForce) != 0;
+    const SlUnit un = units[p / kSlParts];
+    const int w = p % kSlParts, row0 = ((w + kFirstDrainWarp) & 3) * 32, n0 = (w >> 2) * 16;
+    __syncthreads();                        // (the part before is done)
+    if (tid < 16) mask[tid] = fix.mask[p * 16 + tid];
+    __syncthreads();
+    const double* A = un.sel ? src.A1 : src.A;
+    const double* B = un.sel ? src.B1 : src.B;
+    double* Cp = C + un.offC + (int64_t)row0 * un.ldc + n0;
+    // the element's exponent among the scales of the output as a later operand
+    auto keep = [&](int r, int c, double v) {
+      if (un.em < 0) return;
+      const int f = scale_of(v, un.d0 >= 0 ? d[un.d0 + n0 + c] : 0);
+      if (f) atomicMax(collect + un.em + (collect_cols ? n0 + c : row0 + r), f);
+    };
+    const auto listed = [&]() {
+      int n = 0;
+#pragma unroll
+      for (int c = 0; c < 16; ++c) n += __popc(mask[c]);
+      return n;
+    };
+    int total = listed();
+    if (total > kFixFew && !force) {
+      // S of row lane, columns warp and warp + 8
+      if (tid < 16) s_fb[tid] = n0 + tid < un.cols ? eB[un.eb + n0 + tid] + 1 - kSlBias : 0;
+      if (warp == 1) s_fa[lane] = row0 + lane < un.rows ? eA[un.ea + row0 + lane] + un.shift + 1 - kSlBias : 0;
+      __syncthreads();
+      float size[2] = {0.f, 0.f};
+      for (int g = 0; g < un.nseg; ++g) {
+        const SlSeg q = segs[un.seg0 + g];
+        const double cf = q.scale * src.scale;
+        const int ce = exponent_of(cf);
+        const float cm = part_of(cf, ce);
+        for (int k0 = 0; k0 < q.K; k0 += kFixK) {
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const int e = tid + i * kFixThreads;
+            const int r = src.ta ? e & 31 : e >> 5, k = src.ta ? e >> 5 : e & 31;
+            double x = 0.0;
+            if (row0 + r < un.rows && k0 + k < q.K) {
+              const int64_t m = un.m0 + row0 + r, kk = k0 + k;
+              x = src.ta ? A[q.offA + kk * q.lda + m] : A[q.offA + m * q.lda + kk];
+            }
+            sa[k][r] = part_of(x, s_fa[r] - (ce - 1023)) * cm;
+          }
+#pragma unroll
+          for (int i = 0; i < 2; ++i) {
+            const int e = tid + i * kFixThreads;
+            const int c = src.tb ? e >> 5 : e & 15, k = src.tb ? e & 31 : e >> 4;
+            double x = 0.0;
+            if (n0 + c < un.cols && k0 + k < q.K) {
+              const int64_t n = un.n0 + n0 + c, kk = k0 + k;
+              x = src.tb ? B[q.offB + n * q.ldb + kk] : B[q.offB + kk * q.ldb + n];
+            }
+            sb[k][c] = part_of(x, s_fb[c]);
+          }
+          __syncthreads();
+#pragma unroll 4
+          for (int k = 0; k < kFixK; ++k) {
+            size[0] = fmaf(sa[k][lane], sb[k][warp], size[0]);
+            size[1] = fmaf(sa[k][lane], sb[k][warp + 8], size[1]);
+          }
+          __syncthreads();
+        }
+      }
+      const float least = (float)un.least * 0x1p-20f;
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int c = warp + 8 * h;
+        const bool in = (mask[c] >> lane & 1u) != 0;
+        // (rows and columns with Inf or NaN have no scale)
+        const bool special = s_fa[lane] > kSlSpecial / 2 || s_fb[c] > kSlSpecial / 2;
+        const bool form = in && (special || !(size[h] >= least && size[h] < 1e30f));
+        if (in && !form) keep(lane, c, Cp[(int64_t)lane * un.ldc + c]);
+        const uint32_t left = __ballot_sync(0xffffffffu, form);
+        __syncwarp();
+        if (lane == 0) mask[c] = left;
+      }
+      __syncthreads();
+      total = listed();
+    }
+    // `ways` warps an element, each some of its segments
+    const int ways = total > 4 ? 1 : total > 2 ? 2 : total > 1 ? 4 : 8;
+    const int way = warp % ways;
+    for (int e0 = 0; e0 < total; e0 += kFixWarps / ways) {
+      const int e = e0 + warp / ways;
+      int c = 0, left = min(e, total - 1);
+      while (left >= __popc(mask[c])) left -= __popc(mask[c++]);
+      uint32_t bits = mask[c];
+      for (; left > 0; --left) bits &= bits - 1u;
+      const int r = __ffs(bits) - 1;
+      const int64_t m = un.m0 + row0 + r, n = un.n0 + n0 + c;
+      double acc = 0.0, rest = 0.0;
+      for (int g = e < total ? way : un.nseg; g < un.nseg; g += ways) {
+        const SlSeg q = segs[un.seg0 + g];
+        const double* a = A + q.offA + (src.ta ? m : m * q.lda);
+        const double* b = B + q.offB + (src.tb ? n * q.ldb : n);
+        const int64_t da = src.ta ? q.lda : 1, db = src.tb ? 1 : q.ldb;
+        double s0 = 0.0, l0 = 0.0;
+        if (force) {
+          for (int k = lane; k < q.K; k += 32) s0 = dot2(a[k * da], b[k * db], s0, l0);
+          acc = dot2(q.scale, s0, acc, rest);
+          rest = fma(q.scale, l0, rest);
+        } else {
+#pragma unroll 4
+          for (int k = lane; k < q.K; k += 32) s0 = fma(a[k * da], b[k * db], s0);
+          acc = fma(q.scale, s0, acc);
+        }
+      }
+      if (fabs(rest) < 1e308) acc += rest;      // (Inf and NaN: the plain sum)
+      for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+      if (ways > 1) {
+        __syncthreads();
+        if (lane == 0) s_sum[warp] = acc;
+        __syncthreads();
+        for (int x = 1; x < ways; ++x) acc += s_sum[min(warp + x, kFixWarps - 1)];
+      }
+      if (lane == 0 && way == 0 && e < total) {
+        const double v = src.scale * acc;
+        Cp[(int64_t)r * un.ldc + c] = v;
+        keep(r, c, v);
+      }
+    }
+  }
+}
+
 // ---- slicing -----------------------------------------------------------------------
 // One CTA per 8 rows of a scale group (the packed blocks that share row
 // scales): the largest exponent of every row over all blocks of the group,
@@ -585,63 +806,81 @@ __global__ void __launch_bounds__(kThreads, 1)
 // scale and cut into digits.  All operands of a stage that are at hand are
 // sliced by one launch.
 
-// Significand and exponent field of coef * x: |coef x| = m 2^(f - 1075)
-// (m < 2^53) when the coefficient is a power of two, else m 2^(f - 1086)
-// with m < 2^64 (the upper 64 bits of the product of the significands).
+// A coefficient: |c| = m 2^(f - 1086) with its significand m normalised to 64 bits
+// (a subnormal one too).
 struct Coef {
-  unsigned long long m;   // significand << 11
-  int f;                  // exponent field
+  unsigned long long m;
+  int f;                  // exponent field (below 1 for a subnormal)
   bool pow2, neg, bad;
 };
 __device__ __forceinline__ Coef make_coef(double c) {
   Coef r;
   const unsigned long long b = (unsigned long long)__double_as_longlong(c);
   int f = (int)((b >> 52) & 0x7FF);
-  unsigned long long m = b & 0xFFFFFFFFFFFFFull;
+  unsigned long long m = b << 12 >> 1;               // (bit 63: the leading one)
   r.neg = (b >> 63) != 0;
   r.bad = f == 0x7FF;
-  if (f) m |= 1ull << 52;
-  else f = 1;
-  r.pow2 = m == (1ull << 52);
-  r.m = m << 11;
+  if (f) {
+    m |= 1ull << 63;
+  } else {
+    const int z = __clzll((long long)m);             // 64 for a zero
+    f = 1 - z;
+    m = z < 64 ? m << z : 0ull;
+  }
+  r.pow2 = m == (1ull << 63);
+  r.m = m;
   r.f = f;
   return r;
 }
 
-// Effective exponent field of coef * x (see slice digits); kMin for a zero.
+// Effective exponent field of coef * x 2^d, which is below 2^(field - 1022); kMinField
+// for a zero.
 constexpr int kMinField = -1000000;
-__device__ __forceinline__ int eff_field(double x, const Coef& c) {
+__device__ __forceinline__ int eff_field(double x, const Coef& c, int d) {
   const unsigned long long b = (unsigned long long)__double_as_longlong(x);
   const int f = (int)((b >> 52) & 0x7FF);
   if (f == 0x7FF) return kSlSpecial;
-  if ((b << 1) == 0ull) return kMinField;
-  return (f ? f : 1) + c.f - (c.pow2 ? 1023 : 1022);
+  if ((b << 1) == 0ull || c.m == 0ull) return kMinField;
+  return (f ? f : 1) + c.f + d - (c.pow2 ? 1023 : 1022);
 }
 
-// The seven digits of coef * x relative to the row field F, biased by 256 each
-// and packed in one 64-bit word (digit i in bits 54 - 9 i ..; digit 0 takes 10).
-__device__ __forceinline__ unsigned long long digits(double x, const Coef& c, int F) {
+// The eight digits of coef * x 2^d relative to the row field F, biased by 256 each:
+// digit 0 (10 bits) returned, digits 1-7 in *low, digit i in bits 63 - 9 i ...  The
+// significand (of the product: its upper 64 bits) is shifted to the 71 bits below
+// 2^(F - 1022).
+__device__ __forceinline__ uint32_t digits(double x, const Coef& c, int d, int F, unsigned long long* low) {
   constexpr unsigned long long kBias = (256ull << 54) | (256ull << 45) | (256ull << 36) |
                                        (256ull << 27) | (256ull << 18) | (256ull << 9) | 256ull;
   const unsigned long long b = (unsigned long long)__double_as_longlong(x);
   int f = (int)((b >> 52) & 0x7FF);
   unsigned long long m = b & 0xFFFFFFFFFFFFFull;
-  if (f) m |= 1ull << 52;
-  else f = 1;
-  unsigned long long t;
-  int s;
-  if (c.pow2) {
-    t = m << 9;
-    s = F - (f + c.f - 1023);
+  if (f) {
+    m = (m | 1ull << 52) << 11;
   } else {
-    t = __umul64hi(m << 11, c.m);
-    s = F - (f + c.f - 1022) + 2;
+    const int z = __clzll((long long)m);
+    m = z < 64 ? m << z : 0ull;
+    f = 12 - z;
   }
-  unsigned long long v = 0;
-  if (s <= 0) v = t;
-  else if (s < 64) v = (t >> s) + ((t >> (s - 1)) & 1ull);   // to nearest, half away from zero
-  const bool neg = ((b >> 63) != 0) != c.neg;
-  return kBias + (neg ? 0ull - v : v);
+  if (!c.pow2) m = __umul64hi(m, c.m);
+  const int s = F - (f + c.f + d - (c.pow2 ? 1023 : 1022));      // v = m 2^7 >> s
+  unsigned long long lo = 0;
+  uint32_t hi = 0;
+  if (s <= 7) {
+    const int l = 7 - max(s, 0);
+    lo = m << l;
+    hi = (uint32_t)((m >> 32) >> (32 - l));                        // l <= 7
+  } else if (s < 72) {
+    const unsigned long long t = m >> (s - 8);                     // to nearest, half away from zero
+    lo = (t >> 1) + (t & 1ull);
+  }
+  if (((b >> 63) != 0) != c.neg) {
+    lo = 0ull - lo;
+    hi = ~hi + (lo == 0ull ? 1u : 0u);
+  }
+  lo += kBias;
+  hi += 128u + (lo < kBias ? 1u : 0u);
+  *low = lo;
+  return hi << 1 | (uint32_t)(lo >> 63);
 }
 
 constexpr int kTRow = 66;      // doubles per row of a transposed tile (64 + 2 pad)
@@ -681,16 +920,17 @@ __device__ __forceinline__ void load_tile(const double* src, int64_t ld, int K, 
 // The digits of row r of a tile (its scale f; zero: no digits): this lane's
 // pair of k, 4 bytes of the swizzled 16-byte piece lane / 4 of every slice.
 __device__ __forceinline__ void store_row(uint16_t* base, int64_t slice, int r, double x0, double x1,
-                                          const Coef& cf, bool zero, int f, int lane) {
-  const unsigned long long d0 = digits(zero ? 0.0 : x0, cf, zero ? 0 : f);
-  const unsigned long long d1 = digits(zero ? 0.0 : x1, cf, zero ? 0 : f);
+                                          const Coef& cf, int2 d, bool zero, int f, int lane) {
+  unsigned long long d0, d1;
+  const uint32_t t0 = digits(zero ? 0.0 : x0, cf, d.x, zero ? 0 : f, &d0);
+  const uint32_t t1 = digits(zero ? 0.0 : x1, cf, d.y, zero ? 0 : f, &d1);
   uint16_t* row = base + r * 64 + (((lane >> 2) ^ r) << 3) + 2 * (lane & 3);
 #pragma unroll
   for (int i = 0; i < kSlices; ++i) {
     // digit + 256 in 0 .. 512: as FP16, 1024 + (digit + 256) has these bits
     // exactly; one packed subtraction of 1280 leaves the digits
-    const uint32_t f0 = (uint32_t)(d0 >> (54 - 9 * i)) & (i == 0 ? 0x3FFu : 0x1FFu);
-    const uint32_t f1 = (uint32_t)(d1 >> (54 - 9 * i)) & (i == 0 ? 0x3FFu : 0x1FFu);
+    const uint32_t f0 = i == 0 ? t0 : (uint32_t)(d0 >> (63 - 9 * i)) & 0x1FFu;
+    const uint32_t f1 = i == 0 ? t1 : (uint32_t)(d1 >> (63 - 9 * i)) & 0x1FFu;
     const uint32_t hw = (f0 | (f1 << 16)) | 0x64006400u;
     uint32_t res;
     asm("sub.rn.f16x2 %0, %1, %2;" : "=r"(res) : "r"(hw), "r"(0x65006500u));
@@ -711,15 +951,16 @@ __device__ __forceinline__ int member_of(const SlMember* __restrict__ m, int nm,
   return n - 1;
 }
 
-__global__ void __launch_bounds__(256, 3)
+constexpr int kSliceWarps = 8;
+__global__ void __launch_bounds__(32 * kSliceWarps, 3)
     slice_kernel(const SlGroup* __restrict__ groups, const int32_t* __restrict__ cta_group,
-                 const SlMember* __restrict__ members, int cta0,
+                 const SlMember* __restrict__ members,
                  const __grid_constant__ SlOperands ops) {
   grid_next();
   grid_wait();
   __shared__ int smax[8];
-  __shared__ double tr[8][8 * kTRow];
-  const int cta = cta0 + (int)blockIdx.x;
+  __shared__ double tr[kSliceWarps * 8 * kTRow];
+  const int cta = (int)blockIdx.x;
   const SlGroup gr = groups[cta_group[cta]];
   const SlOperand op = ops.op[gr.which];
   const SlMember* mem = members + gr.m0;
@@ -727,11 +968,22 @@ __global__ void __launch_bounds__(256, 3)
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   for (int i = (int)(blockIdx.x * blockDim.x + threadIdx.x); i < ops.nclear; i += (int)(gridDim.x * blockDim.x))
     ops.clear[i] = 0;
+  if (blockIdx.x == 0 && (int)threadIdx.x < ops.nfix) ops.fix[threadIdx.x] = 0;
   if (threadIdx.x < 8) smax[threadIdx.x] = kMinField;
   __syncthreads();
   auto load = [&](const SlMember& mb, int t, double (&x)[16]) {
     load_tile(op.src + mb.src + (mb.trans ? (int64_t)r0 : (int64_t)r0 * mb.ld), mb.ld, mb.K, mb.trans, nr,
-              t - mb.t0, lane, tr[warp], x);
+              t - mb.t0, lane, tr + warp * 8 * kTRow, x);
+  };
+  // the grading of this lane's two k
+  auto grading = [&](const SlMember& mb, int t) {
+    const int k = (t - mb.t0) * 64 + 2 * lane;
+    int2 d = make_int2(0, 0);
+    if (mb.d0 >= 0 && op.d) {
+      if (k < mb.K) d.x = op.sign * op.d[mb.d0 + k];
+      if (k + 1 < mb.K) d.y = op.sign * op.d[mb.d0 + k + 1];
+    }
+    return d;
   };
   double x[16];
   if (nr > 0) {
@@ -739,14 +991,15 @@ __global__ void __launch_bounds__(256, 3)
 #pragma unroll
     for (int r = 0; r < 8; ++r) mx[r] = kMinField;
     // the warp's chunks, the last one first: the first stays in registers
-    const int last = gr.nt > warp ? warp + (gr.nt - 1 - warp) / 8 * 8 : -1;
-    for (int t = last; t >= 0; t -= 8) {
+    const int last = gr.nt > warp ? warp + (gr.nt - 1 - warp) / kSliceWarps * kSliceWarps : -1;
+    for (int t = last; t >= 0; t -= kSliceWarps) {
       const SlMember mb = mem[member_of(mem, gr.nm, t, lane)];
       const Coef cf = make_coef(mb.coef * op.scale);
+      const int2 d = grading(mb, t);
       load(mb, t, x);
 #pragma unroll
       for (int e = 0; e < 16; ++e)
-        mx[e >> 1] = max(mx[e >> 1], cf.bad ? kSlSpecial : eff_field(x[e], cf));
+        mx[e >> 1] = max(mx[e >> 1], cf.bad ? kSlSpecial : eff_field(x[e], cf, e & 1 ? d.y : d.x));
     }
 #pragma unroll
     for (int r = 0; r < 8; ++r) {
@@ -757,19 +1010,67 @@ __global__ void __launch_bounds__(256, 3)
   __syncthreads();
   if ((int)threadIdx.x < nr) {
     const int v = smax[threadIdx.x];
-    op.scales[gr.e0 + r0 + threadIdx.x] = v == kMinField ? 0 : v;
+    op.scales[gr.e0 + r0 + threadIdx.x] = v == kMinField ? 0 : v == kSlSpecial ? v : v + kSlBias;
   }
-  for (int t = warp; t < gr.nt; t += 8) {
+  for (int t = warp; t < gr.nt; t += kSliceWarps) {
     const SlMember mb = mem[member_of(mem, gr.nm, t, lane)];
     const Coef cf = make_coef(mb.coef * op.scale);
+    const int2 d = grading(mb, t);
     if (t != warp || nr <= 0) load(mb, t, x);
     uint16_t* base = op.out + mb.dst + ((int64_t)(t - mb.t0) * kSlices * gr.R8 + (r0 >> 3)) * kSlTile;
 #pragma unroll
     for (int r = 0; r < 8; ++r) {
       const int f = smax[r];             // zero rows and rows with Inf or NaN have no digits
-      store_row(base, (int64_t)gr.R8 * kSlTile, r, x[2 * r], x[2 * r + 1], cf,
+      store_row(base, (int64_t)gr.R8 * kSlTile, r, x[2 * r], x[2 * r + 1], cf, d,
                 f == kMinField || f == kSlSpecial, f + gr.shift, lane);
     }
+  }
+}
+
+// Grading.  The rows of a site tensor carry the Schmidt weights of the bond that the
+// product sums over; in the environment's identity channels only one term of a sum is
+// not zero, and the terms of small weight would be held with few digits beside the
+// others of their column.  So the site tensor's row k is taken as 2^-d_k and the
+// environment's column as 2^d_k, exactly, with d_k the exponent of the largest element
+// (of a sample) of the site tensor at k; and in the same way the stage-2 output of H_eff, whose
+// columns carry the weights of the other bond, and the second environment.  (With any d the results are right; without one, the
+// fix launch would form most of a graded tensor's copies.)  A sample of 32 elements a
+// block makes it one load latency and a little: 3 us.
+__global__ void __launch_bounds__(256)
+    grade_kernel(const SlGrade* __restrict__ items, const SlView* __restrict__ views, const double* src,
+                 int32_t* d) {
+  grid_next();
+  grid_wait();
+  __shared__ int best[32];
+  const SlGrade it = items[blockIdx.x];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (threadIdx.x < 32) best[threadIdx.x] = 0;
+  __syncthreads();
+  // (32 elements of every view and k are enough to see the weights)
+  for (int v = 0; v < it.nv; ++v) {
+    const SlView w = views[it.v0 + v];
+    double x[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int k = w.trans ? warp + 8 * i : lane;
+      const int64_t r = (int64_t)(w.trans ? lane : warp + 8 * i) * max(w.R, 32) / 32;
+      x[i] = k < it.nk && r < w.R ? src[w.src + (w.trans ? k * (int64_t)w.ld + r : r * w.ld + k)] : 0.0;
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int f = exponent_of(x[i]);
+      if (w.trans) {
+        const int m = __reduce_max_sync(0xffffffffu, f);
+        if (lane == 0) atomicMax(&best[warp + 8 * i], m);
+      } else if (f) {
+        atomicMax(&best[lane], f);
+      }
+    }
+  }
+  __syncthreads();
+  if ((int)threadIdx.x < it.nk) {
+    const int f = best[threadIdx.x];
+    d[it.d0 + threadIdx.x] = f == 0 || f == 0x7FF ? 0 : f - 1022;
   }
 }
 
@@ -778,7 +1079,7 @@ __global__ void __launch_bounds__(256, 3)
 __global__ void __launch_bounds__(256)
     slice_known_kernel(const SlPiece* __restrict__ pieces, int npieces,
                        const int32_t* __restrict__ first, int ntiles, const double* src,
-                       uint16_t* out, const int32_t* scales) {
+                       uint16_t* out, const int32_t* scales, const int32_t* d) {
   grid_next();
   grid_wait();
   __shared__ double tr[8][8 * kTRow];
@@ -791,6 +1092,12 @@ __global__ void __launch_bounds__(256)
   const int local = t - p.tile0, c = local / p.R8, g = local - c * p.R8;
   const int r0 = g * 8, nr = min(8, p.R - r0);
   const int fl = lane < nr ? scales[p.e0 + r0 + lane] : 0;
+  const int k = c * 64 + 2 * lane;
+  int2 dk = make_int2(0, 0);
+  if (p.d0 >= 0) {
+    if (k < p.K) dk.x = -d[p.d0 + k];
+    if (k + 1 < p.K) dk.y = -d[p.d0 + k + 1];
+  }
   double x[16];
   load_tile(src + p.src + (p.trans ? (int64_t)r0 : (int64_t)r0 * p.ld), p.ld, p.K, p.trans, nr, c, lane,
             tr[warp], x);
@@ -799,31 +1106,39 @@ __global__ void __launch_bounds__(256)
 #pragma unroll
   for (int r = 0; r < 8; ++r) {
     const int f = __shfl_sync(0xffffffffu, fl, r);
-    store_row(base, (int64_t)p.R8 * kSlTile, r, x[2 * r], x[2 * r + 1], cf, f == 0 || f == kSlSpecial,
-              f + p.shift, lane);
+    store_row(base, (int64_t)p.R8 * kSlTile, r, x[2 * r], x[2 * r + 1], cf, dk, f == 0 || f == kSlSpecial,
+              f - kSlBias + p.shift, lane);
   }
 }
 
 }  // namespace
 
-void launch_slice(const SlGroup* groups, const int32_t* cta_group, int cta0, int nctas,
+void launch_slice(const SlGroup* groups, const int32_t* cta_group, int nctas,
                   const SlMember* members, const SlOperands& ops, cudaStream_t st) {
   if (nctas <= 0) return;
   count_launch();
-  launch_chain(slice_kernel, nctas, 256, 0, st, groups, cta_group, members, cta0, ops);
+  launch_chain(slice_kernel, nctas, 32 * kSliceWarps, 0, st, groups, cta_group, members, ops);
+}
+
+void launch_grade(const SlGrade* items, int nitems, const SlView* views, const double* src, int32_t* d,
+                  cudaStream_t st) {
+  if (nitems <= 0) return;
+  count_launch();
+  launch_chain(grade_kernel, nitems, 256, 0, st, items, views, src, d);
 }
 
 void launch_slice_known(const SlPiece* pieces, int npieces, const int32_t* first, int ntiles,
-                        const double* src, uint16_t* out, const int32_t* scales, cudaStream_t st) {
+                        const double* src, uint16_t* out, const int32_t* scales, const int32_t* d,
+                        cudaStream_t st) {
   if (ntiles <= 0) return;
   count_launch();
-  launch_chain(slice_known_kernel, (ntiles + 7) / 8, 256, 0, st, pieces, npieces, first, ntiles, src, out, scales);
+  launch_chain(slice_known_kernel, (ntiles + 7) / 8, 256, 0, st, pieces, npieces, first, ntiles, src, out, scales, d);
 }
 
 void launch_gemm_sliced(const SlTables& t, const uint16_t* pA, const uint16_t* pB,
                         const int32_t* eA, const int32_t* eB, const SlSource& src, double* C,
-                        int32_t* collect, bool collect_cols, int* err, uint64_t wait_ns,
-                        cudaStream_t st) {
+                        int32_t* collect, bool collect_cols, const int32_t* d, const SlFix& fix, int* err,
+                        uint64_t wait_ns, cudaStream_t st) {
   if (t.ncta <= 0) return;
   // the shared-memory limit is a per-device attribute of the kernel
   static std::atomic<uint64_t> done{0};
@@ -835,9 +1150,15 @@ void launch_gemm_sliced(const SlTables& t, const uint16_t* pA, const uint16_t* p
                          kSmemBytes);
     if (bit) done.fetch_or(bit);
   }
-  count_launch();
-  const PlainLaunches plain(!t.chain);
-  launch_chain(gemm_sliced_kernel, t.ncta, kThreads, kSmemBytes, st, t, pA, pB, eA, eB, src, C, collect, collect_cols ? 1 : 0, err, wait_ns);
+  count_launch(2);
+  {
+    const PlainLaunches plain(!t.chain);
+    launch_chain(gemm_sliced_kernel, t.ncta, kThreads, kSmemBytes, st, t, pA, pB, eA, eB, C, collect,
+                 collect_cols ? 1 : 0, d, fix, err, wait_ns);
+  }
+  const int64_t parts = (int64_t)t.nunits * kSlParts;
+  launch_chain(fix_kernel, (unsigned)std::min<int64_t>(parts, kFixCtas), kFixThreads, 0, st, t.units, t.segs, fix,
+               eA, eB, src, C, collect, collect_cols ? 1 : 0, d);
 }
 
 }  // namespace dmrg3s

@@ -502,6 +502,7 @@ struct Slicer {
     b.m.K = (int32_t)K;
     b.m.KC = (int32_t)((K + 63) / 64);
     b.m.trans = trans;
+    b.m.d0 = -1;
     b.R = (int32_t)R;
     const int id = (int)blks.size();
     blks.push_back(b);
@@ -546,8 +547,73 @@ struct Slicer {
   }
 };
 
-// Sliced form of a stage: GemmSeg.scale is the coefficient of A (coefA) or B.
-bool build_sliced(const GemmStage& g, bool coefA, SlStage* out, std::string* err) {
+// The bound below which a sum of K terms is listed (kernels_sliced.cu): 3 2^54
+// sqrt(K) 0.95 2^-72 of the scales, in units of 2^32 H (2^-20 of the scales).
+constexpr double kSlLeast = 3.0 * 0.95 * 4.0;
+
+// Views of the site tensor along the k of a block (by its source offset): what the
+// grading of those k is taken from.
+using GradeViews = std::map<int64_t, std::vector<SlView>>;
+
+// The grading of the blocks that meet along k (grade_kernel): blocks of A and B in one
+// segment share it, so the classes are the sectors of the contracted bond.  The
+// views are those of A's blocks (of_a) or of B's.
+bool grade_blocks(const GemmStage& g, const std::vector<int>& ia, const std::vector<int>& ib, bool of_a,
+                  const GradeViews& from, Slicer* a, Slicer* b, std::vector<SlGrade>* items,
+                  std::vector<SlView>* views, int32_t* n, std::string* err) {
+  const int na = (int)a->blks.size();
+  std::vector<int> parent(na + b->blks.size());
+  for (size_t i = 0; i < parent.size(); ++i) parent[i] = (int)i;
+  auto find = [&](int i) {
+    while (parent[i] != i) i = parent[i] = parent[parent[i]];
+    return i;
+  };
+  for (size_t k = 0; k < g.segs.size(); ++k) {
+    const int x = find(ia[k]), y = find(na + ib[k]);
+    parent[std::max(x, y)] = std::min(x, y);
+  }
+  auto member = [&](int i) -> SlMember& { return i < na ? a->blks[i].m : b->blks[i - na].m; };
+  std::vector<int32_t> d0(parent.size(), -1);
+  std::vector<std::vector<SlView>> site(parent.size());
+  for (int i = 0; i < (int)parent.size(); ++i) {
+    const int r = find(i);
+    if (d0[r] < 0) {
+      d0[r] = *n;
+      *n += member(i).K;
+    }
+    if (member(i).K != member(r).K) {
+      *err = "sliced stage: blocks of unequal length share a grading";
+      return false;
+    }
+    member(i).d0 = d0[r];
+    if ((i < na) == of_a) {
+      const auto it = from.find(member(i).src);
+      if (it != from.end()) site[r].insert(site[r].end(), it->second.begin(), it->second.end());
+    }
+  }
+  for (size_t r = 0; r < site.size(); ++r) {
+    if (d0[r] < 0) continue;
+    // (a block of the site tensor may be seen through several blocks)
+    std::vector<SlView>& v = site[r];
+    std::sort(v.begin(), v.end(), [](const SlView& x, const SlView& y) { return x.src < y.src; });
+    v.erase(std::unique(v.begin(), v.end(), [](const SlView& x, const SlView& y) { return x.src == y.src; }),
+            v.end());
+    const int K = member((int)r).K;
+    for (int k = 0; k < K; k += 32) {
+      items->push_back(SlGrade{d0[r] + k, std::min(32, K - k), (int32_t)views->size(), (int32_t)v.size()});
+      for (SlView w : v) {
+        w.src += w.trans ? (int64_t)k * w.ld : k;
+        views->push_back(w);
+      }
+    }
+  }
+  return true;
+}
+
+// Sliced form of a stage: GemmSeg.scale is the coefficient of A (coefA) or B.  With
+// `grade`, the blocks take a grading from these views of A's (of_a) or B's blocks.
+bool build_sliced(const GemmStage& g, bool coefA, Plan* grade, bool of_a, const GradeViews& from, SlStage* out,
+                  std::string* err) {
   SlStage& s = *out;
   s = SlStage();
   Slicer a, b;
@@ -578,6 +644,8 @@ bool build_sliced(const GemmStage& g, bool coefA, SlStage* out, std::string* err
       *err = "sliced stage: blocks of unequal rows share scales";
       return false;
     }
+  if (grade && !grade_blocks(g, ia, ib, of_a, from, &a, &b, &grade->grades, &grade->views, &grade->ngrade, err))
+    return false;
   std::vector<int32_t> ea, eb;
   a.layout(true, &s.gA, &s.mA, &s.nA, &s.neA, &ea);
   b.layout(false, &s.gB, &s.mB, &s.nB, &s.neB, &eb);
@@ -590,24 +658,43 @@ bool build_sliced(const GemmStage& g, bool coefA, SlStage* out, std::string* err
   };
   int tile_n = 64;
   while (tile_n > 16 && count(tile_n - 16) <= plan_ctas()) tile_n -= 16;
-  std::vector<TcUnit> units;
-  std::vector<double> cost;
-  for (const GemmTask& t : g.tasks) {
+  // cycles of a unit of nw columns: the MMAs of the 36 digit products (max(100, N / 2)
+  // each, up to 256 columns in one), against the slabs' copies at ~48 B per cycle;
+  // then the drains and the store
+  const auto unit_cost = [&](const GemmTask& t, int tm, int nw) {
+    double mma = 0.0;
+    for (int i = 0; i < kSlices; ++i) {
+      const int all = kSlices - i, n1 = i == 0 ? 4 : all * nw > 256 ? 3 : all;
+      mma += std::max(100.0, 0.5 * n1 * nw) + (n1 < all ? std::max(100.0, 0.5 * (all - n1) * nw) : 0.0);
+    }
     int steps = 0, chunks = 0;
     for (int k = 0; k < t.nseg; ++k) {
       steps += (g.segs[t.seg0 + k].K + 15) / 16;
       chunks += (g.segs[t.seg0 + k].K + 63) / 64;
     }
-    const int id = (int)(&t - g.tasks.data());
+    const int ga = std::min(16, Slicer::groups(t.M) - tm * 16);
+    const double copy = chunks * (double)kSlices * 1024.0 * (ga + nw / 8) / 48.0;
+    return std::max(std::max(mma * steps, copy), 2200.0 * chunks) + 3000.0;
+  };
+  // a task that would keep its SMs busy for longer than the others take in all gets
+  // narrower units, down to 32 columns (H_eff: the block that sums every channel has
+  // eight times the terms of the others)
+  double total = 0.0;
+  for (const GemmTask& t : g.tasks)
+    total += unit_cost(t, 0, tile_n) * ((t.M + 127) / 128) * ((t.N + tile_n - 1) / tile_n);
+  std::vector<int> tile(g.tasks.size(), tile_n);
+  for (size_t i = 0; i < g.tasks.size(); ++i)
+    while (tile[i] > 32 && unit_cost(g.tasks[i], 0, std::min(tile[i], (g.tasks[i].N + 15) / 16 * 16)) >
+                               1.2 * total / plan_ctas())
+      tile[i] -= 16;
+  std::vector<TcUnit> units;
+  std::vector<double> cost;
+  for (const GemmTask& t : g.tasks) {
+    const int id = (int)(&t - g.tasks.data()), tn = tile[id];
     for (int i = 0; i < (t.M + 127) / 128; ++i)
-      for (int j = 0; j < (t.N + tile_n - 1) / tile_n; ++j) {
+      for (int j = 0; j < (t.N + tn - 1) / tn; ++j) {
         units.push_back(TcUnit{id, i, j, 0});
-        // cycles: 14 per column and k16 step of the 28 digit products, against
-        // the slabs' copies at ~48 B per cycle; then the drains and the store
-        const int nw = std::min(tile_n, (t.N + 15) / 16 * 16 - j * tile_n);
-        const int ga = std::min(16, Slicer::groups(t.M) - i * 16);
-        const double mma = 14.0 * nw * steps, copy = chunks * 7.0 * 1024.0 * (ga + nw / 8) / 48.0;
-        cost.push_back(std::max(std::max(mma, copy), 2200.0 * chunks) + 3000.0);
+        cost.push_back(unit_cost(t, i, std::min(tn, (t.N + 15) / 16 * 16 - j * tn)));
       }
   }
   std::vector<int32_t> cta;
@@ -622,12 +709,14 @@ bool build_sliced(const GemmStage& g, bool coefA, SlStage* out, std::string* err
       const GemmTask& t = g.tasks[units[ui].task];
       SlUnit un{};
       un.em = -1;
+      un.d0 = -1;
       un.m0 = units[ui].tm * 128;
-      un.n0 = units[ui].tn * tile_n;
+      const int tn = tile[units[ui].task];
+      un.n0 = units[ui].tn * tn;
       un.offC = t.offC + (int64_t)un.m0 * t.ldc + un.n0;
       un.ldc = t.ldc;
       un.rows = std::min(128, t.M - un.m0);
-      un.cols = std::min(tile_n, t.N - un.n0);
+      un.cols = std::min(tn, t.N - un.n0);
       un.nw = (un.cols + 15) / 16 * 16;
       un.seg0 = t.seg0;
       un.nseg = t.nseg;
@@ -636,6 +725,9 @@ bool build_sliced(const GemmStage& g, bool coefA, SlStage* out, std::string* err
         un.eb = eb[ib[t.seg0]] + un.n0;
         un.shift = a.blks[a.find(ia[t.seg0])].shift;
       }
+      int64_t terms = 0;
+      for (int k = 0; k < t.nseg; ++k) terms += g.segs[t.seg0 + k].K;
+      un.least = (uint32_t)std::ceil(kSlLeast * std::sqrt((double)terms));
       const int ra8 = Slicer::groups(t.M), rb8 = Slicer::groups(t.N);
       const size_t first = s.words.size();
       int used = 0;
@@ -782,7 +874,7 @@ void rechunk(CombStage& c) {
 // every unit of stage 2 collects its row scales (EnvLR: its columns' scales).
 bool plan_t2(Plan* p, const std::vector<SlGroup>& groups, const std::vector<SlMember>& members,
              std::string* err) {
-  std::map<int64_t, int32_t> e0;       // block offset -> its first row scale
+  std::map<int64_t, int32_t> e0, d0;   // block offset -> its first row scale, grading entry
   for (const SlGroup& g : groups)
     for (int k = 0; k < g.nm; ++k) {
       const SlMember& m = members[g.m0 + k];
@@ -797,9 +889,11 @@ bool plan_t2(Plan* p, const std::vector<SlGroup>& groups, const std::vector<SlMe
       q.R8 = g.R8;
       q.e0 = g.e0;
       q.shift = g.shift;
+      q.d0 = m.d0;
       q.tile0 = p->t2_tiles;
       p->t2_tiles += g.R8 * m.KC;
       p->t2.push_back(q);
+      d0[m.src] = m.d0;
       if (!e0.emplace(m.src, g.e0).second) {
         *err = "sliced stage: a stage-2 block with two sets of scales";
         return false;
@@ -815,8 +909,10 @@ bool plan_t2(Plan* p, const std::vector<SlGroup>& groups, const std::vector<SlMe
     // the unit's block: its offset less the unit's place in it
     const auto it = e0.find(u.offC - (int64_t)u.m0 * u.ldc - u.n0);
     u.em = it == e0.end() ? -1 : it->second + (cols ? u.n0 : u.m0);
+    // (a graded operand: A of H_eff, whose k are the block's columns)
+    u.d0 = it == e0.end() || d0[it->first] < 0 ? -1 : d0[it->first] + u.n0;
     const int32_t ne = p->kind == Kind::Heff ? p->s3.neA : p->s3.neB;
-    if (u.em >= 0 && u.em + (cols ? u.cols : u.rows) > ne) {
+    if (u.em >= 0 && (u.em + (cols ? u.cols : u.rows) > ne || (u.d0 >= 0 && u.d0 + u.cols > p->ngrade))) {
       *err = "sliced stage: collected scales out of bounds";
       return false;
     }
@@ -824,12 +920,27 @@ bool plan_t2(Plan* p, const std::vector<SlGroup>& groups, const std::vector<SlMe
   return true;
 }
 
-// Least algorithmic work of a contraction that takes the sliced form, whose time
-// hardly falls below 35 us.  Prepared operators, plain against sliced: XXZ m = 200
-// (10 Mflop) 31 and 37 us, m = 256 (22) 47 and 44, m = 512 (177) 220 and 67; one
-// block, m = 64 (9.5) 25 and 34, m = 96 (32) 53 and 46; Hubbard m = 400 (7) 23 and
-// 42, m = 700 (38) 65 and 53.  Gradients: 11 Mflop 38 and 36, 25 Mflop 59 and 44.
-constexpr double kSlicedMinFlops = 16e6;
+// Least work of a contraction that takes the sliced form, whose time hardly falls
+// below 60 us: flops that fill the products' tiles (128 rows, 16 columns, 16 k; a
+// sector of 40 states wastes two thirds of them).  Plain against sliced calls (us; Mflop,
+// the share that fills): operators, XXZ m = 256 (22, 0.26) 47 and 83, m = 320 (43, 0.34)
+// 78 and 94, m = 400 (84, 0.50) 119 and 99, m = 512 (177, 0.53) 219 and 118; Hubbard m = 700
+// (38, 0.34) 65 and 98, m = 1024 (127, 0.48) 163 and 117; one block, m = 96 (32, 0.75) 52 and
+// 80, m = 128 (76, 1) 93 and 83.  Expansions, Hubbard m = 700 (19, 0.35) 36 and 55, m = 1024 (64,
+// 0.5) 86 and 68; gradients, Hubbard m = 700 (37) 99 and 103, m = 1024 (126) 225 and 168.
+constexpr double kSlicedMinFlops = 11e6;
+double tile_fill(const GemmStage& g, const GemmStage* h) {
+  double work = 0.0, tiles = 0.0;
+  for (const GemmStage* s : {&g, h})
+    if (s)
+      for (const GemmTask& t : s->tasks)
+        for (int k = 0; k < t.nseg; ++k) {
+          const double K = s->segs[t.seg0 + k].K;
+          work += (double)t.M * t.N * K;
+          tiles += std::ceil(t.M / 128.0) * 128.0 * std::ceil(t.N / 16.0) * 16.0 * std::ceil(K / 16.0) * 16.0;
+        }
+  return tiles > 0.0 ? work / tiles : 0.0;
+}
 // Largest ratio of the fused stage's work to stage 1's: the sliced products
 // run 3 (0.2 Gflop) to 16 (13 Gflop) times as fast as the plain ones; a model
 // MPO has a ratio near 1.2.  Below it, the least work grows with the ratio.
@@ -839,16 +950,31 @@ constexpr double kSlicedMaxTerms = 6.0;
 dmrg3s_status finish_sliced(Plan* p, int64_t nA1, int64_t nB1, int64_t nOut2, int64_t nA3,
                             int64_t nB3, int64_t nC3, std::string* err) {
   p->sliced = false;
-  if (p->flops() < kSlicedMinFlops) return DMRG3S_OK;
+  const double flops = p->flops() * tile_fill(p->g1, p->has_g3 ? &p->g3 : nullptr);
+  if (flops < kSlicedMinFlops) return DMRG3S_OK;
   // a dense MPO tensor: too many terms per stage-1 block to form each anew
   double terms = 0.0, blocks = 0.0;
   for (const CombTask& t : p->c2.tasks) terms += (double)t.nt * t.rows * t.cols;
   for (const GemmTask& t : p->g1.tasks) blocks += (double)t.M * t.N;
-  if (terms > kSlicedMaxTerms * blocks || p->flops() * blocks < kSlicedMinFlops * terms)
+  if (terms > kSlicedMaxTerms * blocks || flops * blocks < kSlicedMinFlops * terms)
     return DMRG3S_OK;
   const bool left = p->kind == Kind::Heff || p->kind == Kind::ExpandLR || p->kind == Kind::EnvLR;
-  bool ok = fuse_f64(*p, &p->f12, err) && build_sliced(p->f12, left, &p->s12, err) &&
-            sliced_ok(p->f12, p->s12, nA1, nB1, nOut2, err);
+  bool ok = fuse_f64(*p, &p->f12, err);
+  // the site tensor (B of the left kinds, A of the right ones): along k, and along
+  // the other index of the blocks that H_eff's stage 3 contracts
+  GradeViews along, across;
+  for (const GemmTask& t : p->f12.tasks)
+    for (int k = 0; ok && k < t.nseg; ++k) {
+      const GemmSeg& q = p->f12.segs[t.seg0 + k];
+      if (left) {
+        along[q.offB] = {SlView{q.offB, q.ldb, t.N, 1, 0}};
+        across[t.offC].push_back(SlView{q.offB, q.ldb, q.K, 0, 0});
+      } else {
+        along[q.offA] = {SlView{q.offA, q.lda, t.M, 0, 0}};
+      }
+    }
+  ok = ok && build_sliced(p->f12, left, p, !left, along, &p->s12, err) &&
+       sliced_ok(p->f12, p->s12, nA1, nB1, nOut2, p->ngrade, err);
   if (ok && p->has_g3) {
     int64_t units1 = 0;
     int maxseg = 1;
@@ -866,15 +992,15 @@ dmrg3s_status finish_sliced(Plan* p, int64_t nA1, int64_t nB1, int64_t nOut2, in
       p->f3 = p->g3;
       p->f3.tiles.clear();
     }
-    ok = ok && build_sliced(p->f3, true, &p->s3, err) &&
-         sliced_ok(p->f3, p->s3, nA3, nB3, G > 1 ? std::max<int64_t>(p->ws3s, 1) : nC3, err);
+    ok = ok && build_sliced(p->f3, true, p->kind == Kind::Heff ? p : nullptr, true, across, &p->s3, err) &&
+         sliced_ok(p->f3, p->s3, nA3, nB3, G > 1 ? std::max<int64_t>(p->ws3s, 1) : nC3, p->ngrade, err);
   }
   if (ok) {
     const bool t2_is_a = p->kind == Kind::Heff;
-    p->slices.add(left ? p->s12.gA : p->s12.gB, left ? p->s12.mA : p->s12.mB);
     p->slices.add(t2_is_a ? p->s3.gB : p->s3.gA, t2_is_a ? p->s3.mB : p->s3.mA);
+    p->slices.add(left ? p->s12.gA : p->s12.gB, left ? p->s12.mA : p->s12.mB);
     p->slices.add(left ? p->s12.gB : p->s12.gA, left ? p->s12.mB : p->s12.mA);
-    ok = slice_table_ok(p->slices, err);
+    ok = slice_table_ok(p->slices, err) && grades_ok(p->grades, p->views, left ? nB1 : nA1, p->ngrade, err);
     if (ok && p->has_g3) ok = plan_t2(p, t2_is_a ? p->s3.gA : p->s3.gB, t2_is_a ? p->s3.mA : p->s3.mB, err);
   }
   if (!ok) {
@@ -1286,15 +1412,15 @@ dmrg3s_status plan_mpo_grad(const EnvLayout& le, const MpoLayout& W, const EnvLa
   // sliced form over the virtual operand arrays A = [L | M], B = [M | R] and
   // the output [T1 | Y]; then each operand's blocks back to its own array
   p->sliced = false;
-  if (p->flops() >= kSlicedMinFlops) {
+  if (p->flops() * tile_fill(p->g1, &p->gy) >= kSlicedMinFlops) {
     const int64_t nL = le.size, nM = M.size, nR = re.size;
     GemmStage g;
     g.ta = p->g1.ta;
     g.tb = p->g1.tb;
     append_gemm(g, p->g1, 0, 0, 0);
     append_gemm(g, p->gy, nL, nM, w1);
-    bool ok = p->g1.ta == p->gy.ta && p->g1.tb == p->gy.tb && build_sliced(g, true, &p->s, err) &&
-              sliced_ok(g, p->s, nL + nM, nM + nR, w1 + wy, err);
+    bool ok = p->g1.ta == p->gy.ta && p->g1.tb == p->gy.tb && build_sliced(g, true, nullptr, false, {}, &p->s, err) &&
+              sliced_ok(g, p->s, nL + nM, nM + nR, w1 + wy, 0, err);
     auto split = [&](std::vector<SlGroup>& gs, std::vector<SlMember>& ms, int64_t n0) {
       std::vector<SlGroup> ga, gb;
       for (SlGroup q : gs) {

@@ -129,12 +129,15 @@ struct Plan {
   // term, scaled by its coefficient; the output is the stage-2 output in FP64),
   // stage 3 split-K into FP64 partial blocks and a sum (no split: written to
   // the output directly).  sliced = false: too little work (plan.cpp).
-  // slices: operand 0 = stage 1's environment (L, R), 1 = stage 3's operand that
-  // is at hand (R, M), 2 = stage 1's site tensor.  The stage-2 output is sliced
+  // slices: operand 0 = stage 3's operand that is at hand (R, M), 1 = stage 1's
+  // environment (L, R), 2 = stage 1's site tensor.  The stage-2 output is sliced
   // piece by piece (t2), its row scales collected by stage 2.
   GemmStage f12, f3;
   SlStage s12, s3;
   SliceTable slices;
+  std::vector<SlGrade> grades;     // the site tensor's grading, ngrade entries
+  std::vector<SlView> views;
+  int32_t ngrade = 0;
   std::vector<SlPiece> t2;
   std::vector<int32_t> t2_first;   // piece of every eighth tile
   int32_t t2_tiles = 0;

@@ -130,7 +130,7 @@ inline bool tc_ok(const std::vector<GemmTask>& tasks, const TcStage& tc, int64_t
 // Sliced FP64 tables: every source view, packed block, row scale, bulk copy and
 // output inside its array.
 inline bool slices_ok(const std::vector<SlGroup>& g, const std::vector<SlMember>& m, int64_t nSrc,
-                      int64_t nPacked, int32_t ne, std::string* err) {
+                      int64_t nPacked, int32_t ne, int32_t ngrade, std::string* err) {
   for (const SlGroup& q : g) {
     bool ok = q.R > 0 && q.R8 * 8 >= q.R && q.R8 % 2 == 0 && q.m0 >= 0 && q.nm > 0 &&
               (size_t)q.m0 + q.nm <= m.size() && q.e0 >= 0 && q.e0 + q.R <= ne && q.shift >= 0 &&
@@ -142,7 +142,8 @@ inline bool slices_ok(const std::vector<SlGroup>& g, const std::vector<SlMember>
                                    : (int64_t)(q.R - 1) * b.ld + b.K - 1;
       ok = b.K > 0 && span_ok(b.src, last, nSrc) && b.ld >= (b.trans ? q.R : b.K) &&
            (int64_t)b.KC * 64 >= b.K && b.dst >= 0 && b.dst % kSlTile == 0 &&
-           b.dst + (int64_t)q.R8 * b.KC * kSlices * kSlTile <= nPacked && b.t0 == t;
+           b.dst + (int64_t)q.R8 * b.KC * kSlices * kSlTile <= nPacked && b.t0 == t &&
+           b.d0 >= -1 && (b.d0 < 0 || (int64_t)b.d0 + b.K <= ngrade);
       t += b.KC;
     }
     ok = ok && t == q.nt;
@@ -173,11 +174,30 @@ inline bool slice_table_ok(const SliceTable& t, std::string* err) {
   return true;
 }
 
+inline bool grades_ok(const std::vector<SlGrade>& g, const std::vector<SlView>& v, int64_t nSrc,
+                      int32_t ngrade, std::string* err) {
+  for (const SlGrade& q : g) {
+    bool ok = q.nk >= 1 && q.nk <= 32 && q.d0 >= 0 && (int64_t)q.d0 + q.nk <= ngrade && q.v0 >= 0 &&
+              q.nv >= 0 && (size_t)q.v0 + q.nv <= v.size();
+    for (int k = 0; ok && k < q.nv; ++k) {
+      const SlView& w = v[q.v0 + k];
+      ok = w.R > 0 && w.ld >= (w.trans ? w.R : q.nk) &&
+           span_ok(w.src, w.trans ? (int64_t)(q.nk - 1) * w.ld + w.R - 1 : (int64_t)(w.R - 1) * w.ld + q.nk - 1,
+                   nSrc);
+    }
+    if (!ok) {
+      *err = "site tensor's grading out of bounds";
+      return false;
+    }
+  }
+  return true;
+}
+
 inline bool sliced_ok(const GemmStage& g, const SlStage& s, int64_t nA, int64_t nB, int64_t nC,
-                      std::string* err) {
+                      int32_t ngrade, std::string* err) {
   if (!gemm_ok(g.ta, g.tb, g.tasks, g.segs, nA, nB, nC, err) ||
-      !slices_ok(s.gA, s.mA, nA, s.nA, s.neA, err) ||
-      !slices_ok(s.gB, s.mB, nB, s.nB, s.neB, err))
+      !slices_ok(s.gA, s.mA, nA, s.nA, s.neA, ngrade, err) ||
+      !slices_ok(s.gB, s.mB, nB, s.nB, s.neB, ngrade, err))
     return false;
   bool ok = s.segs.size() == g.segs.size() && s.words.size() == s.chunks.size() &&
             s.cta_unit.size() == s.cta_chunk.size() &&
