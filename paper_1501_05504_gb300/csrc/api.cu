@@ -40,7 +40,8 @@ void Hasher::mpo(const MpoLayout& w) {
 }
 
 DevicePlan::~DevicePlan() {
-  if (mem) cudaFree(mem);
+  for (void* p : {mem, mem_tc, mem_sl})
+    if (p) cudaFree(p);
 }
 DeviceGradPlan::~DeviceGradPlan() {
   if (mem) cudaFree(mem);
@@ -64,17 +65,41 @@ T* place(char* base, size_t* off, const std::vector<T>& v, std::vector<char>* st
   *off += bytes_of(v);
   return v.empty() ? nullptr : p;
 }
-size_t bytes_of(const SlStage& q) {
-  return bytes_of(q.segs) + bytes_of(q.units) + bytes_of(q.chunks) + bytes_of(q.words) +
-         bytes_of(q.cta_unit) + bytes_of(q.cta_chunk);
-}
-void place_sliced(char* base, size_t* off, DeviceSliced* d, const SlStage& q, std::vector<char>* staging) {
-  d->segs = place(base, off, q.segs, staging);
-  d->units = place(base, off, q.units, staging);
-  d->chunks = place(base, off, q.chunks, staging);
-  d->words = place(base, off, q.words, staging);
-  d->cta_unit = place(base, off, q.cta_unit, staging);
-  d->cta_chunk = place(base, off, q.cta_chunk, staging);
+}  // namespace
+
+namespace {
+// Lays tables out in one device allocation: the first walk adds the sizes up, the
+// second places and copies them.
+struct Tables {
+  size_t total = 0, off = 0;
+  void* mem = nullptr;
+  std::vector<char> staging;
+  template <class T>
+  void add(T** p, const std::vector<T>& v) {
+    if (!mem) total += bytes_of(v);
+    else *p = place(static_cast<char*>(mem), &off, v, &staging);
+  }
+  void add(DeviceSliced* d, const SlStage& q) {
+    add(&d->segs, q.segs);
+    add(&d->units, q.units);
+    add(&d->chunks, q.chunks);
+    add(&d->words, q.words);
+    add(&d->cta_unit, q.cta_unit);
+    add(&d->cta_chunk, q.cta_chunk);
+  }
+};
+template <class Walk>
+dmrg3s_status upload(void** mem, Walk walk) {
+  Tables t;
+  walk(t);
+  if (t.total == 0) t.total = 256;
+  if (cudaMalloc(&t.mem, t.total) != cudaSuccess) return DMRG3S_ERR_CUDA;
+  *mem = t.mem;
+  t.staging.assign(t.total, 0);
+  walk(t);
+  return cudaMemcpy(t.mem, t.staging.data(), t.total, cudaMemcpyHostToDevice) == cudaSuccess
+             ? DMRG3S_OK
+             : DMRG3S_ERR_CUDA;
 }
 }  // namespace
 
@@ -82,73 +107,83 @@ dmrg3s_status upload_plan(Plan&& host, std::unique_ptr<DevicePlan>* out) {
   std::unique_ptr<DevicePlan> dp(new (std::nothrow) DevicePlan());
   if (!dp) return DMRG3S_ERR_OOM;
   dp->host = std::move(host);
-  const Plan& h = dp->host;
-  size_t total = bytes_of(h.g1.tiles) + bytes_of(h.g1.tasks) + bytes_of(h.g1.segs) +
-                 bytes_of(h.c2.chunks) + bytes_of(h.c2.tasks) + bytes_of(h.c2.terms) +
-                 bytes_of(h.g3.tiles) + bytes_of(h.g3.tasks) + bytes_of(h.g3.segs) +
-                 bytes_of(h.g3s.tasks) + bytes_of(h.c3r.chunks) + bytes_of(h.c3r.tasks) +
-                 bytes_of(h.c3r.terms) + bytes_of(h.g1.tc.units) + bytes_of(h.g1.tc.segs) +
-                 bytes_of(h.g1.tc.packA) + bytes_of(h.g1.tc.packB) + bytes_of(h.g3s.tc.units) +
-                 bytes_of(h.g3s.tc.segs) + bytes_of(h.g3s.tc.packA) + bytes_of(h.g3s.tc.packB) +
-                 bytes_of(h.c2pack) + bytes_of(h.g12.tasks) + bytes_of(h.g12.tc.units) +
-                 bytes_of(h.g12.tc.segs) + bytes_of(h.g12.tc.packA) + bytes_of(h.g12.tc.packB) +
-                 bytes_of(h.g1.tc.cta_start) + bytes_of(h.g3s.tc.cta_start) +
-                 bytes_of(h.g12.tc.cta_start);
-  total += bytes_of(h.s12) + bytes_of(h.s3);
-  total += bytes_of(h.slices.groups) + bytes_of(h.slices.members) +
-           bytes_of(h.slices.cta_group) + bytes_of(h.grades) + bytes_of(h.views) + bytes_of(h.t2) +
-           bytes_of(h.t2_first);
-  total += bytes_of(h.s3r.chunks) + bytes_of(h.s3r.tasks) + bytes_of(h.s3r.terms);
-  if (total == 0) total = 256;
-  if (cudaMalloc(&dp->mem, total) != cudaSuccess) return DMRG3S_ERR_CUDA;
-  std::vector<char> staging(total, 0);
-  char* base = static_cast<char*>(dp->mem);
-  size_t off = 0;
-  dp->g1_tiles = place(base, &off, h.g1.tiles, &staging);
-  dp->g1_tasks = place(base, &off, h.g1.tasks, &staging);
-  dp->g1_segs = place(base, &off, h.g1.segs, &staging);
-  dp->c2_chunks = place(base, &off, h.c2.chunks, &staging);
-  dp->c2_tasks = place(base, &off, h.c2.tasks, &staging);
-  dp->c2_terms = place(base, &off, h.c2.terms, &staging);
-  dp->g3_tiles = place(base, &off, h.g3.tiles, &staging);
-  dp->g3_tasks = place(base, &off, h.g3.tasks, &staging);
-  dp->g3_segs = place(base, &off, h.g3.segs, &staging);
-  dp->g3s_tasks = place(base, &off, h.g3s.tasks, &staging);
-  dp->g1_units = place(base, &off, h.g1.tc.units, &staging);
-  dp->g1_tsegs = place(base, &off, h.g1.tc.segs, &staging);
-  dp->g1_packA = place(base, &off, h.g1.tc.packA, &staging);
-  dp->g1_packB = place(base, &off, h.g1.tc.packB, &staging);
-  dp->g3s_units = place(base, &off, h.g3s.tc.units, &staging);
-  dp->g3s_tsegs = place(base, &off, h.g3s.tc.segs, &staging);
-  dp->g3s_packA = place(base, &off, h.g3s.tc.packA, &staging);
-  dp->g3s_packB = place(base, &off, h.g3s.tc.packB, &staging);
-  dp->c2_pack = place(base, &off, h.c2pack, &staging);
-  dp->g12_tasks = place(base, &off, h.g12.tasks, &staging);
-  dp->g12_units = place(base, &off, h.g12.tc.units, &staging);
-  dp->g12_tsegs = place(base, &off, h.g12.tc.segs, &staging);
-  dp->g12_packA = place(base, &off, h.g12.tc.packA, &staging);
-  dp->g12_packB = place(base, &off, h.g12.tc.packB, &staging);
-  dp->g1_cta = place(base, &off, h.g1.tc.cta_start, &staging);
-  dp->g3s_cta = place(base, &off, h.g3s.tc.cta_start, &staging);
-  dp->g12_cta = place(base, &off, h.g12.tc.cta_start, &staging);
-  dp->c3r_chunks = place(base, &off, h.c3r.chunks, &staging);
-  dp->c3r_tasks = place(base, &off, h.c3r.tasks, &staging);
-  dp->c3r_terms = place(base, &off, h.c3r.terms, &staging);
-  place_sliced(base, &off, &dp->s12, h.s12, &staging);
-  place_sliced(base, &off, &dp->s3, h.s3, &staging);
-  dp->sl_groups = place(base, &off, h.slices.groups, &staging);
-  dp->sl_members = place(base, &off, h.slices.members, &staging);
-  dp->sl_cta_group = place(base, &off, h.slices.cta_group, &staging);
-  dp->grades = place(base, &off, h.grades, &staging);
-  dp->views = place(base, &off, h.views, &staging);
-  dp->t2 = place(base, &off, h.t2, &staging);
-  dp->t2_first = place(base, &off, h.t2_first, &staging);
-  dp->s3r_chunks = place(base, &off, h.s3r.chunks, &staging);
-  dp->s3r_tasks = place(base, &off, h.s3r.tasks, &staging);
-  dp->s3r_terms = place(base, &off, h.s3r.terms, &staging);
-  if (cudaMemcpy(dp->mem, staging.data(), total, cudaMemcpyHostToDevice) != cudaSuccess)
-    return DMRG3S_ERR_CUDA;
+  DevicePlan* d = dp.get();
+  const Plan& h = d->host;
+  const dmrg3s_status s = upload(&d->mem, [&](Tables& t) {
+    t.add(&d->g1_tiles, h.g1.tiles);
+    t.add(&d->g1_tasks, h.g1.tasks);
+    t.add(&d->g1_segs, h.g1.segs);
+    t.add(&d->c2_chunks, h.c2.chunks);
+    t.add(&d->c2_tasks, h.c2.tasks);
+    t.add(&d->c2_terms, h.c2.terms);
+    t.add(&d->g3_tiles, h.g3.tiles);
+    t.add(&d->g3_tasks, h.g3.tasks);
+    t.add(&d->g3_segs, h.g3.segs);
+  });
+  if (s != DMRG3S_OK) return s;
   *out = std::move(dp);
+  return DMRG3S_OK;
+}
+
+// The plan keeps its address; its forms are filled in when a call needs them.
+dmrg3s_status need_form(Context* c, const DevicePlan& plan, dmrg3s_precision prec) {
+  DevicePlan* d = const_cast<DevicePlan*>(&plan);
+  Plan& h = d->host;
+  if (prec == DMRG3S_FP64) {
+    if (h.sliced_tried) return DMRG3S_OK;
+    plan_sliced(&h);
+    if (!h.sliced) return DMRG3S_OK;
+    const dmrg3s_status s = upload(&d->mem_sl, [&](Tables& t) {
+      t.add(&d->s12, h.s12);
+      t.add(&d->s3, h.s3);
+      t.add(&d->sl_groups, h.slices.groups);
+      t.add(&d->sl_members, h.slices.members);
+      t.add(&d->sl_cta_group, h.slices.cta_group);
+      t.add(&d->grades, h.grades);
+      t.add(&d->views, h.views);
+      t.add(&d->t2, h.t2);
+      t.add(&d->t2_first, h.t2_first);
+      t.add(&d->s3r_chunks, h.s3r.chunks);
+      t.add(&d->s3r_tasks, h.s3r.tasks);
+      t.add(&d->s3r_terms, h.s3r.terms);
+    });
+    if (s != DMRG3S_OK) {             // no memory for the tables: the plain form
+      h.sliced = false;
+      cudaGetLastError();
+    }
+    return DMRG3S_OK;
+  }
+  if (h.tc_built) return DMRG3S_OK;
+  std::string err;
+  dmrg3s_status s = plan_tensor_core(&h, &err);
+  if (s != DMRG3S_OK) return fail(c, s, err);
+  s = upload(&d->mem_tc, [&](Tables& t) {
+    t.add(&d->g3s_tasks, h.g3s.tasks);
+    t.add(&d->g1_units, h.g1.tc.units);
+    t.add(&d->g1_tsegs, h.g1.tc.segs);
+    t.add(&d->g1_packA, h.g1.tc.packA);
+    t.add(&d->g1_packB, h.g1.tc.packB);
+    t.add(&d->g3s_units, h.g3s.tc.units);
+    t.add(&d->g3s_tsegs, h.g3s.tc.segs);
+    t.add(&d->g3s_packA, h.g3s.tc.packA);
+    t.add(&d->g3s_packB, h.g3s.tc.packB);
+    t.add(&d->c2_pack, h.c2pack);
+    t.add(&d->g12_tasks, h.g12.tasks);
+    t.add(&d->g12_units, h.g12.tc.units);
+    t.add(&d->g12_tsegs, h.g12.tc.segs);
+    t.add(&d->g12_packA, h.g12.tc.packA);
+    t.add(&d->g12_packB, h.g12.tc.packB);
+    t.add(&d->g1_cta, h.g1.tc.cta_start);
+    t.add(&d->g3s_cta, h.g3s.tc.cta_start);
+    t.add(&d->g12_cta, h.g12.tc.cta_start);
+    t.add(&d->c3r_chunks, h.c3r.chunks);
+    t.add(&d->c3r_tasks, h.c3r.tasks);
+    t.add(&d->c3r_terms, h.c3r.terms);
+  });
+  if (s != DMRG3S_OK) {
+    h.tc_built = false;
+    return fail(c, s, "uploading a contraction plan failed");
+  }
   return DMRG3S_OK;
 }
 
@@ -359,30 +394,24 @@ dmrg3s_status upload_grad_plan(GradPlan&& host, std::unique_ptr<DeviceGradPlan>*
   std::unique_ptr<DeviceGradPlan> dp(new (std::nothrow) DeviceGradPlan());
   if (!dp) return DMRG3S_ERR_OOM;
   dp->host = std::move(host);
-  const GradPlan& h = dp->host;
-  size_t total = bytes_of(h.tasks) + bytes_of(h.segs) + bytes_of(h.s) + bytes_of(h.slices.groups) +
-                 bytes_of(h.slices.members) + bytes_of(h.slices.cta_group) + 256;
-  for (const GemmStage* g : {&h.g1, &h.gy})
-    total += bytes_of(g->tiles) + bytes_of(g->tasks) + bytes_of(g->segs);
-  if (cudaMalloc(&dp->mem, total) != cudaSuccess) return DMRG3S_ERR_CUDA;
-  std::vector<char> staging(total, 0);
-  char* base = static_cast<char*>(dp->mem);
-  size_t off = 0;
-  DeviceGradPlan::Gemm* dg[2] = {&dp->g1, &dp->gy};
-  const GemmStage* hg[2] = {&h.g1, &h.gy};
-  for (int i = 0; i < 2; ++i) {
-    dg[i]->tiles = place(base, &off, hg[i]->tiles, &staging);
-    dg[i]->tasks = place(base, &off, hg[i]->tasks, &staging);
-    dg[i]->segs = place(base, &off, hg[i]->segs, &staging);
-  }
-  dp->tasks = place(base, &off, h.tasks, &staging);
-  dp->segs = place(base, &off, h.segs, &staging);
-  place_sliced(base, &off, &dp->s, h.s, &staging);
-  dp->sl_groups = place(base, &off, h.slices.groups, &staging);
-  dp->sl_members = place(base, &off, h.slices.members, &staging);
-  dp->sl_cta_group = place(base, &off, h.slices.cta_group, &staging);
-  if (cudaMemcpy(dp->mem, staging.data(), total, cudaMemcpyHostToDevice) != cudaSuccess)
-    return DMRG3S_ERR_CUDA;
+  DeviceGradPlan* d = dp.get();
+  const GradPlan& h = d->host;
+  const dmrg3s_status s = upload(&d->mem, [&](Tables& t) {
+    DeviceGradPlan::Gemm* dg[2] = {&d->g1, &d->gy};
+    const GemmStage* hg[2] = {&h.g1, &h.gy};
+    for (int i = 0; i < 2; ++i) {
+      t.add(&dg[i]->tiles, hg[i]->tiles);
+      t.add(&dg[i]->tasks, hg[i]->tasks);
+      t.add(&dg[i]->segs, hg[i]->segs);
+    }
+    t.add(&d->tasks, h.tasks);
+    t.add(&d->segs, h.segs);
+    t.add(&d->s, h.s);
+    t.add(&d->sl_groups, h.slices.groups);
+    t.add(&d->sl_members, h.slices.members);
+    t.add(&d->sl_cta_group, h.slices.cta_group);
+  });
+  if (s != DMRG3S_OK) return s;
   *out = std::move(dp);
   return DMRG3S_OK;
 }
@@ -814,7 +843,7 @@ dmrg3s_status dmrg3s_apply_heff(dmrg3s_ctx ctx, const dmrg3s_env* L, const dmrg3
   }
   if (!L->data || !R->data || !A->data || !HA->data)
     return fail(c, DMRG3S_ERR_ARG, "NULL device data pointer");
-  if ((st = check_ws(c, p->host, prec)) || (st = use_device(c))) return st;
+  if ((st = use_device(c)) || (st = need_form(c, *p, prec)) || (st = check_ws(c, p->host, prec))) return st;
   double* ws1 = reinterpret_cast<double*>(c->ws);
   double* ws2 = ws1 + p->host.ws1;
   st = run_plan(c, *p, L->data, A->data, ws1, ws2, 1.0, ws2, R->data, HA->data,
@@ -866,7 +895,7 @@ dmrg3s_status dmrg3s_expand(dmrg3s_ctx ctx, int32_t dir, const dmrg3s_env* env,
     remember_plan(c, key, p);
   }
   if (!env->data || !M->data || !P->data) return fail(c, DMRG3S_ERR_ARG, "NULL device data");
-  if ((st = check_ws(c, p->host, prec)) || (st = use_device(c))) return st;
+  if ((st = use_device(c)) || (st = need_form(c, *p, prec)) || (st = check_ws(c, p->host, prec))) return st;
   double* ws1 = reinterpret_cast<double*>(c->ws);
   const double* g1A = dir == 1 ? env->data : M->data;
   const double* g1B = dir == 1 ? M->data : env->data;
@@ -914,7 +943,7 @@ dmrg3s_status dmrg3s_update_env(dmrg3s_ctx ctx, int32_t dir, const dmrg3s_env* e
     remember_plan(c, key, p);
   }
   if (!env->data || !A->data || !out->data) return fail(c, DMRG3S_ERR_ARG, "NULL device data");
-  if ((st = check_ws(c, p->host, prec)) || (st = use_device(c))) return st;
+  if ((st = use_device(c)) || (st = need_form(c, *p, prec)) || (st = check_ws(c, p->host, prec))) return st;
   double* ws1 = reinterpret_cast<double*>(c->ws);
   double* ws2 = ws1 + p->host.ws1;
   const double* g1A = dir == 1 ? env->data : A->data;

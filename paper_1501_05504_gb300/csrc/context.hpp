@@ -48,7 +48,9 @@ constexpr size_t kMaxGradPlans = 256;     // cached per context
 // Device copy of a plan's task tables.
 struct DevicePlan {
   Plan host;
-  void* mem = nullptr;      // one allocation holding every table
+  // the tables of the plain form, and those of the tensor-core and the sliced form once
+  // a call has needed them (need_form), each in one allocation
+  void *mem = nullptr, *mem_tc = nullptr, *mem_sl = nullptr;
   GemmTile* g1_tiles = nullptr;
   GemmTask* g1_tasks = nullptr;
   GemmSeg* g1_segs = nullptr;
@@ -336,6 +338,10 @@ dmrg3s_status pinned_reserve(Context* c, size_t n);
 
 // Upload a host plan (allocates the device tables).  Returns CUDA errors.
 dmrg3s_status upload_plan(Plan&& host, std::unique_ptr<DevicePlan>* out);
+// Builds and uploads what a call in this precision needs beside the plain tables, once
+// (a 3xTF32 operator never reads the sliced tables, and an FP64 one never the TF32
+// tables).  Before plan_ws_doubles, sliced_fits and run_plan.
+dmrg3s_status need_form(Context* c, const DevicePlan& p, dmrg3s_precision prec);
 
 // Enqueue the stages of a plan.  Bases as documented for each plan Kind.
 // Tensor-core mode: the stage-1 and stage-3 operands are packed (hi, lo

@@ -322,7 +322,7 @@ extern "C" dmrg3s_status dmrg3s_eigensolve(dmrg3s_ctx ctx, const dmrg3s_env* L,
   if (a.size == 0) return fail(c, DMRG3S_ERR_SHAPE, "site tensor has no allowed block");
   if ((st = use_device(c))) return st;
   const DevicePlan* p = nullptr;
-  if ((st = heff_plan(c, le, w, re, a, &p))) return st;
+  if ((st = heff_plan(c, le, w, re, a, &p)) || (st = need_form(c, *p, prec))) return st;
   size_t cursor = (size_t)plan_ws_doubles(p->host, prec) * sizeof(double);
   int it = 0;
   double theta = 0.0;

@@ -51,7 +51,7 @@ dmrg3s_status dmrg3s_heff_create(dmrg3s_ctx ctx, const dmrg3s_env* L, const dmrg
   if (!L->data || !R->data) return fail(c, DMRG3S_ERR_ARG, "NULL device data");
   if ((st = use_device(c))) return st;
   const DevicePlan* p = nullptr;
-  if ((st = heff_plan(c, le, w, re, a, &p))) return st;
+  if ((st = heff_plan(c, le, w, re, a, &p)) || (st = need_form(c, *p, prec))) return st;
   if ((size_t)plan_ws_doubles(p->host, prec) * sizeof(double) > c->ws_bytes)
     return fail(c, DMRG3S_ERR_OOM, "context workspace too small for H_eff");
   HeffOp* h = new (std::nothrow) HeffOp();

@@ -8,8 +8,10 @@
 #include <array>
 #include <atomic>
 #include <cmath>
+#include <functional>
 #include <map>
-#include <set>
+#include <queue>
+#include <unordered_map>
 
 namespace dmrg3s {
 
@@ -78,18 +80,23 @@ std::vector<GemmTile> choose_tiles(const GemmStage& g) {
 }
 
 void GemmStage::finalize_bytes(Trans, Trans) {
-  std::set<std::pair<int64_t, int64_t>> a, b;
+  std::vector<std::pair<int64_t, int64_t>> a, b;
+  a.reserve(segs.size());
+  b.reserve(segs.size());
   double elems = 0.0;
   for (const GemmTask& t : tasks) {
     elems += (double)t.M * t.N;
     for (int k = 0; k < t.nseg; ++k) {
       const GemmSeg& g = segs[t.seg0 + k];
-      a.insert({g.offA, (int64_t)t.M * g.K});
-      b.insert({g.offB, (int64_t)t.N * g.K});
+      a.push_back({g.offA, (int64_t)t.M * g.K});
+      b.push_back({g.offB, (int64_t)t.N * g.K});
     }
   }
-  for (auto& x : a) elems += (double)x.second;
-  for (auto& x : b) elems += (double)x.second;
+  for (auto* v : {&a, &b}) {
+    std::sort(v->begin(), v->end());
+    v->erase(std::unique(v->begin(), v->end()), v->end());
+    for (auto& x : *v) elems += (double)x.second;
+  }
   bytes = 8.0 * elems;
 }
 
@@ -151,11 +158,14 @@ void schedule(std::vector<TcUnit>& units, std::vector<int32_t>& cta_start,
   for (int i = 0; i < n; ++i) order[i] = i;
   std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return cost[a] > cost[b]; });
   std::vector<std::vector<int>> lists(nc);
-  std::vector<double> load(nc, 0.0);
+  using Load = std::pair<double, int>;               // (the lowest of equal ones first)
+  std::priority_queue<Load, std::vector<Load>, std::greater<Load>> load;
+  for (int c = 0; c < nc; ++c) load.push({0.0, c});
   for (int i : order) {
-    const int c = (int)(std::min_element(load.begin(), load.end()) - load.begin());
-    lists[c].push_back(i);
-    load[c] += cost[i];
+    const Load l = load.top();
+    load.pop();
+    lists[l.second].push_back(i);
+    load.push({l.first + cost[i], l.second});
   }
   std::vector<TcUnit> out;
   out.reserve(n);
@@ -220,7 +230,7 @@ void left_stages(const EnvLayout& le, const MpoLayout& W, const SiteLayout& M, P
       const Block& blk = M.blocks[mb];
       const int j = blk.c;
       const int64_t rows = le.bond.dim[ip], cols = M.right.dim[j], K = M.left.dim[i];
-      (*t1)[Key{bl, s, i, 0}] = Interm{off, (int)rows, (int)cols};
+      if (t1) (*t1)[Key{bl, s, i, 0}] = Interm{off, (int)rows, (int)cols};
       p->g1.add(off, (int)cols, (int)rows, (int)cols, {seg(lb.off, K, blk.off, cols, K)});
       // stage 2 terms
       for (int so = 0; so < W.d; ++so)
@@ -244,7 +254,7 @@ void left_stages(const EnvLayout& le, const MpoLayout& W, const SiteLayout& M, P
 
 // Stage 1 + 2 of the right side: U1[br, s] = M[s] R[br]^T; U2 terms.
 void right_stages(const EnvLayout& re, const MpoLayout& W, const SiteLayout& M, Plan* p,
-                  std::map<Key, Interm>* u1, std::map<Key, Combo>* u2) {
+                  std::map<Key, Combo>* u2) {
   p->g1.ta = Trans::N;
   p->g1.tb = Trans::T;
   int64_t off = 0;
@@ -256,7 +266,6 @@ void right_stages(const EnvLayout& re, const MpoLayout& W, const SiteLayout& M, 
       const Block& rblk = re.blocks[rb];
       const int jp = rblk.b;
       const int64_t rows = M.left.dim[i], cols = re.bond.dim[jp], K = M.right.dim[j];
-      (*u1)[Key{br, s, i, 0}] = Interm{off, (int)rows, (int)cols};
       p->g1.add(off, (int)cols, (int)rows, (int)cols, {seg(mb.off, K, rblk.off, K, K)});
       for (int so = 0; so < W.d; ++so)
         for (int bl = 0; bl < W.wl; ++bl) {
@@ -486,15 +495,17 @@ struct Slicer {
   };
   std::vector<Blk> blks;
   std::vector<int> parent;
-  std::map<std::pair<std::array<int64_t, 5>, double>, int> seen;   // (view, coef) -> block
+  std::unordered_multimap<int64_t, int> seen;                 // source offset -> blocks
   int find(int i) {
     while (parent[i] != i) i = parent[i] = parent[parent[i]];
     return i;
   }
   int add(int64_t src, int64_t ld, int64_t R, int64_t K, int trans, double coef) {
-    const auto key = std::make_pair(std::array<int64_t, 5>{src, ld, R, K, trans}, coef);
-    auto it = seen.find(key);
-    if (it != seen.end()) return it->second;
+    const auto range = seen.equal_range(src);
+    for (auto it = range.first; it != range.second; ++it) {
+      const Blk& q = blks[it->second];
+      if (q.m.coef == coef && q.m.ld == ld && q.R == R && q.m.K == K && q.m.trans == trans) return it->second;
+    }
     Blk b{};
     b.m.src = src;
     b.m.coef = coef;
@@ -507,7 +518,7 @@ struct Slicer {
     const int id = (int)blks.size();
     blks.push_back(b);
     parent.push_back(id);
-    seen[key] = id;
+    seen.emplace(src, id);
     return id;
   }
   void join(int a, int b) {
@@ -519,21 +530,29 @@ struct Slicer {
   // Places every block and group; e0[block] = first scale of its group.
   void layout(bool headroom, std::vector<SlGroup>* g, std::vector<SlMember>* m, int64_t* n,
               int32_t* ne, std::vector<int32_t>* e0) {
-    std::map<int, std::vector<int>> by;
-    for (int i = 0; i < (int)blks.size(); ++i) by[find(i)].push_back(i);
+    // blocks by their group (a group's first block is its lowest)
+    std::vector<int32_t> first(blks.size() + 1, 0), by(blks.size());
+    for (int i = 0; i < (int)blks.size(); ++i) ++first[find(i) + 1];
+    for (size_t i = 1; i < first.size(); ++i) first[i] += first[i - 1];
+    std::vector<int32_t> at(first.begin(), first.end() - 1);
+    for (int i = 0; i < (int)blks.size(); ++i) by[at[find(i)]++] = i;
     e0->assign(blks.size(), 0);
-    for (const auto& kv : by) {
+    m->reserve(blks.size());
+    for (int root = 0; root < (int)blks.size(); ++root) {
+      const int nm = first[root + 1] - first[root];
+      if (!nm) continue;
       SlGroup gr{};
-      gr.R = blks[kv.first].R;
+      gr.R = blks[root].R;
       gr.R8 = groups(gr.R);
       gr.m0 = (int32_t)m->size();
-      gr.nm = (int32_t)kv.second.size();
+      gr.nm = nm;
       gr.e0 = *ne;
       int spans = 0;
-      for (int i : kv.second) spans = std::max(spans, blks[i].spans);
+      for (int k = 0; k < nm; ++k) spans = std::max(spans, blks[by[first[root] + k]].spans);
       while (headroom && spans > kSlSpans << gr.shift) ++gr.shift;
-      blks[kv.first].shift = gr.shift;
-      for (int i : kv.second) {
+      blks[root].shift = gr.shift;
+      for (int k = 0; k < nm; ++k) {
+        const int i = by[first[root] + k];
         blks[i].m.t0 = gr.nt;
         gr.nt += blks[i].m.KC;
         blks[i].m.dst = *n;
@@ -553,7 +572,7 @@ constexpr double kSlLeast = 3.0 * 0.95 * 4.0;
 
 // Views of the site tensor along the k of a block (by its source offset): what the
 // grading of those k is taken from.
-using GradeViews = std::map<int64_t, std::vector<SlView>>;
+using GradeViews = std::unordered_map<int64_t, std::vector<SlView>>;
 
 // The grading of the blocks that meet along k (grade_kernel): blocks of A and B in one
 // segment share it, so the classes are the sectors of the contracted bond.  The
@@ -774,7 +793,8 @@ bool build_sliced(const GemmStage& g, bool coefA, Plan* grade, bool of_a, const 
 // Stages 1 + 2 as one grouped GEMM in FP64: one task per stage-2 block, one
 // K-segment per MPO term, scaled by its coefficient.
 bool fuse_f64(const Plan& p, GemmStage* out, std::string* err) {
-  std::map<int64_t, int> t1_task;      // T1 element offset -> stage-1 task
+  std::unordered_map<int64_t, int> t1_task;      // T1 element offset -> stage-1 task
+  t1_task.reserve(p.g1.tasks.size());
   for (size_t i = 0; i < p.g1.tasks.size(); ++i) t1_task[p.g1.tasks[i].offC] = (int)i;
   GemmStage& g = *out;
   g = GemmStage();
@@ -874,7 +894,9 @@ void rechunk(CombStage& c) {
 // every unit of stage 2 collects its row scales (EnvLR: its columns' scales).
 bool plan_t2(Plan* p, const std::vector<SlGroup>& groups, const std::vector<SlMember>& members,
              std::string* err) {
-  std::map<int64_t, int32_t> e0, d0;   // block offset -> its first row scale, grading entry
+  // block offset -> its first row scale, grading entry
+  std::unordered_map<int64_t, std::pair<int32_t, int32_t>> e0;
+  e0.reserve(members.size());
   for (const SlGroup& g : groups)
     for (int k = 0; k < g.nm; ++k) {
       const SlMember& m = members[g.m0 + k];
@@ -893,8 +915,7 @@ bool plan_t2(Plan* p, const std::vector<SlGroup>& groups, const std::vector<SlMe
       q.tile0 = p->t2_tiles;
       p->t2_tiles += g.R8 * m.KC;
       p->t2.push_back(q);
-      d0[m.src] = m.d0;
-      if (!e0.emplace(m.src, g.e0).second) {
+      if (!e0.emplace(m.src, std::make_pair(g.e0, m.d0)).second) {
         *err = "sliced stage: a stage-2 block with two sets of scales";
         return false;
       }
@@ -908,9 +929,9 @@ bool plan_t2(Plan* p, const std::vector<SlGroup>& groups, const std::vector<SlMe
   for (SlUnit& u : p->s12.units) {
     // the unit's block: its offset less the unit's place in it
     const auto it = e0.find(u.offC - (int64_t)u.m0 * u.ldc - u.n0);
-    u.em = it == e0.end() ? -1 : it->second + (cols ? u.n0 : u.m0);
+    u.em = it == e0.end() ? -1 : it->second.first + (cols ? u.n0 : u.m0);
     // (a graded operand: A of H_eff, whose k are the block's columns)
-    u.d0 = it == e0.end() || d0[it->first] < 0 ? -1 : d0[it->first] + u.n0;
+    u.d0 = it == e0.end() || it->second.second < 0 ? -1 : it->second.second + u.n0;
     const int32_t ne = p->kind == Kind::Heff ? p->s3.neA : p->s3.neB;
     if (u.em >= 0 && (u.em + (cols ? u.cols : u.rows) > ne || (u.d0 >= 0 && u.d0 + u.cols > p->ngrade))) {
       *err = "sliced stage: collected scales out of bounds";
@@ -947,17 +968,21 @@ double tile_fill(const GemmStage& g, const GemmStage* h) {
 constexpr double kSlicedMaxTerms = 6.0;
 
 // The sliced FP64 form, where there is enough work for it.
-dmrg3s_status finish_sliced(Plan* p, int64_t nA1, int64_t nB1, int64_t nOut2, int64_t nA3,
-                            int64_t nB3, int64_t nC3, std::string* err) {
+}  // namespace
+
+void plan_sliced(Plan* p) {
+  const int64_t nA1 = p->nA1, nB1 = p->nB1, nOut2 = p->nOut2, nA3 = p->nA3, nB3 = p->nB3, nC3 = p->nC3;
+  std::string why, *err = &why;
   p->sliced = false;
+  p->sliced_tried = true;
   const double flops = p->flops() * tile_fill(p->g1, p->has_g3 ? &p->g3 : nullptr);
-  if (flops < kSlicedMinFlops) return DMRG3S_OK;
+  if (flops < kSlicedMinFlops) return;
   // a dense MPO tensor: too many terms per stage-1 block to form each anew
   double terms = 0.0, blocks = 0.0;
   for (const CombTask& t : p->c2.tasks) terms += (double)t.nt * t.rows * t.cols;
   for (const GemmTask& t : p->g1.tasks) blocks += (double)t.M * t.N;
   if (terms > kSlicedMaxTerms * blocks || flops * blocks < kSlicedMinFlops * terms)
-    return DMRG3S_OK;
+    return;
   const bool left = p->kind == Kind::Heff || p->kind == Kind::ExpandLR || p->kind == Kind::EnvLR;
   bool ok = fuse_f64(*p, &p->f12, err);
   // the site tensor (B of the left kinds, A of the right ones): along k, and along
@@ -966,11 +991,11 @@ dmrg3s_status finish_sliced(Plan* p, int64_t nA1, int64_t nB1, int64_t nOut2, in
   for (const GemmTask& t : p->f12.tasks)
     for (int k = 0; ok && k < t.nseg; ++k) {
       const GemmSeg& q = p->f12.segs[t.seg0 + k];
-      if (left) {
-        along[q.offB] = {SlView{q.offB, q.ldb, t.N, 1, 0}};
-        across[t.offC].push_back(SlView{q.offB, q.ldb, q.K, 0, 0});
-      } else {
-        along[q.offA] = {SlView{q.offA, q.lda, t.M, 0, 0}};
+      auto& v = along[left ? q.offB : q.offA];
+      if (v.empty()) v.push_back(left ? SlView{q.offB, q.ldb, t.N, 1, 0} : SlView{q.offA, q.lda, t.M, 0, 0});
+      if (p->kind == Kind::Heff) {
+        auto& w = across[t.offC];
+        if (w.empty() || w.back().src != q.offB) w.push_back(SlView{q.offB, q.ldb, q.K, 0, 0});
       }
     }
   ok = ok && build_sliced(p->f12, left, p, !left, along, &p->s12, err) &&
@@ -1003,23 +1028,39 @@ dmrg3s_status finish_sliced(Plan* p, int64_t nA1, int64_t nB1, int64_t nOut2, in
     ok = slice_table_ok(p->slices, err) && grades_ok(p->grades, p->views, left ? nB1 : nA1, p->ngrade, err);
     if (ok && p->has_g3) ok = plan_t2(p, t2_is_a ? p->s3.gA : p->s3.gB, t2_is_a ? p->s3.mA : p->s3.mB, err);
   }
-  if (!ok) {
-    *err = "internal planning error: " + *err;
-    return DMRG3S_ERR_SHAPE;
-  }
-  p->sliced = true;
-  return DMRG3S_OK;
+  p->sliced = ok;                    // (tables that fail a check: the plain form)
 }
+
+namespace {
 
 // Bounds of every table against the buffers the stages address.
 dmrg3s_status finish(Plan* p, int64_t nA1, int64_t nB1, int64_t nOut2, int64_t nA3, int64_t nB3,
                      int64_t nC3, std::string* err) {
   p->nA1 = nA1;
   p->nB1 = nB1;
+  p->nOut2 = nOut2;
   p->nA3 = p->has_g3 ? nA3 : 0;
   p->nB3 = p->has_g3 ? nB3 : 0;
+  p->nC3 = p->has_g3 ? nC3 : 0;
   p->g1.finalize_bytes(p->g1.ta, p->g1.tb);
   if (p->has_g3) p->g3.finalize_bytes(p->g3.ta, p->g3.tb);
+  const int64_t w1 = p->ws1 > 0 ? p->ws1 : 1;
+  if (!gemm_ok(p->g1.ta, p->g1.tb, p->g1.tasks, p->g1.segs, nA1, nB1, w1, err) ||
+      !comb_ok(p->c2.tasks, p->c2.terms, w1, nOut2, err) ||
+      (p->has_g3 && !gemm_ok(p->g3.ta, p->g3.tb, p->g3.tasks, p->g3.segs, nA3, nB3, nC3, err))) {
+    *err = "internal planning error: " + *err;
+    return DMRG3S_ERR_SHAPE;
+  }
+  p->g1.tiles = choose_tiles(p->g1);
+  p->g3.tiles = choose_tiles(p->g3);
+  rechunk(p->c2);
+  return DMRG3S_OK;
+}
+
+}  // namespace
+
+dmrg3s_status plan_tensor_core(Plan* p, std::string* err) {
+  const int64_t nA1 = p->nA1, nB1 = p->nB1, nA3 = p->nA3, nB3 = p->nB3, nC3 = p->nC3;
   if (p->has_g3) {
     // split-K form of stage 3: the K-segments of every output block in G
     // consecutive groups, G chosen so that the units fill the GPU about twice
@@ -1039,13 +1080,6 @@ dmrg3s_status finish(Plan* p, int64_t nA1, int64_t nB1, int64_t nOut2, int64_t n
       *err = "internal planning error: " + *err;
       return DMRG3S_ERR_SHAPE;
     }
-  }
-  const int64_t w1 = p->ws1 > 0 ? p->ws1 : 1;
-  if (!gemm_ok(p->g1.ta, p->g1.tb, p->g1.tasks, p->g1.segs, nA1, nB1, w1, err) ||
-      !comb_ok(p->c2.tasks, p->c2.terms, w1, nOut2, err) ||
-      (p->has_g3 && !gemm_ok(p->g3.ta, p->g3.tb, p->g3.tasks, p->g3.segs, nA3, nB3, nC3, err))) {
-    *err = "internal planning error: " + *err;
-    return DMRG3S_ERR_SHAPE;
   }
   // tensor-core form.  H_eff: stages 1 and 2 fused (g12) writing T2 packed
   // for stage 3.  The others: stage 1 packs both operands, and stage 3 takes
@@ -1075,14 +1109,10 @@ dmrg3s_status finish(Plan* p, int64_t nA1, int64_t nB1, int64_t nOut2, int64_t n
     *err = "internal planning error: " + *err;
     return DMRG3S_ERR_SHAPE;
   }
-  p->g1.tiles = choose_tiles(p->g1);
-  p->g3.tiles = choose_tiles(p->g3);
-  rechunk(p->c2);
   rechunk(p->c3r);
-  return finish_sliced(p, nA1, nB1, nOut2, nA3, nB3, nC3, err);
+  p->tc_built = true;
+  return DMRG3S_OK;
 }
-
-}  // namespace
 
 namespace {
 // Appends stage `src` to `dst` with its operand offsets moved by oA / oB and
@@ -1212,9 +1242,8 @@ dmrg3s_status check_env(const EnvLayout& e, const Bond& bond, int w, const std::
 dmrg3s_status plan_heff(const EnvLayout& le, const MpoLayout& W, const EnvLayout& re,
                         const SiteLayout& M, Plan* p, std::string* err) {
   p->kind = Kind::Heff;
-  std::map<Key, Interm> t1;
   std::map<Key, Combo> t2c;
-  left_stages(le, W, M, p, &t1, &t2c);
+  left_stages(le, W, M, p, nullptr, &t2c);
   std::map<Key, Interm> t2 = materialise(t2c, p);
   p->has_g3 = true;
   p->g3.ta = Trans::N;
@@ -1241,9 +1270,8 @@ dmrg3s_status plan_expand_lr(const EnvLayout& le, const MpoLayout& W, const Site
                              const SiteLayout& P, const FusedBond& fused, Plan* p,
                              std::string* err) {
   p->kind = Kind::ExpandLR;
-  std::map<Key, Interm> t1;
   std::map<Key, Combo> t2c;
-  left_stages(le, W, M, p, &t1, &t2c);
+  left_stages(le, W, M, p, nullptr, &t2c);
   const int nsrc = M.right.nsec();
   for (const Block& pb : P.blocks) {
     const int so = pb.a, ip = pb.b, k = pb.c;
@@ -1264,9 +1292,8 @@ dmrg3s_status plan_expand_lr(const EnvLayout& le, const MpoLayout& W, const Site
 dmrg3s_status plan_env_lr(const EnvLayout& le, const MpoLayout& W, const SiteLayout& M,
                           const EnvLayout& out, Plan* p, std::string* err) {
   p->kind = Kind::EnvLR;
-  std::map<Key, Interm> t1;
   std::map<Key, Combo> t2c;
-  left_stages(le, W, M, p, &t1, &t2c);
+  left_stages(le, W, M, p, nullptr, &t2c);
   std::map<Key, Interm> t2 = materialise(t2c, p);
   p->has_g3 = true;
   p->g3.ta = Trans::T;
@@ -1293,9 +1320,8 @@ dmrg3s_status plan_expand_rl(const EnvLayout& re, const MpoLayout& W, const Site
                              const SiteLayout& P, const FusedBond& fused, Plan* p,
                              std::string* err) {
   p->kind = Kind::ExpandRL;
-  std::map<Key, Interm> u1;
   std::map<Key, Combo> u2c;
-  right_stages(re, W, M, p, &u1, &u2c);
+  right_stages(re, W, M, p, &u2c);
   const int nsrc = M.left.nsec();
   for (const Block& pb : P.blocks) {
     const int so = pb.a, k = pb.b, jp = pb.c;
@@ -1316,9 +1342,8 @@ dmrg3s_status plan_expand_rl(const EnvLayout& re, const MpoLayout& W, const Site
 dmrg3s_status plan_env_rl(const EnvLayout& re, const MpoLayout& W, const SiteLayout& M,
                           const EnvLayout& out, Plan* p, std::string* err) {
   p->kind = Kind::EnvRL;
-  std::map<Key, Interm> u1;
   std::map<Key, Combo> u2c;
-  right_stages(re, W, M, p, &u1, &u2c);
+  right_stages(re, W, M, p, &u2c);
   std::map<Key, Interm> u2 = materialise(u2c, p);
   p->has_g3 = true;
   p->g3.ta = Trans::N;

@@ -144,6 +144,10 @@ struct Plan {
   CombStage s3r;                // sum of the partials (empty: no split)
   int64_t ws3s = 0;             // doubles of the partial blocks
   bool sliced = false;
+  // The forms beside the plain one are built when a call first needs them
+  // (plan_tensor_core, plan_sliced).
+  bool tc_built = false, sliced_tried = false;
+  int64_t nOut2 = 0, nC3 = 0;   // elements of the stage-2 and stage-3 outputs
   double flops() const { return g1.flops + c2.flops + (has_g3 ? g3.flops : 0.0); }
 };
 
@@ -162,6 +166,10 @@ struct PlanPart {
 // intermediates laid out back to back), then the split-K stage 3 and the
 // tensor-core form built over the whole, so that one launch per stage
 // serves every part.  n* are the sizes of the merged operand arrays.
+// The tensor-core (3xTF32 / TF32) tables of a plan; the sliced FP64 tables, where
+// there is enough work for that form (Plan::sliced).
+dmrg3s_status plan_tensor_core(Plan* p, std::string* err);
+void plan_sliced(Plan* p);
 dmrg3s_status merge_plans(Kind kind, const std::vector<PlanPart>& parts, int64_t nA1, int64_t nB1,
                           int64_t nOut2, int64_t nA3, int64_t nB3, int64_t nC3, Plan* out,
                           std::string* err);

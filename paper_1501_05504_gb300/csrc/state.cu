@@ -224,7 +224,7 @@ dmrg3s_status env_step(State& S, int i, int dir, const EnvLayout& src_lay, const
                 dir == 1 ? a.lay.right : a.lay.left, out_lay);
   const DevicePlan* p;
   dmrg3s_status s = env_plan(c, dir, src_lay, w, a.lay, *out_lay, &p);
-  if (s) return s;
+  if (s || (s = need_form(c, *p, DMRG3S_FP64))) return s;
   if ((size_t)(p->host.ws1 + p->host.ws2) * sizeof(double) > c->ws_bytes)
     return fail(c, DMRG3S_ERR_OOM, "context workspace too small for the environment update");
   if ((s = dalloc(c, out, out_lay->size, st))) return s;
@@ -261,7 +261,7 @@ dmrg3s_status rayleigh(State& S, int i, const double* x, cudaStream_t st, double
   Context* c = S.c;
   const DevicePlan* p;
   dmrg3s_status s = heff_plan(c, S.Lenv[i].lay, S.W[i], S.Renv[i].lay, S.M[i].lay, &p);
-  if (s) return s;
+  if (s || (s = need_form(c, *p, DMRG3S_FP64))) return s;
   if ((size_t)(p->host.ws1 + p->host.ws2) * sizeof(double) > c->ws_bytes)
     return fail(c, DMRG3S_ERR_OOM, "context workspace too small for H_eff");
   const int64_t n = S.M[i].lay.size;
@@ -837,7 +837,8 @@ dmrg3s_status local_update(State& S, int dir, double alpha, const Opts& o, Info*
   int ph = phase(kProfEig);
   if (o.optimise) {
     const DevicePlan* hp;
-    if ((s = heff_plan(c, S.Lenv[i].lay, w, S.Renv[i].lay, m.lay, &hp))) return s;
+    if ((s = heff_plan(c, S.Lenv[i].lay, w, S.Renv[i].lay, m.lay, &hp)) || (s = need_form(c, *hp, o.prec)))
+      return s;
     size_t cursor = (size_t)plan_ws_doubles(hp->host, o.prec) * sizeof(double);
     double lam = 0.0;
     int it = 0;
@@ -866,7 +867,8 @@ dmrg3s_status local_update(State& S, int dir, double alpha, const Opts& o, Info*
       make_site_from(m.lay.nsym, m.lay.d, m.lay.qp, fp.bond, m.lay.right, &pl);
     const DevicePlan* ep;
     const DevEnv& env = dir == 1 ? S.Lenv[i] : S.Renv[i];
-    if ((s = expand_plan(c, dir, env.lay, w, m.lay, pl, fp, &ep))) return s;
+    if ((s = expand_plan(c, dir, env.lay, w, m.lay, pl, fp, &ep)) || (s = need_form(c, *ep, DMRG3S_FP64)))
+      return s;
     if ((size_t)ep->host.ws1 * sizeof(double) > c->ws_bytes)
       return fail(c, DMRG3S_ERR_OOM, "context workspace too small for the expansion");
     if ((s = scr.get(&P, pl.size))) return s;
@@ -958,14 +960,14 @@ struct BItem {
 
 dmrg3s_status upload_merged(Context* c, Kind kind, const std::vector<PlanPart>& parts, int64_t nA1,
                             int64_t nB1, int64_t nOut2, int64_t nA3, int64_t nB3, int64_t nC3,
-                            std::unique_ptr<DevicePlan>* out) {
+                            dmrg3s_precision prec, std::unique_ptr<DevicePlan>* out) {
   Plan mp;
   std::string err;
   dmrg3s_status s = merge_plans(kind, parts, nA1, nB1, nOut2, nA3, nB3, nC3, &mp, &err);
   if (s) return fail(c, s, "merged plan: " + err);
   if ((s = upload_plan(std::move(mp), out)))
     return fail(c, s, "uploading a merged contraction plan failed");
-  return DMRG3S_OK;
+  return need_form(c, **out, prec);
 }
 
 dmrg3s_status copy_in(Context* c, double* dst, const double* src, int64_t n, cudaStream_t st) {
@@ -989,7 +991,9 @@ dmrg3s_status batch_eig(Context* c, std::vector<BItem>& items, cudaStream_t st) 
       State& S = *it.S;
       const int i = S.centre;
       const DevicePlan* hp;
-      if ((s = heff_plan(c, S.Lenv[i].lay, S.W[i], S.Renv[i].lay, S.M[i].lay, &hp))) return s;
+      if ((s = heff_plan(c, S.Lenv[i].lay, S.W[i], S.Renv[i].lay, S.M[i].lay, &hp)) ||
+          (s = need_form(c, *hp, prec)))
+        return s;
       const size_t cursor = (size_t)plan_ws_doubles(hp->host, prec) * sizeof(double);
       if ((s = lanczos_run(c, *hp, S.Lenv[i].data, S.Renv[i].data, S.M[i].data, S.M[i].lay.size,
                            it.o.kmax, lanczos_tol(it.o), cursor, st, &it.info.lambda, &it.info.iters, prec)))
@@ -1016,7 +1020,7 @@ dmrg3s_status batch_eig(Context* c, std::vector<BItem>& items, cudaStream_t st) 
       nX += align32(S.M[i].lay.size);
     }
     std::unique_ptr<DevicePlan> dp;
-    if ((s = upload_merged(c, Kind::Heff, parts, nL, nX, 0, 0, nR, nX, &dp))) return s;
+    if ((s = upload_merged(c, Kind::Heff, parts, nL, nX, 0, 0, nR, nX, prec, &dp))) return s;
     Scratch scr(c, st);
     double *La, *Ra, *Xa;
     if ((s = scr.get(&La, nL)) || (s = scr.get(&Ra, nR)) || (s = scr.get(&Xa, nX))) return s;
@@ -1101,7 +1105,8 @@ dmrg3s_status batch_expand(Context* c, std::vector<BItem>& items, Scratch& keep,
     }
     std::unique_ptr<DevicePlan> dp;
     const Kind kind = dir == 1 ? Kind::ExpandLR : Kind::ExpandRL;
-    if ((s = upload_merged(c, kind, parts, dir == 1 ? nE : nM, dir == 1 ? nM : nE, nP, 0, 0, 0, &dp)))
+    if ((s = upload_merged(c, kind, parts, dir == 1 ? nE : nM, dir == 1 ? nM : nE, nP, 0, 0, 0, DMRG3S_FP64,
+                           &dp)))
       return s;
     if ((size_t)dp->host.ws1 * sizeof(double) > c->ws_bytes)
       return fail(c, DMRG3S_ERR_OOM, "context workspace too small for the expansion");
@@ -1239,7 +1244,7 @@ dmrg3s_status batch_env(Context* c, std::vector<BItem>& items, cudaStream_t st) 
     std::unique_ptr<DevicePlan> dp;
     const Kind kind = dir == 1 ? Kind::EnvLR : Kind::EnvRL;
     if ((s = upload_merged(c, kind, parts, dir == 1 ? nE : nA, dir == 1 ? nA : nE, 0, nA, 0, nO,
-                           &dp)))
+                           DMRG3S_FP64, &dp)))
       return s;
     if ((size_t)(dp->host.ws1 + dp->host.ws2) * sizeof(double) > c->ws_bytes)
       return fail(c, DMRG3S_ERR_OOM, "context workspace too small for the environment update");
@@ -1309,7 +1314,7 @@ dmrg3s_status batch_energy(Context* c, std::vector<BItem>& items, cudaStream_t s
     nX += align32(S.M[i].lay.size);
   }
   std::unique_ptr<DevicePlan> dp;
-  if ((s = upload_merged(c, Kind::Heff, parts, nL, nX, 0, 0, nR, nX, &dp))) return s;
+  if ((s = upload_merged(c, Kind::Heff, parts, nL, nX, 0, 0, nR, nX, DMRG3S_FP64, &dp))) return s;
   if ((size_t)(dp->host.ws1 + dp->host.ws2) * sizeof(double) > c->ws_bytes)
     return fail(c, DMRG3S_ERR_OOM, "context workspace too small for H_eff");
   std::vector<LzChunk> hch;
