@@ -536,9 +536,6 @@ const DevicePlan* known_plan(Context* c, const RawKey& key) {
   auto it = c->by_args.find(key);
   return it == c->by_args.end() ? nullptr : it->second;
 }
-void remember_plan(Context* c, const RawKey& key, const DevicePlan* p) {
-  if (key.ok) c->by_args[key] = p;
-}
 
 dmrg3s_status prec_ok(Context* c, dmrg3s_precision prec) {
   if (prec == DMRG3S_FP64 || prec == DMRG3S_TF32X3 || prec == DMRG3S_TF32) return DMRG3S_OK;
@@ -839,7 +836,7 @@ dmrg3s_status dmrg3s_apply_heff(dmrg3s_ctx ctx, const dmrg3s_env* L, const dmrg3
       return fail(c, DMRG3S_ERR_ARG, "NULL device data pointer");
     st = heff_plan(c, le, w, re, a, &p);
     if (st != DMRG3S_OK) return st;
-    remember_plan(c, key, p);
+    remember(&c->by_args, key, p);
   }
   if (!L->data || !R->data || !A->data || !HA->data)
     return fail(c, DMRG3S_ERR_ARG, "NULL device data pointer");
@@ -892,7 +889,7 @@ dmrg3s_status dmrg3s_expand(dmrg3s_ctx ctx, int32_t dir, const dmrg3s_env* env,
     if (!env->data || !M->data || !P->data) return fail(c, DMRG3S_ERR_ARG, "NULL device data");
     st = expand_plan(c, dir, e, w, m, pl, f, &p);
     if (st != DMRG3S_OK) return st;
-    remember_plan(c, key, p);
+    remember(&c->by_args, key, p);
   }
   if (!env->data || !M->data || !P->data) return fail(c, DMRG3S_ERR_ARG, "NULL device data");
   if ((st = use_device(c)) || (st = need_form(c, *p, prec)) || (st = check_ws(c, p->host, prec))) return st;
@@ -940,7 +937,7 @@ dmrg3s_status dmrg3s_update_env(dmrg3s_ctx ctx, int32_t dir, const dmrg3s_env* e
     if (!env->data || !A->data || !out->data) return fail(c, DMRG3S_ERR_ARG, "NULL device data");
     st = env_plan(c, dir, e, w, a, o, &p);
     if (st != DMRG3S_OK) return st;
-    remember_plan(c, key, p);
+    remember(&c->by_args, key, p);
   }
   if (!env->data || !A->data || !out->data) return fail(c, DMRG3S_ERR_ARG, "NULL device data");
   if ((st = use_device(c)) || (st = need_form(c, *p, prec)) || (st = check_ws(c, p->host, prec))) return st;

@@ -253,6 +253,14 @@ struct RawKeyHash {
   size_t operator()(const RawKey& k) const { return (size_t)(k.a ^ (k.b << 1)); }
 };
 
+constexpr size_t kMaxArgs = 4096;
+template <class Map, class Plan>
+void remember(Map* m, const RawKey& key, const Plan* p) {
+  if (!key.ok) return;
+  if (m->size() >= kMaxArgs) m->clear();
+  (*m)[key] = p;
+}
+
 struct Context {
   Profiler prof;
   int device = 0;
@@ -269,7 +277,9 @@ struct Context {
   std::unordered_map<uint64_t, std::unique_ptr<DevicePlan>> plans;
   std::unordered_map<uint64_t, std::unique_ptr<DeviceGradPlan>> grad_plans;
   // plans by the raw arguments of the calls that use them (entries of `plans`,
-  // which live as long as the context; of `grad_plans`, dropped with them)
+  // which live as long as the context; of `grad_plans`, dropped with them).  At most
+  // kMaxArgs of each: the MPO's values are among the arguments, and a program that
+  // varies them makes a new entry with every call.
   std::unordered_map<RawKey, const DevicePlan*, RawKeyHash> by_args;
   std::unordered_map<RawKey, const DeviceGradPlan*, RawKeyHash> grad_by_args;
   std::string last_error;

@@ -106,7 +106,7 @@ extern "C" dmrg3s_status dmrg3s_mpo_grad_site(dmrg3s_ctx ctx, const dmrg3s_env* 
     if (!L->data || !R->data || !M->data) return fail(c, DMRG3S_ERR_ARG, "NULL device data pointer");
     if ((st = use_device(c))) return st;
     if ((st = grad_plan(c, le, w, re, m, &p))) return st;
-    if (key.ok) c->grad_by_args[key] = p;
+    remember(&c->grad_by_args, key, p);
   }
   if (!L->data || !R->data || !M->data) return fail(c, DMRG3S_ERR_ARG, "NULL device data pointer");
   if ((st = use_device(c))) return st;
