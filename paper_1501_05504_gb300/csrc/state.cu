@@ -531,9 +531,16 @@ void prepare_truncation(const SiteLayout& ml, int dir, bool expand, const FusedB
   // AUTO: the Jacobi SVD, since its QR and left vectors run in this library's
   // kernels.  Whole updates, gesvd against it (ms): XXZ FP64 m = 16 2.8 and 1.7, 128
   // 7.9 and 5.7, 512 39.9 and 14.2, 1024 97 and 52; 3xTF32 m = 64 3.5 and 2.3, 512 37.8
-  // and 12.6; Hubbard FP64 m = 128 9.3 and 3.9, 1024 97 and 24.  Eight sweeps of the
-  // L = 40 chain at m = 128, 3xTF32 (whose noise costs Jacobi sweeps): 3.3 and 1.5 s.
-  if (svd == DMRG3S_SVD_AUTO) svd = DMRG3S_SVD_JACOBI;
+  // and 12.6; Hubbard FP64 m = 128 9.3 and 3.9, 2048 262 and 87; cylinder m = 256 15.1 and
+  // 3.8, 2048 235 and 123; one sector of 256 74 and 31.  57 batched steps of 16 chains at m = 32
+  // 768 and 204, of 8 chains at m = 128 327 and 171.  Eight sweeps of the L = 40 chain at
+  // m = 128, 3xTF32 (whose noise costs Jacobi sweeps): 3.3 and 1.5 s.  Sectors beyond its
+  // limit go to gesvd.
+  if (svd == DMRG3S_SVD_AUTO) {
+    svd = DMRG3S_SVD_JACOBI;
+    for (const Sector& sc : secs)
+      if (sc.n > kJacobiMaxN) svd = DMRG3S_SVD_GESVD;
+  }
   t->method = svd;
   bool any_proj = svd == DMRG3S_SVD_JACOBI;
   for (const Sector& sc : secs) any_proj = any_proj || (sc.vt_only && sc.base > 0);
@@ -1140,10 +1147,11 @@ dmrg3s_status batch_truncate(Context* c, std::vector<BItem>& items, dmrg3s_svd_m
   int64_t nX = 0, nF = 0, nS = 0;
   size_t nsec = 0;
   bool any_proj = false;
-  if (method == DMRG3S_SVD_AUTO) method = DMRG3S_SVD_JACOBI;   // (prepare_truncation)
+  bool gesvd = false;              // (one method for all)
   for (BItem& it : items) {
     State& S = *it.S;
     prepare_truncation(S.M[S.centre].lay, it.dir, it.expand, it.fp, it.pl, method, &it.t);
+    gesvd = gesvd || it.t.method == DMRG3S_SVD_GESVD;
     it.xb = nX;
     it.fb = nF;
     it.sb = nS;
@@ -1153,6 +1161,7 @@ dmrg3s_status batch_truncate(Context* c, std::vector<BItem>& items, dmrg3s_svd_m
     nsec += it.t.secs.size();
     any_proj = any_proj || it.t.any_proj;
   }
+  method = gesvd ? DMRG3S_SVD_GESVD : DMRG3S_SVD_JACOBI;
   any_proj = any_proj || method == DMRG3S_SVD_JACOBI;
   Scratch scr(c, st);
   double *X, *F, *Sv, *dinfo_d, *X0 = nullptr;

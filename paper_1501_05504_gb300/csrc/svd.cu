@@ -897,7 +897,7 @@ dmrg3s_status svd_jacobi(Context* c, std::vector<SvdLane>& lanes, int nlanes,
   size_t smem = 0;
   for (int k = 0; k < nj; ++k) {
     const SvdJob& jb = jobs[k];
-    if (jb.n < 1 || jb.m < jb.n || jb.m > (1 << 30) || jb.n > (1 << 15))
+    if (jb.n < 1 || jb.m < jb.n || jb.m > (1 << 30) || jb.n > kJacobiMaxN)
       return fail(c, DMRG3S_ERR_ARG, "SVD matrix shape (need 1 <= n <= m, n <= 32768)");
     if (jb.offU >= 0 && !U) return fail(c, DMRG3S_ERR_ARG, "SVD left vectors without a buffer");
     JacJob& t = tab[k];

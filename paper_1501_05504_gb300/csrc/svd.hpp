@@ -48,6 +48,7 @@ struct SvdJob {
 // kJacobiMaxSweeps, fewer when the environment variable DMRG3S_JACOBI_SWEEPS
 // (1 .. kJacobiMaxSweeps) is set.
 constexpr int kJacobiMaxSweeps = 40;
+constexpr int64_t kJacobiMaxN = 32768;   // columns of a matrix
 int jacobi_max_sweeps();
 
 // Factorises every job; A is only read (the factorisation works on a copy).
