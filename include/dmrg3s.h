@@ -161,7 +161,7 @@ dmrg3s_status dmrg3s_set_wait_limit(dmrg3s_ctx ctx, double seconds);
  * truncation's S V^dagger products and the MPO-entry gradient), and around
  * each sweep of the truncation's Jacobi SVD (kernel 9: one record per sweep,
  * counting its launches: the sweep-counter kernel and one launch per round;
- * flops: 6n per column-pair test plus, per rotation, 6n (12n when the left
+ * flops: 2n per column-pair test plus, per rotation, 6n (12n when the left
  * vectors' rotations are accumulated too); bytes: 16n per pair test plus,
  * per rotation, 16n (48n with the left vectors)).
  * dmrg3s_profile(ctx, 1) resets and enables, 0 disables;

@@ -1163,7 +1163,7 @@ dmrg3s_status svd_jacobi(Context* c, std::vector<SvdLane>& lanes, int nlanes,
       break;
     }
     // algorithmic cost of the sweep: a pair test reads two columns (16n bytes)
-    // for three dot products (6n flops); a rotation of a column pair of Y and
+    // for a dot product (2n flops); a rotation of a column pair of Y and
     // of V1 takes 6n flops each and writes 16n bytes each (V1 also read)
     double fl = 0.0, by = 0.0;
     bool more = false;
@@ -1171,7 +1171,7 @@ dmrg3s_status svd_jacobi(Context* c, std::vector<SvdLane>& lanes, int nlanes,
       if (!active[k]) continue;
       const double n = tab[k].n, pairs = 0.5 * n * (n - 1.0);
       const bool v = tab[k].offV >= 0;
-      fl += pairs * 6.0 * n + hrot[k] * 6.0 * n * (v ? 2.0 : 1.0);
+      fl += pairs * 2.0 * n + hrot[k] * 6.0 * n * (v ? 2.0 : 1.0);
       by += pairs * 16.0 * n + hrot[k] * 16.0 * n * (v ? 3.0 : 1.0);
       if (hrot[k] == 0) {
         active[k] = 0;
