@@ -33,9 +33,10 @@ __device__ __forceinline__ double inverse_scale(double x) {
   return double_of(1.0f, 1023 - (e < 1 ? 1 : e > 2040 ? 2040 : e));
 }
 
-// 1 / x to about one unit in the last place (|x| within 2^+-1000): an FP32
-// reciprocal r0 of the mantissa, then 1 / x = r0 (1 + e + e^2 + ..) with e = 1 - x r0
-// below 2^-22.  Three dependent FP64 instructions.
+// 1 / x within one unit in the last place of the rounded value (|x| within
+// 2^+-1000): an FP32 reciprocal r0 of the mantissa, then the third-order Newton step
+// 1 / x = r0 (1 + e + e^2 + ..) with e = 1 - x r0 below 2^-21 (e^3 is left out, 2^-63; the
+// last multiply-add rounds once).  Three dependent FP64 instructions.
 __device__ __forceinline__ double recip(double x) {
   const int e = exponent_of(x);
   const double r0 = double_of(1.0f / float_of(x, e), 1023 - e);
@@ -43,9 +44,11 @@ __device__ __forceinline__ double recip(double x) {
   return fma(r0, fma(d, d, d), r0);
 }
 
-// sqrt(x) to about one unit in the last place (0 < x < 2^1000, normal): with x = m
-// 2^(2k), m in [1, 4), the FP32 rsqrt of m and Newton's coupled iteration for
-// sqrt(m) and 1 / (2 sqrt(m)).  Six dependent FP64 instructions.
+// sqrt(x) within one unit in the last place of the rounded value (0 < x < 2^1000,
+// normal): with x = m 2^(2k), m in [1, 4), the FP32 rsqrt of m and Goldschmidt's
+// coupled Newton iteration for g ~ sqrt(m) and h ~ 1 / (2 sqrt(m)), then Markstein's
+// correction g + h (m - g^2) (IBM J. Res. Dev. 34, 1990), which rounds once.  Six
+// dependent FP64 instructions.
 __device__ __forceinline__ double sqrt_of(double x) {
   const int e = exponent_of(x), k = (e - 1023) >> 1;
   const double m = __longlong_as_double(__double_as_longlong(x) - ((long long)(2 * k) << 52));
