@@ -30,8 +30,9 @@
 // inner rounds of kJacB disjoint pairs, one warp each (in round 0 all pairs of
 // the 2 kJacB columns, in the circle schedule); columns >= n are skipped.  One
 // launch runs a round of every matrix of the batch; one sweep (a launch per
-// round) is a CUDA graph.  A matrix with no rotation in a sweep is converged and
-// its CTAs exit at once in later sweeps.
+// round) is a CUDA graph.  A matrix with no rotation in a sweep is converged: in later
+// sweeps its CTAs exit after their loads (the loads do not wait for the count of the
+// sweep before, which would cost the CTAs still rotating a memory latency a round).
 #include <cuda_runtime.h>
 
 #include <algorithm>

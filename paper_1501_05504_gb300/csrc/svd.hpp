@@ -2,7 +2,8 @@
 // truncation step of the local update (Sec. IV A, Sec. V step 4).
 //
 // Each matrix A (m x n, m >= n), its columns ordered by descending norm
-// (A P), is factorised A P = Q R by cuSOLVER's Householder QR; R^T is then
+// (A P), is factorised A P = Q R by Householder reflections (qr_kernel; cuSOLVER's
+// for matrices that the SMs' shared memory does not hold); R^T is then
 // orthogonalised by the one-sided (Hestenes) Jacobi method in this library's
 // kernels, R^T V1 = W with orthogonal columns, which gives R^T = U1 S V1^T
 // (U1 = W S^-1) and
@@ -52,7 +53,7 @@ constexpr int64_t kJacobiMaxN = 32768;   // columns of a matrix
 int jacobi_max_sweeps();
 
 // Factorises every job; A is only read (the factorisation works on a copy).
-// `lanes[0 .. nlanes)` run the QR factorisations (and Q V1) concurrently
+// `lanes[0 .. nlanes)` run the QR factorisations left to cuSOLVER concurrently
 // after the work already queued on `st`; `st` waits for all results.
 // info[k] (host) = 0, or 1 when job k did not converge within the sweep
 // limit (its outputs are then invalid; *diag, when given, names the first

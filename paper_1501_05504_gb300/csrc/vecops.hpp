@@ -82,7 +82,7 @@ inline void lz_layout(const std::vector<std::pair<int64_t, int64_t>>& ranges, in
 
 // Device-counter form: the kernels below that take `kdev` (non-null) read the
 // iteration k from that device word instead of their k1 argument (k1 = k + 1),
-// so that one captured launch sequence serves every iteration.
+// which they also advance (lz_advance), so that every iteration's launches are the same.
 //
 // partial[b * kp + j] = <V_j, w> over chunk b, for j < k1 (V_j = V + j * ldv).
 void launch_lz_dots(const double* V, int64_t ldv, int k1, const double* w, const LzChunk* chunks,
