@@ -121,11 +121,12 @@ struct SlView {
   int64_t src;             // of the first k
   int32_t ld, R, trans, pad;
 };
-// Blocks with the same rows whose rows share scales: scales[e0 + r]; one CTA
-// of the slicing kernel per row group, from cta0 on.
+// Blocks with the same rows whose rows share scales: scales[e0 + r]; a CTA of the
+// slicing kernel per `per` row groups (1, 2, 4 or 8), from cta0 on.
 // `shift` raises the scales by that power of two: headroom of the integer sums.
 struct SlGroup {
-  int32_t R, R8, m0, nm, nt, e0, cta0, shift, which, pad;   // nt: chunks; which: its operand
+  int32_t R, R8, m0, nm, nt, e0, cta0, shift, which, per;   // nt: chunks; which: its operand
+  int32_t ctas() const { return (R8 + per - 1) / per; }
 };
 // Spans a unit may sum before the headroom has to grow (the levels of a span
 // stay below 2^58.1 in the 64-bit sum).
@@ -203,7 +204,7 @@ struct SlPiece {
   int64_t src, dst;
   int32_t ld, K, KC, trans, R, R8, e0, shift, tile0, d0;   // d0: as in SlMember (sign -1)
 };
-// Row scales and slices of every block of every group (a group has R8 CTAs from its
+// Row scales and slices of every block of every group (a group has ctas() CTAs from its
 // cta0 on; cta_group[c] = the group of CTA c).
 void launch_slice(const SlGroup* groups, const int32_t* cta_group, int nctas,
                   const SlMember* members, const SlOperands& ops, cudaStream_t st);

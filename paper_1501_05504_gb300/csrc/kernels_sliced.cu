@@ -684,11 +684,18 @@ __global__ void __launch_bounds__(kFixThreads, 4)
       const int f = scale_of(v, un.d0 >= 0 ? d[un.d0 + n0 + c] : 0);
       if (f) atomicMax(collect + un.em + (collect_cols ? n0 + c : row0 + r), f);
     };
+    // this lane's column of the mask, and how many elements it and those before it list
+    uint32_t word = 0;
+    int upto = 0;
     const auto listed = [&]() {
-      int n = 0;
+      word = lane < 16 ? mask[lane] : 0u;
+      upto = __popc(word);
 #pragma unroll
-      for (int c = 0; c < 16; ++c) n += __popc(mask[c]);
-      return n;
+      for (int o = 1; o < 16; o *= 2) {
+        const int v = __shfl_up_sync(0xffffffffu, upto, o);
+        if (lane >= o) upto += v;
+      }
+      return __shfl_sync(0xffffffffu, upto, 15);
     };
     int total = listed();
     if (total > kFixFew && !force) {
@@ -755,10 +762,10 @@ __global__ void __launch_bounds__(kFixThreads, 4)
     const int way = warp % ways;
     for (int e0 = 0; e0 < total; e0 += kFixWarps / ways) {
       const int e = e0 + warp / ways;
-      int c = 0, left = min(e, total - 1);
-      while (left >= __popc(mask[c])) left -= __popc(mask[c++]);
-      uint32_t bits = mask[c];
-      for (; left > 0; --left) bits &= bits - 1u;
+      const int at = min(e, total - 1);
+      const int c = __ffs(__ballot_sync(0xffffffffu, upto > at)) - 1;
+      uint32_t bits = __shfl_sync(0xffffffffu, word, c);
+      for (int left = at - (__shfl_sync(0xffffffffu, upto, c) - __popc(bits)); left > 0; --left) bits &= bits - 1u;
       const int r = __ffs(bits) - 1;
       const int64_t m = un.m0 + row0 + r, n = un.n0 + n0 + c;
       double acc = 0.0, rest = 0.0;
@@ -797,7 +804,8 @@ __global__ void __launch_bounds__(kFixThreads, 4)
 
 // ---- slicing -----------------------------------------------------------------------
 // One CTA per 8 rows of a scale group (the packed blocks that share row
-// scales): the largest exponent of every row over all blocks of the group,
+// scales; of several row groups where there are few chunks: with idle warps the
+// kernel was at 20 % of its issue rate, XXZ m = 512 operator 23 us): the largest exponent of every row over all blocks of the group,
 // then the slices.  A warp handles 8 rows x 64 k of one block at a time, lane l
 // k = 2 l and 2 l + 1 of every row, so that the reads of a row and the writes
 // of a slice's row are whole 128-byte lines; blocks stored with k as the slow
@@ -921,10 +929,15 @@ __device__ __forceinline__ void load_tile(const double* src, int64_t ld, int K, 
 // pair of k, 4 bytes of the swizzled 16-byte piece lane / 4 of every slice.
 __device__ __forceinline__ void store_row(uint16_t* base, int64_t slice, int r, double x0, double x1,
                                           const Coef& cf, int2 d, bool zero, int f, int lane) {
-  unsigned long long d0, d1;
-  const uint32_t t0 = digits(zero ? 0.0 : x0, cf, d.x, zero ? 0 : f, &d0);
-  const uint32_t t1 = digits(zero ? 0.0 : x1, cf, d.y, zero ? 0 : f, &d1);
   uint16_t* row = base + r * 64 + (((lane >> 2) ^ r) << 3) + 2 * (lane & 3);
+  if (zero) {                            // (the same for the whole warp)
+#pragma unroll
+    for (int i = 0; i < kSlices; ++i) *reinterpret_cast<uint32_t*>(row + i * slice) = 0u;
+    return;
+  }
+  unsigned long long d0, d1;
+  const uint32_t t0 = digits(x0, cf, d.x, f, &d0);
+  const uint32_t t1 = digits(x1, cf, d.y, f, &d1);
 #pragma unroll
   for (int i = 0; i < kSlices; ++i) {
     // digit + 256 in 0 .. 512: as FP16, 1024 + (digit + 256) has these bits
@@ -958,18 +971,21 @@ __global__ void __launch_bounds__(32 * kSliceWarps, 3)
                  const __grid_constant__ SlOperands ops) {
   grid_next();
   grid_wait();
-  __shared__ int smax[8];
+  __shared__ int smax[8 * 8];                        // of up to eight row groups
   __shared__ double tr[kSliceWarps * 8 * kTRow];
   const int cta = (int)blockIdx.x;
   const SlGroup gr = groups[cta_group[cta]];
   const SlOperand op = ops.op[gr.which];
   const SlMember* mem = members + gr.m0;
-  const int r0 = (cta - gr.cta0) * 8, nr = min(8, gr.R - r0);      // rows of this CTA (<= 0: padding)
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  // the warp's row group, and its place among the `nw` warps of that group
+  const int nw = kSliceWarps / gr.per, sub = warp / nw, wi = warp % nw;
+  const int r0 = ((cta - gr.cta0) * gr.per + sub) * 8, nr = min(8, gr.R - r0);   // (<= 0: padding)
+  int* gmax = smax + 8 * sub;
   for (int i = (int)(blockIdx.x * blockDim.x + threadIdx.x); i < ops.nclear; i += (int)(gridDim.x * blockDim.x))
     ops.clear[i] = 0;
   if (blockIdx.x == 0 && (int)threadIdx.x < ops.nfix) ops.fix[threadIdx.x] = 0;
-  if (threadIdx.x < 8) smax[threadIdx.x] = kMinField;
+  if (threadIdx.x < 64) smax[threadIdx.x] = kMinField;
   __syncthreads();
   auto load = [&](const SlMember& mb, int t, double (&x)[16]) {
     load_tile(op.src + mb.src + (mb.trans ? (int64_t)r0 : (int64_t)r0 * mb.ld), mb.ld, mb.K, mb.trans, nr,
@@ -991,8 +1007,8 @@ __global__ void __launch_bounds__(32 * kSliceWarps, 3)
 #pragma unroll
     for (int r = 0; r < 8; ++r) mx[r] = kMinField;
     // the warp's chunks, the last one first: the first stays in registers
-    const int last = gr.nt > warp ? warp + (gr.nt - 1 - warp) / kSliceWarps * kSliceWarps : -1;
-    for (int t = last; t >= 0; t -= kSliceWarps) {
+    const int last = gr.nt > wi ? wi + (gr.nt - 1 - wi) / nw * nw : -1;
+    for (int t = last; t >= 0; t -= nw) {
       const SlMember mb = mem[member_of(mem, gr.nm, t, lane)];
       const Coef cf = make_coef(mb.coef * op.scale);
       const int2 d = grading(mb, t);
@@ -1004,23 +1020,24 @@ __global__ void __launch_bounds__(32 * kSliceWarps, 3)
 #pragma unroll
     for (int r = 0; r < 8; ++r) {
       const int w = __reduce_max_sync(0xffffffffu, mx[r]);
-      if (lane == r && w != kMinField) atomicMax(&smax[r], w);
+      if (lane == r && w != kMinField) atomicMax(&gmax[r], w);
     }
   }
   __syncthreads();
-  if ((int)threadIdx.x < nr) {
-    const int v = smax[threadIdx.x];
-    op.scales[gr.e0 + r0 + threadIdx.x] = v == kMinField ? 0 : v == kSlSpecial ? v : v + kSlBias;
+  if (wi == 0 && lane < nr) {
+    const int v = gmax[lane];
+    op.scales[gr.e0 + r0 + lane] = v == kMinField ? 0 : v == kSlSpecial ? v : v + kSlBias;
   }
-  for (int t = warp; t < gr.nt; t += kSliceWarps) {
+  if (r0 >= 8 * gr.R8) return;
+  for (int t = wi; t < gr.nt; t += nw) {
     const SlMember mb = mem[member_of(mem, gr.nm, t, lane)];
     const Coef cf = make_coef(mb.coef * op.scale);
     const int2 d = grading(mb, t);
-    if (t != warp || nr <= 0) load(mb, t, x);
+    if (t != wi || nr <= 0) load(mb, t, x);
     uint16_t* base = op.out + mb.dst + ((int64_t)(t - mb.t0) * kSlices * gr.R8 + (r0 >> 3)) * kSlTile;
 #pragma unroll
     for (int r = 0; r < 8; ++r) {
-      const int f = smax[r];             // zero rows and rows with Inf or NaN have no digits
+      const int f = gmax[r];             // zero rows and rows with Inf or NaN have no digits
       store_row(base, (int64_t)gr.R8 * kSlTile, r, x[2 * r], x[2 * r + 1], cf, d,
                 f == kMinField || f == kSlSpecial, f + gr.shift, lane);
     }

@@ -107,8 +107,10 @@ void SliceTable::add(const std::vector<SlGroup>& g, const std::vector<SlMember>&
     q.which = which;
     q.m0 += m0;
     q.cta0 = at;
-    at += q.R8;
-    cta_group.insert(cta_group.end(), q.R8, (int32_t)groups.size());
+    // eight warps for one row group's chunks, or for two, four or eight groups with few
+    q.per = q.nt > 4 ? 1 : q.nt > 2 ? 2 : q.nt > 1 ? 4 : 8;
+    at += q.ctas();
+    cta_group.insert(cta_group.end(), q.ctas(), (int32_t)groups.size());
     groups.push_back(q);
   }
   members.insert(members.end(), m.begin(), m.end());

@@ -161,11 +161,12 @@ inline bool slice_table_ok(const SliceTable& t, std::string* err) {
             (int32_t)t.cta_group.size() == t.cta.back();
   for (const SlGroup& q : t.groups) {
     ok = ok && q.cta0 == at && q.which >= 0 && (size_t)q.which + 1 < t.cta.size() &&
-         q.cta0 >= t.cta[q.which] && q.cta0 + q.R8 <= t.cta[q.which + 1] && q.m0 >= 0 &&
+         q.cta0 >= t.cta[q.which] && (q.per == 1 || q.per == 2 || q.per == 4 || q.per == 8) &&
+         q.cta0 + q.ctas() <= t.cta[q.which + 1] && q.m0 >= 0 &&
          (size_t)q.m0 + q.nm <= t.members.size();
-    for (int32_t c = at; ok && c < at + q.R8; ++c)
+    for (int32_t c = at; ok && c < at + q.ctas(); ++c)
       ok = t.cta_group[c] == (int32_t)(&q - t.groups.data());
-    at += q.R8;
+    at += q.ctas();
   }
   if (!ok || at != t.cta.back()) {
     *err = "slicing table";
