@@ -111,3 +111,24 @@ def test_on_a_stream_behind_the_callers_kernel(b, prec):
         st.synchronize()
         assert torch.equal(out.data, ref)
     ctx.close()
+
+
+@pytest.mark.parametrize("prec", ["fp64", "tf32x3"])
+def test_captured_call_replays(b, prec):
+    """A structure planned before can be captured; the replays see the tensors' contents."""
+    p = Problem(b, *_bonds(b, DIMS, 1), seed=44)
+    ctx = b.dmrg3s_create(0, 1 << 30)
+    first = _apply(b, ctx, p, prec)
+    out = b.empty_site_like(p.qp, p.left, p.right)
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        b.dmrg3s_apply_heff(ctx, p.L, p.W, p.R, p.M, out, prec)
+    g.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(out.data, first)
+    p.M.data.mul_(-2.0)
+    g.replay()
+    torch.cuda.synchronize()
+    replayed = out.data.clone()
+    assert torch.equal(replayed, _apply(b, ctx, p, prec))
+    ctx.close()
