@@ -188,7 +188,8 @@ dmrg3s_status lanczos_batch(Context* c, const DevicePlan& heff, const double* Ld
   // of the m = 512 XXZ chain in 3xTF32; 72 us an iteration against 73 at m = 32,
   // where the host's share is largest).  In all, with the one-launch
   // orthogonalisation and the tridiagonal solve beside the product: 4745 -> 3469 us
-  // (3xTF32) and 5288 -> 4590 us (FP64).
+  // (3xTF32) and, with sliced products of seven slices, 5288 -> 4590 us (FP64; with
+  // eight and gradings 6400).
   // A stream with fewer SMs than chunks (of a green context, say) refuses the
   // cooperative launch: then the separate launches, which add in the same order.
   auto orthogonalise = [&]() {

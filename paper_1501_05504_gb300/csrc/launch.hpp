@@ -8,10 +8,10 @@
 // product slowed it).
 //
 // A product is itself chained only while it is short (kChainChunks k-chunks a
-// CTA, about 40 us): chained, the XXZ m = 512 operator takes 72 us instead of 75
-// and a sliced one of 10 Mflop 33 instead of 37, but the cylinder's products slow
-// down (environment 782 instead of 756 us, 3xTF32 operator by 2 %), whose launch
-// latency does not count.  Every kernel launched this way calls grid_wait()
+// CTA, about 40 us): chained, the XXZ m = 512 operator in 3xTF32 takes 37.6 us instead of
+// 43.0, the Hubbard m = 1024 one in FP64 113 instead of 117 and the FP64 eigensolver 6.38 ms
+// instead of 6.48 (an expansion 66 instead of 63), but the cylinder's products slow
+// down (environment 991 instead of 917 us), whose launch latency does not count.  Every kernel launched this way calls grid_wait()
 // before its first access to global memory, whatever the data: the chain stays
 // ordered as plain launches would be.  Pointers that a predecessor may write
 // through are not declared __restrict__: a load from a const __restrict__

@@ -965,7 +965,7 @@ double tile_fill(const GemmStage& g, const GemmStage* h) {
   return tiles > 0.0 ? work / tiles : 0.0;
 }
 // Largest ratio of the fused stage's work to stage 1's: the sliced products
-// run 3 (0.2 Gflop) to 16 (13 Gflop) times as fast as the plain ones; a model
+// run 2 (0.2 Gflop) to 13 (13 Gflop) times as fast as the plain ones; a model
 // MPO has a ratio near 1.2.  Below it, the least work grows with the ratio.
 constexpr double kSlicedMaxTerms = 6.0;
 
