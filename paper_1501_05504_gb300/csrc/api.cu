@@ -97,7 +97,10 @@ dmrg3s_status upload(void** mem, Walk walk) {
   *mem = t.mem;
   t.staging.assign(t.total, 0);
   walk(t);
-  return cudaMemcpy(t.mem, t.staging.data(), t.total, cudaMemcpyHostToDevice) == cudaSuccess
+  // a copy from pageable memory returns when its source is staged, and the caller's
+  // stream need not wait for the default stream: the copy has to be complete
+  return cudaMemcpy(t.mem, t.staging.data(), t.total, cudaMemcpyHostToDevice) == cudaSuccess &&
+                 cudaStreamSynchronize(cudaStreamLegacy) == cudaSuccess
              ? DMRG3S_OK
              : DMRG3S_ERR_CUDA;
 }
@@ -573,7 +576,8 @@ dmrg3s_status dmrg3s_create(dmrg3s_ctx* ctx, int device, size_t workspace_bytes)
     cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &thr);
   }
   if (cudaMalloc(&c->d_err, sizeof(int)) != cudaSuccess ||
-      cudaMemset(c->d_err, 0, sizeof(int)) != cudaSuccess) {
+      cudaMemset(c->d_err, 0, sizeof(int)) != cudaSuccess ||
+      cudaStreamSynchronize(cudaStreamLegacy) != cudaSuccess) {
     cudaFree(c->ws);
     delete c;
     return DMRG3S_ERR_CUDA;

@@ -11,12 +11,12 @@
 // CTA, about 40 us): chained, the XXZ m = 512 operator in 3xTF32 takes 37.6 us instead of
 // 43.0, the Hubbard m = 1024 one in FP64 113 instead of 117 and the FP64 eigensolver 6.38 ms
 // instead of 6.48 (an expansion 66 instead of 63), but the cylinder's products slow
-// down (environment 991 instead of 917 us), whose launch latency does not count.  Every kernel launched this way calls grid_wait()
-// before its first access to global memory, whatever the data: the chain stays
-// ordered as plain launches would be.  Pointers that a predecessor may write
-// through are not declared __restrict__: a load from a const __restrict__
-// pointer counts as invariant for the whole kernel, and the compiler may move
-// it before the wait.
+// down (environment 991 instead of 917 us), whose launch latency does not count.  Every
+// kernel launched this way calls grid_wait() before its first access to global
+// memory, whatever the data: the chain stays ordered as plain launches would be.
+// Pointers that a predecessor may write through are not declared __restrict__: a
+// load from a const __restrict__ pointer counts as invariant for the whole kernel,
+// and the compiler may move it before the wait.
 #pragma once
 
 #include <cuda_runtime.h>

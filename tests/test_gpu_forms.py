@@ -132,3 +132,22 @@ def test_captured_call_replays(b, prec):
     replayed = out.data.clone()
     assert torch.equal(replayed, _apply(b, ctx, p, prec))
     ctx.close()
+
+
+@pytest.mark.parametrize("call", ("heff", "expand+", "env-"))
+def test_first_call_on_a_stream_of_its_own(b, call):
+    """The plan's tables are on the device before a stream that does not wait for the
+    default stream reads them: first calls on new structures, one after the other."""
+    st = torch.cuda.Stream()
+    for k in range(12):
+        dims = (120 + k, 127, 129 - k, 16)
+        p = Problem(b, *_bonds(b, dims, 1), seed=45)
+        torch.cuda.synchronize()
+        ref_ctx, ctx = b.dmrg3s_create(0, 1 << 29), b.dmrg3s_create(0, 1 << 29)
+        p.run(ref_ctx, call)
+        ref = p.run(ref_ctx, call)                # (tables long in place)
+        with torch.cuda.stream(st):
+            got = p.run(ctx, call)
+        assert torch.equal(got, ref)
+        ctx.close()
+        ref_ctx.close()
