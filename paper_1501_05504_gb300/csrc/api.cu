@@ -191,8 +191,8 @@ dmrg3s_status need_form(Context* c, const DevicePlan& plan, dmrg3s_precision pre
 }
 
 namespace {
-SlSource source(const GemmStage& g, const double* A, const double* B, double scale) {
-  return SlSource{A, B, A, B, g.ta == Trans::T ? 1 : 0, g.tb == Trans::T ? 1 : 0, scale};
+SlSource source(const GemmStage& g, const double* A, const double* B, double scale, int sign) {
+  return SlSource{A, B, A, B, g.ta == Trans::T ? 1 : 0, g.tb == Trans::T ? 1 : 0, scale, sign, 0};
 }
 
 // FP64 by exact FP16 slices (kernels_sliced.cu): slice the operands, stages
@@ -231,7 +231,7 @@ dmrg3s_status run_sliced(Context* c, const DevicePlan& p, const double* g1A, con
   launch_slice(p.sl_groups, p.sl_cta_group, h.slices.cta.back(), p.sl_members, ops, st);
   if (!h.s12.units.empty()) {
     const int id = pr.on ? pr.begin(kProfGemm, h.f12.flops, h.f12.bytes, st) : -1;
-    launch_gemm_sliced(sliced_tables(p.s12, h.s12), pk(sl.a1), pk(sl.b1), e1A, e1B, source(h.f12, g1A, g1B, scale), t2, et2,
+    launch_gemm_sliced(sliced_tables(p.s12, h.s12), pk(sl.a1), pk(sl.b1), e1A, e1B, source(h.f12, g1A, g1B, scale, left ? 1 : -1), t2, et2,
                        h.kind == Kind::EnvLR, d, sl_fix(fix, 0, 2, fix_units), c->d_err, c->wait_ns, st);
     if (id >= 0) pr.end(id, st);
   }
@@ -244,7 +244,7 @@ dmrg3s_status run_sliced(Context* c, const DevicePlan& p, const double* g1A, con
     double* c3 = split ? base + sl.p3 : g3C;
     if (!h.s3.units.empty()) {
       const int id = pr.on ? pr.begin(kProfGemm, h.g3.flops, h.g3.bytes, st) : -1;
-      launch_gemm_sliced(sliced_tables(p.s3, h.s3), pk(sl.a3), pk(sl.b3), e3A, e3B, source(h.f3, a3, b3, 1.0), c3, nullptr, false, d,
+      launch_gemm_sliced(sliced_tables(p.s3, h.s3), pk(sl.a3), pk(sl.b3), e3A, e3B, source(h.f3, a3, b3, 1.0, -1), c3, nullptr, false, d,
                          sl_fix(fix, 1, 2, fix_units), c->d_err, c->wait_ns, st);
       if (id >= 0) pr.end(id, st);
     }

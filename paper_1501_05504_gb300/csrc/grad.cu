@@ -48,7 +48,7 @@ dmrg3s_status run_mpo_grad(Context* c, const DeviceGradPlan& dp, const double* L
     ops.nfix = 1;
     launch_slice(dp.sl_groups, dp.sl_cta_group, p.slices.cta.back(), dp.sl_members, ops, st);
     const int id = pr.on ? pr.begin(kProfAuxGemm, p.g1.flops + p.gy.flops, p.g1.bytes + p.gy.bytes, st) : -1;
-    launch_gemm_sliced(sliced_tables(dp.s, p.s), pA, pB, eA, eB, SlSource{L, M, M, R, 0, 0, 1.0}, ws1,
+    launch_gemm_sliced(sliced_tables(dp.s, p.s), pA, pB, eA, eB, SlSource{L, M, M, R, 0, 0, 1.0, 0, 0}, ws1,
                        nullptr, false, nullptr, sl_fix(ops.fix, 0, 1, p.s.units.size()), c->d_err, c->wait_ns, st);
     if (id >= 0) pr.end(id, st);
   } else {

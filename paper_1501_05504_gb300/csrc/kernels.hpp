@@ -131,12 +131,12 @@ struct SlGroup {
 // Spans a unit may sum before the headroom has to grow (the levels of a span
 // stay below 2^58.1 in the 64-bit sum).
 constexpr int kSlSpans = 28;
-// One K-segment of a task where its FP64 operands are (read for rows with Inf
-// or NaN only); GemmTask / GemmSeg order.
+// One K-segment of a task where its FP64 operands are (read for listed elements
+// only), and the first entry of its grading or -1; GemmTask / GemmSeg order.
 struct SlSeg {
   int64_t offA, offB;
   double scale;
-  int32_t lda, ldb, K, pad;
+  int32_t lda, ldb, K, d0;
 };
 // One output tile of up to 128 rows x tile_n columns (rows and cols: what lies
 // inside the block), written at C + offC with leading dimension ldc; row scales
@@ -234,6 +234,7 @@ struct SlSource {
   const double *A, *B, *A1, *B1;     // A1, B1: of the units with sel = 1
   int32_t ta, tb;                    // stored transposed (as in launch_gemm_f64)
   double scale;
+  int32_t sign, pad;                 // of A's grading (SlOperand.sign); B has the other one
 };
 // d: the gradings (SlUnit.d0; the scales of column c are collected as those of the
 // elements times 2^-d).  fix (its count cleared before): receives the elements to form from the FP64

@@ -633,18 +633,24 @@ __global__ void __launch_bounds__(kThreads, 1)
 // ---- listed elements ---------------------------------------------------------------
 // One CTA per listed part (32 rows x 16 columns) at a time.  More than a few elements:
 // a first pass forms S = sum |a| |b| of the whole part relative to the scales, on the
-// FP32 pipe (truncated operands: a lower bound to K 2^-24), and those whose S reaches
-// the bound are done.  The others are formed by a warp each, or by several, its lanes
-// over k.  Empty lists cost the launch.
+// FP32 pipe (truncated operands: a lower bound to K 2^-24, what is below 2^-60 of a
+// scale taken as that); those whose S reaches the bound are done, and those whose S
+// is zero, since every product then has a factor zero.  The others are formed by a
+// warp each, or by several, its lanes over k, or, where they are many, by the part's
+// FP64 sums.  Empty lists cost the launch.  XXZ operator m = 512, plain form
+// 220 us: a site tensor log-uniform over 40 decades, nearly all elements formed, 695 us
+// with a warp an element alone and 461 so; one with 2 % of its elements not zero, 1187
+// and 615; one with normal elements 113 both ways.
 constexpr int kFixThreads = 256, kFixWarps = kFixThreads / 32;
-constexpr int kFixFew = 16;
+constexpr int kFixFew = 16, kFixMany = 96;
 constexpr int kFixK = 32;
 constexpr int kFixCtas = 4 * 152;
 
-// |x| / 2^(e - 1023) truncated (0 for a subnormal; Inf beyond the range)
+// |x| / 2^(e - 1023) truncated, at least 2^-60 unless zero; Inf beyond the range
 __device__ __forceinline__ float part_of(double x, int e) {
   const int f = exponent_of(x);
-  return f == 0 ? 0.f : f - e > 127 ? INFINITY : fabsf(float_of(x, e));
+  if ((__double_as_longlong(x) << 1) == 0ll) return 0.f;
+  return f == 0 || f - e < -60 ? 0x1p-60f : f - e > 127 ? INFINITY : fabsf(float_of(x, e));
 }
 
 // acc + a b, with what its roundings leave added to lo (Ogita, Rump and Oishi, 2005).
@@ -655,13 +661,81 @@ __device__ __forceinline__ double dot2(double a, double b, double acc, double& l
   return s;
 }
 
+// acc[h] = sum of the segments' products for row lane, column warp + 8 h of a part, or
+// (SIZE) of their magnitudes relative to the scales.
+template <bool SIZE, class T>
+__device__ __forceinline__ void part_sums(const SlUnit& un, const SlSeg* __restrict__ segs, const double* A,
+                                          const double* B, const SlSource& src, const int32_t* d, int row0,
+                                          int n0, const int* s_fa, const int* s_fb, T (*sa)[33], T (*sb)[16],
+                                          T (&acc)[2]) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  acc[0] = acc[1] = (T)0;
+  for (int g = 0; g < un.nseg; ++g) {
+    const SlSeg q = segs[un.seg0 + g];
+    const double cf = SIZE ? q.scale * src.scale : q.scale;
+    const int ce = exponent_of(cf);
+    // (a subnormal coefficient: no S, the elements are formed)
+    const T w = !SIZE ? (T)cf : cf == 0.0 ? (T)0 : ce == 0 ? (T)NAN : (T)part_of(cf, ce);
+    T part[2] = {(T)0, (T)0}, low[2] = {(T)0, (T)0};
+    for (int k0 = 0; k0 < q.K; k0 += kFixK) {
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const int e = tid + i * kFixThreads;
+        const int r = src.ta ? e & 31 : e >> 5, k = src.ta ? e >> 5 : e & 31;
+        double x = 0.0;
+        int dk = 0;
+        if (row0 + r < un.rows && k0 + k < q.K) {
+          const int64_t m = un.m0 + row0 + r, kk = k0 + k;
+          x = src.ta ? A[q.offA + kk * q.lda + m] : A[q.offA + m * q.lda + kk];
+          if (SIZE && q.d0 >= 0) dk = src.sign * d[q.d0 + kk];
+        }
+        sa[k][r] = SIZE ? (T)part_of(x, s_fa[r] - (ce - 1023) - dk) : (T)x;
+      }
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        const int e = tid + i * kFixThreads;
+        const int c = src.tb ? e >> 5 : e & 15, k = src.tb ? e & 31 : e >> 4;
+        double x = 0.0;
+        int dk = 0;
+        if (n0 + c < un.cols && k0 + k < q.K) {
+          const int64_t n = un.n0 + n0 + c, kk = k0 + k;
+          x = src.tb ? B[q.offB + n * q.ldb + kk] : B[q.offB + kk * q.ldb + n];
+          if (SIZE && q.d0 >= 0) dk = -src.sign * d[q.d0 + kk];
+        }
+        sb[k][c] = SIZE ? (T)part_of(x, s_fb[c] - dk) : (T)x;
+      }
+      __syncthreads();
+      // (columns beyond the segment are zero.)  The 32 terms in four sums, and their sum
+      // into the total with its rounding kept
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        T r[4] = {(T)0, (T)0, (T)0, (T)0};
+#pragma unroll
+        for (int k = 0; k < kFixK; ++k) r[k & 3] = fma(sa[k][lane], sb[k][warp + 8 * h], r[k & 3]);
+        const T t = (r[0] + r[1]) + (r[2] + r[3]), sum = part[h] + t, z = sum - part[h];
+        if (!SIZE) low[h] += (part[h] - (sum - z)) + (t - z);
+        part[h] = sum;
+      }
+      __syncthreads();
+    }
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      if (!SIZE && fabs(low[h]) < (T)1e308) part[h] += low[h];      // (Inf and NaN: the plain sum)
+      acc[h] = fma(w, part[h], acc[h]);
+    }
+  }
+}
+
 __global__ void __launch_bounds__(kFixThreads, 4)
     fix_kernel(const SlUnit* __restrict__ units, const SlSeg* __restrict__ segs, const SlFix fix,
                const int32_t* eA, const int32_t* eB, const __grid_constant__ SlSource src, double* C,
                int32_t* collect, int collect_cols, const int32_t* d) {
   grid_next();
   grid_wait();
-  __shared__ float sa[kFixK][33], sb[kFixK][16];
+  __shared__ union {
+    struct { double a[kFixK][33], b[kFixK][16]; } d;
+    struct { float a[kFixK][33], b[kFixK][16]; } f;
+  } tile;
   __shared__ uint32_t mask[16];
   __shared__ int s_fa[32], s_fb[16];
   __shared__ double s_sum[kFixWarps];
@@ -703,44 +777,8 @@ __global__ void __launch_bounds__(kFixThreads, 4)
       if (tid < 16) s_fb[tid] = n0 + tid < un.cols ? eB[un.eb + n0 + tid] + 1 - kSlBias : 0;
       if (warp == 1) s_fa[lane] = row0 + lane < un.rows ? eA[un.ea + row0 + lane] + un.shift + 1 - kSlBias : 0;
       __syncthreads();
-      float size[2] = {0.f, 0.f};
-      for (int g = 0; g < un.nseg; ++g) {
-        const SlSeg q = segs[un.seg0 + g];
-        const double cf = q.scale * src.scale;
-        const int ce = exponent_of(cf);
-        const float cm = part_of(cf, ce);
-        for (int k0 = 0; k0 < q.K; k0 += kFixK) {
-#pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            const int e = tid + i * kFixThreads;
-            const int r = src.ta ? e & 31 : e >> 5, k = src.ta ? e >> 5 : e & 31;
-            double x = 0.0;
-            if (row0 + r < un.rows && k0 + k < q.K) {
-              const int64_t m = un.m0 + row0 + r, kk = k0 + k;
-              x = src.ta ? A[q.offA + kk * q.lda + m] : A[q.offA + m * q.lda + kk];
-            }
-            sa[k][r] = part_of(x, s_fa[r] - (ce - 1023)) * cm;
-          }
-#pragma unroll
-          for (int i = 0; i < 2; ++i) {
-            const int e = tid + i * kFixThreads;
-            const int c = src.tb ? e >> 5 : e & 15, k = src.tb ? e & 31 : e >> 4;
-            double x = 0.0;
-            if (n0 + c < un.cols && k0 + k < q.K) {
-              const int64_t n = un.n0 + n0 + c, kk = k0 + k;
-              x = src.tb ? B[q.offB + n * q.ldb + kk] : B[q.offB + kk * q.ldb + n];
-            }
-            sb[k][c] = part_of(x, s_fb[c]);
-          }
-          __syncthreads();
-#pragma unroll 4
-          for (int k = 0; k < kFixK; ++k) {
-            size[0] = fmaf(sa[k][lane], sb[k][warp], size[0]);
-            size[1] = fmaf(sa[k][lane], sb[k][warp + 8], size[1]);
-          }
-          __syncthreads();
-        }
-      }
+      float size[2];
+      part_sums<true, float>(un, segs, A, B, src, d, row0, n0, s_fa, s_fb, tile.f.a, tile.f.b, size);
       const float least = (float)un.least * 0x1p-20f;
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
@@ -748,7 +786,7 @@ __global__ void __launch_bounds__(kFixThreads, 4)
         const bool in = (mask[c] >> lane & 1u) != 0;
         // (rows and columns with Inf or NaN have no scale)
         const bool special = s_fa[lane] > kSlSpecial / 2 || s_fb[c] > kSlSpecial / 2;
-        const bool form = in && (special || !(size[h] >= least && size[h] < 1e30f));
+        const bool form = in && (special || !(size[h] == 0.f || (size[h] >= least && size[h] < 1e30f)));
         if (in && !form) keep(lane, c, Cp[(int64_t)lane * un.ldc + c]);
         const uint32_t left = __ballot_sync(0xffffffffu, form);
         __syncwarp();
@@ -756,6 +794,20 @@ __global__ void __launch_bounds__(kFixThreads, 4)
       }
       __syncthreads();
       total = listed();
+    }
+    if (total > kFixMany && !force) {
+      double sum[2];
+      part_sums<false, double>(un, segs, A, B, src, d, row0, n0, s_fa, s_fb, tile.d.a, tile.d.b, sum);
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int c = warp + 8 * h;
+        if (mask[c] >> lane & 1u) {
+          const double v = src.scale * sum[h];
+          Cp[(int64_t)lane * un.ldc + c] = v;
+          keep(lane, c, v);
+        }
+      }
+      continue;
     }
     // `ways` warps an element, each some of its segments
     const int ways = total > 4 ? 1 : total > 2 ? 2 : total > 1 ? 4 : 8;

@@ -670,7 +670,10 @@ bool build_sliced(const GemmStage& g, bool coefA, Plan* grade, bool of_a, const 
   std::vector<int32_t> ea, eb;
   a.layout(true, &s.gA, &s.mA, &s.nA, &s.neA, &ea);
   b.layout(false, &s.gB, &s.mB, &s.nB, &s.neB, &eb);
-  for (const GemmSeg& q : g.segs) s.segs.push_back(SlSeg{q.offA, q.offB, q.scale, q.lda, q.ldb, q.K, 0});
+  for (size_t k = 0; k < g.segs.size(); ++k) {
+    const GemmSeg& q = g.segs[k];
+    s.segs.push_back(SlSeg{q.offA, q.offB, q.scale, q.lda, q.ldb, q.K, a.blks[ia[k]].m.d0});
+  }
   // narrower units when the 64-wide ones leave SMs without work
   auto count = [&](int tn) {
     int64_t n = 0;

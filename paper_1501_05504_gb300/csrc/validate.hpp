@@ -206,6 +206,7 @@ inline bool sliced_ok(const GemmStage& g, const SlStage& s, int64_t nA, int64_t 
              (s.cta_unit.size() >= 2 && s.cta_unit.front() == 0 && s.cta_chunk.front() == 0 &&
               s.cta_unit.back() == (int32_t)s.units.size() &&
               s.cta_chunk.back() == (int32_t)s.chunks.size()));
+  for (const SlSeg& q : s.segs) ok = ok && q.d0 >= -1 && (q.d0 < 0 || (int64_t)q.d0 + q.K <= ngrade);
   for (const SlChunk& c : s.chunks) {
     ok = ok && c.ga >= 1 && c.ga <= 16 && c.gb >= 2 && c.gb <= 8 && c.gb % 2 == 0 && c.a >= 0 &&
          c.b >= 0 && c.sa >= c.ga * kSlTile && c.sb >= c.gb * kSlTile && c.a % kSlTile == 0 &&

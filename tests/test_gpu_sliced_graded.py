@@ -79,6 +79,24 @@ def test_componentwise_bound(b, call, decades):
     assert bool(((x - y).abs() <= n * 2.0 ** -53 * size).all())
 
 
+@pytest.mark.parametrize("kind", ("loguniform", "sparse"))
+@pytest.mark.parametrize("call", CALLS)
+def test_whole_parts_listed(b, call, kind):
+    """Elements over 40 decades without an order along any bond, and few that are not
+    zero: nearly every element of a part is listed, and formed or found to be zero."""
+    p = Problem(b, *_bonds(b, DIMS, 2), seed=34)
+    g = torch.Generator(device="cuda").manual_seed(7)
+    u = torch.rand(p.M.data.shape, dtype=torch.float64, device="cuda", generator=g)
+    p.M.data.mul_(10.0 ** (40 * u - 20) if kind == "loguniform" else (u < 0.02).double())
+    x, y, counts = _both(b, p, call)
+    assert counts[0] != counts[1]
+    q = Problem(b, p.left, p.right, W=np.abs(XXZ_W), seed=34)
+    q.L.data, q.R.data, q.M.data = p.L.data.abs(), p.R.data.abs(), p.M.data.abs()
+    _, size, _ = _both(b, q, call)
+    n = 257 + 4 + 2 * 5 * 257 + 4
+    assert bool(((x - y).abs() <= n * 2.0 ** -53 * size).all())
+
+
 def test_repeating_digits(b):
     """Data that repeat along k: every digit product has the same sign in all terms, so
     the lower levels' sums leave the range that FP32 holds exactly."""
